@@ -4,7 +4,7 @@
 //
 //   potrf  : one CTA factors the diagonal tile in shared memory and also forms
 //            inv(L_KK) and its transpose (kept for the panel solve and for the
-//            block triangular solves).
+//            block triangular solves); the FP32 tile's kernel is in k_potrf.cu.
 //   trsm   : panel tiles L_IK = A_IK inv(L_KK)^T as a small GEMM (in place).
 //   syrk   : CUDA-core trailing update C_IJ -= sum_k L_Ik L_Jk^T over a set of
 //            tiles (the tensor-core version lives in k_update_tc.cu).
@@ -172,247 +172,6 @@ __global__ void __launch_bounds__(512) k_potrf_diag(T* __restrict__ Z, T* __rest
       Y[r * TILE + c] = v;
       YT[c * TILE + r] = v;
     }
-  }
-}
-
-// ------------------------------------------------- blocked potrf (FP32)
-// The same factor and inverse for the FP32 factor, organised in 32 x 32
-// blocks of the tile held in shared memory (A: the tile becoming L; Y: inv(L);
-// row stride LDB = 132 floats so that rows are 16-byte aligned for float4
-// loads):
-//   for kb = 0..3 (o = 32 kb):
-//     warp 0 factors the diagonal block A[o:o+32, o:o+32] with lane l owning
-//       column l: lane c scales column c (1/sqrt of the pivot from rsqrtf)
-//       and publishes it in shared memory, the lanes to its right update
-//       their columns from it (broadcast float4 reads, no barrier beyond
-//       __syncwarp); then it inverts the block into the diagonal block of Y,
-//       lane l solving for column l of the identity right-looking in
-//       registers from the published columns;
-//     all warps: blocks below it, A_ib,kb <- A_ib,kb Yd_kb^T (panel solve);
-//     all warps: trailing blocks A_ib,jb -= A_ib,kb A_jb,kb^T (kb < jb <= ib).
-//   Off-diagonal blocks of Y by block diagonals d = ib - jb = 1, 2, 3:
-//     Y_ib,jb = -Yd_ib (sum_{kb=jb}^{ib-1} L_ib,kb Y_kb,jb).
-// The block products read four consecutive k per float4 (one shared-memory
-// wavefront serves the warp's broadcast operand).  A non-positive pivot
-// raises ST_NOTPD with its row (1-based, smallest wins) and is replaced by 1
-// so the kernel finishes without NaNs.
-constexpr int PB = 32;   // block edge
-constexpr int LDB = 132; // shared-memory row stride (floats), 16-byte aligned rows
-
-__device__ __forceinline__ float dot4(float4 a, float4 b, float acc) {
-  acc = fmaf(a.x, b.x, acc);
-  acc = fmaf(a.y, b.y, acc);
-  acc = fmaf(a.z, b.z, acc);
-  return fmaf(a.w, b.w, acc);
-}
-
-__global__ void __launch_bounds__(512, 1) k_potrf_blk(float* __restrict__ Z, float* __restrict__ Dinv,
-                                                      float* __restrict__ DinvT, int64_t K, DevStatus* st) {
-  extern __shared__ __align__(16) float psm[];
-  float* A = psm;                // [TILE][LDB]
-  float* Y = psm + TILE * LDB;   // [TILE][LDB]
-  __shared__ __align__(16) float colL[PB][PB];  // finished columns of the current diagonal block
-  __shared__ int skip;
-  const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
-  if (tid == 0) skip = (st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE)) != 0;  // set by earlier kernels
-  __syncthreads();
-  if (skip) return;  // uniform across the CTA
-  float* tile = Z + tri_index(K, K) * TILE_ELEMS;
-  for (int e = tid; e < TILE * TILE / 4; e += 512) {
-    const int r = e >> 5, c = (e & 31) * 4;
-    *reinterpret_cast<float4*>(A + r * LDB + c) = reinterpret_cast<const float4*>(tile)[e];
-  }
-  __syncthreads();
-
-  for (int kb = 0; kb < TILE / PB; ++kb) {
-    const int o = kb * PB;
-    if (w == 0) {
-      // lane l owns column l of the diagonal block: a[i] = A[o+i][o+l] (i >= l
-      // matter; entries above the diagonal are never read and stored as 0)
-      float a[PB];
-#pragma unroll
-      for (int i = 0; i < PB; ++i) a[i] = A[(o + i) * LDB + o + l];
-#pragma unroll
-      for (int c = 0; c < PB; ++c) {
-        // lane c: column c is final; scale it and publish it in colL[c]
-        if (l == c) {
-          const float piv = a[c];
-          const bool bad = !(piv > 0.f);
-          if (bad) {
-            atomicOr(&st->flags, ST_NOTPD);
-            atomicMin(&st->notpd_index, (int)(K * TILE + o + c + 1));
-          }
-          const float rs = bad ? 1.f : rsqrtf(piv);
-          a[c] = bad ? 1.f : piv * rs;
-#pragma unroll
-          for (int i = c + 1; i < PB; ++i) a[i] *= rs;
-#pragma unroll
-          for (int i = 0; i < PB; i += 4)
-            *reinterpret_cast<float4*>(&colL[c][i]) =
-                make_float4(i >= c ? a[i] : 0.f, i + 1 >= c ? a[i + 1] : 0.f, i + 2 >= c ? a[i + 2] : 0.f,
-                            i + 3 >= c ? a[i + 3] : 0.f);
-        }
-        __syncwarp();
-        // lanes l > c: A[i][l] -= L[i][c] L[l][c] (broadcast reads of column c)
-        if (l > c) {
-          const float llc = colL[c][l];
-#pragma unroll
-          for (int i4 = (c + 1) & ~3; i4 < PB; i4 += 4) {  // aligned float4 groups from row c+1
-            const float4 v = *reinterpret_cast<const float4*>(&colL[c][i4]);
-            const float lv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (i4 + q > c) a[i4 + q] -= lv[q] * llc;
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < PB; ++i) A[(o + i) * LDB + o + l] = i >= l ? a[i] : 0.f;
-      const float myinv = 1.f / colL[l][l];  // every lane its own pivot: one division per lane
-      // column l of inv(L_D), right-looking: once y_k is final (scaled by
-      // 1/L[k][k]), y_i -= L[i][k] y_k for i > k; L's column k is read from
-      // colL by broadcast, so the dependence chain is one multiply and one
-      // FMA per k
-      float y[PB];
-#pragma unroll
-      for (int i = 0; i < PB; ++i) y[i] = i == l ? 1.f : 0.f;
-#pragma unroll
-      for (int k = 0; k < PB; ++k) {
-        y[k] *= __shfl_sync(0xffffffffu, myinv, k);
-#pragma unroll
-        for (int i4 = (k + 1) & ~3; i4 < PB; i4 += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(&colL[k][i4]);
-          const float lv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (i4 + q > k) y[i4 + q] -= lv[q] * y[k];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < PB; ++i) Y[(o + i) * LDB + o + l] = y[i];
-      __syncwarp();  // colL is rewritten by the next block's factor
-    }
-    __syncthreads();
-    // panel solve of the blocks below: X[r][c] = sum_k A[r][o+k] Yd[c][k]
-    float xb[3][2];
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int ro = o + PB * (b + 1);
-      if (ro < TILE) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int r = ro + w + 16 * q;
-          float acc = 0.f;
-#pragma unroll
-          for (int k = 0; k < PB; k += 4)
-            acc = dot4(*reinterpret_cast<const float4*>(A + r * LDB + o + k),
-                       *reinterpret_cast<const float4*>(Y + (o + l) * LDB + o + k), acc);
-          xb[b][q] = acc;
-        }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int ro = o + PB * (b + 1);
-      if (ro < TILE) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) A[(ro + w + 16 * q) * LDB + o + l] = xb[b][q];
-      }
-    }
-    __syncthreads();
-    // trailing blocks
-    for (int ib = kb + 1; ib < TILE / PB; ++ib)
-      for (int jb = kb + 1; jb <= ib; ++jb) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int r = ib * PB + w + 16 * q, c = jb * PB + l;
-          float acc = 0.f;
-#pragma unroll
-          for (int k = 0; k < PB; k += 4)
-            acc = dot4(*reinterpret_cast<const float4*>(A + r * LDB + o + k),
-                       *reinterpret_cast<const float4*>(A + c * LDB + o + k), acc);
-          A[r * LDB + c] -= acc;
-        }
-      }
-    __syncthreads();
-  }
-
-  // off-diagonal blocks of Y = inv(L), one block diagonal at a time
-  for (int dd = 1; dd < TILE / PB; ++dd) {
-    float tv[3][2];
-#pragma unroll
-    for (int jb = 0; jb < 3; ++jb) {
-      const int ib = jb + dd;
-      if (ib < TILE / PB) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int r = ib * PB + w + 16 * q, c = jb * PB + l;
-          float acc = 0.f;
-          for (int kb = jb; kb < ib; ++kb) {
-#pragma unroll
-            for (int k = 0; k < PB; k += 4) {
-              const float4 lr = *reinterpret_cast<const float4*>(A + r * LDB + kb * PB + k);
-              const float* yc = Y + (kb * PB + k) * LDB + c;
-              acc = fmaf(lr.x, yc[0], acc);
-              acc = fmaf(lr.y, yc[LDB], acc);
-              acc = fmaf(lr.z, yc[2 * LDB], acc);
-              acc = fmaf(lr.w, yc[3 * LDB], acc);
-            }
-          }
-          tv[jb][q] = acc;
-        }
-      }
-    }
-#pragma unroll
-    for (int jb = 0; jb < 3; ++jb) {
-      const int ib = jb + dd;
-      if (ib < TILE / PB) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) Y[(ib * PB + w + 16 * q) * LDB + jb * PB + l] = tv[jb][q];
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int jb = 0; jb < 3; ++jb) {
-      const int ib = jb + dd;
-      if (ib < TILE / PB) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int r = ib * PB + w + 16 * q, c = jb * PB + l;
-          float acc = 0.f;
-#pragma unroll
-          for (int k = 0; k < PB; k += 4) {
-            const float4 yr = *reinterpret_cast<const float4*>(Y + r * LDB + ib * PB + k);
-            const float* tc = Y + (ib * PB + k) * LDB + c;
-            acc = fmaf(yr.x, tc[0], acc);
-            acc = fmaf(yr.y, tc[LDB], acc);
-            acc = fmaf(yr.z, tc[2 * LDB], acc);
-            acc = fmaf(yr.w, tc[3 * LDB], acc);
-          }
-          tv[jb][q] = -acc;
-        }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int jb = 0; jb < 3; ++jb) {
-      const int ib = jb + dd;
-      if (ib < TILE / PB) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) Y[(ib * PB + w + 16 * q) * LDB + jb * PB + l] = tv[jb][q];
-      }
-    }
-    __syncthreads();
-  }
-
-  float* Yg = Dinv + K * TILE_ELEMS;
-  float* YTg = DinvT + K * TILE_ELEMS;
-  for (int e = tid; e < TILE * TILE; e += 512) {
-    const int r = e >> 7, c = e & 127;
-    tile[e] = c <= r ? A[r * LDB + c] : 0.f;
-    Yg[e] = c <= r ? Y[r * LDB + c] : 0.f;
-    YTg[e] = r <= c ? Y[c * LDB + r] : 0.f;
   }
 }
 
@@ -653,10 +412,7 @@ cudaError_t launch_potrf_diag(T* Z, T* Dinv, int64_t K, int64_t n, DevStatus* st
   const int64_t N = (n + TILE - 1) / TILE;
   // Dinv holds N tiles of inv(L_KK) followed by N tiles of inv(L_KK)^T.
   if constexpr (sizeof(T) == 4) {
-    const size_t smem = (size_t)2 * TILE * LDB * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_potrf_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_potrf_blk<<<1, 512, smem, s>>>(Z, Dinv, Dinv + N * TILE_ELEMS, K, st);
+    return launch_potrf_f32(Z, Dinv, Dinv + N * TILE_ELEMS, K, st, s);
   } else {
     const size_t smem = (size_t)TILE * LDA * sizeof(T);
     cudaError_t e = cudaFuncSetAttribute(k_potrf_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -156,6 +156,9 @@ cudaError_t launch_rowsum_max(const double* rowsum, int64_t n, DevStatus* st, cu
 // K2: blocked right-looking Cholesky pieces (T = float or double).
 template <typename T>
 cudaError_t launch_potrf_diag(T* Z, T* Dinv, int64_t K, int64_t n, DevStatus* st, cudaStream_t s);
+// The FP32 diagonal tile (k_potrf.cu): L in place, inv(L_KK) into tile K of
+// Dinv, its transpose into tile K of DinvT.
+cudaError_t launch_potrf_f32(float* Z, float* Dinv, float* DinvT, int64_t K, DevStatus* st, cudaStream_t s);
 // Panel solve: tiles (I, K) for I in [K+1, N): A_IK <- A_IK inv(L_KK)^T.
 template <typename T>
 cudaError_t launch_trsm_col(T* Z, const T* Dinv, int64_t K, int64_t N, DevStatus* st,

@@ -1,0 +1,73 @@
+"""Kernels against plain FP64 arithmetic at the sizes where their tiling can go
+wrong (edges of the 128-row tile and of its 32-column panels, remainders, the
+smallest and the largest sizes)."""
+import numpy as np
+import pytest
+import torch
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+M = pytest.importorskip("paper_2607_23354_gb300")
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return M.Context()
+
+
+def _dev(X):
+    return torch.from_numpy(np.ascontiguousarray(X)).cuda()
+
+
+def _z(X, t):
+    d = torch.cdist(X, X, compute_mode="donot_use_mm_for_euclid_dist")
+    return torch.exp(-t * d)
+
+
+# The diagonal tile's factor, by the Cholesky backward error |Z - L L^T| <=
+# (n + 1) u |L| |L^T| (Higham, Accuracy and Stability of Numerical Algorithms,
+# Theorem 10.3; the diagonal of |L| |L^T| is Z's, so every entry of it is at
+# most 1) with u = 2^-23 for the split products, plus 4 u for the FP32 entries
+# of Z and the reciprocal square roots.
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 64, 97, 127, 128])
+@pytest.mark.parametrize("prec", ["fp32", "fp16x3"])
+def test_diagonal_tile_factor(ctx, n, prec):
+    X = _dev(workloads.unit_cube_cloud(n=n, m=5, seed=n))
+    t = 1.5
+    L = ctx.cholesky_factor(X, t, prec).double()
+    Z = _z(X, t)
+    u = 2.0 ** -23
+    assert float((L @ L.T - Z).abs().max()) <= (n + 5) * u
+    assert bool((torch.triu(L, 1) == 0).all())
+
+
+# A solve within one tile uses the factor and its inverse in both sweeps.
+@pytest.mark.parametrize("n", [2, 5, 63, 96, 128, 129, 161])
+def test_small_solves(ctx, n):
+    X = _dev(workloads.unit_cube_cloud(n=n, m=4, seed=100 + n))
+    t = 2.0
+    w, mag, info = ctx.solve(X, t)
+    Z = _z(X, t)
+    r = 1.0 - Z @ w
+    assert info["fallback"] == 0
+    assert float(r.abs().max()) <= 1e-14 * float(Z.sum(1).max()) * float(w.abs().max())
+    assert abs(mag - float(w.sum())) <= 1e-13 * abs(mag)
+
+
+# A pivot that is exactly zero in FP32, in any place of a pivot block and in
+# any panel: points far apart (every other entry below e^-15, its square below
+# half a unit in the last place of 1) but for one pair 1e-13 apart, whose entry
+# rounds to 1.
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 30, 33, 66, 127])
+def test_zero_pivot_is_reported_with_its_row(ctx, p):
+    X = np.zeros((128, 2))
+    X[:, 0] = 16.0 * np.arange(128)
+    X[p] = X[p - 1] + [0.0, 1e-13]
+    with pytest.raises(M.MagnitudeError) as e:
+        ctx.cholesky_factor(_dev(X), 1.0, "fp32")
+    assert e.value.status == M.MAG_ENOTPD
+    assert f"row {p} " in str(e.value)
