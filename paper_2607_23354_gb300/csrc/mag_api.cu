@@ -1107,7 +1107,13 @@ int mag_min_distance(mag_ctx* ctx, const double* points, int64_t n, int32_t m, d
   // Only the status block and vectors are needed; reuse whatever layout fits.
   if (!ctx->ws || ctx->lay.np < ((n + TILE - 1) / TILE) * TILE) TRY(ensure_workspace(ctx, n, false, false));
   TRY(reset_status(ctx));
-  CU(launch_min_distance(points, n, m, ctx->st(), ctx->stream));
+  // the quantized coordinates' buffer holds the FP32 copy of the points; with
+  // no memory for it, FP64 differences for every pair
+  ctx->xq_ok = false;
+  if (grow_buffer(ctx, &ctx->xq, &ctx->xq_bytes, min_distance_scratch_bytes(n, m), 0))
+    CU(launch_min_distance_filtered(points, n, m, ctx->xq, ctx->st(), ctx->stream));
+  else
+    CU(launch_min_distance(points, n, m, ctx->st(), ctx->stream));
   TRY(read_status(ctx));
   const int fl = ctx->h_st->flags;
   const double d2 = bits_to_double(ctx->h_st->min_d2_bits);

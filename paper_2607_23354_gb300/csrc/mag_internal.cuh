@@ -150,6 +150,12 @@ cudaError_t launch_generate_from_dist(const double* Dd, int64_t n, double t, int
 cudaError_t launch_far_from_first(const double* X, int64_t n, int m, DevStatus* st, cudaStream_t s);
 // min_{j != k} d^2 over all pairs (FP64) into st->min_d2_bits.
 cudaError_t launch_min_distance(const double* X, int64_t n, int m, DevStatus* st, cudaStream_t s);
+// The same minimum and flags from an FP32 comparison of all pairs and the FP64
+// evaluation of those that could hold the minimum (k_mindist.cu); scratch:
+// min_distance_scratch_bytes of device memory, 256-byte aligned.
+size_t min_distance_scratch_bytes(int64_t n, int m);
+cudaError_t launch_min_distance_filtered(const double* X, int64_t n, int m, void* scratch, DevStatus* st,
+                                         cudaStream_t s);
 // off-diagonal row-sum maximum (Gershgorin) from rowsum into st->off_max_bits.
 cudaError_t launch_rowsum_max(const double* rowsum, int64_t n, DevStatus* st, cudaStream_t s);
 

@@ -71,3 +71,60 @@ def test_zero_pivot_is_reported_with_its_row(ctx, p):
         ctx.cholesky_factor(_dev(X), 1.0, "fp32")
     assert e.value.status == M.MAG_ENOTPD
     assert f"row {p} " in str(e.value)
+
+
+def _clouds():
+    rng = np.random.default_rng(11)
+    far = rng.random((300, 3)) * 1e-9  # close pairs below FP32's resolution of the span
+    far[150:] += 1.0
+    grid = np.stack(np.meshgrid(np.arange(9), np.arange(8), np.arange(5)), -1).reshape(-1, 3).astype(float)
+    return {
+        "two points": np.array([[0.0, 1.0], [3.0, 5.0]]),
+        "one dimension": rng.random((129, 1)),
+        "ragged": rng.standard_normal((385, 7)),
+        "more dimensions than a chunk": rng.standard_normal((200, 70)),
+        "more dimensions than threads": rng.standard_normal((150, 300)),
+        "offset": rng.random((260, 4)) + 1e6,
+        "far clusters": far,
+        "lattice": grid,
+    }
+
+
+# The closest distance from FP32 comparisons is the FP64 one bit for bit: the
+# generator's own minimum (FP64 differences of every pair) of a solve near the
+# identity, where it cannot fail.
+@pytest.mark.parametrize("name", sorted(_clouds()))
+def test_min_distance_is_the_generators(ctx, name):
+    X = _clouds()[name]
+    dmin, bound = ctx.min_distance(_dev(X))
+    c = M.Context(M.Options(exact_distances=False, deflate=-1))
+    _, _, info = c.solve(_dev(X), 40.0 / dmin)
+    assert dmin == info["min_distance"]
+    assert bound == np.log(len(X) - 1) / dmin
+
+
+# Scaling the points by a power of two scales every step exactly, inside the
+# FP32 path's range of spans and beyond it (2^+-400).
+@pytest.mark.parametrize("k", [-430, -380, 380, 430])
+def test_min_distance_scales_exactly(ctx, k):
+    X = np.random.default_rng(5).random((140, 3))
+    assert ctx.min_distance(_dev(np.ldexp(X, k)))[0] == np.ldexp(ctx.min_distance(_dev(X))[0], k)
+
+
+def test_min_distance_errors(ctx):
+    X = np.random.default_rng(2).random((300, 5))
+    for bad, status in ((np.inf, M.MAG_EINVAL), (np.nan, M.MAG_EINVAL)):
+        Y = X.copy()
+        Y[299, 4] = bad
+        with pytest.raises(M.MagnitudeError) as e:
+            ctx.min_distance(_dev(Y))
+        assert e.value.status == status
+    for a, b in ((0, 1), (5, 299), (290, 299)):
+        Y = X.copy()
+        Y[a] = Y[b]
+        with pytest.raises(M.MagnitudeError) as e:
+            ctx.min_distance(_dev(Y))
+        assert e.value.status == M.MAG_EDUPLICATE
+    with pytest.raises(M.MagnitudeError) as e:  # every distance overflows
+        ctx.min_distance(_dev(X * 1e300))
+    assert e.value.status == M.MAG_EINVAL
