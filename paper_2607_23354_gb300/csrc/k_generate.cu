@@ -17,6 +17,7 @@
 // Side outputs, all fused: full row sums of Z (for ||Z||inf and the Gershgorin
 // bound used to choose the factor precision), min off-diagonal d^2 (the Sec. 1
 // bound), and flags for non-finite coordinates and coincident points.
+#include "mag_fx.cuh"
 #include "mag_internal.cuh"
 #include "mag_math.cuh"
 
@@ -194,17 +195,22 @@ __global__ void __launch_bounds__(GEN_THREADS, 1)
   }
 }
 
-// Z from stored FP64 distances (same layout): one CTA per lower tile, FP64
-// exp only, 16-byte reads and stores (lane l: columns 4 l .. 4 l + 3).
-// Tiles of the padding get the identity, as in k_generate.
-template <bool WF, bool WD>
+// Z from stored FP64 distances (same layout): one CTA per lower tile, the
+// exponential of mag_fx.cuh (EXP: Z = exp(-t d)) or FP64, 16-byte reads and
+// stores (lane l: columns 4 l .. 4 l + 3).  Tiles of the padding get the
+// identity, as in k_generate.
+template <bool WF, bool WD, bool EXP>
 __global__ void __launch_bounds__(256) k_generate_from_dist(const double* __restrict__ Dd, int64_t n, double t,
-                                                            float* __restrict__ Zf, double* __restrict__ Zd,
-                                                            double* __restrict__ rowsum, int kind, double dcut,
-                                                            double kc) {
-  __shared__ __align__(16) double exptab[EXPT_SMEM];
+                                                            FxScale sc, float* __restrict__ Zf,
+                                                            double* __restrict__ Zd, double* __restrict__ rowsum,
+                                                            int kind, double dcut, double kc) {
+  __shared__ __align__(16) double exptab[EXP ? 2 : 2 * EXPT_SIZE];
+  __shared__ fx_u64 fxtab[EXP ? FX_TABLE_SIZE : 2];
   __shared__ float colpart[8][TILE];
-  load_exp_table(exptab);
+  if (EXP)
+    load_fx_table(fxtab);
+  else
+    load_exp_table_d(exptab);
   __syncthreads();
   int64_t I, J;
   tri_coords((int64_t)blockIdx.x, &I, &J);
@@ -212,8 +218,9 @@ __global__ void __launch_bounds__(256) k_generate_from_dist(const double* __rest
   const int64_t off = tri_index(I, J) * TILE_ELEMS;
   const float tf = (float)t;
   const unsigned long long tiny_bits = (unsigned long long)__double_as_longlong(dcut);
-  // row/column partial sums in FP32 (a norm; the FP64 pipe is the limit)
+  // row/column partial sums in FP32 (a norm)
   float cs[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
   for (int i = 0; i < 16; ++i) {
     const int r = warp * 16 + i;
     const int64_t gr = I * TILE + r;
@@ -238,15 +245,14 @@ __global__ void __launch_bounds__(256) k_generate_from_dist(const double* __rest
         if (gr == gc && gr < n) rs += 1.0f;  // the diagonal counts in its row sum
       } else {
         const double d = dv[q];
-        if (WD && !kind && (unsigned long long)__double_as_longlong(d) > tiny_bits) {
+        const unsigned long long db = (unsigned long long)__double_as_longlong(d);
+        if (EXP && db > tiny_bits) {
           zf = exp_neg_tiny_td(tf, t, d);
           zd = f32_to_f64_nonneg(zf);
         } else {
-          zd = WD ? mat_entry(kind, t, kc, d, exptab) : 0.0;
-          zf = WD ? (kind == MAT_DEFLATED ? __double2float_rn(zd) : f64_to_f32_nonneg(zd))
-                  : (kind == MAT_EXP ? expf(-tf * (float)d)
-                                     : (kind == MAT_SHIFTED_DIST ? 1.0f - tf * (float)d
-                                                                 : fmaf((float)kc, expm1f(-tf * (float)d), 1.0f)));
+          zd = EXP ? __longlong_as_double((long long)fx_exp_neg_d(db, sc.kg, sc.g, fxtab))
+                   : mat_entry(kind, t, kc, d, exptab);
+          zf = !EXP && kind == MAT_DEFLATED ? __double2float_rn(zd) : f64_to_f32_nonneg(zd);
         }
         rs += zf;
         cs[q] += zf;
@@ -302,77 +308,28 @@ __global__ void k_rowsum_max(const double* __restrict__ rowsum, int64_t n, DevSt
   if ((threadIdx.x & 31) == 0) atomic_max_nonneg(&st->off_max_bits, fmax(v, 0.0));
 }
 
-// FP64 distances of the packed lower tiles from the quantized coordinates
-// (m <= GEN_MC; MQ8: m <= 8, a column's coordinates held in registers),
-// with min d^2 and the coincident-point flag as k_generate: one CTA per
-// tile, warp w on tile rows w + 16 i (i < 8), lane l on columns 32 q + l
-// (q < 4), each pair finished and stored on its own (a warp's store covers
-// 32 consecutive entries of a row).  Rows and columns of the padding get
-// d = 0 (the generator from distances gives them the identity by index).
-template <bool MQ8>
-__global__ void __launch_bounds__(GEN_THREADS, 1)
-    k_dist_q(const long long* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, QuantParams qp,
-             double* __restrict__ Dd, DevStatus* st) {
-  extern __shared__ double smem[];
-  long long* xr = reinterpret_cast<long long*>(smem);  // [TILE][GEN_MC] row points (broadcast reads)
-  long long* xc = xr + TILE * GEN_MC;                  // [GEN_MC][TILE] column points (conflict free)
-  __shared__ unsigned long long warpmin[GEN_THREADS / 32];
-  int64_t I, J;
-  tri_coords((int64_t)blockIdx.x, &I, &J);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t row0 = I * TILE, col0 = J * TILE;
-  const int mc = MQ8 ? 8 : m;  // MQ8: dimensions m .. 7 staged as zeros
-  for (int e = threadIdx.x; e < TILE * mc; e += GEN_THREADS) {
-    const int r = e / mc, l = e - r * mc;
-    const int64_t gr = row0 + r, gc = col0 + r;
-    xr[r * GEN_MC + l] = gr < n && l < m ? Xq[gr * m + l] : 0ll;
-    xc[l * TILE + r] = gc < n && l < m ? Xq[gc * m + l] : 0ll;
+// Pairs of quantized points that are too close for them (fx_close): d^2 from
+// the FP64 differences, as k_generate, with the coincident-point flag.
+__device__ __noinline__ double close_square(const double* __restrict__ X, int64_t gr, int64_t gc, int m, int* flags,
+                                            unsigned long long* mind2b) {
+  double v = 0.0;
+  for (int l = 0; l < m; ++l) {
+    const double diff = X[gr * m + l] - X[gc * m + l];
+    v = fma(diff, diff, v);
   }
-  __syncthreads();
-  const unsigned long long mask = (1ull << qp.L) - 1ull;
-  const unsigned long long tau2_bits = (unsigned long long)__double_as_longlong(qp.tau2);
-  const int64_t tile_off = tri_index(I, J) * TILE_ELEMS;
-  unsigned long long mind2b = 0x7ff0000000000000ull;  // +inf
-  int flags = 0;
-  for (int q = 0; q < 4; ++q) {
-    const int c = 32 * q + lane;
-    const int64_t gc = col0 + c;
-    long long cv[8];
-    if (MQ8) {
-#pragma unroll
-      for (int l = 0; l < 8; ++l) cv[l] = xc[l * TILE + c];
-    }
-#pragma unroll 4
-    for (int i = 0; i < 8; ++i) {
-      const int r = warp + 16 * i;
-      const int64_t gr = row0 + r;
-      const long long* xrow = xr + r * GEN_MC;
-      unsigned long long A = 0ull, Bx = 0ull, C = 0ull;
-      if (MQ8) {
-#pragma unroll
-        for (int l = 0; l < 8; ++l) q_accumulate(xrow[l], cv[l], mask, qp.L, A, Bx, C);
-      } else {
-        for (int l = 0; l < m; ++l) q_accumulate(xrow[l], xc[l * TILE + c], mask, qp.L, A, Bx, C);
-      }
-      double dd = 0.0;
-      if (gr < n && gc < n && gr != gc) {
-        double v = q128_to_f64(A, Bx, C, qp.L, qp.e);
-        unsigned long long vb = (unsigned long long)__double_as_longlong(v);
-        if (vb < tau2_bits) {
-          // close pair: the FP64 differences of the points, as k_generate
-          v = 0.0;
-          for (int l = 0; l < m; ++l) {
-            const double diff = X[gr * m + l] - X[gc * m + l];
-            v = fma(diff, diff, v);
-          }
-          vb = (unsigned long long)__double_as_longlong(v);
-        }
-        if (vb == 0ull) flags |= ST_DUPLICATE;
-        else mind2b = vb < mind2b ? vb : mind2b;
-        dd = sqrt_pos(v);
-      }
-      Dd[tile_off + (int64_t)r * TILE + c] = dd;
-    }
+  const unsigned long long vb = (unsigned long long)__double_as_longlong(v);
+  if (vb == 0ull) *flags |= ST_DUPLICATE;
+  else *mind2b = vb < *mind2b ? vb : *mind2b;
+  return v;
+}
+
+// A CTA's flags and min d^2 (mq: the least square of this thread's pairs that
+// were not close, h = ~0 if none) into the status.
+__device__ __forceinline__ void finish_min(unsigned long long mind2b, const FxSquare& mq, int e, int flags,
+                                           unsigned long long* warpmin, DevStatus* st) {
+  if (mq.h != ~0ull) {
+    const unsigned long long b = fx_square_bits(mq, e);
+    mind2b = b < mind2b ? b : mind2b;
   }
   if (flags) atomicOr(&st->flags, flags);
 #pragma unroll
@@ -380,108 +337,140 @@ __global__ void __launch_bounds__(GEN_THREADS, 1)
     const unsigned long long other = __shfl_xor_sync(0xffffffffu, mind2b, o);
     mind2b = other < mind2b ? other : mind2b;
   }
-  if (lane == 0) warpmin[warp] = mind2b;
+  if ((threadIdx.x & 31) == 0) warpmin[threadIdx.x >> 5] = mind2b;
   __syncthreads();
   if (threadIdx.x == 0) {
     unsigned long long v = warpmin[0];
-    for (int w = 1; w < GEN_THREADS / 32; ++w) v = warpmin[w] < v ? warpmin[w] : v;
+    for (int w = 1; w < FX_THREADS / 32; ++w) v = warpmin[w] < v ? warpmin[w] : v;
     if (v < 0x7ff0000000000000ull) atomicMin(&st->min_d2_bits, v);
   }
 }
 
-// k_generate with the pair distances from the quantized coordinates (the
-// exact integer d^2 of mag_math.cuh; pairs with d^2 < tau2 from the FP64
-// differences of X), row sums when rowsum is given: the same entries,
-// checks and outputs in one pass, each pair finished on its own (row
-// r = w + 16 i outer, column 4 l + q inner, so a thread still stores its
-// four entries of a row with 16-byte stores), tiles in the slab layout of
-// k_generate.  Used where no distances are kept (a single t, the slabs of
-// the out-of-core factor); a multi-t call keeps them with k_dist_q, then
-// k_generate_from_dist.
-template <bool WF, bool WD>
-__global__ void __launch_bounds__(GEN_THREADS, 1)
-    k_generate_q(const long long* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, QuantParams qp,
+// FP64 distances of the packed lower tiles from the quantized coordinates
+// (mag_fx.cuh; pairs too close for them from the FP64 differences of X), with
+// min d^2 and the coincident-point flag as k_generate: one CTA per tile.  Rows
+// and columns of the padding get d = 0 (the generator from distances gives
+// them the identity by index).
+template <int R>
+__global__ void __launch_bounds__(FX_THREADS, 2)
+    k_dist_q(const fx_coord* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, int qe,
+             double* __restrict__ Dd, DevStatus* st) {
+  extern __shared__ __align__(16) unsigned char gen_smem[];
+  __shared__ unsigned long long warpmin[FX_THREADS / 32];
+  int64_t I, J;
+  tri_coords((int64_t)blockIdx.x, &I, &J);
+  const int lane = threadIdx.x & 31;
+  const int64_t row0 = I * TILE, col0 = J * TILE;
+  const int64_t tile_off = tri_index(I, J) * TILE_ELEMS;
+  unsigned long long mind2b = 0x7ff0000000000000ull;  // +inf
+  FxSquare mq{~0ull, ~0ull};
+  int flags = 0;
+  fx_tile_pairs<R>(Xq, n, m, row0, col0, reinterpret_cast<fx_coord*>(gen_smem), [&](int r, FxSquare(&q)[4]) {
+    const int64_t gr = row0 + r;
+    double ddv[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int64_t gc = col0 + 4 * lane + c;
+      double dd = 0.0;
+      if (gr < n && gc < n && gr != gc) {
+        if (fx_close(q[c], m)) {
+          dd = sqrt_pos(close_square(X, gr, gc, m, &flags, &mind2b));
+        } else {
+          if (q[c].h < mq.h || (q[c].h == mq.h && q[c].l < mq.l)) mq = q[c];
+          const FxRoot rt = fx_root_start(q[c]);
+          dd = __longlong_as_double((long long)fx_dist_bits(fx_root(rt), rt.j, qe));
+        }
+      }
+      ddv[c] = dd;
+    }
+    const int64_t e = tile_off + (int64_t)r * TILE + 4 * lane;
+    *reinterpret_cast<double2*>(Dd + e) = make_double2(ddv[0], ddv[1]);
+    *reinterpret_cast<double2*>(Dd + e + 2) = make_double2(ddv[2], ddv[3]);
+  });
+  finish_min(mind2b, mq, qe, flags, warpmin, st);
+}
+
+// k_generate with the pair distances from the quantized coordinates and, for
+// Z = exp(-t d) (EXP), the exponential of mag_fx.cuh from the unrounded
+// distance: no FP64 operation but in the pairs too close for the quantized
+// coordinates.  The same entries, checks and outputs in one pass (row sums
+// when rowsum is given), tiles in the slab layout of k_generate.  Used where
+// no distances are kept (a single t, the slabs of the out-of-core factor); a
+// multi-t call keeps them with k_dist_q, then k_generate_from_dist.
+template <int R, bool WF, bool WD, bool EXP>
+__global__ void __launch_bounds__(FX_THREADS, 2)
+    k_generate_q(const fx_coord* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, FxScale sc,
                  double t, float* __restrict__ Zf, double* __restrict__ Zd, double* __restrict__ rowsum,
-                 DevStatus* st, int kind, double dcut, double kc, int64_t t0, int64_t W) {
-  extern __shared__ double smem[];
-  long long* xr = reinterpret_cast<long long*>(smem);  // [TILE][GEN_MC] row points (broadcast reads)
-  long long* xc = xr + TILE * GEN_MC;                  // [GEN_MC][TILE] column points (conflict free)
-  __shared__ double colpart[GEN_THREADS / 32][TILE];
-  __shared__ unsigned long long warpmin[GEN_THREADS / 32];
-  __shared__ __align__(16) double exptab[EXPT_SMEM];
-  if (WD) load_exp_table(exptab);
+                 DevStatus* st, int kind, float tiny, double kc, int64_t t0, int64_t W) {
+  extern __shared__ __align__(16) unsigned char gen_smem[];
+  __shared__ float colpart[FX_THREADS / 32][TILE];
+  __shared__ unsigned long long warpmin[FX_THREADS / 32];
+  __shared__ __align__(16) double exptab[EXP ? 2 : 2 * EXPT_SIZE];
+  __shared__ fx_u64 fxtab[EXP ? FX_TABLE_SIZE : 2];
+  if (EXP)
+    load_fx_table(fxtab);
+  else
+    load_exp_table_d(exptab);
   int64_t I, J;
   tile_coords((int64_t)blockIdx.x, W, &I, &J);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t row0 = (t0 + I) * TILE, col0 = (t0 + J) * TILE;
-  for (int e = threadIdx.x; e < TILE * m; e += GEN_THREADS) {
-    const int r = e / m, l = e - r * m;
-    const int64_t gr = row0 + r, gc = col0 + r;
-    xr[r * GEN_MC + l] = gr < n ? Xq[gr * m + l] : 0ll;
-    xc[l * TILE + 32 * (r & 3) + (r >> 2)] = gc < n ? Xq[gc * m + l] : 0ll;
-  }
-  __syncthreads();
-  const unsigned long long mask = (1ull << qp.L) - 1ull;
-  const unsigned long long tau2_bits = (unsigned long long)__double_as_longlong(qp.tau2);
   const int64_t tile_off = tile_index(I, J, W) * TILE_ELEMS;
   float cs[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   unsigned long long mind2b = 0x7ff0000000000000ull;  // +inf
+  FxSquare mq{~0ull, ~0ull};
   int flags = 0;
-  const float tf = (float)t;
-  const unsigned long long tiny_bits = (unsigned long long)__double_as_longlong(dcut);
-#pragma unroll 1
-  for (int i = 0; i < 8; ++i) {
-    const int r = warp + 16 * i;
+  fx_tile_pairs<R>(Xq, n, m, row0, col0, reinterpret_cast<fx_coord*>(gen_smem), [&](int r, FxSquare(&q)[4]) {
     const int64_t gr = row0 + r;
-    const long long* xrow = xr + r * GEN_MC;
     float rs = 0.0f;
     float zfv[4];
     double zdv[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int64_t gc = col0 + 4 * lane + q;
-      unsigned long long A = 0ull, Bx = 0ull, C = 0ull;
-      for (int l = 0; l < m; ++l) q_accumulate(xrow[l], xc[l * TILE + 32 * q + lane], mask, qp.L, A, Bx, C);
+    for (int c = 0; c < 4; ++c) {
+      const int64_t gc = col0 + 4 * lane + c;
       double zd = 0.0;
       float zf = 0.0f;
       if (gr >= n || gc >= n || gr == gc) {
         zd = (gr == gc) ? 1.0 : 0.0;
         zf = (float)zd;
       } else {
-        double v = q128_to_f64(A, Bx, C, qp.L, qp.e);
-        unsigned long long vb = (unsigned long long)__double_as_longlong(v);
-        if (vb < tau2_bits) {
-          v = 0.0;
-          for (int l = 0; l < m; ++l) {
-            const double diff = X[gr * m + l] - X[gc * m + l];
-            v = fma(diff, diff, v);
-          }
-          vb = (unsigned long long)__double_as_longlong(v);
-        }
-        if (vb == 0ull) flags |= ST_DUPLICATE;
-        else mind2b = vb < mind2b ? vb : mind2b;
-        if (WD) {
-          const double dd = sqrt_pos(v);
-          if (!kind && (unsigned long long)__double_as_longlong(dd) > tiny_bits) {
-            zf = exp_neg_tiny_td(tf, t, dd);
-            zd = f32_to_f64_nonneg(zf);
-          } else {
-            zd = mat_entry(kind, t, kc, dd, exptab);
-            if (WF) zf = kind == MAT_DEFLATED ? __double2float_rn(zd) : f64_to_f32_nonneg(zd);
+        fx_u64 s = 0, db = 0;
+        int j = 0;
+        bool done = false;
+        if (fx_close(q[c], m)) {
+          db = (fx_u64)__double_as_longlong(sqrt_pos(close_square(X, gr, gc, m, &flags, &mind2b)));
+          if (EXP) {
+            zd = __longlong_as_double((long long)fx_exp_neg_d(db, sc.kg, sc.g, fxtab));
+            done = true;
           }
         } else {
-          const float df = sqrtf(f64_to_f32_nonneg(v));
-          zf = kind == MAT_EXP ? expf(-tf * df)
-                               : (kind == MAT_SHIFTED_DIST ? 1.0f - tf * df
-                                                           : fmaf((float)kc, expm1f(-tf * df), 1.0f));
+          if (q[c].h < mq.h || (q[c].h == mq.h && q[c].l < mq.l)) mq = q[c];
+          const FxRoot rt = fx_root_start(q[c]);
+          // t d in FP32: beyond `tiny` the entry is evaluated on the FP32 pipe
+          const float td = fx_float(fx_bits(rt.sf) + ((uint32_t)(rt.j - 63) << 23)) * sc.t63;
+          if (EXP && td > tiny) {
+            zf = exp_neg_tiny_f(td);
+            zd = f32_to_f64_nonneg(zf);
+            done = true;
+          } else {
+            s = fx_root(rt);
+            j = rt.j;
+            if (EXP)
+              zd = __longlong_as_double((long long)fx_exp_neg(s, j - sc.e + sc.kg, sc.g, fxtab));
+            else
+              db = fx_dist_bits(s, j, sc.e);
+          }
         }
+        (void)done;
+        if (!EXP) zd = mat_entry(kind, t, kc, __longlong_as_double((long long)db), exptab);
+        if (WF || !WD) zf = !EXP && kind == MAT_DEFLATED ? __double2float_rn(zd) : f64_to_f32_nonneg(zd);
       }
-      zfv[q] = zf;
-      zdv[q] = zd;
+      zfv[c] = zf;
+      zdv[c] = zd;
       if (gr < n && gc < n) {
         const float zs = WF ? zf : (float)zd;
         rs += zs;
-        cs[q] += zs;
+        cs[c] += zs;
       }
     }
     const int64_t e = tile_off + (int64_t)r * TILE + 4 * lane;
@@ -491,83 +480,37 @@ __global__ void __launch_bounds__(GEN_THREADS, 1)
       *reinterpret_cast<double2*>(Zd + e + 2) = make_double2(zdv[2], zdv[3]);
     }
     // the row's sum: an FP32 lane tree, one FP64 atomic per row
+    if (rowsum) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
-    if (rowsum && lane == 0 && gr < n) atomicAdd(rowsum + gr, (double)rs);
-  }
-  if (flags) atomicOr(&st->flags, flags);
+      for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
+      if (lane == 0 && gr < n) atomicAdd(rowsum + gr, (double)rs);
+    }
+  });
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long other = __shfl_xor_sync(0xffffffffu, mind2b, o);
-    mind2b = other < mind2b ? other : mind2b;
-  }
-  if (lane == 0) warpmin[warp] = mind2b;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) colpart[warp][4 * lane + q] = (double)cs[q];
-  __syncthreads();
+  for (int c = 0; c < 4; ++c) colpart[warp][4 * lane + c] = cs[c];
+  finish_min(mind2b, mq, sc.e, flags, warpmin, st);  // synchronizes
   if (rowsum && I != J && threadIdx.x < TILE) {
     double v = 0.0;
-    for (int w = 0; w < GEN_THREADS / 32; ++w) v += colpart[w][threadIdx.x];
+    for (int w = 0; w < FX_THREADS / 32; ++w) v += (double)colpart[w][threadIdx.x];
     const int64_t gc = col0 + threadIdx.x;
     if (gc < n) atomicAdd(rowsum + gc, v);
-  }
-  if (threadIdx.x == 0) {
-    unsigned long long v = warpmin[0];
-    for (int w = 1; w < GEN_THREADS / 32; ++w) v = warpmin[w] < v ? warpmin[w] : v;
-    if (v < 0x7ff0000000000000ull) atomicMin(&st->min_d2_bits, v);
-  }
-}
-
-// Per dimension l < m (one CTA each): min and max of X[:, l] into
-// out[2 l], out[2 l + 1]; out[2 m] = 1 if a coordinate is not finite.
-__global__ void k_coord_range(const double* __restrict__ X, int64_t n, int m, double* __restrict__ out) {
-  const int l = blockIdx.x;
-  double lo = INFINITY, hi = -INFINITY;
-  int bad = 0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    const double v = X[i * m + l];
-    if (!isfinite(v)) bad = 1;
-    lo = fmin(lo, v);
-    hi = fmax(hi, v);
-  }
-  __shared__ double slo[32], shi[32];
-  __shared__ int sbad;
-  if (threadIdx.x == 0) sbad = 0;
-  __syncthreads();
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-  }
-  if (bad) atomicOr(&sbad, 1);
-  if ((threadIdx.x & 31) == 0) {
-    slo[threadIdx.x >> 5] = lo;
-    shi[threadIdx.x >> 5] = hi;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-      lo = fmin(lo, slo[w]);
-      hi = fmax(hi, shi[w]);
-    }
-    out[2 * l] = lo;
-    out[2 * l + 1] = hi;
-    if (sbad) out[2 * m] = 1.0;
   }
 }
 
 // q = round(2^e (x - lo_l)) with x - lo_l taken exactly as s + err (TwoSum):
-// round(2^e s) + round(2^e err), within one unit of 2^e (x - lo_l).
-__global__ void k_quantize(const double* __restrict__ X, int64_t n, int m, const double* __restrict__ range,
-                           int e, long long* __restrict__ Xq) {
+// round(2^e s) + round(2^e err), within one unit of 2^e (x - lo_l); stored as
+// its limbs.
+__global__ void k_quantize(const double* __restrict__ X, int64_t n, int m,
+                           const unsigned long long* __restrict__ range, int e, fx_coord* __restrict__ Xq) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n * m) return;
   const int l = (int)(k % m);
-  const double x = X[k], b = -range[2 * l];
+  const double x = X[k], b = -ordered_value(range[2 * l]);
   const double s = x + b;
   const double bv = s - x;
   const double err = (x - (s - bv)) + (b - bv);
-  Xq[k] = __double2ll_rn(ldexp(s, e)) + __double2ll_rn(ldexp(err, e));
+  const long long q = __double2ll_rn(ldexp(s, e)) + __double2ll_rn(ldexp(err, e));
+  Xq[k] = fx_coord{(int)(q & ((1ll << FX_LIMB) - 1)), (int)(q >> FX_LIMB)};
 }
 
 template <bool WF, bool WD, bool ROWSUM, bool WDIST = false>
@@ -613,87 +556,104 @@ cudaError_t launch_generate_dist(const double* X, int64_t n, int m, double t, in
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_generate_q(const long long* Xq, const double* X, int64_t n, int m, int L, int e, double tau2,
-                              double t, int64_t N, float* Zf, double* Zd, double* rowsum, DevStatus* st,
-                              cudaStream_t s, int kind, double tiny_arg, double kc, int64_t t0, int64_t W) {
-  if (m < 1 || m > GEN_MC) return cudaErrorInvalidValue;
-  const size_t smem = 2 * (size_t)TILE * GEN_MC * sizeof(long long);
-  const QuantParams qp{L, e, tau2};
+namespace {
+
+template <int R, bool WF, bool WD, bool EXP>
+cudaError_t launch_gen_q(const fx_coord* Xq, const double* X, int64_t n, int m, const FxScale& sc, double t,
+                         unsigned tiles, float* Zf, double* Zd, double* rowsum, DevStatus* st, cudaStream_t s,
+                         int kind, float tiny, double kc, int64_t t0, int64_t W) {
+  auto kern = k_generate_q<R, WF, WD, EXP>;
+  const size_t smem = fx_tile_smem(m);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<tiles, FX_THREADS, smem, s>>>(Xq, X, n, m, sc, t, Zf, Zd, rowsum, st, kind, tiny, kc, t0, W);
+  note_launch();
+  return cudaGetLastError();
+}
+
+template <int R, bool EXP>
+cudaError_t launch_gen_q_out(const fx_coord* Xq, const double* X, int64_t n, int m, const FxScale& sc, double t,
+                             unsigned tiles, float* Zf, double* Zd, double* rowsum, DevStatus* st, cudaStream_t s,
+                             int kind, float tiny, double kc, int64_t t0, int64_t W) {
+  if (Zf && Zd)
+    return launch_gen_q<R, true, true, EXP>(Xq, X, n, m, sc, t, tiles, Zf, Zd, rowsum, st, s, kind, tiny, kc, t0, W);
+  if (Zf)  // FP32 tiles alone: rounded from the FP64 entries
+    return launch_gen_q<R, true, false, EXP>(Xq, X, n, m, sc, t, tiles, Zf, Zd, rowsum, st, s, kind, INFINITY, kc, t0,
+                                             W);
+  if (Zd)
+    return launch_gen_q<R, false, true, EXP>(Xq, X, n, m, sc, t, tiles, Zf, Zd, rowsum, st, s, kind, tiny, kc, t0, W);
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+cudaError_t launch_generate_q(const void* Xq, const double* X, int64_t n, int m, int e, double t, int64_t N,
+                              float* Zf, double* Zd, double* rowsum, DevStatus* st, cudaStream_t s, int kind,
+                              double tiny_arg, double kc, int64_t t0, int64_t W) {
+  if (m < 1 || m > FX_MAX_DIM) return cudaErrorInvalidValue;
   // N: tile rows of the (slab) matrix from global tile t0; W < 0: all columns
   if (W < 0) W = N;
   const int64_t tiles = num_slab_tiles(N, W);
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-  const double dcut = tiny_arg / t;
-  cudaError_t err;
-  if (Zf && Zd) {
-    err = cudaFuncSetAttribute(k_generate_q<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    k_generate_q<true, true><<<(unsigned)tiles, GEN_THREADS, smem, s>>>(Xq, X, n, m, qp, t, Zf, Zd, rowsum, st,
-                                                                         kind, dcut, kc, t0, W);
-  } else if (Zf) {
-    err = cudaFuncSetAttribute(k_generate_q<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    k_generate_q<true, false><<<(unsigned)tiles, GEN_THREADS, smem, s>>>(Xq, X, n, m, qp, t, Zf, Zd, rowsum, st,
-                                                                          kind, INFINITY, kc, t0, W);
-  } else if (Zd) {
-    err = cudaFuncSetAttribute(k_generate_q<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    k_generate_q<false, true><<<(unsigned)tiles, GEN_THREADS, smem, s>>>(Xq, X, n, m, qp, t, Zf, Zd, rowsum, st,
-                                                                          kind, dcut, kc, t0, W);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  note_launch();
-  return cudaGetLastError();
+  const FxScale sc = fx_scale(t, e);
+  const fx_coord* q = static_cast<const fx_coord*>(Xq);
+  const unsigned g = (unsigned)tiles;
+  const float ta = (float)tiny_arg;
+  if (m <= FX_SPILL)
+    return kind == MAT_EXP
+               ? launch_gen_q_out<1, true>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W)
+               : launch_gen_q_out<1, false>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W);
+  return kind == MAT_EXP ? launch_gen_q_out<2, true>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W)
+                         : launch_gen_q_out<2, false>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W);
 }
 
-cudaError_t launch_coord_range(const double* X, int64_t n, int m, double* out, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(out + 2 * m, 0, sizeof(double), s);
-  if (e != cudaSuccess) return e;
-  k_coord_range<<<m, 1024, 0, s>>>(X, n, m, out);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_quantize(const double* X, int64_t n, int m, const double* range, int e, long long* Xq,
+cudaError_t launch_quantize(const double* X, int64_t n, int m, const unsigned long long* range, int e, void* Xq,
                             cudaStream_t s) {
   const int64_t k = n * m;
-  k_quantize<<<(unsigned)((k + 255) / 256), 256, 0, s>>>(X, n, m, range, e, Xq);
+  k_quantize<<<(unsigned)((k + 255) / 256), 256, 0, s>>>(X, n, m, range, e, static_cast<fx_coord*>(Xq));
   note_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_dist_q(const long long* Xq, const double* X, int64_t n, int m, int L, int e, double tau2,
-                          int64_t N, double* Dd, DevStatus* st, cudaStream_t s) {
-  if (m < 1 || m > GEN_MC) return cudaErrorInvalidValue;
-  const size_t smem = 2 * (size_t)TILE * GEN_MC * sizeof(long long);
-  const QuantParams qp{L, e, tau2};
+cudaError_t launch_dist_q(const void* Xq, const double* X, int64_t n, int m, int e, int64_t N, double* Dd,
+                          DevStatus* st, cudaStream_t s) {
+  if (m < 1 || m > FX_MAX_DIM) return cudaErrorInvalidValue;
+  const size_t smem = fx_tile_smem(m);
   const int64_t tiles = num_lower_tiles(N);
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-  cudaError_t err;
-  if (m <= 8) {
-    err = cudaFuncSetAttribute(k_dist_q<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    k_dist_q<true><<<(unsigned)tiles, GEN_THREADS, smem, s>>>(Xq, X, n, m, qp, Dd, st);
-  } else {
-    err = cudaFuncSetAttribute(k_dist_q<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    k_dist_q<false><<<(unsigned)tiles, GEN_THREADS, smem, s>>>(Xq, X, n, m, qp, Dd, st);
-  }
+  const fx_coord* q = static_cast<const fx_coord*>(Xq);
+  auto kern = m <= FX_SPILL ? k_dist_q<1> : k_dist_q<2>;
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err != cudaSuccess) return err;
+  kern<<<(unsigned)tiles, FX_THREADS, smem, s>>>(q, X, n, m, e, Dd, st);
   note_launch();
   return cudaGetLastError();
 }
+
+namespace {
+
+template <bool WF, bool WD>
+void launch_from_dist(unsigned tiles, const double* Dd, int64_t n, double t, const FxScale& sc, float* Zf, double* Zd,
+                      double* rowsum, cudaStream_t s, int kind, double dcut, double kc) {
+  if (kind == MAT_EXP)
+    k_generate_from_dist<WF, WD, true><<<tiles, 256, 0, s>>>(Dd, n, t, sc, Zf, Zd, rowsum, kind, dcut, kc);
+  else
+    k_generate_from_dist<WF, WD, false><<<tiles, 256, 0, s>>>(Dd, n, t, sc, Zf, Zd, rowsum, kind, dcut, kc);
+}
+
+}  // namespace
 
 cudaError_t launch_generate_from_dist(const double* Dd, int64_t n, double t, int64_t N, float* Zf, double* Zd,
                                      double* rowsum, cudaStream_t s, int kind, double tiny_arg, double kc) {
   const unsigned tiles = (unsigned)num_lower_tiles(N);
   const double dcut = tiny_arg / t;
+  const FxScale sc = fx_scale(t, 0);
   if (Zf && Zd)
-    k_generate_from_dist<true, true><<<tiles, 256, 0, s>>>(Dd, n, t, Zf, Zd, rowsum, kind, dcut, kc);
+    launch_from_dist<true, true>(tiles, Dd, n, t, sc, Zf, Zd, rowsum, s, kind, dcut, kc);
   else if (Zf)
-    k_generate_from_dist<true, false><<<tiles, 256, 0, s>>>(Dd, n, t, Zf, Zd, rowsum, kind, INFINITY, kc);
+    launch_from_dist<true, false>(tiles, Dd, n, t, sc, Zf, Zd, rowsum, s, kind, INFINITY, kc);
   else if (Zd)
-    k_generate_from_dist<false, true><<<tiles, 256, 0, s>>>(Dd, n, t, Zf, Zd, rowsum, kind, dcut, kc);
+    launch_from_dist<false, true>(tiles, Dd, n, t, sc, Zf, Zd, rowsum, s, kind, dcut, kc);
   else
     return cudaErrorInvalidValue;
   note_launch();
@@ -701,13 +661,11 @@ cudaError_t launch_generate_from_dist(const double* Dd, int64_t n, double t, int
 }
 
 cudaError_t launch_generate_slab(const double* X, int64_t n, int m, double t, int64_t t0, int64_t W, float* Zf,
-                                 DevStatus* st, cudaStream_t s, double tiny_arg, const long long* Xq, int qL, int qe,
-                                 double qtau2) {
+                                 DevStatus* st, cudaStream_t s, double tiny_arg, const void* Xq, int qe) {
   const int64_t N = (n + TILE - 1) / TILE;
   if (t0 < 0 || t0 >= N || W < 1) return cudaErrorInvalidValue;
   if (Xq)
-    return launch_generate_q(Xq, X, n, m, qL, qe, qtau2, t, N - t0, Zf, nullptr, nullptr, st, s, MAT_EXP, tiny_arg,
-                             0.0, t0, W);
+    return launch_generate_q(Xq, X, n, m, qe, t, N - t0, Zf, nullptr, nullptr, st, s, MAT_EXP, tiny_arg, 0.0, t0, W);
   return launch_gen_t<true, false, false>(X, n, m, t, N - t0, Zf, nullptr, nullptr, st, s, nullptr, MAT_EXP,
                                           tiny_arg, t0, W);
 }

@@ -44,12 +44,12 @@ __device__ __forceinline__ unsigned long long ordered_bits(double v) {
   return (b >> 63) ? ~b : b | 0x8000000000000000ull;
 }
 
-// Starting values of the range and of the least d32^2.
-__global__ void k_mindist_init(unsigned long long* range, int m, unsigned* best32) {
+// Starting values of the range and (if given) of the least d32^2.
+__global__ void k_range_init(unsigned long long* range, int m, unsigned* best32) {
   for (int e = threadIdx.x; e < 2 * m; e += blockDim.x) range[e] = (e & 1) ? 0ull : ~0ull;
   if (threadIdx.x == 0) {
     range[2 * m] = 0ull;
-    *best32 = 0x7f800000u;
+    if (best32) *best32 = 0x7f800000u;
   }
 }
 
@@ -99,10 +99,6 @@ __global__ void __launch_bounds__(256) k_range_ordered(const double* __restrict_
     }
   }
   if (bad) range[2 * m] = 1ull;
-}
-
-__device__ __forceinline__ double ordered_value(unsigned long long u) {
-  return __longlong_as_double((long long)((u >> 63) ? u & 0x7fffffffffffffffull : ~u));
 }
 
 // A[tile][l][r] = (x_l - lo_l) 2^-E of point r of each 128-point tile in FP32
@@ -242,7 +238,21 @@ __global__ void __launch_bounds__(MD_THREADS, 2)
   }
 }
 
+cudaError_t range_ordered(const double* X, int64_t n, int m, unsigned long long* range, unsigned* best32,
+                          cudaStream_t s) {
+  k_range_init<<<1, 256, 0, s>>>(range, m, best32);
+  note_launch();
+  const int64_t passes = (n * m + 255) / 256;
+  k_range_ordered<<<(unsigned)(passes < 304 ? passes : 304), 256, 0, s>>>(X, n, m, range);
+  note_launch();
+  return cudaGetLastError();
+}
+
 }  // namespace
+
+cudaError_t launch_range_ordered(const double* X, int64_t n, int m, unsigned long long* range, cudaStream_t s) {
+  return range_ordered(X, n, m, range, nullptr, s);
+}
 
 size_t min_distance_scratch_bytes(int64_t n, int m) {
   const int64_t N = (n + TILE - 1) / TILE;
@@ -257,11 +267,8 @@ cudaError_t launch_min_distance_filtered(const double* X, int64_t n, int m, void
   unsigned* best32 = reinterpret_cast<unsigned*>(range + 2 * m + 1);
   const size_t head = ((size_t)(2 * m + 2) * sizeof(unsigned long long) + 255) & ~(size_t)255;
   float* A = reinterpret_cast<float*>(static_cast<char*>(scratch) + head);
-  k_mindist_init<<<1, 256, 0, s>>>(range, m, best32);
-  note_launch();
-  const int64_t passes = (n * m + 255) / 256;
-  k_range_ordered<<<(unsigned)(passes < 304 ? passes : 304), 256, 0, s>>>(X, n, m, range);
-  note_launch();
+  cudaError_t e = range_ordered(X, n, m, range, best32, s);
+  if (e != cudaSuccess) return e;
   k_scale_points<<<(unsigned)N, 256, 0, s>>>(X, n, m, range, A, st);
   note_launch();
   k_min_dist<false><<<(unsigned)N, MD_THREADS, 0, s>>>(X, A, n, m, best32, st);

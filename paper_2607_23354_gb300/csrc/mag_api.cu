@@ -26,7 +26,9 @@
 #include <cuda_fp16.h>
 
 #include "../../include/magnitude.h"
+#include "mag_fx.cuh"
 #include "mag_internal.cuh"
+#include "mag_math.cuh"
 
 using namespace mag;
 
@@ -139,17 +141,16 @@ struct mag_ctx {
   // tiles that the panel solve of the one-product factor writes
   float* chain_s = nullptr;
   size_t chain_s_bytes = 0;
-  // quantized coordinates of the exact distance pass: 2m + 1 doubles of
-  // ranges (and a flag), then n m int64
+  // quantized coordinates of the exact distances: 2m + 1 words of ranges (and
+  // a flag), then n m coordinates of two 30-bit limbs
   void* xq = nullptr;
   size_t xq_bytes = 0;
   bool xq_ok = false;                // xq holds the quantization of (xq_pts, xq_n, xq_m) for this solve
   const double* xq_pts = nullptr;
   int64_t xq_n = 0;
   int32_t xq_m = 0;
-  int xq_L = 0, xq_e = 0;
-  double xq_tau2 = 0.0;
-  const long long* xq_q = nullptr;
+  int xq_e = 0;
+  const void* xq_q = nullptr;
   void* lh = nullptr;
   size_t lh_bytes = 0;
   bool chain_ready = false;          // chain_s holds the B tiles of the current factor
@@ -903,7 +904,7 @@ int plan_out_of_core(mag_ctx* ctx, int64_t n, int prec, int64_t* pool_tiles) {
 }
 
 // The quantized coordinates of this solve's points (defined with generate).
-const long long* quantized(mag_ctx* ctx, const double* X, int64_t n, int32_t m);
+const void* quantized(mag_ctx* ctx, const double* X, int64_t n, int32_t m);
 
 // The out-of-core factor of Z = exp[-t d] in an FP16 kind (UPD_FP16X3 or
 // UPD_FP16).  slab0_ready: slab 0 is already generated (the precision probe
@@ -919,9 +920,8 @@ int factor_ooc(mag_ctx* ctx, const double* X, int32_t m, double t, int mode, boo
     float* Zs = ctx->slab_dev(sl);
     const int64_t rows = L.N - sl.c0;
     if (!(si == 0 && slab0_ready)) {
-      const long long* q = quantized(ctx, X, L.n, m);
-      CU(launch_generate_slab(X, L.n, m, t, sl.c0, sl.S, Zs, ctx->st(), s, INFINITY, q, ctx->xq_L, ctx->xq_e,
-                              ctx->xq_tau2));
+      const void* q = quantized(ctx, X, L.n, m);
+      CU(launch_generate_slab(X, L.n, m, t, sl.c0, sl.S, Zs, ctx->st(), s, INFINITY, q, ctx->xq_e));
     }
     if (ctx->slab_cmap_base != Zs || ctx->slab_cmap_tiles != sl.tiles) {
       if (!make_c_map(&ctx->slab_cmap, Zs, sl.tiles))
@@ -1197,44 +1197,36 @@ float elapsed(mag_ctx* ctx, int a, int b) {
   return ms;
 }
 
-// Generate the tiles for the given precision into the current layout.
-// tiny_fp32: entries below e^-46 in FP32 (exp_neg_tiny_td), for the solve path;
-// the entry points that return Z or differentiate it keep FP64 everywhere.
-// Coordinates quantized for the exact distance pass (launch_dist_q): per
-// dimension the minimum lo_l, the largest span S < 2^E, limbs of L bits with
-// m 2^(2L) <= 2^63 (the kernel's 64-bit sums cannot wrap), B = 2L - 1 bits
-// per coordinate, scale 2^e with e = B - E (every coordinate offset below
-// 2^B), and tau2 = m 2^(106 - 2e): at d >= sqrt(tau2) the quantization
-// (at most 2 sqrt(m) 2^-e in d) is below 2^-52 d.  false: FP64 differences
-// instead (a non-finite coordinate, every dimension constant, m > 32, a
-// scale beyond 2^+-400, or no memory for the copy).
-bool quantize_points(mag_ctx* ctx, const double* X, int64_t n, int32_t m, int* L, int* e, double* tau2,
-                     const long long** Xq) {
+// Coordinates quantized for the exact distances (mag_fx.cuh): per dimension
+// the minimum lo_l, the largest span S < 2^E, 59 bits per coordinate, unit
+// 2^-e with e = 59 - E (every coordinate offset below 2^59).  At d >= sqrt(m)
+// 2^(53-e) the quantization (at most 2 sqrt(m) 2^-e in d) is below 2^-52 d;
+// closer pairs take the FP64 differences.  false: FP64 differences for all (a
+// non-finite coordinate, every dimension constant, m > 512, a scale beyond
+// 2^+-400, or no memory for the copy).
+bool quantize_points(mag_ctx* ctx, const double* X, int64_t n, int32_t m, int* e, const void** Xq) {
   ctx->xq_ok = false;
-  if (!ctx->opt.exact_distances || m > 32 || m < 1) return false;
-  const size_t head = ((size_t)(2 * m + 1) * sizeof(double) + 255) & ~(size_t)255;
-  if (!grow_buffer(ctx, &ctx->xq, &ctx->xq_bytes, head + (size_t)n * m * sizeof(long long), 0)) return false;
-  double* range = (double*)ctx->xq;
-  long long* q = (long long*)((char*)ctx->xq + head);
+  if (!ctx->opt.exact_distances || m > FX_MAX_DIM || m < 1) return false;
+  const size_t head = ((size_t)(2 * m + 1) * sizeof(unsigned long long) + 255) & ~(size_t)255;
+  if (!grow_buffer(ctx, &ctx->xq, &ctx->xq_bytes, head + (size_t)n * m * sizeof(fx_coord), 0)) return false;
+  unsigned long long* range = (unsigned long long*)ctx->xq;
+  void* q = (char*)ctx->xq + head;
   cudaStream_t s = ctx->stream;
-  std::vector<double> h(2 * m + 1);
-  if (launch_coord_range(X, n, m, range, s) != cudaSuccess ||
-      cudaMemcpyAsync(h.data(), range, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+  std::vector<unsigned long long> h(2 * m + 1);
+  if (launch_range_ordered(X, n, m, range, s) != cudaSuccess ||
+      cudaMemcpyAsync(h.data(), range, h.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s) !=
+          cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  if (h[2 * m] != 0.0) return false;
+  if (h[2 * m] != 0) return false;
   double S = 0.0;
-  for (int l = 0; l < m; ++l) S = std::max(S, h[2 * l + 1] - h[2 * l]);
+  for (int l = 0; l < m; ++l) S = std::max(S, ordered_value(h[2 * l + 1]) - ordered_value(h[2 * l]));
   if (!(S > 0.0) || !std::isfinite(S)) return false;
   const int E = std::ilogb(S) + 1;  // S < 2^E
-  int mb = 0;
-  while ((1 << mb) < m) ++mb;
-  *L = (63 - mb) / 2;
-  *e = (2 * *L - 1) - E;
+  *e = FX_COORD_BITS - E;
   if (*e < -400 || *e > 400) return false;
-  *tau2 = std::ldexp((double)m, 106 - 2 * *e);
   if (launch_quantize(X, n, m, range, *e, q, s) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -1244,27 +1236,27 @@ bool quantize_points(mag_ctx* ctx, const double* X, int64_t n, int32_t m, int* L
   ctx->xq_pts = X;
   ctx->xq_n = n;
   ctx->xq_m = m;
-  ctx->xq_L = *L;
   ctx->xq_e = *e;
-  ctx->xq_tau2 = *tau2;
   ctx->xq_q = q;
   return true;
 }
 
 // The quantized coordinates of this solve's points for the matrix-free
 // residual (quantize_points on first use; null: FP64 differences).
-const long long* quantized(mag_ctx* ctx, const double* X, int64_t n, int32_t m) {
+const void* quantized(mag_ctx* ctx, const double* X, int64_t n, int32_t m) {
   if (ctx->xq_ok && ctx->xq_pts == X && ctx->xq_n == n && ctx->xq_m == m) return ctx->xq_q;
-  int L = 0, e = 0;
-  double tau2 = 0.0;
-  const long long* q = nullptr;
-  if (!quantize_points(ctx, X, n, m, &L, &e, &tau2, &q)) {
+  int e = 0;
+  const void* q = nullptr;
+  if (!quantize_points(ctx, X, n, m, &e, &q)) {
     ctx->xq_ok = false;
     return nullptr;
   }
   return q;
 }
 
+// Generate the tiles for the given precision into the current layout.
+// tiny_fp32: entries below e^-46 in FP32 (exp_neg_tiny_td), for the solve path;
+// the entry points that return Z or differentiate it keep FP64 everywhere.
 int generate(mag_ctx* ctx, const double* X, int32_t m, double t, bool f32, bool f64, SolveResult* R,
              bool tiny_fp32 = false) {
   const double tiny_arg = tiny_fp32 ? kTinyArg : INFINITY;
@@ -1279,12 +1271,11 @@ int generate(mag_ctx* ctx, const double* X, int32_t m, double t, bool f32, bool 
     CU(launch_generate_from_dist(ctx->dist(), L.n, t, L.N, f32 ? ctx->zf() : nullptr, f64 ? ctx->zd() : nullptr,
                                  ctx->vd(V_ROWSUM), s, ctx->kind, tiny_arg, ctx->kind_c));
   } else if (ctx->dist_active && L.dist) {
-    int qL = 0, qe = 0;
-    double qtau2 = 0.0;
-    const long long* Xq = nullptr;
-    if (quantize_points(ctx, X, L.n, m, &qL, &qe, &qtau2, &Xq)) {
+    int qe = 0;
+    const void* Xq = nullptr;
+    if (quantize_points(ctx, X, L.n, m, &qe, &Xq)) {
       // exact d^2 on the integer pipe, then Z from the distances
-      CU(launch_dist_q(Xq, X, L.n, m, qL, qe, qtau2, L.N, ctx->dist(), ctx->st(), s));
+      CU(launch_dist_q(Xq, X, L.n, m, qe, L.N, ctx->dist(), ctx->st(), s));
       CU(launch_generate_from_dist(ctx->dist(), L.n, t, L.N, f32 ? ctx->zf() : nullptr, f64 ? ctx->zd() : nullptr,
                                    ctx->vd(V_ROWSUM), s, ctx->kind, tiny_arg, ctx->kind_c));
       R->exact_distances = 1;
@@ -1293,11 +1284,10 @@ int generate(mag_ctx* ctx, const double* X, int32_t m, double t, bool f32, bool 
                               ctx->dist(), ctx->vd(V_ROWSUM), ctx->st(), s, ctx->kind, tiny_arg, ctx->kind_c));
     }
   } else {
-    int qL = 0, qe = 0;
-    double qtau2 = 0.0;
-    const long long* Xq = nullptr;
-    if (quantize_points(ctx, X, L.n, m, &qL, &qe, &qtau2, &Xq)) {
-      CU(launch_generate_q(Xq, X, L.n, m, qL, qe, qtau2, t, L.N, f32 ? ctx->zf() : nullptr,
+    int qe = 0;
+    const void* Xq = nullptr;
+    if (quantize_points(ctx, X, L.n, m, &qe, &Xq)) {
+      CU(launch_generate_q(Xq, X, L.n, m, qe, t, L.N, f32 ? ctx->zf() : nullptr,
                            f64 ? ctx->zd() : nullptr, ctx->vd(V_ROWSUM), ctx->st(), s, ctx->kind, tiny_arg,
                            ctx->kind_c));
       R->exact_distances = 1;
@@ -1506,9 +1496,9 @@ int residual(mag_ctx* ctx, const double* X, int32_t m, double t, const double* w
     CU(launch_residual_stored(ctx->zd(), L.n, L.N, w, b, ctx->vd(V_ROWSUM), r, ctx->spart(), L.np,
                               ctx->st(), s));
   else {
-    const long long* q = ctx->kind == MAT_EXP ? quantized(ctx, X, L.n, m) : nullptr;
+    const void* q = ctx->kind == MAT_EXP ? quantized(ctx, X, L.n, m) : nullptr;
     CU(launch_residual_sym(X, L.n, m, t, w, b, r, ctx->spart(), ctx->vd(V_ROWSUM), L.np, ctx->st(), s, ctx->kind,
-                           ctx->kind_c, q, ctx->xq_L, ctx->xq_e, ctx->xq_tau2));
+                           ctx->kind_c, q, ctx->xq_e));
   }
   CU(cudaEventRecord(ctx->ev[1], s));
   TRY(read_status(ctx));
@@ -1697,9 +1687,9 @@ int gmres_ir(mag_ctx* ctx, int prec, const double* X, int32_t m, double t, const
     else if (stored)
       CU(launch_residual_stored(ctx->zd(), n, L.N, v, zeros, ctx->vd(V_ROWSUM), tmp, ctx->spart(), np, ctx->st(), s));
     else {
-      const long long* q = ctx->kind == MAT_EXP ? quantized(ctx, X, n, m) : nullptr;
+      const void* q = ctx->kind == MAT_EXP ? quantized(ctx, X, n, m) : nullptr;
       CU(launch_residual_sym(X, n, m, t, v, zeros, tmp, ctx->spart(), ctx->vd(V_ROWSUM), np, ctx->st(), s,
-                             ctx->kind, ctx->kind_c, q, ctx->xq_L, ctx->xq_e, ctx->xq_tau2));
+                             ctx->kind, ctx->kind_c, q, ctx->xq_e));
     }
     TRY(correction(ctx, prec, tmp, out, /*init=*/true, R));
     CU(launch_scale(out, -1.0, out, n, s));
@@ -1980,9 +1970,9 @@ int solve_ooc(mag_ctx* ctx, const double* X, int64_t n, int32_t m, double t, con
     const int64_t K = std::min<int64_t>(L.nb, kProbeTiles);
     if (ctx->slabs[0].S >= K && L.N >= 3 * K) {
       CU(cudaEventRecord(ctx->ev[0], s));
-      const long long* q = quantized(ctx, X, n, m);
+      const void* q = quantized(ctx, X, n, m);
       CU(launch_generate_slab(X, n, m, t, 0, ctx->slabs[0].S, ctx->slab_dev(ctx->slabs[0]), ctx->st(), s, INFINITY,
-                              q, ctx->xq_L, ctx->xq_e, ctx->xq_tau2));
+                              q, ctx->xq_e));
       CU(cudaEventRecord(ctx->ev[1], s));
       TRY(read_status(ctx));
       R->ms_gen += elapsed(ctx, 0, 1);

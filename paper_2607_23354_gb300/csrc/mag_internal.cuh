@@ -114,25 +114,27 @@ cudaError_t launch_generate(const double* X, int64_t n, int m, double t, int64_t
 cudaError_t launch_generate_dist(const double* X, int64_t n, int m, double t, int64_t N, float* Zf,
                                  double* Zd, double* Dd, double* rowsum, DevStatus* st, cudaStream_t s,
                                  int kind = MAT_EXP, double tiny_arg = INFINITY, double kc = 0.0);
-// Exact pair distances from quantized coordinates (k_generate.cu).
-// launch_coord_range: per dimension min and max of X into out[2l], out[2l+1]
-// and out[2m] = 1 if a coordinate is not finite (2m + 1 doubles).
-// launch_quantize: Xq[i m + l] = round(2^e (X[i m + l] - out[2l])) (int64).
-// launch_dist_q: FP64 distances Dd of the packed lower tiles (m <= 32) from
-// Xq (limb bits L, scale 2^e; pairs with d^2 < tau2 from the FP64
-// differences of X), min d^2 and ST_DUPLICATE into st as the generator.
-cudaError_t launch_coord_range(const double* X, int64_t n, int m, double* out, cudaStream_t s);
-cudaError_t launch_quantize(const double* X, int64_t n, int m, const double* range, int e, long long* Xq,
+// Exact pair distances from quantized coordinates (mag_fx.cuh).
+// launch_range_ordered (k_mindist.cu): per dimension min and max of X in the
+// order-preserving encoding of ordered_value, range[2l], range[2l+1], and
+// range[2m] = 1 if a coordinate is not finite (2m + 1 words).
+// launch_quantize: Xq[i m + l] = round(2^e (X[i m + l] - min_l)) as two 30-bit
+// limbs (8 bytes a coordinate).
+// launch_dist_q: FP64 distances Dd of the packed lower tiles (m <= 512) from Xq
+// (pairs closer than sqrt(m) 2^(53-e) from the FP64 differences of X), min
+// d^2 and ST_DUPLICATE into st as the generator.
+cudaError_t launch_range_ordered(const double* X, int64_t n, int m, unsigned long long* range, cudaStream_t s);
+cudaError_t launch_quantize(const double* X, int64_t n, int m, const unsigned long long* range, int e, void* Xq,
                             cudaStream_t s);
-cudaError_t launch_dist_q(const long long* Xq, const double* X, int64_t n, int m, int L, int e, double tau2,
-                          int64_t N, double* Dd, DevStatus* st, cudaStream_t s);
+cudaError_t launch_dist_q(const void* Xq, const double* X, int64_t n, int m, int e, int64_t N, double* Dd,
+                          DevStatus* st, cudaStream_t s);
 // launch_generate (row sums, min d^2, flags) with the distances of
 // launch_dist_q, in one pass (no distances kept).
 // rowsum may be null (none); t0, W: the slab layout of launch_generate_slab.
-cudaError_t launch_generate_q(const long long* Xq, const double* X, int64_t n, int m, int L, int e, double tau2,
-                              double t, int64_t N, float* Zf, double* Zd, double* rowsum, DevStatus* st,
-                              cudaStream_t s, int kind = MAT_EXP, double tiny_arg = INFINITY, double kc = 0.0,
-                              int64_t t0 = 0, int64_t W = -1);
+cudaError_t launch_generate_q(const void* Xq, const double* X, int64_t n, int m, int e, double t, int64_t N,
+                              float* Zf, double* Zd, double* rowsum, DevStatus* st, cudaStream_t s,
+                              int kind = MAT_EXP, double tiny_arg = INFINITY, double kc = 0.0, int64_t t0 = 0,
+                              int64_t W = -1);
 // FP32 tiles of one slab for the out-of-core factor: global tile columns
 // [t0, t0 + W) of rows [t0, N), in the slab layout (tile_index with column
 // cap W, tile (0, 0) = global (t0, t0)); no row sums; min d^2 and flags as
@@ -141,7 +143,7 @@ cudaError_t launch_generate_q(const long long* Xq, const double* X, int64_t n, i
 // distances from their exact integer d^2 (launch_generate_q).
 cudaError_t launch_generate_slab(const double* X, int64_t n, int m, double t, int64_t t0, int64_t W, float* Zf,
                                  DevStatus* st, cudaStream_t s, double tiny_arg = INFINITY,
-                                 const long long* Xq = nullptr, int qL = 0, int qe = 0, double qtau2 = 0.0);
+                                 const void* Xq = nullptr, int qe = 0);
 // Z from stored FP64 distance tiles: Zf (may be null) and Zd (may be null), row sums.
 cudaError_t launch_generate_from_dist(const double* Dd, int64_t n, double t, int64_t N, float* Zf, double* Zd,
                                      double* rowsum, cudaStream_t s, int kind = MAT_EXP,
@@ -322,13 +324,11 @@ cudaError_t launch_residual_mf(const double* X, int64_t n, int m, double t, cons
 // Matrix free over the lower triangle (each Z entry computed once, used for
 // its row and its column): P is scratch of N * N * 128 doubles, rowsum of n
 // doubles (overwritten with the row sums of Z).  Same outputs as above.
-// Xq (optional, Z = exp(-t d) with m <= 32): the quantized coordinates of
-// launch_quantize (limb bits qL, scale 2^qe, FP64 differences below qtau2),
-// the pair distances from their exact integer d^2.
+// Xq (optional, Z = exp(-t d) with m <= 512): the quantized coordinates of
+// launch_quantize (scale 2^qe), the pairs from their exact integer d^2.
 cudaError_t launch_residual_sym(const double* X, int64_t n, int m, double t, const double* w, const double* b,
                                 double* r, double* P, double* rowsum, int64_t np, DevStatus* st, cudaStream_t s,
-                                int kind = MAT_EXP, double kc = 0.0, const long long* Xq = nullptr, int qL = 0,
-                                int qe = 0, double qtau2 = 0.0);
+                                int kind = MAT_EXP, double kc = 0.0, const void* Xq = nullptr, int qe = 0);
 // Stored: P is scratch of N * N * 128 doubles (one partial per row block,
 // tile and row); rowsum holds the row sums of Z from the generator.
 cudaError_t launch_residual_stored(const double* Zd, int64_t n, int64_t N, const double* w,
