@@ -351,8 +351,8 @@ __device__ __forceinline__ void finish_min(unsigned long long mind2b, const FxSq
 // min d^2 and the coincident-point flag as k_generate: one CTA per tile.  Rows
 // and columns of the padding get d = 0 (the generator from distances gives
 // them the identity by index).
-template <int R>
-__global__ void __launch_bounds__(FX_THREADS, 2)
+template <int KIND>
+__global__ void __launch_bounds__(FX_THREADS, fx_ctas(KIND))
     k_dist_q(const fx_coord* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, int qe,
              double* __restrict__ Dd, DevStatus* st) {
   extern __shared__ __align__(16) unsigned char gen_smem[];
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
   unsigned long long mind2b = 0x7ff0000000000000ull;  // +inf
   FxSquare mq{~0ull, ~0ull};
   int flags = 0;
-  fx_tile_pairs<R>(Xq, n, m, row0, col0, reinterpret_cast<fx_coord*>(gen_smem), [&](int r, FxSquare(&q)[4]) {
+  fx_tile_pairs<KIND>(Xq, n, m, row0, col0, reinterpret_cast<fx_coord*>(gen_smem), [&](int r, FxSquare(&q)[4]) {
     const int64_t gr = row0 + r;
     double ddv[4];
 #pragma unroll
@@ -397,8 +397,8 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
 // when rowsum is given), tiles in the slab layout of k_generate.  Used where
 // no distances are kept (a single t, the slabs of the out-of-core factor); a
 // multi-t call keeps them with k_dist_q, then k_generate_from_dist.
-template <int R, bool WF, bool WD, bool EXP>
-__global__ void __launch_bounds__(FX_THREADS, 2)
+template <int KIND, bool WF, bool WD, bool EXP>
+__global__ void __launch_bounds__(FX_THREADS, fx_ctas(KIND))
     k_generate_q(const fx_coord* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, FxScale sc,
                  double t, float* __restrict__ Zf, double* __restrict__ Zd, double* __restrict__ rowsum,
                  DevStatus* st, int kind, float tiny, double kc, int64_t t0, int64_t W) {
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
   unsigned long long mind2b = 0x7ff0000000000000ull;  // +inf
   FxSquare mq{~0ull, ~0ull};
   int flags = 0;
-  fx_tile_pairs<R>(Xq, n, m, row0, col0, reinterpret_cast<fx_coord*>(gen_smem), [&](int r, FxSquare(&q)[4]) {
+  fx_tile_pairs<KIND>(Xq, n, m, row0, col0, reinterpret_cast<fx_coord*>(gen_smem), [&](int r, FxSquare(&q)[4]) {
     const int64_t gr = row0 + r;
     float rs = 0.0f;
     float zfv[4];
@@ -497,6 +497,72 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
   }
 }
 
+// Z = exp(-t d) as the dense n x n row-major matrix, both triangles, from the
+// quantized coordinates: one CTA per lower tile writes it and its transpose
+// (eight rows at a time through shared memory, 64 contiguous bytes per column
+// in FP64), with the checks of k_generate.  In one pass; packed tiles first and
+// a copy of them afterwards took twice the time.
+template <int KIND, typename T>
+__global__ void __launch_bounds__(FX_THREADS, fx_ctas(KIND))
+    k_dense_q(const fx_coord* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, FxScale sc,
+              T* __restrict__ Z, DevStatus* st) {
+  extern __shared__ __align__(16) unsigned char gen_smem[];
+  __shared__ unsigned long long warpmin[FX_THREADS / 32];
+  __shared__ fx_u64 fxtab[FX_TABLE_SIZE];
+  __shared__ T rows[2][FX_THREADS / 32][TILE + 1];  // two passes' rows, by the parity of the pass
+  load_fx_table(fxtab);
+  int64_t I, J;
+  tri_coords((int64_t)blockIdx.x, &I, &J);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t row0 = I * TILE, col0 = J * TILE;
+  unsigned long long mind2b = 0x7ff0000000000000ull;  // +inf
+  FxSquare mq{~0ull, ~0ull};
+  int flags = 0;
+  fx_tile_pairs<KIND>(Xq, n, m, row0, col0, reinterpret_cast<fx_coord*>(gen_smem), [&](int r, FxSquare(&q)[4]) {
+    const int64_t gr = row0 + r;
+    const int pass = r >> 3;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int64_t gc = col0 + 4 * lane + c;
+      double z = 1.0;
+      if (gr < n && gc < n && gr != gc) {
+        fx_u64 b;
+        if (fx_close(q[c], m)) {
+          const double d = sqrt_pos(close_square(X, gr, gc, m, &flags, &mind2b));
+          b = fx_exp_neg_d((fx_u64)__double_as_longlong(d), sc.kg, sc.g, fxtab);
+        } else {
+          if (q[c].h < mq.h || (q[c].h == mq.h && q[c].l < mq.l)) mq = q[c];
+          const FxRoot rt = fx_root_start(q[c]);
+          b = fx_exp_neg(fx_root(rt), rt.j - sc.e + sc.kg, sc.g, fxtab);
+        }
+        z = __longlong_as_double((long long)b);
+      }
+      T v;
+      if constexpr (sizeof(T) == 8)
+        v = z;
+      else
+        v = f64_to_f32_nonneg(z);
+      rows[pass & 1][warp][4 * lane + c] = v;
+    }
+    __syncthreads();  // every warp is on the same pass
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t gc = col0 + lane + 32 * k;
+      if (gr < n && gc < n) Z[gr * n + gc] = rows[pass & 1][warp][lane + 32 * k];
+    }
+    if (I != J) {  // the transpose: column (tid / 8) + 32 k, row tid % 8 of the pass
+      const int rr = threadIdx.x & 7;
+      const int64_t tr = row0 + 8 * pass + rr;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int c = (threadIdx.x >> 3) + 32 * k;
+        if (tr < n && col0 + c < n) Z[(col0 + c) * n + tr] = rows[pass & 1][rr][c];
+      }
+    }
+  });
+  finish_min(mind2b, mq, sc.e, flags, warpmin, st);
+}
+
 // q = round(2^e (x - lo_l)) with x - lo_l taken exactly as s + err (TwoSum):
 // round(2^e s) + round(2^e err), within one unit of 2^e (x - lo_l); stored as
 // its limbs.
@@ -510,7 +576,8 @@ __global__ void k_quantize(const double* __restrict__ X, int64_t n, int m,
   const double bv = s - x;
   const double err = (x - (s - bv)) + (b - bv);
   const long long q = __double2ll_rn(ldexp(s, e)) + __double2ll_rn(ldexp(err, e));
-  Xq[k] = fx_coord{(int)(q & ((1ll << FX_LIMB) - 1)), (int)(q >> FX_LIMB)};
+  const int lb = fx_limb_of(m);
+  Xq[k] = fx_coord{(int)(q & ((1ll << lb) - 1)), (int)(q >> lb)};
 }
 
 template <bool WF, bool WD, bool ROWSUM, bool WDIST = false>
@@ -558,11 +625,11 @@ cudaError_t launch_generate_dist(const double* X, int64_t n, int m, double t, in
 
 namespace {
 
-template <int R, bool WF, bool WD, bool EXP>
+template <int KIND, bool WF, bool WD, bool EXP>
 cudaError_t launch_gen_q(const fx_coord* Xq, const double* X, int64_t n, int m, const FxScale& sc, double t,
                          unsigned tiles, float* Zf, double* Zd, double* rowsum, DevStatus* st, cudaStream_t s,
                          int kind, float tiny, double kc, int64_t t0, int64_t W) {
-  auto kern = k_generate_q<R, WF, WD, EXP>;
+  auto kern = k_generate_q<KIND, WF, WD, EXP>;
   const size_t smem = fx_tile_smem(m);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -571,17 +638,16 @@ cudaError_t launch_gen_q(const fx_coord* Xq, const double* X, int64_t n, int m, 
   return cudaGetLastError();
 }
 
-template <int R, bool EXP>
+template <int KIND, bool EXP>
 cudaError_t launch_gen_q_out(const fx_coord* Xq, const double* X, int64_t n, int m, const FxScale& sc, double t,
                              unsigned tiles, float* Zf, double* Zd, double* rowsum, DevStatus* st, cudaStream_t s,
                              int kind, float tiny, double kc, int64_t t0, int64_t W) {
   if (Zf && Zd)
-    return launch_gen_q<R, true, true, EXP>(Xq, X, n, m, sc, t, tiles, Zf, Zd, rowsum, st, s, kind, tiny, kc, t0, W);
+    return launch_gen_q<KIND, true, true, EXP>(Xq, X, n, m, sc, t, tiles, Zf, Zd, rowsum, st, s, kind, tiny, kc, t0, W);
   if (Zf)  // FP32 tiles alone: rounded from the FP64 entries
-    return launch_gen_q<R, true, false, EXP>(Xq, X, n, m, sc, t, tiles, Zf, Zd, rowsum, st, s, kind, INFINITY, kc, t0,
-                                             W);
+    return launch_gen_q<KIND, true, false, EXP>(Xq, X, n, m, sc, t, tiles, Zf, Zd, rowsum, st, s, kind, tiny, kc, t0, W);
   if (Zd)
-    return launch_gen_q<R, false, true, EXP>(Xq, X, n, m, sc, t, tiles, Zf, Zd, rowsum, st, s, kind, tiny, kc, t0, W);
+    return launch_gen_q<KIND, false, true, EXP>(Xq, X, n, m, sc, t, tiles, Zf, Zd, rowsum, st, s, kind, tiny, kc, t0, W);
   return cudaErrorInvalidValue;
 }
 
@@ -599,13 +665,48 @@ cudaError_t launch_generate_q(const void* Xq, const double* X, int64_t n, int m,
   const fx_coord* q = static_cast<const fx_coord*>(Xq);
   const unsigned g = (unsigned)tiles;
   const float ta = (float)tiny_arg;
-  if (m <= FX_SPILL)
-    return kind == MAT_EXP
-               ? launch_gen_q_out<1, true>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W)
-               : launch_gen_q_out<1, false>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W);
-  return kind == MAT_EXP ? launch_gen_q_out<2, true>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W)
-                         : launch_gen_q_out<2, false>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W);
+#define MAG_GEN_Q(KIND_)                                                                                               \
+  return kind == MAT_EXP                                                                                               \
+             ? launch_gen_q_out<KIND_, true>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W)         \
+             : launch_gen_q_out<KIND_, false>(q, X, n, m, sc, t, g, Zf, Zd, rowsum, st, s, kind, ta, kc, t0, W)
+  switch (fx_kind(m)) {
+    case 0: MAG_GEN_Q(0);
+    case 1: MAG_GEN_Q(1);
+    default: MAG_GEN_Q(2);
+  }
+#undef MAG_GEN_Q
 }
+
+template <int KIND, typename T>
+static cudaError_t launch_dense_t(const fx_coord* Xq, const double* X, int64_t n, int m, const FxScale& sc, T* Z,
+                                  unsigned tiles, DevStatus* st, cudaStream_t s) {
+  auto kern = k_dense_q<KIND, T>;
+  const size_t smem = fx_tile_smem(m);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<tiles, FX_THREADS, smem, s>>>(Xq, X, n, m, sc, Z, st);
+  note_launch();
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_dense_q(const void* Xq, const double* X, int64_t n, int m, int e, double t, T* Z, DevStatus* st,
+                           cudaStream_t s) {
+  if (m < 1 || m > FX_MAX_DIM) return cudaErrorInvalidValue;
+  const int64_t tiles = num_lower_tiles((n + TILE - 1) / TILE);
+  if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  const FxScale sc = fx_scale(t, e);
+  const fx_coord* q = static_cast<const fx_coord*>(Xq);
+  switch (fx_kind(m)) {
+    case 0: return launch_dense_t<0, T>(q, X, n, m, sc, Z, (unsigned)tiles, st, s);
+    case 1: return launch_dense_t<1, T>(q, X, n, m, sc, Z, (unsigned)tiles, st, s);
+    default: return launch_dense_t<2, T>(q, X, n, m, sc, Z, (unsigned)tiles, st, s);
+  }
+}
+template cudaError_t launch_dense_q<float>(const void*, const double*, int64_t, int, int, double, float*, DevStatus*,
+                                           cudaStream_t);
+template cudaError_t launch_dense_q<double>(const void*, const double*, int64_t, int, int, double, double*,
+                                            DevStatus*, cudaStream_t);
 
 cudaError_t launch_quantize(const double* X, int64_t n, int m, const unsigned long long* range, int e, void* Xq,
                             cudaStream_t s) {
@@ -622,7 +723,8 @@ cudaError_t launch_dist_q(const void* Xq, const double* X, int64_t n, int m, int
   const int64_t tiles = num_lower_tiles(N);
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   const fx_coord* q = static_cast<const fx_coord*>(Xq);
-  auto kern = m <= FX_SPILL ? k_dist_q<1> : k_dist_q<2>;
+  const int kd = fx_kind(m);
+  auto kern = kd == 0 ? k_dist_q<0> : (kd == 1 ? k_dist_q<1> : k_dist_q<2>);
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   kern<<<(unsigned)tiles, FX_THREADS, smem, s>>>(q, X, n, m, e, Dd, st);

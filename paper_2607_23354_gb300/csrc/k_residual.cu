@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(SYM_THREADS, 1)
 // instead of five shuffle levels each).
 constexpr int SYMQ_LD = 33;
 
-template <int R>
+template <int KIND>
 __global__ void __launch_bounds__(FX_THREADS, 2)
     k_resid_sym_q(const fx_coord* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, FxScale sc,
                   const double* __restrict__ w, double* __restrict__ P, double* __restrict__ rowsum, int64_t N) {
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
     cs[c] = 0.0;
     zc[c] = 0.0f;
   }
-  fx_tile_pairs<R>(Xq, n, m, row0, col0, stage, [&](int r, FxSquare(&q)[4]) {
+  fx_tile_pairs<KIND>(Xq, n, m, row0, col0, stage, [&](int r, FxSquare(&q)[4]) {
     const int64_t gr = row0 + r;
     const double wr = s_wr[r];
     double v = 0.0;
@@ -973,7 +973,8 @@ cudaError_t launch_residual_sym(const double* X, int64_t n, int m, double t, con
   if (Xq && kind == MAT_EXP && m <= FX_MAX_DIM) {
     const FxScale sc = fx_scale(t, qe);
     const size_t sq = (size_t)TILE * SYMQ_LD * sizeof(double) + fx_tile_smem(m);
-    auto kern = m <= FX_SPILL ? k_resid_sym_q<1> : k_resid_sym_q<2>;
+    const int kd = fx_kind(m);
+    auto kern = kd == 0 ? k_resid_sym_q<0> : (kd == 1 ? k_resid_sym_q<1> : k_resid_sym_q<2>);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sq);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)tiles, FX_THREADS, sq, s>>>(static_cast<const fx_coord*>(Xq), X, n, m, sc, w, P, rowsum, N);

@@ -1198,9 +1198,10 @@ float elapsed(mag_ctx* ctx, int a, int b) {
 }
 
 // Coordinates quantized for the exact distances (mag_fx.cuh): per dimension
-// the minimum lo_l, the largest span S < 2^E, 59 bits per coordinate, unit
-// 2^-e with e = 59 - E (every coordinate offset below 2^59).  At d >= sqrt(m)
-// 2^(53-e) the quantization (at most 2 sqrt(m) 2^-e in d) is below 2^-52 d;
+// the minimum lo_l, the largest span S < 2^E, B = 61 (m <= 4) or 59 bits per
+// coordinate, unit 2^-e with e = B - E (every coordinate offset below 2^B).  At
+// d >= sqrt(m) 2^(53-e) the quantization (at most 2 sqrt(m) 2^-e in d) is
+// below 2^-52 d;
 // closer pairs take the FP64 differences.  false: FP64 differences for all (a
 // non-finite coordinate, every dimension constant, m > 512, a scale beyond
 // 2^+-400, or no memory for the copy).
@@ -1225,7 +1226,7 @@ bool quantize_points(mag_ctx* ctx, const double* X, int64_t n, int32_t m, int* e
   for (int l = 0; l < m; ++l) S = std::max(S, ordered_value(h[2 * l + 1]) - ordered_value(h[2 * l]));
   if (!(S > 0.0) || !std::isfinite(S)) return false;
   const int E = std::ilogb(S) + 1;  // S < 2^E
-  *e = FX_COORD_BITS - E;
+  *e = fx_coord_bits(m) - E;
   if (*e < -400 || *e > 400) return false;
   if (launch_quantize(X, n, m, range, *e, q, s) != cudaSuccess) {
     cudaGetLastError();
@@ -2282,6 +2283,21 @@ int mag_similarity_matrix(mag_ctx* ctx, const double* points, int64_t n, int32_t
   const bool f64 = precision == MAG_PREC_FP64;
   SolveResult R;
   ctx->fac_valid = false;
+  // straight into Z_out from the quantized coordinates; the packed tiles and a
+  // copy of them where the points do not admit those
+  if (!ctx->ws || ctx->lay.np < ((n + TILE - 1) / TILE) * TILE) TRY(ensure_workspace(ctx, n, false, false));
+  int qe = 0;
+  const void* Xq = nullptr;
+  if (n <= 65535 && quantize_points(ctx, points, n, m, &qe, &Xq)) {  // the copy's limit on n
+    TRY(reset_status(ctx));
+    if (f64)
+      CU(launch_dense_q<double>(Xq, points, n, m, qe, t, (double*)Z_out, ctx->st(), ctx->stream));
+    else
+      CU(launch_dense_q<float>(Xq, points, n, m, qe, t, (float*)Z_out, ctx->st(), ctx->stream));
+    TRY(read_status(ctx));
+    if (ctx->h_st->flags & ST_DUPLICATE) return fail(ctx, MAG_EDUPLICATE, "two points coincide (min d = 0)");
+    return MAG_OK;
+  }
   TRY(ensure_workspace(ctx, n, !f64, f64));
   TRY(generate(ctx, points, m, t, !f64, f64, &R));
   const Layout& L = ctx->lay;

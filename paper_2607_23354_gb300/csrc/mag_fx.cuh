@@ -7,9 +7,9 @@
 // nine FP64 operations (and a hundred others) it replaces, and rounded to FP64
 // once.
 //
-//   d^2   exact: coordinates as two limbs of 30 bits, q = hi 2^30 + lo, the
-//         differences of both limbs, and three 64-bit sums (lo lo, hi lo,
-//         hi hi) of signed 32 x 32-bit products;
+//   d^2   exact: coordinates as two limbs, q = hi 2^30 + lo, the differences
+//         of both limbs, and three 64-bit sums (lo lo, hi lo, hi hi) of signed
+//         32 x 32-bit products;
 //   d     sqrt of the leading 64 bits: an FP32 reciprocal square root, then two
 //         corrections s += (v - s^2) / (2 s) with the residual exact in 64-bit
 //         integers and the quotient in FP32 (P. Markstein, "Computation of
@@ -43,12 +43,21 @@ namespace mag {
 
 typedef unsigned long long fx_u64;
 
-constexpr int FX_LIMB = 30;              // bits of a coordinate limb
-constexpr int FX_COORD_BITS = 59;        // bits of a quantized coordinate
 constexpr int FX_MAX_DIM = 512;          // d^2 < 512 2^118 fits 128 bits
-constexpr int FX_SPILL = 16;             // dimensions whose products fit the 64-bit sums
 
-struct fx_coord {  // q = hi 2^30 + lo
+// Limbs by the dimension: a coordinate of fx_coord_bits(m) bits, q = hi 2^LB + lo
+// with LB = fx_limb_of(m).  31 + 30 bits while four dimensions' products fit
+// the 64-bit sums, 30 + 29 bits for 16 dimensions and, with the sums emptied
+// every 16, any more.  The finer grid at m <= 4 is for the pairs too close for
+// it (fx_close), which are common in few dimensions: the 8-component cloud of
+// 16,384 points in R^3 sends 20% of its warps to FP64 with 59 bits, 0.3% with
+// 61 (generation 2.35 and 1.7 ms).
+constexpr int FX_LOW_DIM = 4;
+constexpr int FX_SPILL = 16;
+FX_HD int fx_limb_of(int m) { return m <= FX_LOW_DIM ? 31 : 30; }
+FX_HD int fx_coord_bits(int m) { return 2 * fx_limb_of(m) - 1; }
+
+struct fx_coord {
   int lo, hi;
 };
 
@@ -132,16 +141,17 @@ struct FxSquare {
   fx_u64 h, l;
 };
 FX_HD void fx_square_clear(FxSquare& q) { q.h = 0, q.l = 0; }
-// q += C 2^60 + Bx 2^31 + A
+// q += C 2^(2 LB) + Bx 2^(LB + 1) + A
+template <int LB>
 FX_HD void fx_add(FxSquare& q, const FxSums& s) {
   fx_u64 l = q.l + s.A;
   fx_u64 h = q.h + (l < s.A ? 1 : 0);
-  const fx_u64 bl = (fx_u64)s.Bx << 31;
+  const fx_u64 bl = (fx_u64)s.Bx << (LB + 1);
   l += bl;
-  h += (fx_u64)(s.Bx >> 33) + (l < bl ? 1 : 0);
-  const fx_u64 cl = s.C << 60;
+  h += (fx_u64)(s.Bx >> (63 - LB)) + (l < bl ? 1 : 0);
+  const fx_u64 cl = s.C << (2 * LB);
   l += cl;
-  h += (s.C >> 4) + (l < cl ? 1 : 0);
+  h += (s.C >> (64 - 2 * LB)) + (l < cl ? 1 : 0);
   q.h = h, q.l = l;
 }
 // Pairs this close (d < sqrt(m) 2^(53-e)) take the FP64 differences.
@@ -312,16 +322,23 @@ __device__ __forceinline__ void load_fx_table(fx_u64* tab) {
 // The pairs of one 128 x 128 tile (rows row0 .., columns col0 .. of the n
 // quantized points Xq), 256 threads: f(r, q) is called once for every row r =
 // warp + 8 i of the tile with the squares q[4] of the lane's columns 4 lane ..
-// 4 lane + 3.  R rows are accumulated together: one while the dimensions fit
-// the 64-bit sums (the column reads then hide behind the finishing work), two
-// beyond, where the reads would set the pace.  smem: fx_tile_smem bytes.
+// 4 lane + 3.  KIND: 0 for m <= FX_LOW_DIM, 1 for m <= FX_SPILL, 2 beyond.
+// Beyond FX_SPILL two rows are accumulated together, where the column reads
+// would set the pace; below, one (they hide behind the finishing work).  smem:
+// fx_tile_smem bytes.
 constexpr int FX_THREADS = 256;
+inline int fx_kind(int m) { return m <= FX_LOW_DIM ? 0 : (m <= FX_SPILL ? 1 : 2); }
+// CTAs per SM the kernels over tiles are compiled for: one row at a time fits
+// 80 registers, and three CTAs hide more of the multiplier's latency than two
+// (n = 16,384, m = 8: 1.79 against 1.95 ms); two rows need 128.
+constexpr int fx_ctas(int kind) { return kind < 2 ? 3 : 2; }
 constexpr int FX_CHUNK = 32;  // dimensions staged at a time
 inline size_t fx_tile_smem(int m) { return 2 * (size_t)128 * (m < FX_CHUNK ? m : FX_CHUNK) * sizeof(fx_coord); }
 
-template <int R, class F>
+template <int KIND, class F>
 __device__ __forceinline__ void fx_tile_pairs(const fx_coord* __restrict__ Xq, int64_t n, int m, int64_t row0,
                                               int64_t col0, fx_coord* smem, F&& f) {
+  constexpr int R = KIND < 2 ? 1 : 2, LB = KIND == 0 ? 31 : 30;
   const int mc = m < FX_CHUNK ? m : FX_CHUNK;
   fx_coord* xr = smem;              // [128][mc] row points (broadcast reads)
   fx_coord* xc = smem + 128 * mc;   // [mc][128]: column 4 l + q at 32 q + l (conflict free)
@@ -374,7 +391,7 @@ __device__ __forceinline__ void fx_tile_pairs(const fx_coord* __restrict__ Xq, i
         for (int k = 0; k < R; ++k)
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            fx_add(q[k][c], s[k][c]);
+            fx_add<LB>(q[k][c], s[k][c]);
             if (R > 1) fx_clear(s[k][c]);
           }
       }

@@ -135,6 +135,12 @@ cudaError_t launch_generate_q(const void* Xq, const double* X, int64_t n, int m,
                               float* Zf, double* Zd, double* rowsum, DevStatus* st, cudaStream_t s,
                               int kind = MAT_EXP, double tiny_arg = INFINITY, double kc = 0.0, int64_t t0 = 0,
                               int64_t W = -1);
+// Z = exp(-t d) as the dense n x n row-major matrix from the quantized
+// coordinates, entries as launch_generate_q with every entry exact; min d^2
+// and ST_DUPLICATE into st.
+template <typename T>
+cudaError_t launch_dense_q(const void* Xq, const double* X, int64_t n, int m, int e, double t, T* Z, DevStatus* st,
+                           cudaStream_t s);
 // FP32 tiles of one slab for the out-of-core factor: global tile columns
 // [t0, t0 + W) of rows [t0, N), in the slab layout (tile_index with column
 // cap W, tile (0, 0) = global (t0, t0)); no row sums; min d^2 and flags as

@@ -128,3 +128,26 @@ def test_min_distance_errors(ctx):
     with pytest.raises(M.MagnitudeError) as e:  # every distance overflows
         ctx.min_distance(_dev(X * 1e300))
     assert e.value.status == M.MAG_EINVAL
+
+
+# The integer-pipe distances and exponential on the GPU, by the three limb
+# layouts (m <= 4, m <= 16, beyond, with and without a second chunk of 32
+# dimensions), ragged and whole tiles, pairs too close for the quantized
+# coordinates among them, through the dense output and through a solve's tiles:
+# |dZ| <= 1 ulp of exp + t |d d|, each side's d within (m / 2 + 3) u of exact.
+@pytest.mark.parametrize("n", [2, 127, 128, 131, 300])
+@pytest.mark.parametrize("m", [1, 4, 5, 16, 17, 32, 33, 100])
+def test_similarity_entries(ctx, n, m):
+    rng = np.random.default_rng(n * 1000 + m)
+    X = rng.standard_normal((n, m))
+    X[n // 2] = X[0] + 1e-9 * rng.standard_normal(m)  # closer than the quantized coordinates resolve
+    t = 1.5 / np.sqrt(m)
+    d = np.sqrt(((X[:, None, :].astype(np.longdouble) - X[None, :, :]) ** 2).sum(-1))
+    Z = np.exp(-t * d.astype(np.float64))
+    tol = 2.0 ** -52 * (1.0 + (m / 2 + 4) * t * d) * Z
+    Zg = ctx.similarity_matrix(_dev(X), t, "fp64").cpu().numpy()
+    assert np.all(np.abs(Zg - Z) <= tol)
+    Zf = ctx.similarity_matrix(_dev(X), t, "fp32").cpu().numpy()
+    assert np.all(np.abs(Zf - Z) <= 2.0 ** -24 * Z + tol)
+    L = ctx.cholesky_factor(_dev(X), t, "fp64").cpu().numpy()
+    assert np.abs(L @ L.T - Z).max() <= (n + 5) * 2.0 ** -53 + tol.max()
