@@ -446,14 +446,28 @@ __global__ void __launch_bounds__(SYM_THREADS, 1)
 }
 
 // k_resid_sym with the pairs from quantized coordinates (mag_fx.cuh; pairs too
-// close for them from the FP64 differences of X), Z = exp(-t d) only: the two
-// products of an entry are its only FP64 operations.  Thread layout of
-// fx_tile_pairs: warp w takes rows w + 8 i, lane l columns 4 l .. 4 l + 3; a
-// row's lane sums are added from shared memory (one FP64 addition per 32
-// instead of five shuffle levels each).
+// close for them from the FP64 differences of X), Z = exp(-t d) only: the
+// products and sums of an entry are its only FP64 operations, and run beside
+// its integer ones.  Thread layout of fx_tile_pairs: warp w takes rows w + 8 i,
+// lane l columns 4 l .. 4 l + 3; a row's 32 lane sums are added from shared
+// memory.
+//
+// COMP (the residual entry points): every sum compensated beyond chains of
+// four FMAs -- a row's lane sums and a column's groups of four rows by TwoSum
+// with the errors carried along, P as (sum, error) pairs, the row sums of Z
+// exact in 128-bit fixed point up to 2^-64 an entry -- which costs five FP64
+// operations a pair instead of two and still stays below the integer work's
+// time.  The solver's own residual (COMP false) takes FMA chains and FP32 norms.
 constexpr int SYMQ_LD = 33;
 
-template <int KIND>
+// s + c <- s + c + x with the rounding of s collected in c
+__device__ __forceinline__ void add_comp(double& s, double& c, double x) {
+  const double t = s + x, bv = t - s;
+  c += (s - (t - bv)) + (x - bv);
+  s = t;
+}
+
+template <int KIND, bool COMP>
 __global__ void __launch_bounds__(FX_THREADS, 2)
     k_resid_sym_q(const fx_coord* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, FxScale sc,
                   const double* __restrict__ w, double* __restrict__ P, double* __restrict__ rowsum, int64_t N) {
@@ -461,7 +475,9 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
   double* rowacc = reinterpret_cast<double*>(symq_smem);  // [TILE][SYMQ_LD]: a row's lane sums
   fx_coord* stage = reinterpret_cast<fx_coord*>(rowacc + TILE * SYMQ_LD);
   __shared__ double colpart[FX_THREADS / 32][TILE];
+  __shared__ double colerr[COMP ? FX_THREADS / 32 : 1][TILE];
   __shared__ float zcol[FX_THREADS / 32][TILE];
+  __shared__ fx_u64 zcol_l[COMP ? TILE : 1], zcol_h[COMP ? TILE : 1];
   __shared__ fx_u64 fxtab[FX_TABLE_SIZE];
   __shared__ double s_wr[TILE];
   load_fx_table(fxtab);
@@ -469,80 +485,208 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
   tri_coords((int64_t)blockIdx.x, &I, &J);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t row0 = I * TILE, col0 = J * TILE;
-  if (threadIdx.x < TILE) s_wr[threadIdx.x] = row0 + threadIdx.x < n ? w[row0 + threadIdx.x] : 0.0;
-  double wc[4], cs[4];
+  if (threadIdx.x < TILE) {
+    s_wr[threadIdx.x] = row0 + threadIdx.x < n ? w[row0 + threadIdx.x] : 0.0;
+    if (COMP) zcol_l[threadIdx.x] = zcol_h[threadIdx.x] = 0;
+  }
+  double wc[4], cs[4], cc[4], ch[4];  // column sums: this group's chain, the sum and its error
   float zc[4];
+  fx_u64 zcl[4];   // COMP: column sums of Z in units of 2^-63 (16 entries of at most 2^63: the top in zch)
+  unsigned zch[4];
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const int64_t gc = col0 + 4 * lane + c;
     wc[c] = gc < n ? w[gc] : 0.0;
-    cs[c] = 0.0;
+    cs[c] = cc[c] = ch[c] = 0.0;
     zc[c] = 0.0f;
+    zcl[c] = 0;
+    zch[c] = 0;
   }
   fx_tile_pairs<KIND>(Xq, n, m, row0, col0, stage, [&](int r, FxSquare(&q)[4]) {
     const int64_t gr = row0 + r;
     const double wr = s_wr[r];
     double v = 0.0;
     float zv = 0.0f;
+    fx_u64 zl = 0;
+    unsigned zh = 0;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int64_t gc = col0 + 4 * lane + c;
       double z = 0.0;
+      fx_u64 zx = 0;  // the entry in units of 2^-63
       if (gr < n && gc < n) {
         if (gr == gc) {
           z = 1.0;
-        } else if (fx_close(q[c], m)) {
-          double d2 = 0.0;
-          for (int l = 0; l < m; ++l) {
-            const double diff = X[gr * m + l] - X[gc * m + l];
-            d2 = fma(diff, diff, d2);
-          }
-          const fx_u64 db = (fx_u64)__double_as_longlong(sqrt_pos(d2));
-          z = __longlong_as_double((long long)fx_exp_neg_d(db, sc.kg, sc.g, fxtab));
+          zx = 1ull << 63;
         } else {
-          const FxRoot rt = fx_root_start(q[c]);
-          const float td = fx_float(fx_bits(rt.sf) + ((uint32_t)(rt.j - 63) << 23)) * sc.t63;
-          z = td > (float)kTinyArg
-                  ? f32_to_f64_nonneg(exp_neg_tiny_f(td))
-                  : __longlong_as_double((long long)fx_exp_neg(fx_root(rt), rt.j - sc.e + sc.kg, sc.g, fxtab));
+          fx_u64 dm;
+          int k;
+          bool tiny = false;
+          if (fx_close(q[c], m)) {
+            double d2 = 0.0;
+            for (int l = 0; l < m; ++l) {
+              const double diff = X[gr * m + l] - X[gc * m + l];
+              d2 = fma(diff, diff, d2);
+            }
+            const fx_u64 db = (fx_u64)__double_as_longlong(sqrt_pos(d2));
+            dm = (db >> 52 ? (db & 0xfffffffffffffull) | 0x10000000000000ull : db) << 10;
+            k = (db >> 52 ? (int)(db >> 52) : 1) - 1023 + sc.kg;
+          } else {
+            const FxRoot rt = fx_root_start(q[c]);
+            const float td = fx_float(fx_bits(rt.sf) + ((uint32_t)(rt.j - 63) << 23)) * sc.t63;
+            tiny = !COMP && td > (float)kTinyArg;
+            if (tiny) z = f32_to_f64_nonneg(exp_neg_tiny_f(td));
+            dm = tiny ? 0 : fx_root(rt);
+            k = rt.j - sc.e + sc.kg;
+          }
+          if (!tiny) {
+            int shift;
+            const fx_u64 zf = fx_exp_fixed(dm, k, sc.g, fxtab, &shift);
+            z = __longlong_as_double((long long)fx_pack(zf, shift));
+            if (COMP) zx = shift < 64 ? zf >> shift : 0;
+          }
         }
       }
       v = fma(z, wc[c], v);
-      cs[c] = fma(z, wr, cs[c]);
-      const float zf = f64_to_f32_nonneg(z);
-      zv += zf;
-      zc[c] += zf;
+      ch[c] = fma(z, wr, ch[c]);
+      if (COMP) {
+        zl += zx;
+        zh += zl < zx ? 1u : 0u;
+        zcl[c] += zx;
+        zch[c] += zcl[c] < zx ? 1u : 0u;
+      } else {
+        const float zf = f64_to_f32_nonneg(z);
+        zv += zf;
+        zc[c] += zf;
+      }
     }
     rowacc[r * SYMQ_LD + lane] = v;
+    if (COMP) {
+      if ((r >> 3 & 3) == 3) {  // four rows of this warp: fold the chains
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) zv += __shfl_xor_sync(0xffffffffu, zv, o);
-    if (lane == 0 && gr < n) atomicAdd(rowsum + gr, (double)zv);
+        for (int c = 0; c < 4; ++c) {
+          add_comp(cs[c], cc[c], ch[c]);
+          ch[c] = 0.0;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const fx_u64 ol = __shfl_xor_sync(0xffffffffu, zl, o);
+        zh += __shfl_xor_sync(0xffffffffu, zh, o);
+        zl += ol;
+        zh += zl < ol ? 1u : 0u;
+      }
+      // units of 2^-63, 2^64 of them in zh: to FP64 from the two halves
+      if (lane == 0 && gr < n) atomicAdd(rowsum + gr, fma((double)zh, 2.0, (double)zl * 0x1p-63));
+    } else {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) zv += __shfl_xor_sync(0xffffffffu, zv, o);
+      if (lane == 0 && gr < n) atomicAdd(rowsum + gr, (double)zv);
+    }
   });
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    colpart[warp][4 * lane + c] = cs[c];
-    zcol[warp][4 * lane + c] = zc[c];
+    const int col = 4 * lane + c;
+    colpart[warp][col] = COMP ? cs[c] : ch[c];
+    if (COMP) {
+      colerr[warp][col] = cc[c];
+      if (I != J) {  // two words of 32-bit halves: neither sum can wrap
+        atomicAdd(&zcol_l[col], zcl[c] & 0xffffffffull);
+        atomicAdd(&zcol_h[col], (zcl[c] >> 32) + ((fx_u64)zch[c] << 32));
+      }
+    } else {
+      zcol[warp][col] = zc[c];
+    }
   }
   __syncthreads();
   if (threadIdx.x < TILE) {
     // rows of block I: P[I][J]
     const double* ra = rowacc + threadIdx.x * SYMQ_LD;
-    double v0 = 0.0, v1 = 0.0;
+    if (COMP) {
+      double s = ra[0], e = 0.0;
 #pragma unroll 4
-    for (int k = 0; k < 32; k += 2) v0 += ra[k], v1 += ra[k + 1];
-    P[(I * N + J) * TILE + threadIdx.x] = v0 + v1;
+      for (int k = 1; k < 32; ++k) add_comp(s, e, ra[k]);
+      reinterpret_cast<double2*>(P)[(I * N + J) * TILE + threadIdx.x] = make_double2(s, e);
+    } else {
+      double v0 = 0.0, v1 = 0.0;
+#pragma unroll 4
+      for (int k = 0; k < 32; k += 2) v0 += ra[k], v1 += ra[k + 1];
+      P[(I * N + J) * TILE + threadIdx.x] = v0 + v1;
+    }
   } else if (I != J) {
     // rows of block J (the transposed tile): P[J][I]; a diagonal tile's rows cover both triangles
     const int c = threadIdx.x - TILE;
-    double v = 0.0;
-    float z = 0.0f;
+    if (COMP) {
+      double s = colpart[0][c], e = colerr[0][c];
 #pragma unroll
-    for (int k = 0; k < FX_THREADS / 32; ++k) {
-      v += colpart[k][c];
-      z += zcol[k][c];
+      for (int k = 1; k < FX_THREADS / 32; ++k) {
+        add_comp(s, e, colpart[k][c]);
+        e += colerr[k][c];
+      }
+      reinterpret_cast<double2*>(P)[(J * N + I) * TILE + c] = make_double2(s, e);
+      if (col0 + c < n)
+        atomicAdd(rowsum + col0 + c, fma((double)zcol_h[c], 0x1p-31, (double)zcol_l[c] * 0x1p-63));
+    } else {
+      double v = 0.0;
+      float z = 0.0f;
+#pragma unroll
+      for (int k = 0; k < FX_THREADS / 32; ++k) {
+        v += colpart[k][c];
+        z += zcol[k][c];
+      }
+      P[(J * N + I) * TILE + c] = v;
+      if (col0 + c < n) atomicAdd(rowsum + col0 + c, (double)z);
     }
-    P[(J * N + I) * TILE + c] = v;
-    if (col0 + c < n) atomicAdd(rowsum + col0 + c, (double)z);
+  }
+}
+
+// r_j = b_j - (the N partial pairs of row j, compensated), and the three
+// norms; eight threads a row, each every eighth partial.
+__global__ void __launch_bounds__(256) k_resid_comp_finish(const double2* __restrict__ P, int64_t n, int64_t N,
+                                                           const double* __restrict__ w, const double* __restrict__ b,
+                                                           const double* __restrict__ rowsum, double* __restrict__ r,
+                                                           DevStatus* st) {
+  __shared__ double2 part[8][32];
+  const int row = threadIdx.x & 31, k = threadIdx.x >> 5;
+  const int64_t j = (int64_t)blockIdx.x * 32 + row;
+  double s = 0.0, e = 0.0;
+  if (j < n) {
+    const int64_t I = j / TILE, rr = j % TILE;
+    const double2* p = P + I * N * TILE + rr;
+#pragma unroll 4
+    for (int64_t J = k; J < N; J += 8) {
+      const double2 v = p[J * TILE];
+      add_comp(s, e, v.x);
+      e += v.y;
+    }
+  }
+  part[k][row] = make_double2(s, e);
+  __syncthreads();
+  if (k) return;
+  double ra = 0.0, za = 0.0, wa = 0.0;
+  if (j < n) {
+#pragma unroll
+    for (int i = 1; i < 8; ++i) {
+      add_comp(s, e, part[i][row].x);
+      e += part[i][row].y;
+    }
+    const double bj = b ? b[j] : 1.0;
+    const double rj = (bj - s) - e;
+    r[j] = rj;
+    ra = fabs(rj);
+    za = rowsum[j];
+    wa = fabs(w[j]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    ra = fmax(ra, __shfl_xor_sync(0xffffffffu, ra, o));
+    za = fmax(za, __shfl_xor_sync(0xffffffffu, za, o));
+    wa = fmax(wa, __shfl_xor_sync(0xffffffffu, wa, o));
+  }
+  if (row == 0) {
+    atomic_max_nonneg(&st->r_max_bits, ra);
+    atomic_max_nonneg(&st->z_max_bits, za);
+    atomic_max_nonneg(&st->w_max_bits, wa);
   }
 }
 
@@ -933,13 +1077,14 @@ cudaError_t launch_residual_mf(const double* X, int64_t n, int m, double t, cons
                                const double* b, double* r, double* part, int chunks, int64_t np,
                                DevStatus* st, cudaStream_t s, int kind, double kc) {
   if (m < 1 || m > MAG_MAX_DIM) return cudaErrorInvalidValue;
+  // with the 8 KB exponential table within the default 48 KB
   int ct = 128;
-  while (ct > 8 && (size_t)ct * (m + 1) * sizeof(double) > 44 * 1024) ct /= 2;
+  while (ct > 8 && (size_t)ct * (m + 1) * sizeof(double) > 40 * 1024) ct /= 2;
   const size_t smem = (size_t)ct * (m + 1) * sizeof(double);
   const dim3 grid(blocks_for(n, RES_THREADS), (unsigned)chunks);
-  if (smem > 44 * 1024) {
+  if (smem > 40 * 1024) {
     // large m: eight column points per stage need more than the default
-    // 48 KB of static (4 KB exp table) plus dynamic shared memory; at most
+    // 48 KB of static (8 KB exp table) plus dynamic shared memory; at most
     // 8 x 2049 doubles = 131 KB
     cudaError_t e = cudaFuncSetAttribute(k_resid_mf<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -974,7 +1119,7 @@ cudaError_t launch_residual_sym(const double* X, int64_t n, int m, double t, con
     const FxScale sc = fx_scale(t, qe);
     const size_t sq = (size_t)TILE * SYMQ_LD * sizeof(double) + fx_tile_smem(m);
     const int kd = fx_kind(m);
-    auto kern = kd == 0 ? k_resid_sym_q<0> : (kd == 1 ? k_resid_sym_q<1> : k_resid_sym_q<2>);
+    auto kern = kd == 0 ? k_resid_sym_q<0, false> : (kd == 1 ? k_resid_sym_q<1, false> : k_resid_sym_q<2, false>);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sq);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)tiles, FX_THREADS, sq, s>>>(static_cast<const fx_coord*>(Xq), X, n, m, sc, w, P, rowsum, N);
@@ -987,6 +1132,35 @@ cudaError_t launch_residual_sym(const double* X, int64_t n, int m, double t, con
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_resid_sym_finish<<<blocks_for(np, 256), 256, 0, s>>>(P, n, N, np, w, b, rowsum, r, st);
+  note_launch();
+  return cudaGetLastError();
+}
+
+size_t residual_comp_bytes(int64_t n) {
+  const size_t N = (size_t)((n + TILE - 1) / TILE);
+  return N * N * TILE * sizeof(double2) + N * TILE * sizeof(double);
+}
+
+cudaError_t launch_residual_comp(const void* Xq, const double* X, int64_t n, int m, int qe, double t, const double* w,
+                                 const double* b, double* r, void* scratch, DevStatus* st, cudaStream_t s) {
+  if (m < 1 || m > FX_MAX_DIM) return cudaErrorInvalidValue;
+  const int64_t N = (n + TILE - 1) / TILE, tiles = num_lower_tiles(N);
+  if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  double* P = static_cast<double*>(scratch);
+  double* rowsum = P + 2 * N * N * TILE;
+  cudaError_t e = cudaMemsetAsync(rowsum, 0, (size_t)n * sizeof(double), s);
+  if (e != cudaSuccess) return e;
+  const FxScale sc = fx_scale(t, qe);
+  const size_t sq = (size_t)TILE * SYMQ_LD * sizeof(double) + fx_tile_smem(m);
+  const int kd = fx_kind(m);
+  auto kern = kd == 0 ? k_resid_sym_q<0, true> : (kd == 1 ? k_resid_sym_q<1, true> : k_resid_sym_q<2, true>);
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sq);
+  if (e != cudaSuccess) return e;
+  kern<<<(unsigned)tiles, FX_THREADS, sq, s>>>(static_cast<const fx_coord*>(Xq), X, n, m, sc, w, P, rowsum, N);
+  note_launch();
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_resid_comp_finish<<<blocks_for(n, 32), 256, 0, s>>>(reinterpret_cast<const double2*>(P), n, N, w, b, rowsum, r, st);
   note_launch();
   return cudaGetLastError();
 }
@@ -1097,7 +1271,7 @@ cudaError_t launch_grad(const double* X, int64_t n, int m, double t, const doubl
                         cudaStream_t s) {
   (void)np;
   int ct = 128;
-  while (ct > 8 && (size_t)ct * (m + 2) * sizeof(double) > 44 * 1024) ct /= 2;  // + 4 KB exp table
+  while (ct > 8 && (size_t)ct * (m + 2) * sizeof(double) > 40 * 1024) ct /= 2;  // + 8 KB exp table
   const size_t smem = (size_t)ct * (m + 2) * sizeof(double);
   const unsigned grid = blocks_for(n, RES_THREADS);
   if (m <= 8)

@@ -151,6 +151,8 @@ struct mag_ctx {
   int32_t xq_m = 0;
   int xq_e = 0;
   const void* xq_q = nullptr;
+  void* rp = nullptr;                // partial sums of mag_residual
+  size_t rp_bytes = 0;
   void* lh = nullptr;
   size_t lh_bytes = 0;
   bool chain_ready = false;          // chain_s holds the B tiles of the current factor
@@ -1069,6 +1071,7 @@ int mag_ctx_destroy(mag_ctx* ctx) {
   if (ctx->probe_z) cudaFree(ctx->probe_z);
   if (ctx->chain_s) cudaFree(ctx->chain_s);
   if (ctx->xq) cudaFree(ctx->xq);
+  if (ctx->rp) cudaFree(ctx->rp);
   if (ctx->lh) cudaFree(ctx->lh);
   if (ctx->host_L) cudaFreeHost(ctx->host_L);
   for (auto& kv : ctx->task_tables)
@@ -2488,7 +2491,18 @@ int mag_residual(mag_ctx* ctx, const double* points, int64_t n, int32_t m, doubl
   // r_out holds exactly n entries, so the residual kernel gets n as its row
   // stride and padding length.
   double* r = r_out ? r_out : ctx->vd(V_R);
-  CU(launch_residual_mf(points, n, m, t, w, b, r, ctx->part(), L.chunks, n, ctx->st(), s));
+  // every pair once, from the quantized coordinates, where they and the
+  // partial sums (16 bytes per tile and row) fit in an eighth of the free
+  // memory; else every entry of the square from FP64 differences
+  const size_t need = residual_comp_bytes(n);
+  int qe = 0;
+  const void* Xq = nullptr;
+  const bool fits = ctx->opt.workspace_limit_bytes <= 0 ||
+                    (double)(ctx->ws_bytes + need) <= ctx->opt.workspace_limit_bytes;
+  if (fits && quantize_points(ctx, points, n, m, &qe, &Xq) && grow_buffer(ctx, &ctx->rp, &ctx->rp_bytes, need, 7 * need))
+    CU(launch_residual_comp(Xq, points, n, m, qe, t, w, b, r, ctx->rp, ctx->st(), s));
+  else
+    CU(launch_residual_mf(points, n, m, t, w, b, r, ctx->part(), L.chunks, n, ctx->st(), s));
   TRY(read_status(ctx));
   const double rn = bits_to_double(ctx->h_st->r_max_bits);
   const double zn = bits_to_double(ctx->h_st->z_max_bits);

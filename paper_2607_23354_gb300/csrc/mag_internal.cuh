@@ -335,6 +335,11 @@ cudaError_t launch_residual_mf(const double* X, int64_t n, int m, double t, cons
 cudaError_t launch_residual_sym(const double* X, int64_t n, int m, double t, const double* w, const double* b,
                                 double* r, double* P, double* rowsum, int64_t np, DevStatus* st, cudaStream_t s,
                                 int kind = MAT_EXP, double kc = 0.0, const void* Xq = nullptr, int qe = 0);
+// The compensated residual of the entry point from quantized coordinates (m <=
+// 512): scratch of residual_comp_bytes.  Same outputs; r has n entries.
+size_t residual_comp_bytes(int64_t n);
+cudaError_t launch_residual_comp(const void* Xq, const double* X, int64_t n, int m, int qe, double t, const double* w,
+                                 const double* b, double* r, void* scratch, DevStatus* st, cudaStream_t s);
 // Stored: P is scratch of N * N * 128 doubles (one partial per row block,
 // tile and row); rowsum holds the row sums of Z from the generator.
 cudaError_t launch_residual_stored(const double* Zd, int64_t n, int64_t N, const double* w,

@@ -151,3 +151,44 @@ def test_similarity_entries(ctx, n, m):
     assert np.all(np.abs(Zf - Z) <= 2.0 ** -24 * Z + tol)
     L = ctx.cholesky_factor(_dev(X), t, "fp64").cpu().numpy()
     assert np.abs(L @ L.T - Z).max() <= (n + 5) * 2.0 ** -53 + tol.max()
+
+
+# The residual entry point over the lower triangle: rows and columns of every
+# tile, ragged ones, each limb layout, coincident and close pairs, an explicit
+# b, weights of both signs over twelve decades.  Against FP64 sums of the same
+# entries: |dr_j| <= sum_k (|dZ_jk| + 2^-52 Z_jk) |w_k|, dZ as for the entries.
+@pytest.mark.parametrize("n", [2, 128, 129, 300, 1000])
+@pytest.mark.parametrize("m", [2, 9, 40])
+def test_residual_rows(ctx, n, m):
+    rng = np.random.default_rng(n + m)
+    X = rng.standard_normal((n, m))
+    X[n - 1] = X[0]
+    if n > 2:
+        X[n // 2] = X[1] + 1e-10
+    t = 2.0 / np.sqrt(m)
+    w = rng.standard_normal(n) * 10.0 ** rng.uniform(-6, 6, n)
+    b = rng.standard_normal(n)
+    d = np.sqrt(((X[:, None, :].astype(np.longdouble) - X[None, :, :]) ** 2).sum(-1))
+    Z = np.exp(-t * d.astype(np.float64))
+    tol = (2.0 ** -52 * (2.0 + (m / 2 + 4) * (t * d).astype(np.float64)) * Z) @ np.abs(w) + 2.0 ** -52 * np.abs(b)
+    for bb in (None, b):
+        r, nr = ctx.residual(_dev(X), t, _dev(w), b=None if bb is None else _dev(bb))
+        ref = ((1.0 if bb is None else bb) - Z.astype(np.longdouble) @ w).astype(np.float64)
+        assert np.all(np.abs(r.cpu().numpy() - ref) <= tol)
+        assert abs(nr["z_norm_inf"] - Z.sum(1).max()) <= 1e-14 * Z.sum(1).max()
+        assert nr["w_norm_inf"] == np.abs(w).max()
+        assert nr["r_norm_inf"] == float(r.abs().max())
+
+
+# Dimensions at which the column stage, beside the exponential's 8 KB table,
+# reaches the default 48 KB of shared memory (both refused the launch before).
+@pytest.mark.parametrize("m", [38, 40, 42, 83, 86, 640])
+def test_staging_fits_shared_memory(ctx, m):
+    X = _dev(np.random.default_rng(m).standard_normal((70, m)))
+    w = _dev(np.random.default_rng(1).standard_normal(70))
+    t = 1.0 / np.sqrt(m)
+    r, _ = M.residual_noalloc(X, t, w)
+    assert float((r - (1.0 - _z(X, t) @ w)).abs().max()) <= 1e-13
+    if m <= 64:
+        _, dx = ctx.grad(X, t, w=w)
+        assert bool(torch.isfinite(dx).all())
