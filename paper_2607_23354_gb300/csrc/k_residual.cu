@@ -897,72 +897,221 @@ __global__ void __launch_bounds__(1024) k_reduce_w(const double* __restrict__ w,
   }
 }
 
-// K7: for row i, with u_ik = (x_i - x_k)/d_ik,
-//   part_t[i] = sum_{k != i} lam_i d_ik Z_ik w_k          (sum_i part_t[i] = lam^T (d o Z) w)
-//   dL_dx[i]  = t sum_{k != i} Z_ik u_ik (lam_i w_k + lam_k w_i).
-// One thread per row i, columns staged in shared memory, coordinates in FP64.
-template <int MR>
-__global__ void __launch_bounds__(RES_THREADS) k_grad(const double* __restrict__ X, int64_t n,
-                                                      int m, double t,
-                                                      const double* __restrict__ w,
-                                                      const double* __restrict__ lam,
-                                                      double* __restrict__ dL_dx,
-                                                      double* __restrict__ part_t, int ct) {
-  extern __shared__ double sm[];
-  double* xc = sm;                 // [ct][m]
-  double* wc = sm + ct * m;        // [ct]
-  double* lc = sm + ct * (m + 1);  // [ct]
-  __shared__ __align__(16) double exptab[EXPT_SMEM];
-  load_exp_table(exptab);
-  const int64_t i = (int64_t)blockIdx.x * RES_THREADS + threadIdx.x;
-  const bool live = i < n;
-  double xi[MR], g[MR];
-#pragma unroll
-  for (int l = 0; l < MR; ++l) {
-    xi[l] = (live && l < m) ? X[i * m + l] : 0.0;
-    g[l] = 0.0;
+// K7: gradients.  With u_ik = (x_i - x_k)/d_ik and s_ik = lam_i w_k + lam_k w_i,
+//   dL/dt    = sum_{i < k} d_ik Z_ik s_ik                  (lam^T (d o Z) w)
+//   dL/dx_i  = t sum_{k != i} Z_ik s_ik u_ik.
+// One CTA per lower tile: the coefficients G = Z s / d of its 128 x 128 pairs
+// go to shared memory, each pair once (fx: distance, exponential and reciprocal
+// in fixed point from the quantized coordinates; else FP64 from the points),
+// then every dimension's differences times G are summed along the rows and
+// along the columns: three FP64 operations per pair and dimension, which bound
+// the kernel.  Tiles leave their row and column sums in P (slot of the other
+// block, like the residual's), added by k_grad_finish; the order of every sum
+// is fixed.  A thread per row over all columns, with FP64 distances, a division
+// and twice the pairs, took 31 ms at n = 8192, m = 16 on 64 of the 152 SMs; 3.9
+// now.
+constexpr int GRAD_THREADS = 512;
+constexpr int GRAD_LD = TILE + 2;
+constexpr int GRAD_MC = 16;  // dimensions staged per chunk
+constexpr size_t GRAD_STAGE = (2 * GRAD_MC + 2 * (GRAD_THREADS / 32)) * (size_t)TILE * sizeof(double);  // 64 KB
+
+template <bool FX, int KIND>
+__global__ void __launch_bounds__(GRAD_THREADS, 1)
+    k_grad_tile(const fx_coord* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, FxScale sc, double t,
+                const double* __restrict__ w, const double* __restrict__ lam, double* __restrict__ P,
+                double* __restrict__ part_t, int64_t N, int64_t q0, int64_t I0) {
+  extern __shared__ __align__(16) unsigned char grad_smem[];
+  double* G = reinterpret_cast<double*>(grad_smem);  // [TILE][GRAD_LD]
+  unsigned char* stage = grad_smem + (size_t)TILE * GRAD_LD * sizeof(double);
+  __shared__ fx_u64 fxtab[FX ? FX_TABLE_SIZE : 2];
+  __shared__ __align__(16) double exptab[FX ? 2 : EXPT_SMEM];
+  __shared__ double s_w[TILE], s_l[TILE], s_t[GRAD_THREADS / 32];
+  if (FX)
+    load_fx_table(fxtab);
+  else
+    load_exp_table(exptab);
+  int64_t I, J;
+  tri_coords(q0 + (int64_t)blockIdx.x, &I, &J);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t row0 = I * TILE, col0 = J * TILE;
+  if (threadIdx.x < TILE) {
+    const int64_t gr = row0 + threadIdx.x;
+    s_w[threadIdx.x] = gr < n ? w[gr] : 0.0;
+    s_l[threadIdx.x] = gr < n ? lam[gr] : 0.0;
   }
-  const double wi = live ? w[i] : 0.0, li = live ? lam[i] : 0.0;
-  double st_s = 0.0, st_c = 0.0;
-  for (int64_t k0 = 0; k0 < n; k0 += ct) {
-    const int cnt = (int)min((int64_t)ct, n - k0);
+  double wc[4], lc[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int64_t gc = col0 + 4 * lane + c;
+    wc[c] = gc < n ? w[gc] : 0.0;
+    lc[c] = gc < n ? lam[gc] : 0.0;
+  }
+  double ts = 0.0, te = 0.0;  // dL/dt over this thread's pairs, compensated
+  // the pair's Z / d and its share of dL/dt from FP64 differences
+  auto by_differences = [&](int64_t gr, int64_t gc, double sik, double* tsum) {
+    double d2 = 0.0;
+    for (int l = 0; l < m; ++l) {
+      const double diff = X[gr * m + l] - X[gc * m + l];
+      d2 = fma(diff, diff, d2);
+    }
+    const double d = sqrt_pos(d2);
+    double z;
+    if constexpr (FX)
+      z = __longlong_as_double((long long)fx_exp_neg_d((fx_u64)__double_as_longlong(d), sc.kg, sc.g, fxtab));
+    else
+      z = exp_neg_td(t, d, exptab);
+    *tsum = fma(d * z, sik, *tsum);
+    return z / d * sik;
+  };
+  if constexpr (FX) {
+    fx_tile_pairs<KIND, GRAD_THREADS>(
+        Xq, n, m, row0, col0, reinterpret_cast<fx_coord*>(stage), [&](int r, FxSquare(&q)[4]) {
+          const int64_t gr = row0 + r;
+          double g[4], tsum = 0.0;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const int64_t gc = col0 + 4 * lane + c;
+            g[c] = 0.0;
+            if (gr < n && gc < n && gr != gc) {
+              const double sik = fma(s_l[r], wc[c], lc[c] * s_w[r]);
+              if (fx_close(q[c], m)) {
+                g[c] = by_differences(gr, gc, sik, &tsum);
+              } else {
+                const FxRoot rt = fx_root_start(q[c]);
+                const fx_u64 s = fx_root(rt);
+                int shift;
+                const fx_u64 z = fx_exp_fixed(s, rt.j - sc.e + sc.kg, sc.g, fxtab, &shift);
+                const fx_u64 zd = fx_mul_low(z, fx_recip(s, rt.y)) << 1;
+                g[c] = __longlong_as_double((long long)fx_pack_any(zd, shift + rt.j - sc.e)) * sik;
+                const double d2 = __longlong_as_double(
+                    (long long)(((fx_u64)(uint32_t)(2 * (rt.j - sc.e) + rt.par + 1022) << 52) + (rt.v >> 11) + ((rt.v >> 10) & 1u)));
+                tsum = fma(g[c], d2, tsum);
+              }
+            }
+          }
+          add_comp(ts, te, tsum);
+          *reinterpret_cast<double2*>(G + r * GRAD_LD + 4 * lane) = make_double2(g[0], g[1]);
+          *reinterpret_cast<double2*>(G + r * GRAD_LD + 4 * lane + 2) = make_double2(g[2], g[3]);
+        });
+  } else {
     __syncthreads();
-    for (int e = threadIdx.x; e < cnt * m; e += RES_THREADS) xc[e] = X[k0 * m + e];
-    for (int e = threadIdx.x; e < cnt; e += RES_THREADS) {
-      wc[e] = w[k0 + e];
-      lc[e] = lam[k0 + e];
+#pragma unroll 1
+    for (int i = 0; i < TILE / (GRAD_THREADS / 32); ++i) {
+      const int r = warp + GRAD_THREADS / 32 * i;
+      const int64_t gr = row0 + r;
+      double tsum = 0.0;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int64_t gc = col0 + 4 * lane + c;
+        double g = 0.0;
+        if (gr < n && gc < n && gr != gc)
+          g = by_differences(gr, gc, fma(s_l[r], wc[c], lc[c] * s_w[r]), &tsum);
+        G[r * GRAD_LD + 4 * lane + c] = g;
+      }
+      add_comp(ts, te, tsum);
+    }
+  }
+  // the tile's share of dL/dt (a diagonal tile holds every pair twice)
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double os = __shfl_xor_sync(0xffffffffu, ts, o), oe = __shfl_xor_sync(0xffffffffu, te, o);
+    add_comp(ts, te, os);
+    te += oe;
+  }
+  if (lane == 0) s_t[warp] = ts + te;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0, e = 0.0;
+    for (int k = 0; k < GRAD_THREADS / 32; ++k) add_comp(s, e, s_t[k]);
+    part_t[q0 + blockIdx.x] = I == J ? 0.5 * (s + e) : s + e;
+  }
+
+  // lane: columns lane + 32 j (j < 4), warp: rows warp + 16 i (i < 8)
+  double* xr = reinterpret_cast<double*>(stage);  // [GRAD_MC][TILE] row points
+  double* xc = xr + GRAD_MC * TILE;               // [GRAD_MC][TILE] column points
+  double* colp = xc + GRAD_MC * TILE;             // [2][warps][TILE] column sums of a dimension, by its parity
+  constexpr int NW = GRAD_THREADS / 32;
+  double g[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) g[i][j] = G[(warp + NW * i) * GRAD_LD + lane + 32 * j];
+  double* prow = P + ((I - I0) * 2 * N + J) * m * TILE;          // this tile's row sums
+  double* pcol = P + ((I - I0) * 2 * N + N + J) * m * TILE;      // and column sums
+  for (int l0 = 0; l0 < m; l0 += GRAD_MC) {
+    const int mc = min(GRAD_MC, m - l0);
+    __syncthreads();  // the previous chunk, or the squares' staging, has been read
+    for (int e = threadIdx.x; e < TILE * mc; e += GRAD_THREADS) {
+      const int r = e / mc, l = e - r * mc;
+      xr[l * TILE + r] = row0 + r < n ? X[(row0 + r) * m + l0 + l] : 0.0;
+      xc[l * TILE + r] = col0 + r < n ? X[(col0 + r) * m + l0 + l] : 0.0;
     }
     __syncthreads();
-    if (!live) continue;
-    for (int q = 0; q < cnt; ++q) {
-      if (k0 + q == i) continue;
-      const double* xk = xc + q * m;
-      double d2 = 0.0;
+    for (int l = 0; l < mc; ++l) {
+      double rs[8], cs[4], b[4];
 #pragma unroll
-      for (int l = 0; l < MR; ++l)
-        if (l < m) {
-          const double diff = xi[l] - xk[l];
-          d2 = fma(diff, diff, d2);
+      for (int j = 0; j < 4; ++j) {
+        b[j] = xc[l * TILE + lane + 32 * j];
+        cs[j] = 0.0;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const double a = xr[l * TILE + warp + NW * i];
+        rs[i] = 0.0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const double diff = a - b[j];
+          rs[i] = fma(g[i][j], diff, rs[i]);
+          cs[j] = fma(g[i][j], diff, cs[j]);
         }
-      const double d = sqrt_pos(d2);
-      const double z = exp_neg_td(t, d, exptab);
-      // dL/dt contribution with Kahan compensation
-      const double y = fma(li * d * z, wc[q], -st_c);
-      const double tt = st_s + y;
-      st_c = (tt - st_s) - y;
-      st_s = tt;
-      const double coef = t * z * (li * wc[q] + lc[q] * wi) / d;
+      }
+      // eight row sums over 32 lanes: halve the rows with the lanes, then the
+      // last two levels; lane 4 k ends with row k' = its three top bits
 #pragma unroll
-      for (int l = 0; l < MR; ++l)
-        if (l < m) g[l] = fma(coef, xi[l] - xk[l], g[l]);
+      for (int h = 4, o = 16; h > 0; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < h) {
+            const double send = up ? rs[i] : rs[i + h], keep = up ? rs[i + h] : rs[i];
+            rs[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+      }
+      rs[0] += __shfl_xor_sync(0xffffffffu, rs[0], 2);
+      rs[0] += __shfl_xor_sync(0xffffffffu, rs[0], 1);
+      if ((lane & 3) == 0) prow[(l0 + l) * TILE + warp + NW * (lane >> 2)] = rs[0];
+      if (I != J) {
+        double* cp = colp + (l & 1) * NW * TILE;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cp[warp * TILE + lane + 32 * j] = cs[j];
+        __syncthreads();
+        if (threadIdx.x < TILE) {
+          double s = 0.0;
+#pragma unroll
+          for (int k = 0; k < NW; ++k) s += cp[k * TILE + threadIdx.x];
+          pcol[(l0 + l) * TILE + threadIdx.x] = -s;
+        }
+      }
     }
   }
-  if (live) {
-    part_t[i] = st_s - st_c;
-#pragma unroll
-    for (int l = 0; l < MR; ++l)
-      if (l < m) dL_dx[i * m + l] = g[l];
-  }
+}
+
+// dL/dx += t times the sums of the tiles of row blocks [I0, I1): those of row
+// block b's own tiles (b, J) and, transposed, of the tiles (I, b), in that
+// order; init: the first band.
+__global__ void __launch_bounds__(TILE) k_grad_finish(const double* __restrict__ P, int64_t n, int m, double t,
+                                                      int64_t N, int64_t I0, int64_t I1, int init,
+                                                      double* __restrict__ dL_dx) {
+  const int64_t b = blockIdx.x, i = b * TILE + threadIdx.x;
+  const int l = blockIdx.y;
+  if (i >= n) return;
+  double s = 0.0, e = 0.0;
+  if (b >= I0 && b < I1)
+    for (int64_t J = 0; J <= b; ++J) add_comp(s, e, P[(((b - I0) * 2 * N + J) * m + l) * TILE + threadIdx.x]);
+  for (int64_t I = (b + 1 > I0 ? b + 1 : I0); I < I1; ++I)
+    add_comp(s, e, P[(((I - I0) * 2 * N + N + b) * m + l) * TILE + threadIdx.x]);
+  const double v = t * (s + e);
+  dL_dx[i * m + l] = init ? v : dL_dx[i * m + l] + v;
 }
 
 __global__ void __launch_bounds__(1024) k_sum_f64(const double* __restrict__ v, int64_t n,
@@ -1266,26 +1415,58 @@ cudaError_t launch_fill(double* v, int64_t n, double value, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_grad(const double* X, int64_t n, int m, double t, const double* w,
-                        const double* lam, double* dL_dx, double* part_t, int64_t np,
-                        cudaStream_t s) {
-  (void)np;
-  int ct = 128;
-  while (ct > 8 && (size_t)ct * (m + 2) * sizeof(double) > 40 * 1024) ct /= 2;  // + 8 KB exp table
-  const size_t smem = (size_t)ct * (m + 2) * sizeof(double);
-  const unsigned grid = blocks_for(n, RES_THREADS);
-  if (m <= 8)
-    k_grad<8><<<grid, RES_THREADS, smem, s>>>(X, n, m, t, w, lam, dL_dx, part_t, ct);
-  else if (m <= 16)
-    k_grad<16><<<grid, RES_THREADS, smem, s>>>(X, n, m, t, w, lam, dL_dx, part_t, ct);
-  else if (m <= 32)
-    k_grad<32><<<grid, RES_THREADS, smem, s>>>(X, n, m, t, w, lam, dL_dx, part_t, ct);
-  else if (m <= 64)
-    k_grad<64><<<grid, RES_THREADS, smem, s>>>(X, n, m, t, w, lam, dL_dx, part_t, ct);
-  else
-    return cudaErrorInvalidValue;
+size_t grad_band_bytes(int64_t n, int m) {
+  const size_t N = (size_t)((n + TILE - 1) / TILE);
+  return 2 * N * (size_t)m * TILE * sizeof(double);
+}
+size_t grad_head_bytes(int64_t n) {
+  const size_t N = (size_t)((n + TILE - 1) / TILE);
+  return (N * (N + 1) / 2 * sizeof(double) + 255) & ~(size_t)255;
+}
+
+template <bool FX, int KIND>
+static cudaError_t launch_grad_t(const fx_coord* Xq, const double* X, int64_t n, int m, const FxScale& sc, double t,
+                                 const double* w, const double* lam, double* P, double* part_t, int64_t N, int64_t I0,
+                                 int64_t I1, cudaStream_t s) {
+  const size_t fx = fx_tile_smem(m);
+  const size_t smem = (size_t)TILE * GRAD_LD * sizeof(double) + (fx > GRAD_STAGE ? fx : GRAD_STAGE);
+  auto kern = k_grad_tile<FX, KIND>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int64_t q0 = num_lower_tiles(I0);
+  kern<<<(unsigned)(num_lower_tiles(I1) - q0), GRAD_THREADS, smem, s>>>(Xq, X, n, m, sc, t, w, lam, P, part_t, N, q0,
+                                                                       I0);
   note_launch();
   return cudaGetLastError();
+}
+
+cudaError_t launch_grad(const void* Xq, int qe, const double* X, int64_t n, int m, double t, const double* w,
+                        const double* lam, double* dL_dx, void* scratch, int64_t bands, cudaStream_t s) {
+  if (m < 1 || m > 64 || bands < 1) return cudaErrorInvalidValue;
+  const int64_t N = (n + TILE - 1) / TILE;
+  double* part_t = static_cast<double*>(scratch);
+  double* P = reinterpret_cast<double*>(static_cast<char*>(scratch) + grad_head_bytes(n));
+  const FxScale sc = fx_scale(t, Xq ? qe : 0);
+  const fx_coord* q = static_cast<const fx_coord*>(Xq);
+  for (int64_t I0 = 0; I0 < N; I0 += bands) {
+    const int64_t I1 = std::min(N, I0 + bands);
+    if (num_lower_tiles(I1) - num_lower_tiles(I0) > 0x7fffffffLL) return cudaErrorInvalidValue;
+    cudaError_t e;
+    if (!q)
+      e = launch_grad_t<false, 0>(q, X, n, m, sc, t, w, lam, P, part_t, N, I0, I1, s);
+    else if (fx_kind(m) == 0)
+      e = launch_grad_t<true, 0>(q, X, n, m, sc, t, w, lam, P, part_t, N, I0, I1, s);
+    else if (fx_kind(m) == 1)
+      e = launch_grad_t<true, 1>(q, X, n, m, sc, t, w, lam, P, part_t, N, I0, I1, s);
+    else
+      e = launch_grad_t<true, 2>(q, X, n, m, sc, t, w, lam, P, part_t, N, I0, I1, s);
+    if (e != cudaSuccess) return e;
+    k_grad_finish<<<dim3((unsigned)N, (unsigned)m), TILE, 0, s>>>(P, n, m, t, N, I0, I1, I0 == 0 ? 1 : 0, dL_dx);
+    note_launch();
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_sum_f64(const double* v, int64_t n, double* out, cudaStream_t s) {

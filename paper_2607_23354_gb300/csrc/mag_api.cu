@@ -151,7 +151,7 @@ struct mag_ctx {
   int32_t xq_m = 0;
   int xq_e = 0;
   const void* xq_q = nullptr;
-  void* rp = nullptr;                // partial sums of mag_residual
+  void* rp = nullptr;                // partial sums of mag_residual and mag_grad
   size_t rp_bytes = 0;
   void* lh = nullptr;
   size_t lh_bytes = 0;
@@ -192,7 +192,7 @@ struct mag_ctx {
 enum { V_ROWSUM = 0, V_R = 1, V_X = 2, V_E = 3, V_BEST = 4, V_T2 = 5 };
 enum { F_V = 0, F_Y = 1, F_T = 2 };
 // FP64 vectors of the aux buffer (sweep probes, gradients)
-enum { A_W = 0, A_LAM = 1, A_G = 2, A_PART = 3, A_COUNT = 4 };
+enum { A_W = 0, A_LAM = 1, A_G = 2, A_COUNT = 3 };
 
 namespace {
 
@@ -2689,9 +2689,20 @@ int mag_grad(mag_ctx* ctx, const double* points, int64_t n, int32_t m, double t,
     CU(cudaMemcpyAsync(lam, wv, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
   if (!ctx->ws) TRY(ensure_workspace(ctx, n, false, false));
-  double* part_t = ctx->aux + (size_t)A_PART * ctx->aux_np;
-  CU(launch_grad(points, n, m, t, wv, lam, dL_dx, part_t, ctx->aux_np, s));
-  CU(launch_sum_f64(part_t, n, &ctx->st()->aux[0], s));
+  // partial sums of the tiles, a band of row blocks at a time within 1 GB
+  const int64_t N = (n + TILE - 1) / TILE;
+  const size_t band = grad_band_bytes(n, m), head = grad_head_bytes(n);
+  int64_t bands = std::max<int64_t>(1, std::min<int64_t>(N, (int64_t)(((size_t)1 << 30) / band)));
+  int qe = 0;
+  const void* Xq = nullptr;
+  if (!quantize_points(ctx, points, n, m, &qe, &Xq)) Xq = nullptr;
+  if (!grow_buffer(ctx, &ctx->rp, &ctx->rp_bytes, head + (size_t)bands * band, 0)) {
+    bands = 1;
+    if (!grow_buffer(ctx, &ctx->rp, &ctx->rp_bytes, head + band, 0))
+      return fail(ctx, MAG_ENOMEM, "gradient partial sums of %.3g bytes", (double)(head + band));
+  }
+  CU(launch_grad(Xq, qe, points, n, m, t, wv, lam, dL_dx, ctx->rp, bands, s));
+  CU(launch_sum_f64(static_cast<const double*>(ctx->rp), num_lower_tiles(N), &ctx->st()->aux[0], s));
   TRY(read_status(ctx));
   *dL_dt = ctx->h_st->aux[0];
   if (info) *info = si;

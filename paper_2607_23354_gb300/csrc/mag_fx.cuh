@@ -258,6 +258,26 @@ FX_HD fx_u64 fx_pack(fx_u64 z, int shift) {
   const fx_u64 m = (fx_make(ml, mh) >> 11) + ((ml >> 10) & 1u);
   return ((fx_u64)(uint32_t)ex << 52) + m;
 }
+// 1 / (s 2^-62) in units of 2^-63 for 2^62 <= s <= 2^63, from its FP32 value y
+// (relative error below 2^-21): q0 = y, r = 1 - s q0 exact, q0 (1 + r + r^2);
+// within 2^-59.
+FX_HD fx_u64 fx_recip(fx_u64 s, float y) {
+  const uint32_t q0 = fx_bits(y + 1.0f) - 0x3f800000u;  // y 2^23
+  const long long r = -(long long)((s >> 2) * q0);      // 1 - s q0, scale 2^83 (mod 2^64)
+  const int rh = (int)(r >> 32);
+  const long long p = r + (long long)((fx_u64)((long long)rh * rh) >> 19);
+  const long long hi = (long long)(int)(p >> 32) * (long long)q0;  // scale 2^74 above the low half
+  return ((fx_u64)q0 << 40) + (fx_u64)(hi >> 11) + (((fx_u64)fx_lo((fx_u64)p) * q0) >> 43);
+}
+// z 2^-63 2^-shift rounded to FP64 for any z > 0 with its leading bit in the
+// high word
+FX_HD fx_u64 fx_pack_any(fx_u64 z, int shift) {
+  const int s = fx_clz(fx_hi(z));
+  const uint32_t mh = fx_shl(fx_lo(z), fx_hi(z), s), ml = fx_lo(z) << s;
+  const int ex = 1022 - s - shift;
+  if (ex < 1) return 0;
+  return ((fx_u64)(uint32_t)ex << 52) + (fx_make(ml, mh) >> 11) + ((ml >> 10) & 1u);
+}
 FX_HD fx_u64 fx_exp_neg(fx_u64 dm, int k, fx_u64 g, const fx_u64* T) {
   int shift;
   const fx_u64 z = fx_exp_fixed(dm, k, g, T, &shift);
@@ -320,8 +340,8 @@ __device__ __forceinline__ void load_fx_table(fx_u64* tab) {
 }
 
 // The pairs of one 128 x 128 tile (rows row0 .., columns col0 .. of the n
-// quantized points Xq), 256 threads: f(r, q) is called once for every row r =
-// warp + 8 i of the tile with the squares q[4] of the lane's columns 4 lane ..
+// quantized points Xq), THREADS threads (NW warps): f(r, q) is called once for
+// every row r = warp + NW i of the tile with the squares q[4] of the lane's columns 4 lane ..
 // 4 lane + 3.  KIND: 0 for m <= FX_LOW_DIM, 1 for m <= FX_SPILL, 2 beyond.
 // Beyond FX_SPILL two rows are accumulated together, where the column reads
 // would set the pace; below, one (they hide behind the finishing work).  smem:
@@ -335,16 +355,16 @@ constexpr int fx_ctas(int kind) { return kind < 2 ? 3 : 2; }
 constexpr int FX_CHUNK = 32;  // dimensions staged at a time
 inline size_t fx_tile_smem(int m) { return 2 * (size_t)128 * (m < FX_CHUNK ? m : FX_CHUNK) * sizeof(fx_coord); }
 
-template <int KIND, class F>
+template <int KIND, int THREADS = FX_THREADS, class F>
 __device__ __forceinline__ void fx_tile_pairs(const fx_coord* __restrict__ Xq, int64_t n, int m, int64_t row0,
                                               int64_t col0, fx_coord* smem, F&& f) {
-  constexpr int R = KIND < 2 ? 1 : 2, LB = KIND == 0 ? 31 : 30;
+  constexpr int R = KIND < 2 ? 1 : 2, LB = KIND == 0 ? 31 : 30, NW = THREADS / 32;
   const int mc = m < FX_CHUNK ? m : FX_CHUNK;
   fx_coord* xr = smem;              // [128][mc] row points (broadcast reads)
   fx_coord* xc = smem + 128 * mc;   // [mc][128]: column 4 l + q at 32 q + l (conflict free)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   auto stage = [&](int l0, int cnt) {
-    for (int e = threadIdx.x; e < 128 * cnt; e += FX_THREADS) {
+    for (int e = threadIdx.x; e < 128 * cnt; e += THREADS) {
       const int r = e / cnt, l = e - r * cnt;
       const int64_t gr = row0 + r, gc = col0 + r;
       xr[r * mc + l] = gr < n ? Xq[gr * m + l0 + l] : fx_coord{0, 0};
@@ -356,7 +376,7 @@ __device__ __forceinline__ void fx_tile_pairs(const fx_coord* __restrict__ Xq, i
     __syncthreads();
   }
 #pragma unroll 1
-  for (int i = 0; i < 16; i += R) {
+  for (int i = 0; i < 128 / NW; i += R) {
     FxSquare q[R][4];
     FxSums s[R][4];
 #pragma unroll
@@ -371,7 +391,7 @@ __device__ __forceinline__ void fx_tile_pairs(const fx_coord* __restrict__ Xq, i
         stage(l0, cnt);
         __syncthreads();
       }
-      const fx_coord* xrow = xr + (warp + 8 * i) * mc;
+      const fx_coord* xrow = xr + (warp + NW * i) * mc;
 #pragma unroll 1
       for (int la = 0; la < cnt; la += FX_SPILL) {
         const int lb = cnt - la < FX_SPILL ? cnt : la + FX_SPILL;
@@ -382,7 +402,7 @@ __device__ __forceinline__ void fx_tile_pairs(const fx_coord* __restrict__ Xq, i
           for (int c = 0; c < 4; ++c) b[c] = xc[l * 128 + 32 * c + lane];
 #pragma unroll
           for (int k = 0; k < R; ++k) {
-            const fx_coord a = xrow[8 * k * mc + l];
+            const fx_coord a = xrow[NW * k * mc + l];
 #pragma unroll
             for (int c = 0; c < 4; ++c) fx_accumulate(s[k][c], a, b[c]);
           }
@@ -398,7 +418,7 @@ __device__ __forceinline__ void fx_tile_pairs(const fx_coord* __restrict__ Xq, i
     }
 #pragma unroll 1
     for (int k = 0; k < R; ++k) {
-      f(warp + 8 * (i + k), q[0]);
+      f(warp + NW * (i + k), q[0]);
       if (R > 1) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) q[0][c] = q[R - 1][c];

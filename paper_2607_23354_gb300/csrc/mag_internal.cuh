@@ -412,10 +412,15 @@ cudaError_t launch_batch_solve(int shape, const BatchProblem* probs, const int* 
                                int64_t nmax, double* w_out, double* mag_out, int* status, int* queue, double tol,
                                int max_iter, int grid, unsigned long long* busy_cycles, cudaStream_t s);
 
-// K7 gradients: dL/dt partial sums and dL/dx.
-cudaError_t launch_grad(const double* X, int64_t n, int m, double t, const double* w,
-                        const double* lam, double* dL_dx, double* part_t, int64_t np,
-                        cudaStream_t s);
+// K7 gradients (m <= 64): dL/dx, and dL/dt as one partial sum per lower tile at
+// the front of scratch (N (N + 1) / 2 doubles, for launch_sum_f64).  Xq: the
+// quantized coordinates (scale 2^qe), null: FP64 differences.  The tiles go in
+// bands of `bands` row blocks; scratch: grad_head_bytes + bands *
+// grad_band_bytes, 256-byte aligned.
+size_t grad_head_bytes(int64_t n);
+size_t grad_band_bytes(int64_t n, int m);
+cudaError_t launch_grad(const void* Xq, int qe, const double* X, int64_t n, int m, double t, const double* w,
+                        const double* lam, double* dL_dx, void* scratch, int64_t bands, cudaStream_t s);
 cudaError_t launch_sum_f64(const double* v, int64_t n, double* out, cudaStream_t s);
 // *out += an order-independent 64-bit mix of the bits of v[0..count) and
 // their positions (a checksum: *out must be zeroed first).

@@ -192,3 +192,33 @@ def test_staging_fits_shared_memory(ctx, m):
     if m <= 64:
         _, dx = ctx.grad(X, t, w=w)
         assert bool(torch.isfinite(dx).all())
+
+
+# The gradient kernel over the lower triangle, by limb layout and by chunk of
+# 16 dimensions, ragged tiles, a close pair, and with FP64 differences.  Against
+# FP64 sums: every term within (m / 2 + 12) (1 + t d) u of its value, the sums
+# within n u of the sum of the terms' magnitudes.
+@pytest.mark.parametrize("n", [2, 128, 129, 300])
+@pytest.mark.parametrize("m", [1, 4, 5, 16, 17, 33, 64])
+@pytest.mark.parametrize("exact", [True, False])
+def test_gradient_sums(n, m, exact):
+    rng = np.random.default_rng(n * 100 + m)
+    X = rng.standard_normal((n, m))
+    if n > 2:
+        X[n // 2] = X[1] + 1e-8 * rng.standard_normal(m)
+    t = 1.5 / np.sqrt(m)
+    c = M.Context(M.Options(exact_distances=exact))
+    w = rng.standard_normal(n)
+    g = rng.standard_normal() * np.ones(n)  # a constant dL/dw: lam = g w, no solve
+    dt, dx = c.grad(_dev(X), t, w=_dev(w), dL_dw=_dev(g))
+    D = X[:, None, :] - X[None, :, :]
+    d = np.sqrt((D.astype(np.longdouble) ** 2).sum(-1)).astype(np.float64)
+    Z = np.exp(-t * d)
+    lam = g[0] * w
+    s = np.outer(lam, w) + np.outer(w, lam)
+    e = 2.0 ** -53 * ((m / 2 + 12) * (1 + t * d) + n)
+    assert abs(dt - (0.5 * d * Z * s).sum()) <= (0.5 * e * d * Z * abs(s)).sum()
+    np.fill_diagonal(d, 1.0)
+    G = t * Z * s / d
+    ref = (G[:, :, None] * D).sum(1)
+    assert np.all(np.abs(dx.cpu().numpy() - ref) <= ((e * abs(G))[:, :, None] * abs(D)).sum(1))
