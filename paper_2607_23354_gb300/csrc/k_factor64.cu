@@ -1,0 +1,579 @@
+// K2, FP64: the plain dense method's blocked Cholesky on the tensor cores.
+//
+// GB300 runs FP64 at 1.2 TFLOP/s, so the matrix products are taken on the FP16
+// tensor cores by splitting (K. Ozaki, T. Ogita, S. Oishi, S. M. Rump,
+// "Error-free transformations of matrix multiplication by using fast routines
+// of matrix multiplication and its applications", Numer. Algorithms 59(1),
+// 2012): every row of an operand is scaled by a power of two to 62-bit integers
+// (entries within 2^-9 of the row's largest keep all their bits), written as
+// eight balanced base-256 digits (|d| <= 128, exact in FP16), and the digit
+// products of equal weight are summed in one FP32 accumulator:
+//
+//   sum_k a_k b_k = 256^14 sum_l D_l 256^-l,  D_l = sum_k sum_{i + j = l} a_ik b_jk
+//
+// for l = 0..7 (36 products).  The leading digit is at most 64, so |D_l| < 8 *
+// 128 * 2^14 = 2^24 and the sums are exact whatever their order; the levels are
+// combined in integers and rounded to FP64 once.  What is dropped (l > 7) is
+// about 2^-67 of the product of the two rows' largest entries, against 2^-53 of
+// every partial sum in FP64 arithmetic.  (Seven digits of 55 bits: backward
+// errors 10 to 40% above the FP64 products'.)
+//
+// Per tile column K: the diagonal tile (FP64, k_potrf_f64), the digits of
+// inv(L_KK) and of the panel's tiles, the panel solve L_IK = A_IK inv(L_KK)^T,
+// the digits of the solved panel and the trailing update C_IJ -= L_IK L_JK^T.
+// n = 5001: 123 ms with FP64 products throughout, 20.9 ms this way (12.8 of
+// them the 40 diagonal tiles); backward error 5e-16 -> 0.6e-16.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "mag_internal.cuh"
+#include "mag_tc.cuh"
+
+namespace mag {
+
+namespace {
+
+// ---------------------------------------------------------- diagonal tile
+// The elimination of [A; I] of k_potrf.cu in FP64, in four panels of 32
+// columns, four columns at a time.  A's lower and W = inv(L)^T's upper
+// triangle share one 128 x 128 array, W's diagonal blocks have their own.
+// Bound: the FP64 pipe (555,000 SM cycles of warp operations, two thirds of
+// them the trailing updates) and, within a panel, the pivots' chain.
+constexpr int PB = 32;
+constexpr int NPB = TILE / PB;
+constexpr int LDM = TILE + 2;
+constexpr int LDW = PB + 2;
+constexpr int P64_THREADS = 512;
+constexpr int PANEL_WARPS = NPB + 1;
+constexpr int BG_WARPS = P64_THREADS / 32 - PANEL_WARPS;
+
+struct Potrf64Smem {
+  double M[TILE * LDM];          // block (i, j): A, becoming L (i >= j); W (i < j)
+  double Wd[NPB][PB * LDW];      // W's diagonal blocks
+  double rinv[TILE];             // 1 / L[c][c]
+};
+
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// s = sqrt(p) and its reciprocal, p > 0: the FP32 seed, two Newton steps, s
+// from p r by its exact residual, then r as the reciprocal of that s (both
+// within 0.51 units and consistent: the column is scaled by 1 / L_jj).
+__device__ __forceinline__ double rsqrt64(double p, double* sq) {
+  // p scaled to FP32's range by an even power of two
+  const int ex = (__double2hiint(p) >> 20) - 1023;
+  const int h = ex >> 1;
+  const double ps = __hiloint2double(__double2hiint(p) - h * (1 << 21), __double2loint(p));  // in [1, 4)
+  double r = (double)rsqrtf((float)ps);
+  const double hp = 0.5 * ps;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) r = fma(r, fma(-hp * r, r, 0.5), r);
+  double s = ps * r;
+  s = fma(0.5 * r, fma(-s, s, ps), s);
+  r = fma(r, fma(-s, r, 1.0), r);
+  *sq = __hiloint2double(__double2hiint(s) + h * (1 << 20), __double2loint(s));
+  return __hiloint2double(__double2hiint(r) - h * (1 << 20), __double2loint(r));
+}
+
+struct Pivot64 {
+  double r0, r1, r2, r3, s0, s1, s2, s3, l10, l20, l30, l21, l31, l32;
+  int bad;
+};
+
+__device__ __forceinline__ void pivot_factor64(const double* a, int j, Pivot64& q) {
+  const unsigned full = 0xffffffffu;
+  const double d00 = __shfl_sync(full, a[0], j), d10 = __shfl_sync(full, a[0], j + 1);
+  const double d20 = __shfl_sync(full, a[0], j + 2), d30 = __shfl_sync(full, a[0], j + 3);
+  const double d11 = __shfl_sync(full, a[1], j + 1), d21 = __shfl_sync(full, a[1], j + 2);
+  const double d31 = __shfl_sync(full, a[1], j + 3), d22 = __shfl_sync(full, a[2], j + 2);
+  const double d32 = __shfl_sync(full, a[2], j + 3), d33 = __shfl_sync(full, a[3], j + 3);
+  // a pivot that is not positive (or below FP64's normal range) is reported
+  // and replaced by 1, so that the kernel finishes on finite values
+  constexpr double kMin = 2.2250738585072014e-308;
+  const bool b0 = !(d00 >= kMin);
+  q.r0 = rsqrt64(b0 ? 1.0 : d00, &q.s0);
+  q.l10 = d10 * q.r0, q.l20 = d20 * q.r0, q.l30 = d30 * q.r0;
+  const double p1 = fma(-q.l10, q.l10, d11);
+  const bool b1 = !(p1 >= kMin);
+  q.r1 = rsqrt64(b1 ? 1.0 : p1, &q.s1);
+  q.l21 = fma(-q.l20, q.l10, d21) * q.r1, q.l31 = fma(-q.l30, q.l10, d31) * q.r1;
+  const double p2 = fma(-q.l21, q.l21, fma(-q.l20, q.l20, d22));
+  const bool b2 = !(p2 >= kMin);
+  q.r2 = rsqrt64(b2 ? 1.0 : p2, &q.s2);
+  q.l32 = fma(-q.l31, q.l21, fma(-q.l30, q.l20, d32)) * q.r2;
+  const double p3 = fma(-q.l32, q.l32, fma(-q.l31, q.l31, fma(-q.l30, q.l30, d33)));
+  const bool b3 = !(p3 >= kMin);
+  q.r3 = rsqrt64(b3 ? 1.0 : p3, &q.s3);
+  q.bad = (int)b0 | (int)b1 << 1 | (int)b2 << 2 | (int)b3 << 3;
+}
+
+// A panel row's steps (DIAG: the diagonal block's rows); own: this lane's 32
+// entries, Ld: the panel's diagonal block of M.
+template <bool DIAG>
+__device__ __forceinline__ void panel_rows64(Potrf64Smem& S, int o, double* own, int lane, int64_t K, DevStatus* st) {
+  constexpr int NBAR = 32 * PANEL_WARPS;
+  const double* Ld = S.M + o * LDM + o;
+  double a[PB];
+#pragma unroll
+  for (int c = 0; c < PB; ++c) a[c] = own[c];
+  Pivot64 q;
+  q.bad = 0;
+#pragma unroll 1
+  for (int g = 0; g < PB / 4; ++g) {
+    const int j = 4 * g;
+    if (DIAG) {
+      pivot_factor64(a, j, q);
+    } else {
+      bar_sync(1 + g, NBAR);
+      q.r0 = S.rinv[o + j], q.r1 = S.rinv[o + j + 1], q.r2 = S.rinv[o + j + 2], q.r3 = S.rinv[o + j + 3];
+      const double* r1 = Ld + (j + 1) * LDM + j;
+      q.l10 = r1[0];
+      q.l20 = r1[LDM], q.l21 = r1[LDM + 1];
+      q.l30 = r1[2 * LDM], q.l31 = r1[2 * LDM + 1], q.l32 = r1[2 * LDM + 2];
+    }
+    double x0 = a[0] * q.r0;
+    double x1 = fma(-x0, q.l10, a[1]) * q.r1;
+    double x2 = fma(-x1, q.l21, fma(-x0, q.l20, a[2])) * q.r2;
+    double x3 = fma(-x2, q.l32, fma(-x1, q.l31, fma(-x0, q.l30, a[3]))) * q.r3;
+    if (DIAG) {
+      x0 = lane < j ? 0.0 : (lane == j ? q.s0 : x0);
+      x1 = lane < j + 1 ? 0.0 : (lane == j + 1 ? q.s1 : x1);
+      x2 = lane < j + 2 ? 0.0 : (lane == j + 2 ? q.s2 : x2);
+      x3 = lane < j + 3 ? 0.0 : (lane == j + 3 ? q.s3 : x3);
+    }
+    own[j] = x0, own[j + 1] = x1, own[j + 2] = x2, own[j + 3] = x3;
+    if (DIAG) {
+      if (lane == 0) {
+        S.rinv[o + j] = q.r0, S.rinv[o + j + 1] = q.r1, S.rinv[o + j + 2] = q.r2, S.rinv[o + j + 3] = q.r3;
+        if (q.bad) {
+          atomicOr(&st->flags, ST_NOTPD);
+          atomicMin(&st->notpd_index, (int)(K * TILE + o + j) + __ffs(q.bad));
+        }
+      }
+      __syncwarp();
+      bar_arrive(1 + g, NBAR);
+    }
+    // the remaining columns, rotated by four; beyond the panel's end nothing
+    // is needed any more
+#pragma unroll
+    for (int c4 = 0; c4 < PB - 4; c4 += 4) {
+      if (j + 4 + c4 < PB) {
+        const double* Lq = Ld + (j + 4 + c4) * LDM + j;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const double2 v01 = *reinterpret_cast<const double2*>(Lq + c * LDM);
+          const double2 v23 = *reinterpret_cast<const double2*>(Lq + c * LDM + 2);
+          a[c4 + c] = fma(-x3, v23.y, fma(-x2, v23.x, fma(-x1, v01.y, fma(-x0, v01.x, a[c4 + c + 4]))));
+        }
+      }
+    }
+  }
+}
+
+// 8 x 32 outputs: C -= P Q^T, K = 32 (P: row stride ldp; Q, C in M).  The sums
+// start from C: the partial sums shrink towards the Schur complement, where a
+// sum taken apart rises to C's size and cancels (backward error 1.9e-16 for
+// 0.5e-16 at 128 points of the unit cube).
+__device__ __forceinline__ void trailing_job64(const double* P, int ldp, const double* Q, double* C, int lane) {
+  const double* p = P + (lane >> 3) * ldp;
+  const double* q = Q + (lane & 7) * LDM;
+  double* c = C + (lane >> 3) * LDM + (lane & 7);
+  double acc[2][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = c[4 * i * LDM + 8 * j];
+#pragma unroll 4
+  for (int k = 0; k < PB; ++k) {
+    double b[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) b[j] = q[8 * j * LDM + k];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const double a = -p[4 * i * ldp + k];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = fma(a, b[j], acc[i][j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) c[4 * i * LDM + 8 * j] = acc[i][j];
+}
+
+// Quarter h (8 rows) of the trailing update with panel kb of column block jb,
+// row block number b of: A's jb .. 3, then W's 0 .. kb.
+__device__ __forceinline__ void trailing_block64(Potrf64Smem& S, int kb, int jb, int b, int h, int lane) {
+  const int ib = jb + b;
+  const double* Q = S.M + jb * PB * LDM + kb * PB;
+  if (ib < NPB) {
+    double* row = S.M + (ib * PB + 8 * h) * LDM;
+    trailing_job64(row + kb * PB, LDM, Q, row + jb * PB, lane);
+  } else {
+    const int wb = ib - NPB;
+    double* row = S.M + (wb * PB + 8 * h) * LDM;
+    if (wb == kb)
+      trailing_job64(S.Wd[kb] + 8 * h * LDW, LDW, Q, row + jb * PB, lane);
+    else
+      trailing_job64(row + kb * PB, LDM, Q, row + jb * PB, lane);
+  }
+}
+
+__global__ void __launch_bounds__(P64_THREADS, 1)
+    k_potrf_f64(double* __restrict__ Z, double* __restrict__ Dinv, double* __restrict__ DinvT, int64_t K,
+                DevStatus* st) {
+  extern __shared__ __align__(16) unsigned char p64_smem[];
+  Potrf64Smem& S = *reinterpret_cast<Potrf64Smem*>(p64_smem);
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  if (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) return;  // uniform
+  double* tile = Z + tri_index(K, K) * TILE_ELEMS;
+#pragma unroll 8
+  for (int e = tid; e < TILE * TILE / 2; e += P64_THREADS) {
+    const int r = e >> 6, c = (e & 63) * 2;
+    const double2 v = c / PB <= r / PB ? reinterpret_cast<const double2*>(tile)[e] : make_double2(0.0, 0.0);
+    *reinterpret_cast<double2*>(S.M + r * LDM + c) = v;
+  }
+  for (int e = tid; e < NPB * PB * PB; e += P64_THREADS) {
+    const int b = e / (PB * PB), r = e / PB % PB, c = e % PB;
+    S.Wd[b][r * LDW + c] = r == c ? 1.0 : 0.0;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int kb = 0; kb < NPB; ++kb) {
+    const int o = kb * PB;
+    // the panel's warps: A's row blocks kb .. 3, W's 0 .. kb - 1 (warp = row
+    // block), W's kb-th on warp 4 + (kb + 1) % 4, away from the diagonal's scheduler
+    const int wk = NPB + ((kb + 1) & 3);
+    if (w < NPB) {
+      double* own = S.M + (w * PB + lane) * LDM + o;
+      if (w == kb)
+        panel_rows64<true>(S, o, own, lane, K, st);
+      else
+        panel_rows64<false>(S, o, own, lane, K, st);
+    } else if (w == wk) {
+      panel_rows64<false>(S, o, S.Wd[kb] + lane * LDW, lane, K, st);
+    } else if (kb > 0) {
+      // the rest of the previous panel's trailing update
+      const int bw = w < wk ? w - NPB : w - PANEL_WARPS;
+      int job = bw;
+#pragma unroll 1
+      for (int jb = kb + 1; jb < NPB; ++jb) {
+        const int jobs = 4 * (NPB - jb + kb);
+        for (; job < jobs; job += BG_WARPS) trailing_block64(S, kb - 1, jb, job >> 2, job & 3, lane);
+        job -= jobs;
+      }
+    }
+    __syncthreads();
+    if (kb < NPB - 1) {
+      trailing_block64(S, kb, kb + 1, w >> 2, w & 3, lane);  // the next panel's four row blocks
+      __syncthreads();
+    }
+  }
+  double* Y = Dinv + K * TILE_ELEMS;
+  double* YT = DinvT + K * TILE_ELEMS;
+  // W[c][r] = inv(L)[r][c]
+  auto wv = [&](int c, int r) -> double {
+    const int bc = c / PB, br = r / PB;
+    return bc == br ? S.Wd[bc][(c % PB) * LDW + r % PB] : (br > bc ? S.M[c * LDM + r] : 0.0);
+  };
+  for (int e = tid; e < TILE * TILE; e += P64_THREADS) {
+    const int r = e >> 7, c = e & 127;
+    tile[e] = c <= r ? S.M[r * LDM + c] : 0.0;
+    YT[e] = c >= r ? wv(r, c) : 0.0;
+  }
+  for (int e = tid; e < TILE * TILE; e += P64_THREADS) {
+    const int r = e >> 7, c = e & 127;
+    Y[e] = c <= r ? wv(c, r) : 0.0;
+  }
+}
+
+// ----------------------------------------------------------------- digits
+constexpr int NDIG = 8;
+constexpr int64_t CHUNK_BYTES = 128 * 128;                     // 128 rows x 64 FP16 columns
+constexpr int64_t DIGIT_BYTES = 2 * NDIG * CHUNK_BYTES;        // a tile's digits: [K chunk][digit][128 rows]
+constexpr int64_t DIGIT_STRIDE = DIGIT_BYTES + 1024;           // then 128 row exponents
+
+// Digits of the FP64 tiles of column K: slot 0 from `first` (inv(L_KK), when
+// given), the following slots from tiles (I, K), I = K + 1 ....  Row r of a
+// tile is x = X 2^(e_r - 62), |X| < 2^62, X = sum_i d_i 256^(7 - i).  A row
+// whose largest entry is below 2^-450 counts as zero.
+__global__ void __launch_bounds__(256) k_digits(const double* __restrict__ first, const double* __restrict__ Z,
+                                                int64_t K, unsigned char* __restrict__ out, const DevStatus* st) {
+  if (st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) return;
+  const int64_t slot = blockIdx.x, I = K + 1 + slot - (first ? 1 : 0);
+  const double* src = first && slot == 0 ? first : Z + tri_index(I, K) * TILE_ELEMS;
+  unsigned char* dst = out + slot * DIGIT_STRIDE;
+  int* exps = reinterpret_cast<int*>(dst + DIGIT_BYTES);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 2
+  for (int r = warp; r < TILE; r += 8) {
+    const double2 v01 = *reinterpret_cast<const double2*>(src + r * TILE + 4 * lane);
+    const double2 v23 = *reinterpret_cast<const double2*>(src + r * TILE + 4 * lane + 2);
+    const unsigned long long b[4] = {
+        (unsigned long long)__double_as_longlong(v01.x), (unsigned long long)__double_as_longlong(v01.y),
+        (unsigned long long)__double_as_longlong(v23.x), (unsigned long long)__double_as_longlong(v23.y)};
+    unsigned mx = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) mx = max(mx, (unsigned)(b[q] >> 52) & 0x7ffu);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    const bool zero = mx < 1023 - 450;
+    if (lane == 0) exps[r] = zero ? 0 : (int)mx - 1022;
+    __half d[NDIG][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int ex = (int)(b[q] >> 52) & 0x7ff, s = (int)mx - ex;
+      long long X = 0;
+      if (!zero && ex > 0 && s < 63) {
+        X = (long long)(((b[q] & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
+        if (s > 0) X = (X + (1ll << (s - 1))) >> s;
+        if (b[q] >> 63) X = -X;
+      }
+#pragma unroll
+      for (int i = NDIG - 1; i > 0; --i) {
+        const int g = (int)((unsigned)(X + 128) & 255u) - 128;
+        X = (X - g) >> 8;
+        d[i][q] = __int2half_rn(g);
+      }
+      d[0][q] = __int2half_rn((int)X);
+    }
+    const int chunk = lane >> 4, unit = (lane & 15) >> 1;
+    unsigned char* p = dst + chunk * NDIG * CHUNK_BYTES + swizzled_unit(r, unit) + (lane & 1) * 8;
+#pragma unroll
+    for (int i = 0; i < NDIG; ++i) {
+      uint2 u;
+      const __half2 lo = __halves2half2(d[i][0], d[i][1]), hi = __halves2half2(d[i][2], d[i][3]);
+      u.x = *reinterpret_cast<const uint32_t*>(&lo);
+      u.y = *reinterpret_cast<const uint32_t*>(&hi);
+      *reinterpret_cast<uint2*>(p + i * CHUNK_BYTES) = u;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- products
+// 128 x 64 outputs (half h of a tile) of A B^T from the digits, K = 128 in two
+// chunks of 64 columns: 128 KB of A's digits and 64 KB of B's in shared memory
+// at a time, the eight levels in 8 x 64 TMEM columns.  ASSIGN: tile (I, K) of
+// the panel, A = its own digits (slot 1 + i), B = inv(L_KK) (slot 0); else the
+// trailing update of tile (I, J), A and B the panel's digits.
+constexpr int OZ_THREADS = 256;
+constexpr uint32_t OZ_TMEM = 512;
+constexpr int OZ_SMEM = NDIG * (128 * 128 + 64 * 128);
+constexpr int OZ_LD = 66;
+
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ void mma_f16_128x64(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
+  constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+template <bool ASSIGN>
+__global__ void __launch_bounds__(OZ_THREADS, 1)
+    k_oz_gemm(double* __restrict__ Z, int64_t N, int64_t K, const unsigned char* __restrict__ digits, DevStatus* st,
+              uint64_t timeout_ns) {
+  extern __shared__ __align__(1024) unsigned char oz_raw[];
+  unsigned char* smem = (unsigned char*)(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t full_bar, done_bar[2];  // done_bar[c]: the products of chunk c
+  __shared__ uint32_t tmem_base_sh;
+  __shared__ int abort_flag;
+  __shared__ int ea[128], eb[64];
+  __shared__ int skip;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) skip = (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) != 0;
+  __syncthreads();
+  if (skip) return;  // uniform across the CTA
+  const int h = blockIdx.x & 1;
+  int64_t I, J;
+  const unsigned char *da, *db;
+  if (ASSIGN) {
+    I = K + 1 + (blockIdx.x >> 1), J = K;
+    da = digits + (1 + (int64_t)(blockIdx.x >> 1)) * DIGIT_STRIDE;
+    db = digits;
+  } else {
+    int64_t i, j;
+    tri_coords((int64_t)(blockIdx.x >> 1), &i, &j);
+    I = K + 1 + i, J = K + 1 + j;
+    da = digits + i * DIGIT_STRIDE;
+    db = digits + j * DIGIT_STRIDE;
+  }
+  if (tid == 0) {
+    abort_flag = 0;
+    mbar_init(&full_bar, 1);
+    mbar_init(&done_bar[0], 1);
+    mbar_init(&done_bar[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_sh)),
+                 "r"(OZ_TMEM)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid < 128) ea[tid] = reinterpret_cast<const int*>(da + DIGIT_BYTES)[tid];
+  if (tid >= 128 && tid < 192) eb[tid - 128] = reinterpret_cast<const int*>(db + DIGIT_BYTES)[64 * h + tid - 128];
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base_sh;
+  const uint64_t deadline = globaltimer() + timeout_ns;
+  if (tid == 0) {
+    bool ok = true;
+    for (int c = 0; c < 2 && ok; ++c) {
+      if (c > 0) ok = mbar_wait(&done_bar[0], 0, &abort_flag, deadline);  // chunk 0's operands have been read
+      if (!ok) break;
+      mbar_expect_tx(&full_bar, OZ_SMEM);
+      for (int i = 0; i < NDIG; ++i) {
+        bulk_load(smem + i * CHUNK_BYTES, da + (c * NDIG + i) * CHUNK_BYTES, CHUNK_BYTES, &full_bar);
+        bulk_load(smem + NDIG * CHUNK_BYTES + i * 8192, db + (c * NDIG + i) * CHUNK_BYTES + h * 8192, 8192, &full_bar);
+      }
+      ok = mbar_wait(&full_bar, c, &abort_flag, deadline);
+      if (!ok) {
+        const uint64_t dl = globaltimer() + 200000000ull;  // let the loads land before the CTA ends
+        while (!mbar_try_wait(&full_bar, c) && globaltimer() < dl) {
+        }
+        break;
+      }
+      tc_fence_after();
+      for (int l = 0; l < NDIG; ++l)
+        for (int i = 0; i <= l; ++i) {
+          const uint32_t sa = smem_u32(smem + i * CHUNK_BYTES);
+          const uint32_t sb = smem_u32(smem + NDIG * CHUNK_BYTES + (l - i) * 8192);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            mma_f16_128x64(tmem + l * 64, smem_desc<128>(sa + 32 * k), smem_desc<128>(sb + 32 * k),
+                           (c | i | k) != 0);
+        }
+      mma_commit(&done_bar[c]);
+    }
+  }
+  __syncwarp();
+  const bool waited = mbar_wait(&done_bar[1], 0, &abort_flag, deadline);
+  const bool fine = __syncthreads_and(waited ? 1 : 0) != 0;  // one decision for the whole CTA
+  tc_fence_after();
+  double* stage = reinterpret_cast<double*>(smem);  // [128][OZ_LD], once the MMAs have read the operands
+  if (fine) {
+    const int r = 32 * (warp & 3) + lane, c0 = 32 * (warp >> 2);
+    const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
+    const int er = ea[r] - 36 + 1023;
+#pragma unroll 1
+    for (int g = 0; g < 4; ++g) {
+      float v[NDIG][8];
+#pragma unroll
+      for (int l = 0; l < NDIG; ++l) tmem_ld8(base + l * 64 + 8 * g, v[l]);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int l = 0; l < NDIG; ++l)  // no use of the values moves above the wait
+        asm volatile("" : "+f"(v[l][0]), "+f"(v[l][1]), "+f"(v[l][2]), "+f"(v[l][3]), "+f"(v[l][4]), "+f"(v[l][5]),
+                          "+f"(v[l][6]), "+f"(v[l][7]));
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        // sum_l D_l 256^(7 - l) = t 2^32 + f, |t| < 2^46
+        const long long lo = (long long)__float2int_rn(v[4][q]) * 16777216 +
+                             ((long long)__float2int_rn(v[5][q]) * 65536 +
+                              ((long long)__float2int_rn(v[6][q]) * 256 + __float2int_rn(v[7][q])));
+        const long long t = (long long)__float2int_rn(v[0][q]) * 16777216 +
+                            ((long long)__float2int_rn(v[1][q]) * 65536 +
+                             ((long long)__float2int_rn(v[2][q]) * 256 + __float2int_rn(v[3][q]))) +
+                            (lo >> 32);
+        // the leading 62 bits or more: left-aligned by k <= 32
+        const int k = min(__clzll((long long)(t ^ (t >> 63))) - 1, 32);
+        const long long X = (long long)(((unsigned long long)t << k) | ((unsigned long long)(unsigned)lo << k >> 32));
+        const int c = c0 + 8 * g + q;
+        const int sc = er + eb[c] - k;  // positive: rows below 2^-450 are zero
+        stage[r * OZ_LD + c] = __ll2double_rn(X) * __hiloint2double(sc << 20, 0);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (fine) {
+    double* C = Z + tri_index(I, J) * TILE_ELEMS + 64 * h;
+#pragma unroll 4
+    for (int i = 0; i < 16; ++i) {
+      const int r = warp + 8 * i;
+      const double2 v = *reinterpret_cast<const double2*>(stage + r * OZ_LD + 2 * lane);
+      double2* p = reinterpret_cast<double2*>(C + r * TILE + 2 * lane);
+      if (ASSIGN) {
+        *p = v;
+      } else {
+        double2 c = *p;
+        c.x -= v.x, c.y -= v.y;
+        *p = c;
+      }
+    }
+  }
+  if (tid == 0 && abort_flag) atomicOr(&st->flags, ST_TIMEOUT);
+  tc_fence_after();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_TMEM) : "memory");
+}
+
+constexpr uint64_t kOzTimeout = 10000000000ull;
+
+}  // namespace
+
+size_t factor64_scratch_bytes(int64_t N) { return (size_t)(N + 1) * DIGIT_STRIDE; }
+
+cudaError_t launch_potrf_f64(double* Z, double* Dinv, double* DinvT, int64_t K, DevStatus* st, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(k_potrf_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(Potrf64Smem));
+  if (e != cudaSuccess) return e;
+  k_potrf_f64<<<1, P64_THREADS, sizeof(Potrf64Smem), s>>>(Z, Dinv, DinvT, K, st);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_factor64_panel(double* Z, const double* Dinv, int64_t K, int64_t N, void* scratch, DevStatus* st,
+                                  cudaStream_t s) {
+  unsigned char* dg = static_cast<unsigned char*>(scratch);
+  cudaError_t e;
+  const int64_t below = N - K - 1;
+  if (below <= 0) return cudaSuccess;
+  const int smem = OZ_SMEM + 1024;
+  e = cudaFuncSetAttribute(k_oz_gemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  k_digits<<<(unsigned)(below + 1), 256, 0, s>>>(Dinv + K * TILE_ELEMS, Z, K, dg, st);
+  note_launch();
+  k_oz_gemm<true><<<(unsigned)(2 * below), OZ_THREADS, smem, s>>>(Z, N, K, dg, st, kOzTimeout);
+  note_launch();
+  k_digits<<<(unsigned)below, 256, 0, s>>>(nullptr, Z, K, dg, st);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_factor64_update(double* Z, int64_t K, int64_t N, const void* scratch, DevStatus* st,
+                                   cudaStream_t s) {
+  const int64_t below = N - K - 1, tiles = num_lower_tiles(below);
+  if (below <= 0) return cudaSuccess;
+  if (2 * tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  const int smem = OZ_SMEM + 1024;
+  cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  k_oz_gemm<false><<<(unsigned)(2 * tiles), OZ_THREADS, smem, s>>>(Z, N, K, static_cast<const unsigned char*>(scratch),
+                                                                  st, kOzTimeout);
+  note_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace mag

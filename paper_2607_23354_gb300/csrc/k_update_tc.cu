@@ -43,6 +43,7 @@
 #include <cuda_fp16.h>
 
 #include "mag_internal.cuh"
+#include "mag_tc.cuh"
 
 namespace mag {
 
@@ -102,52 +103,6 @@ __host__ __device__ constexpr int chunk_bytes_of(int mode) {
   return (mode == UPD_TF32X3 || mode == UPD_FP16X3) ? 128 : 128;
 }
 
-// ------------------------------------------------------------ PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait for the phase with `parity` to complete.  Returns false if the
-// deadline passed (then raises the CTA abort flag) or another role aborted.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                          uint64_t deadline) {
-  uint32_t it = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if ((++it & 255u) == 0) {
-      if (*abort_flag) return false;
-      if (globaltimer() > deadline) {
-        *abort_flag = 1;
-        return false;
-      }
-    }
-  }
-  return true;
-}
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x,
                                             int y) {
   asm volatile(
@@ -166,25 +121,6 @@ __device__ __forceinline__ void tma_load_2d_peer_bar(void* dst, const CUtensorMa
       "%3}], [%4];" ::"r"(smem_u32(dst)),
       "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar_cluster)
       : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-// Shared-memory matrix descriptor, K-major, version 1, base offset 0:
-// 128-byte rows -> SWIZZLE_128B (layout 2), 8-row groups 1024 B apart;
-// 64-byte rows  -> SWIZZLE_64B (layout 4), 8-row groups 512 B apart.
-template <int CHUNK>
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);         // start address
-  d |= (uint64_t)1 << 16;                           // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)((8 * CHUNK) >> 4) << 32;          // stride byte offset: 8 rows
-  d |= (uint64_t)1 << 46;                           // descriptor version
-  d |= (uint64_t)(CHUNK == 128 ? 2 : 4) << 61;      // SWIZZLE_128B / SWIZZLE_64B
-  return d;
 }
 // Instruction descriptor: D = F32, A/B format `fmt`, both K-major, M = 128, N = 256.
 __host__ __device__ constexpr uint32_t instr_desc(uint32_t fmt) {
@@ -208,28 +144,6 @@ __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uin
         : "memory");
   }
 }
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
-      "%13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, "
-      "[%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // Bulk reduce-add of a 32 x 32 FP32 box from shared memory into global
 // memory (the L2 performs the read-modify-write), tracked by bulk groups.
 __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* map, uint32_t saddr, int x, int y, int z) {

@@ -151,6 +151,8 @@ struct mag_ctx {
   int32_t xq_m = 0;
   int xq_e = 0;
   const void* xq_q = nullptr;
+  void* dg = nullptr;                // digits of a panel of the FP64 factor
+  size_t dg_bytes = 0;
   void* rp = nullptr;                // partial sums of mag_residual and mag_grad
   size_t rp_bytes = 0;
   void* lh = nullptr;
@@ -461,16 +463,25 @@ double update_flops(int64_t N, int64_t k0, int64_t k1, int64_t j0, int64_t j1) {
   return tiles * (double)(k1 - k0) * 2.0 * TILE * TILE * TILE;
 }
 
+// FP64 products by digits on the tensor cores while their scratch (230 KB a
+// tile row) fits; else, and for FP32, on the CUDA cores.
 template <typename T>
 int factor_blocked(mag_ctx* ctx, T* Z, T* Dinv, int* launches, double* flops) {
   const Layout& L = ctx->lay;
   cudaStream_t s = ctx->stream;
+  const bool digits = sizeof(T) == 8 && grow_buffer(ctx, &ctx->dg, &ctx->dg_bytes, factor64_scratch_bytes(L.N), 0);
   for (int64_t K = 0; K < L.N; ++K) {
     CU(launch_potrf_diag<T>(Z, Dinv, K, L.n, ctx->st(), s));
-    CU(launch_trsm_col<T>(Z, Dinv, K, L.N, ctx->st(), s));
+    if (digits)
+      CU(launch_factor64_panel((double*)Z, (const double*)Dinv, K, L.N, ctx->dg, ctx->st(), s));
+    else
+      CU(launch_trsm_col<T>(Z, Dinv, K, L.N, ctx->st(), s));
     if (K + 1 < L.N) {
       TRY(prof_begin(ctx));
-      CU(launch_syrk_simt<T>(Z, L.N, K, K + 1, K + 1, L.N, ctx->st(), s));
+      if (digits)
+        CU(launch_factor64_update((double*)Z, K, L.N, ctx->dg, ctx->st(), s));
+      else
+        CU(launch_syrk_simt<T>(Z, L.N, K, K + 1, K + 1, L.N, ctx->st(), s));
       TRY(prof_end(ctx));
       ++*launches;
       *flops += update_flops(L.N, K, K + 1, K + 1, L.N);
@@ -1072,6 +1083,7 @@ int mag_ctx_destroy(mag_ctx* ctx) {
   if (ctx->chain_s) cudaFree(ctx->chain_s);
   if (ctx->xq) cudaFree(ctx->xq);
   if (ctx->rp) cudaFree(ctx->rp);
+  if (ctx->dg) cudaFree(ctx->dg);
   if (ctx->lh) cudaFree(ctx->lh);
   if (ctx->host_L) cudaFreeHost(ctx->host_L);
   for (auto& kv : ctx->task_tables)

@@ -222,3 +222,30 @@ def test_gradient_sums(n, m, exact):
     G = t * Z * s / d
     ref = (G[:, :, None] * D).sum(1)
     assert np.all(np.abs(dx.cpu().numpy() - ref) <= ((e * abs(G))[:, :, None] * abs(D)).sum(1))
+
+
+# The FP64 factor: its diagonal tile, and the panel solve and trailing update
+# from digits, at tile edges and remainders, with rows whose entries span many
+# decades (t = 40: below e^-40).  By the theorem above with u = 2^-53, 4 u for
+# the entries of Z.
+@pytest.mark.parametrize("n", [2, 31, 33, 127, 128, 129, 161, 256, 257, 400, 641])
+@pytest.mark.parametrize("t", [0.5, 5.0, 40.0])
+def test_fp64_factor(ctx, n, t):
+    X = _dev(workloads.unit_cube_cloud(n=n, m=3, seed=n))
+    L = ctx.cholesky_factor(X, t, "fp64").cpu().numpy().astype(np.longdouble)
+    Z = ctx.similarity_matrix(X, t, "fp64").cpu().numpy()
+    assert np.abs(L @ L.T - Z).max() <= (n + 5) * 2.0 ** -53
+    assert not np.triu(L, 1).any()
+
+
+# A zero pivot of the FP64 factor, as above: other entries below e^-40, a pair
+# 1e-17 apart, within the diagonal tile, across two tiles and in the last one.
+@pytest.mark.parametrize("p", [1, 3, 33, 127, 128, 129, 255, 299])
+def test_fp64_zero_pivot_is_reported_with_its_row(ctx, p):
+    X = np.zeros((300, 2))
+    X[:, 0] = 40.0 * np.arange(300)
+    X[p] = X[p - 1] + [0.0, 1e-17]
+    with pytest.raises(M.MagnitudeError) as e:
+        ctx.cholesky_factor(_dev(X), 1.0, "fp64")
+    assert e.value.status == M.MAG_ENOTPD
+    assert f"row {p} " in str(e.value)
