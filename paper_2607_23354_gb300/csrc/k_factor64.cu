@@ -365,12 +365,6 @@ constexpr uint32_t OZ_TMEM = 512;
 constexpr int OZ_SMEM = NDIG * (128 * 128 + 64 * 128);
 constexpr int OZ_LD = 66;
 
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
 __device__ __forceinline__ void mma_f16_128x64(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
   constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
   asm volatile(

@@ -339,17 +339,16 @@ __device__ __forceinline__ void write_zeros(float* __restrict__ tile, float* __r
   }
 }
 
-__global__ void __launch_bounds__(POTRF_THREADS, 1)
-    k_potrf_f32(float* __restrict__ Z, float* __restrict__ Dinv, float* __restrict__ DinvT, int64_t K, DevStatus* st) {
+// One tile: Y = inv(L), YT = inv(L)^T; K: the tile column (for the report of a
+// pivot that is not positive).
+__device__ __forceinline__ void potrf_tile(float* __restrict__ tile, float* __restrict__ Y, float* __restrict__ YT,
+                                           int64_t K, DevStatus* st) {
   extern __shared__ __align__(16) unsigned char potrf_smem[];
   PotrfSmem& S = *reinterpret_cast<PotrfSmem*>(potrf_smem);
   float* W = S.M + TILE * LDP;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   // set by earlier kernels of the stream: uniform across the CTA
-  if (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE)) return;
-  float* tile = Z + tri_index(K, K) * TILE_ELEMS;
-  float* Y = Dinv + K * TILE_ELEMS;
-  float* YT = DinvT + K * TILE_ELEMS;
+  if (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) return;
   // A's blocks on and below the diagonal, I's on and above it
 #pragma unroll
   for (int i = 0; i < TILE * TILE / 4 / POTRF_THREADS; ++i) {
@@ -420,6 +419,20 @@ __global__ void __launch_bounds__(POTRF_THREADS, 1)
   write_inv(W, Y, YT, NPB - 1, w, POTRF_THREADS / 32, lane);
 }
 
+__global__ void __launch_bounds__(POTRF_THREADS, 1)
+    k_potrf_f32(float* __restrict__ Z, float* __restrict__ Dinv, float* __restrict__ DinvT, int64_t K, DevStatus* st) {
+  potrf_tile(Z + tri_index(K, K) * TILE_ELEMS, Dinv + K * TILE_ELEMS, DinvT + K * TILE_ELEMS, K, st);
+}
+
+// Diagonal tile K of each of a batch's problems (one CTA each).
+__global__ void __launch_bounds__(POTRF_THREADS, 1)
+    k_potrf_batch(const TiledProblem* __restrict__ probs, float* __restrict__ Z, float* __restrict__ Dinv,
+                  float* __restrict__ DinvT, int64_t K, DevStatus* st) {
+  const TiledProblem& P = probs[blockIdx.x];
+  potrf_tile(Z + (P.tile0 + tri_index(K, K)) * TILE_ELEMS, Dinv + (P.diag0 + K) * TILE_ELEMS,
+             DinvT + (P.diag0 + K) * TILE_ELEMS, K, st + blockIdx.x);
+}
+
 }  // namespace
 
 cudaError_t launch_potrf_f32(float* Z, float* Dinv, float* DinvT, int64_t K, DevStatus* st, cudaStream_t s) {
@@ -427,6 +440,16 @@ cudaError_t launch_potrf_f32(float* Z, float* Dinv, float* DinvT, int64_t K, Dev
                                        (int)sizeof(PotrfSmem));
   if (e != cudaSuccess) return e;
   k_potrf_f32<<<1, POTRF_THREADS, sizeof(PotrfSmem), s>>>(Z, Dinv, DinvT, K, st);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_potrf_batch(const TiledProblem* probs, int count, float* Z, float* Dinv, float* DinvT, int64_t K,
+                               DevStatus* st, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(k_potrf_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(PotrfSmem));
+  if (e != cudaSuccess) return e;
+  k_potrf_batch<<<(unsigned)count, POTRF_THREADS, sizeof(PotrfSmem), s>>>(probs, Z, Dinv, DinvT, K, st);
   note_launch();
   return cudaGetLastError();
 }

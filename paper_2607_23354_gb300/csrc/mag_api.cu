@@ -151,6 +151,8 @@ struct mag_ctx {
   int32_t xq_m = 0;
   int xq_e = 0;
   const void* xq_q = nullptr;
+  void* btws = nullptr;              // tiled batch workspace
+  size_t btws_bytes = 0;
   void* dg = nullptr;                // digits of a panel of the FP64 factor
   size_t dg_bytes = 0;
   void* rp = nullptr;                // partial sums of mag_residual and mag_grad
@@ -226,6 +228,8 @@ int fail(mag_ctx* c, int status, const char* fmt, ...) {
 // tolerance, so that an independent FP64 evaluation of the same residual
 // (which differs in rounding by far less than 10%) also meets the tolerance.
 constexpr double kStopMargin = 0.9;
+constexpr int kBatchTiledMin = 97;                     // see mag_solve_batch
+constexpr size_t kBatchTiledBytes = (size_t)16 << 30;  // a tiled group's workspace at most
 
 double bits_to_double(unsigned long long b) {
   double d;
@@ -1084,6 +1088,7 @@ int mag_ctx_destroy(mag_ctx* ctx) {
   if (ctx->xq) cudaFree(ctx->xq);
   if (ctx->rp) cudaFree(ctx->rp);
   if (ctx->dg) cudaFree(ctx->dg);
+  if (ctx->btws) cudaFree(ctx->btws);
   if (ctx->lh) cudaFree(ctx->lh);
   if (ctx->host_L) cudaFreeHost(ctx->host_L);
   for (auto& kv : ctx->task_tables)
@@ -2721,6 +2726,193 @@ int mag_grad(mag_ctx* ctx, const double* points, int64_t n, int32_t m, double t,
   return MAG_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// A group of a batch's problems through the tile kernels (k_batch_tiled.cu);
+// ids: indices into desc, sorted by decreasing n, a cloud's problems together;
+// cloud_of[i]: problem i's cloud.  Statuses (BatchStatus) into st_host.  *done
+// = false (and nothing else) when the workspace cannot be had.
+int batch_tiled_group(mag_ctx* ctx, const mag_batch_desc* desc, const int* ids, int count,
+                      const std::vector<BatchProblem>& all, const double* points, double* w_out, double* mag_out,
+                      std::vector<int>* st_host, bool* done) {
+  *done = false;
+  cudaStream_t s = ctx->stream;
+  std::vector<TiledProblem> probs(count);
+  std::vector<TiledCloud> clouds;
+  std::vector<int> order;                  // per cloud its problems
+  std::vector<int> first;                  // a cloud's first entry of order
+  int64_t tiles = 0, diags = 0, coords = 0, dims = 0;
+  int mmax[3] = {0, 0, 0};
+  std::vector<int2> gen[3];
+  int last = -1;
+  for (int i = 0; i < count; ++i) {
+    const mag_batch_desc& d = desc[ids[i]];
+    const int N = (d.n + TILE - 1) / TILE;
+    TiledProblem& p = probs[i];
+    p.tile0 = tiles, p.diag0 = diags, p.w_offset = d.w_offset, p.t = d.t, p.n = d.n, p.pid = ids[i];
+    tiled_scale(d.t, &p.g, &p.kg);
+    tiles += num_lower_tiles(N);
+    diags += N;
+    if (all[ids[i]].cloud != last) {
+      last = all[ids[i]].cloud;
+      TiledCloud c{};
+      c.point_offset = d.point_offset, c.xq_offset = coords, c.n = d.n, c.m = d.m, c.flag = (int)clouds.size();
+      c.range_offset = 2 * dims;
+      coords += (int64_t)d.n * d.m;
+      dims += d.m;
+      const int k = tiled_kind(d.m);
+      mmax[k] = std::max(mmax[k], (int)d.m);
+      for (int I = 0; I < N; ++I)
+        for (int J = 0; J <= I; ++J) gen[k].push_back(make_int2((int)clouds.size(), I << 8 | J));
+      clouds.push_back(c);
+      first.push_back(i);
+    }
+    p.flag = (int)clouds.size() - 1;
+    ++clouds.back().nprob;
+    order.push_back(i);
+  }
+  // tasks per tile column
+  const int Nmax = (probs[0].n + TILE - 1) / TILE;
+  std::vector<int2> upd, res;
+  std::vector<int4> pan;
+  std::vector<int> upd0(Nmax + 1, 0), pan0(Nmax + 1, 0), active(Nmax, 0);
+  for (int J = 0; J < Nmax; ++J) {
+    int64_t below = 0;
+    int& a = active[J];
+    for (; a < count && (probs[a].n + TILE - 1) / TILE > J; ++a) below += (probs[a].n + TILE - 1) / TILE - J - 1;
+    // tiles that share a split inverse: as many as leave two CTAs for every SM
+    const int share = (int)std::max<int64_t>(1, std::min<int64_t>(4, below / (2 * ctx->sm_count)));
+    upd0[J] = (int)upd.size();
+    pan0[J] = (int)pan.size();
+    for (int p = 0; p < a; ++p) {
+      const int N = (probs[p].n + TILE - 1) / TILE;
+      if (J > 0)
+        for (int I = J; I < N; ++I) upd.push_back(make_int2(p, I));
+      for (int I = J + 1; I < N; I += share) pan.push_back(make_int4(p, I, std::min(share, N - I), 0));
+      for (int I = J; I < N; ++I) res.push_back(make_int2(p, I << 8 | J));
+    }
+  }
+  upd0[Nmax] = (int)upd.size();
+  pan0[Nmax] = (int)pan.size();
+  // workspace: host-built tables (copied at once), then device arrays
+  size_t off = 0;
+  auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
+  const size_t o_cl = take(clouds.size() * sizeof(TiledCloud)), o_pr = take(probs.size() * sizeof(TiledProblem));
+  const size_t o_or = take(order.size() * sizeof(int));
+  size_t o_gen[3];
+  for (int k = 0; k < 3; ++k) o_gen[k] = take(gen[k].size() * sizeof(int2));
+  const size_t o_up = take(upd.size() * sizeof(int2)), o_pa = take(pan.size() * sizeof(int4));
+  const size_t o_re = take(res.size() * sizeof(int2));
+  const size_t tables = off;
+  const size_t o_z = off;  // zeroed: statuses, flags, counter
+  const size_t o_st = take((size_t)count * sizeof(DevStatus)), o_cf = take(clouds.size() * sizeof(int));
+  const size_t o_rem = take(sizeof(int)), o_ra = take((size_t)dims * 2 * sizeof(unsigned long long));
+  const size_t zeroed = off - o_z;
+  const size_t o_bs = take(all.size() * sizeof(int)), o_ts = take((size_t)count * sizeof(TiledState));
+  const size_t o_xq = take((size_t)coords * tiled_coord_bytes());
+  const size_t o_zf = take((size_t)tiles * TILE_ELEMS * 4), o_op = take((size_t)tiles * TILE_ELEMS * 4);
+  const size_t o_zi = take((size_t)tiles * TILE_ELEMS * 8);
+  const size_t o_p = take((size_t)tiles * 3 * TILE * sizeof(longlong2)), o_s = take((size_t)tiles * 3 * TILE * 4);
+  const size_t o_y = take((size_t)diags * TILE_ELEMS * 4), o_yt = take((size_t)diags * TILE_ELEMS * 4);
+  const size_t o_w = take((size_t)diags * TILE * 8), o_wi = take((size_t)diags * TILE * sizeof(int2));
+  if (!grow_buffer(ctx, &ctx->btws, &ctx->btws_bytes, off, 0)) return MAG_OK;
+  char* base = (char*)ctx->btws;
+  TiledBatch B{};
+  B.clouds = (TiledCloud*)(base + o_cl), B.probs = (TiledProblem*)(base + o_pr), B.state = (TiledState*)(base + o_ts);
+  B.st = (DevStatus*)(base + o_st), B.cloud_flags = (int*)(base + o_cf), B.remaining = (int*)(base + o_rem);
+  B.range = (unsigned long long*)(base + o_ra);
+  B.Xq = base + o_xq, B.Zf = (float*)(base + o_zf), B.Dinv = (float*)(base + o_y), B.DinvT = (float*)(base + o_yt);
+  B.Zi = (unsigned long long*)(base + o_zi), B.oper = (unsigned char*)(base + o_op);
+  B.P = (longlong2*)(base + o_p), B.S = (unsigned*)(base + o_s);
+  B.w = (double*)(base + o_w), B.W = (int2*)(base + o_wi);
+  int* d_bs = (int*)(base + o_bs);
+  for (size_t c = 0; c < clouds.size(); ++c) clouds[c].prob = (const int*)(base + o_or) + first[c];
+  std::vector<char> blob(tables);
+  auto put = [&](size_t o, const void* p, size_t bytes) { if (bytes) std::memcpy(blob.data() + o, p, bytes); };
+  put(o_cl, clouds.data(), clouds.size() * sizeof(TiledCloud));
+  put(o_pr, probs.data(), probs.size() * sizeof(TiledProblem));
+  put(o_or, order.data(), order.size() * sizeof(int));
+  for (int k = 0; k < 3; ++k) put(o_gen[k], gen[k].data(), gen[k].size() * sizeof(int2));
+  put(o_up, upd.data(), upd.size() * sizeof(int2));
+  put(o_pa, pan.data(), pan.size() * sizeof(int4));
+  put(o_re, res.data(), res.size() * sizeof(int2));
+  CU(cudaMemcpyAsync(base, blob.data(), tables, cudaMemcpyHostToDevice, s));
+  CU(cudaMemsetAsync(base + o_z, 0, zeroed, s));
+  CU(launch_bt_quantize(B, points, (int)clouds.size(), s));
+  for (int k = 0; k < 3; ++k)
+    CU(launch_bt_generate(B, points, k, (const int2*)(base + o_gen[k]), (int)gen[k].size(), mmax[k], s));
+  for (int J = 0; J < Nmax; ++J) {
+    CU(launch_bt_update(B, J, (const int2*)(base + o_up) + upd0[J], upd0[J + 1] - upd0[J], s));
+    CU(launch_potrf_batch(B.probs, active[J], B.Zf, B.Dinv, B.DinvT, J, B.st, s));
+    CU(launch_bt_panel(B, J, (const int4*)(base + o_pa) + pan0[J], pan0[J + 1] - pan0[J], s));
+  }
+  const double tol = kStopMargin * ctx->opt.ir_tol;
+  const int max_iter = std::max(ctx->opt.ir_max_iters, 1);
+  CU(launch_bt_solve(B, true, count, w_out, mag_out, d_bs, tol, max_iter, s));
+  int rem = 1;
+  for (int it = 0; rem > 0; ++it) {
+    CU(cudaMemsetAsync(B.remaining, 0, sizeof(int), s));
+    CU(launch_bt_residual(B, it == 0, (const int2*)(base + o_re), (int)res.size(), s));
+    CU(launch_bt_solve(B, false, count, w_out, mag_out, d_bs, tol, max_iter, s));
+    if (it == 0) continue;  // a problem rarely stops at its first residual
+    CU(cudaMemcpyAsync(&rem, B.remaining, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CU(cudaStreamSynchronize(s));
+  }
+  std::vector<int> bs(all.size());
+  CU(cudaMemcpyAsync(bs.data(), d_bs, bs.size() * sizeof(int), cudaMemcpyDeviceToHost, s));
+  CU(cudaStreamSynchronize(s));
+  for (int i = 0; i < count; ++i) (*st_host)[ids[i]] = bs[ids[i]];
+  *done = true;
+  return MAG_OK;
+}
+
+// The device bytes a problem adds to a group (its cloud's coordinates apart).
+size_t batch_tiled_bytes(int n) {
+  const size_t N = (n + TILE - 1) / TILE, T = (size_t)num_lower_tiles(N);
+  return T * (TILE_ELEMS * 16 + 3 * TILE * 20 + 64) + N * (TILE_ELEMS * 8 + TILE * 16) + 1024;
+}
+
+// Problems `ids` (sorted as for a group) in groups that fit the workspace;
+// those that could not be taken are left in *rest.
+int batch_tiled(mag_ctx* ctx, const mag_batch_desc* desc, const std::vector<int>& ids,
+                const std::vector<BatchProblem>& all, const double* points, double* w_out, double* mag_out,
+                std::vector<int>* st_host, std::vector<int>* rest) {
+  size_t budget = ctx->btws_bytes, want = 0;
+  for (int i : ids)
+    want += batch_tiled_bytes(desc[i].n) + 4096 + (size_t)desc[i].n * desc[i].m * tiled_coord_bytes() + 16 * desc[i].m + 512;
+  if (want > budget) {
+    size_t fre = 0, tot = 0;
+    CU(cudaMemGetInfo(&fre, &tot));
+    budget = std::max<size_t>(budget, std::min<size_t>(kBatchTiledBytes, (fre + budget) / 2));
+  }
+  for (size_t i = 0; i < ids.size();) {
+    size_t bytes = 0, k = i;
+    for (; k < ids.size(); ++k) {
+      const mag_batch_desc& d = desc[ids[k]];
+      size_t b = batch_tiled_bytes(d.n) + 4096;
+      if (k == i || all[ids[k]].cloud != all[ids[k - 1]].cloud) b += (size_t)d.n * d.m * tiled_coord_bytes() + 16 * d.m + 512;
+      if (k > i && bytes + b > budget) break;
+      bytes += b;
+    }
+    bool done = false;
+    TRY(batch_tiled_group(ctx, desc, ids.data() + i, (int)(k - i), all, points, w_out, mag_out, st_host, &done));
+    if (done) {
+      i = k;
+    } else if (k - i > 1) {
+      budget = bytes / 2;
+    } else {
+      rest->push_back(ids[i++]);
+    }
+  }
+  return MAG_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, const double* points,
                     double* w_out, double* mag_out, int32_t* status_out, mag_info* info) {
   if (!ctx) return MAG_EINVAL;
@@ -2738,8 +2930,7 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
   // group problems by cloud (same points, n, m): distances are shared across t
   std::vector<BatchCloud> clouds;
   std::vector<BatchProblem> probs(count);
-  std::vector<int> small, large;
-  int64_t dist_total = 0, max_pairs = 0, nmax = 0;
+  std::vector<int> small, tiled;
   {
     std::vector<std::pair<std::pair<int64_t, int64_t>, int>> keys;  // ((offset, n*65536+m), cloud)
     for (int32_t i = 0; i < count; ++i) {
@@ -2748,7 +2939,6 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
       probs[i].n = d.n;
       probs[i].t = d.t;
       if (d.n > BATCH_NMAX) {
-        large.push_back(i);
         probs[i].cloud = -1;
         continue;
       }
@@ -2757,27 +2947,44 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
       for (auto& k : keys)
         if (k.first == key) cid = k.second;
       if (cid < 0) {
-        BatchCloud c;
-        c.point_offset = d.point_offset;
-        c.dist_offset = dist_total;
-        c.n = d.n;
-        c.m = d.m;
-        cid = (int)clouds.size();
-        clouds.push_back(c);
+        cid = (int)keys.size();
         keys.push_back({key, cid});
+      }
+      probs[i].cloud = cid;
+      // more than a factor block: the tile kernels (unless a launch shape of
+      // the one-CTA kernel, or FP64 distances, are asked for)
+      if (ctx->opt.batch_shape == 0 && ctx->opt.exact_distances && d.n >= kBatchTiledMin && d.m <= 512)
+        tiled.push_back(i);
+      else
+        small.push_back(i);
+    }
+  }
+  auto by_size = [&](int a, int b) {
+    return probs[a].n != probs[b].n ? probs[a].n > probs[b].n : probs[a].cloud < probs[b].cloud;
+  };
+  std::vector<int> st_host(count, MAG_BATCH_OK);
+  if (!tiled.empty()) {
+    std::stable_sort(tiled.begin(), tiled.end(), by_size);
+    TRY(batch_tiled(ctx, desc, tiled, probs, points, w_out, mag_out, &st_host, &small));
+  }
+  if (!small.empty()) {
+    std::stable_sort(small.begin(), small.end(), by_size);
+    int64_t dist_total = 0, max_pairs = 0;
+    const int64_t nmax = probs[small[0]].n;
+    int last = -1, cid = -1;
+    for (int i : small) {  // a cloud's problems are consecutive
+      if (probs[i].cloud != last) {
+        last = probs[i].cloud;
+        const mag_batch_desc& d = desc[i];
+        cid = (int)clouds.size();
+        clouds.push_back({d.point_offset, dist_total, d.n, d.m});
         const int64_t pairs = (int64_t)d.n * (d.n - 1) / 2;
         dist_total += pairs;
         max_pairs = std::max(max_pairs, pairs);
       }
       probs[i].cloud = cid;
       probs[i].dist_offset = clouds[cid].dist_offset;
-      nmax = std::max<int64_t>(nmax, d.n);
-      small.push_back(i);
     }
-  }
-  std::vector<int> st_host(count, MAG_BATCH_OK);
-  if (!small.empty()) {
-    std::sort(small.begin(), small.end(), [&](int a, int b) { return probs[a].n > probs[b].n; });
     // launch shape (threads per CTA, CTAs per SM): options.batch_shape, else
     // the one tuned for this size class, else tuned below on a sample
     int cls = 0;
@@ -2880,8 +3087,10 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
     CU(cudaMemsetAsync(d_st, 0, (size_t)count * sizeof(int), s));
     CU(launch_batch_solve(shape, d_pr, d_or, (int)small.size(), d_D, d_cf, d_sf, d_sd, nmax, w_out,
                           mag_out, d_st, d_q, tol, max_iter, grids[shape], nullptr, s));
-    CU(cudaMemcpyAsync(st_host.data(), d_st, (size_t)count * sizeof(int), cudaMemcpyDeviceToHost, s));
+    std::vector<int> st_small(count);
+    CU(cudaMemcpyAsync(st_small.data(), d_st, (size_t)count * sizeof(int), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
+    for (int i : small) st_host[i] = st_small[i];
   }
   // problems too large for one CTA, or that the FP32 batch path could not
   // finish, go through the single-problem solver (which escalates precision)

@@ -399,6 +399,63 @@ struct BatchProblem {
 enum BatchStatus { MAG_BATCH_OK = 0, MAG_BATCH_NOTPD = 1, MAG_BATCH_NOCONV = 2, MAG_BATCH_DUPLICATE = 3,
                    MAG_BATCH_NONFINITE = 4 };
 constexpr int BATCH_NMAX = 2048;  // largest n solved inside one CTA
+
+// The tiled batch (k_batch_tiled.cu): arrays over a group of problems sorted by
+// decreasing n.  tile0, diag0: a problem's first tile (packed lower tiles) and
+// first diagonal tile.
+struct TiledCloud {
+  const int* prob;       // its problems (indices into probs), device
+  int64_t point_offset;  // doubles into the points array
+  int64_t xq_offset;     // coordinates into Xq
+  int64_t range_offset;  // into range
+  int32_t n, m, nprob, flag, e;  // flag: its entry of cloud_flags; e: set by the quantization
+};
+struct TiledProblem {
+  int64_t tile0, diag0, w_offset;
+  double t;
+  unsigned long long g;  // t as mag_fx.cuh's FxScale takes it
+  int32_t kg, n, pid, flag;  // flag: its cloud's entry of cloud_flags
+  float t63;                 // t 2^(63 - e), set by the quantization
+};
+struct TiledState {
+  double prev, zn;       // the last relative residual, ||Z||inf
+  int it, slow, ew, done;
+};
+struct TiledBatch {
+  TiledCloud* clouds;
+  TiledProblem* probs;
+  TiledState* state;
+  DevStatus* st;         // one per problem
+  int* cloud_flags;      // per cloud of the call: 1 non-finite, 2 coincident points, 4 no fixed-point range
+  int* remaining;        // problems that took a correction
+  unsigned long long* range; // per cloud and dimension
+  void* Xq;
+  float *Zf, *Dinv, *DinvT;  // per tile; per diagonal tile
+  unsigned long long* Zi;    // per tile: Z in units of 2^-60, two limbs
+  unsigned char* oper;       // per tile: 64 KB of FP16 operands
+  longlong2* P;              // per tile: row sums of Z w, column sums by halves
+  unsigned* S;               // ... of Z, units of 2^-24
+  double* w;
+  int2* W;
+};
+size_t tiled_coord_bytes();
+void tiled_scale(double t, unsigned long long* g, int* kg);
+int tiled_kind(int m);  // the generator's limb layout: clouds of one launch share it
+cudaError_t launch_bt_quantize(const TiledBatch& B, const double* points, int clouds, cudaStream_t s);
+// tasks: (cloud, I << 8 | J)
+cudaError_t launch_bt_generate(const TiledBatch& B, const double* points, int kind, const int2* tasks, int count,
+                               int mmax, cudaStream_t s);
+// tasks: (problem, I), I >= J
+cudaError_t launch_bt_update(const TiledBatch& B, int J, const int2* tasks, int count, cudaStream_t s);
+cudaError_t launch_potrf_batch(const TiledProblem* probs, int count, float* Z, float* Dinv, float* DinvT, int64_t K,
+                               DevStatus* st, cudaStream_t s);
+// tasks: (problem, first I, tiles, -)
+cudaError_t launch_bt_panel(const TiledBatch& B, int J, const int4* tasks, int count, cudaStream_t s);
+// tasks: (problem, I << 8 | J)
+cudaError_t launch_bt_residual(const TiledBatch& B, bool first, const int2* tasks, int count, cudaStream_t s);
+cudaError_t launch_bt_solve(const TiledBatch& B, bool first, int count, double* w_out, double* mag_out, int* status,
+                            double tol, int max_iter, cudaStream_t s);
+
 // Also sets cloud_flags[c] |= 1 (non-finite coordinate) / 2 (coincident points);
 // cloud_flags must be zeroed.
 cudaError_t launch_batch_dist(const double* X, const BatchCloud* clouds, int nclouds, int64_t max_pairs,

@@ -2,8 +2,11 @@
 // shared-memory matrix descriptor, MMA commit and TMEM loads.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include "mag_internal.cuh"
 
 namespace mag {
 
@@ -99,5 +102,87 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 // its chunk, 16-byte unit u (columns 8u .. 8u + 7 of the chunk) at unit
 // u ^ (r & 7).
 __device__ __forceinline__ uint32_t swizzled_unit(int r, int u) { return (uint32_t)(r * 128 + ((u ^ (r & 7)) << 4)); }
+
+// Untiled bulk copy to shared memory (16-byte aligned addresses, a multiple of
+// 16 bytes), completing on `bar`.
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+
+// ------------------------------------------- FP32 tiles as FP16 operands
+// A 128-row x 128-column FP16 operand in the layout the K-major SWIZZLE_128B
+// descriptors read: two chunks of 64 columns (16 KB each), row r at byte
+// 128 r of its chunk, 16-byte unit u (columns 8u .. 8u + 7 of the chunk) at
+// unit u ^ (r & 7).
+__device__ __forceinline__ uint32_t trsm_unit_offset(int r, int u16) {
+  const int chunk = u16 >> 3, u = u16 & 7;
+  return (uint32_t)(chunk * 16384 + r * 128 + ((u ^ (r & 7)) << 4));
+}
+
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
+
+// Power-of-two exponent e with max |x| * 2^e in [2^13, 2^14): 0 for a row of
+// zeros, subnormals or non-finite values.
+__device__ __forceinline__ int row_scale_exp(float m) {
+  const int ex = (int)((__float_as_uint(m) >> 23) & 0xffu);
+  if (ex == 0 || ex == 255) return 0;
+  const int e = 14 - (ex - 126);
+  return e < -100 ? -100 : (e > 100 ? 100 : e);
+}
+
+// 128 x 128 FP32 tile (row-major) in registers: warp w holds rows
+// 2 (w + 8 i) + (lane >> 4), i = 0..7, lane & 15 holds its columns
+// 8 (lane & 15) .. + 7.
+__device__ __forceinline__ void trsm_load(const float* __restrict__ src, float4 (&x)[16]) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = 2 * (warp + 8 * i) + (lane >> 4);
+    const float4* p = reinterpret_cast<const float4*>(src + r * TILE + 8 * (lane & 15));
+    x[2 * i] = __ldcg(p);
+    x[2 * i + 1] = __ldcg(p + 1);
+  }
+}
+
+// Split the register tile into scaled FP16 hi / lo operands and the row
+// exponents.
+__device__ __forceinline__ void trsm_split(const float4 (&x)[16], unsigned char* hi, unsigned char* lo, int* rexp) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = 2 * (warp + 8 * i) + (lane >> 4);
+    const float4 a = x[2 * i], b = x[2 * i + 1];
+    float m = fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))),
+                    fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w))));
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const int e = row_scale_exp(m);
+    const float sc = pow2f(e);
+    const float v[8] = {a.x * sc, a.y * sc, a.z * sc, a.w * sc, b.x * sc, b.y * sc, b.z * sc, b.w * sc};
+    __align__(16) __half h[8], l[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      h[q] = __float2half_rn(v[q]);
+      l[q] = __float2half_rn(v[q] - __half2float(h[q]));
+    }
+    const uint32_t off = trsm_unit_offset(r, lane & 15);
+    *reinterpret_cast<uint4*>(hi + off) = *reinterpret_cast<const uint4*>(h);
+    *reinterpret_cast<uint4*>(lo + off) = *reinterpret_cast<const uint4*>(l);
+    if ((lane & 15) == 0) rexp[r] = e;
+  }
+}
+
+__device__ __forceinline__ void mma_f16_128x128(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
+  // D = F32, A = B = F16, both K-major, M = 128, N = 128
+  constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
 
 }  // namespace mag

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import workloads
 
 pytestmark = pytest.mark.gpu
@@ -249,3 +250,45 @@ def test_fp64_zero_pivot_is_reported_with_its_row(ctx, p):
         ctx.cholesky_factor(_dev(X), 1.0, "fp64")
     assert e.value.status == M.MAG_ENOTPD
     assert f"row {p} " in str(e.value)
+
+
+# The batch's tile kernels: tile edges and remainders, one to sixteen tile
+# columns, each limb layout, one and several problems of a cloud, t from nearly
+# singular to nearly the identity.  The library's own bound on the relative
+# residual, by the oracle, and the magnitude as the weighting's sum (n u |w|_1).
+@pytest.mark.parametrize("m,ts", [(1, [3.0]), (4, [0.5, 2.0]), (6, [0.05, 40.0]), (17, [0.3]), (33, [0.1, 1.0, 5.0])])
+def test_batch_tiles(ctx, m, ts):
+    rng = np.random.default_rng(m)
+    sizes = [2, 96, 97, 127, 128, 129, 200, 255, 256, 257, 384, 641, 1000] + ([2048] if m == 4 else [])
+    clouds = [rng.standard_normal((n, m)) for n in sizes]
+    clouds[4][7] = clouds[4][3] + 1e-9  # closer than the quantized coordinates resolve
+    ws, mags, sts = ctx.solve_batch([_dev(c) for c in clouds], ts)
+    assert int(sts.abs().sum()) == 0
+    for i, c in enumerate(clouds):
+        for j, t in enumerate(ts):
+            w = ws[i * len(ts) + j].cpu().numpy()
+            assert oracle.relative_residual(c, t, w) <= 1e-14
+            assert abs(mags[i, j].item() - w.sum()) <= len(c) * 2.0 ** -53 * np.abs(w).sum()
+
+
+# What a cloud of several tiles is refused for, beside clouds that are solved:
+# the same statuses as from the one-CTA kernel (launch shape 1).
+def test_batch_tiles_statuses():
+    rng = np.random.default_rng(3)
+    clouds = [rng.standard_normal((300, 3)) for _ in range(7)]
+    clouds[1][299] = clouds[1][0]
+    clouds[2][150, 1] = np.nan
+    clouds[3][0, 0] = np.inf
+    clouds[4][:] = 1.5
+    clouds[5] *= 1e-200
+    out = []
+    for opt in (M.Options(), M.Options(batch_shape=1)):
+        c = M.Context(opt)
+        _, mags, sts = c.solve_batch([_dev(x) for x in clouds], [0.5, 4.0])
+        out.append((sts.cpu().numpy(), mags.cpu().numpy()))
+        c.close()
+    assert np.array_equal(out[0][0], out[1][0])
+    ok = out[0][0] == M.MAG_OK
+    assert ok[0].all() and ok[6].all()
+    assert not ok[1].any() and not ok[2].any() and not ok[3].any() and not ok[4].any()
+    assert np.allclose(out[0][1][ok], out[1][1][ok], rtol=1e-12)
