@@ -404,32 +404,34 @@ class Context:
         this device; ts: list of t values.  Returns (list of w per (cloud, t),
         mags tensor [len(clouds), len(ts)], statuses)."""
         flat = [c.to(torch.float64).contiguous() for c in clouds]
-        offs, descs, w_off = [], [], 0
-        p_off = 0
-        for c in flat:
-            offs.append(p_off)
-            p_off += c.numel()
         P = torch.cat([c.reshape(-1) for c in flat]) if flat else torch.empty(0, dtype=torch.float64,
                                                                             device=self.device)
-        for i, c in enumerate(flat):
-            for t in ts:
-                descs.append(mag_batch_desc(offs[i], w_off, c.shape[0], c.shape[1], float(t)))
-                w_off += c.shape[0]
-        D = (mag_batch_desc * len(descs))(*descs)
+        # mag_batch_desc as the rows of one int64 array (n and m share a word): a
+        # struct and a slice at a time took 3 us a problem
+        ts = torch.tensor([float(t) for t in ts], dtype=torch.float64)
+        n = torch.tensor([c.shape[0] for c in flat], dtype=torch.int64)
+        m = torch.tensor([c.shape[1] for c in flat], dtype=torch.int64)
+        size = torch.tensor([c.numel() for c in flat], dtype=torch.int64)
+        ns = n.repeat_interleave(len(ts))
+        count, w_off = len(ns), int(ns.sum())
+        desc = torch.empty(len(flat), len(ts), 4, dtype=torch.int64)
+        desc[:, :, 0] = (size.cumsum(0) - size)[:, None]
+        desc[:, :, 1] = (ns.cumsum(0) - ns).reshape(len(flat), len(ts))
+        desc[:, :, 2] = (n + (m << 32))[:, None]
+        desc[:, :, 3] = ts.view(torch.int64)
+        D = ctypes.cast(desc.data_ptr(), ctypes.POINTER(mag_batch_desc))
         W = torch.empty(w_off, dtype=torch.float64, device=self.device)
-        M = torch.empty(len(descs), dtype=torch.float64, device=self.device)
-        S = torch.empty(len(descs), dtype=torch.int32, device=self.device)
+        M = torch.empty(count, dtype=torch.float64, device=self.device)
+        S = torch.empty(count, dtype=torch.int32, device=self.device)
         info = mag_info()
         S.fill_(-1)
-        st = self._lib.mag_solve_batch(self._h, D, len(descs), _P(P.data_ptr()), _P(W.data_ptr()),
+        st = self._lib.mag_solve_batch(self._h, D, count, _P(P.data_ptr()), _P(W.data_ptr()),
                                        _P(M.data_ptr()), _P(S.data_ptr()), ctypes.byref(info))
         self.last_batch_info = info.as_dict()
         # per-problem failures are reported in S; raise only for a call-level error
         if st != MAG_OK and not bool((S == st).any()):
             self._check(st)
-        ws = []
-        for d in descs:
-            ws.append(W[d.w_offset:d.w_offset + d.n])
+        ws = list(torch.unsafe_split_with_sizes(W, ns.tolist())) if count else []
         return ws, M.reshape(len(flat), len(ts)), S.reshape(len(flat), len(ts))
 
 

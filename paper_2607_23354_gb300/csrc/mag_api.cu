@@ -2932,7 +2932,7 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
   std::vector<BatchProblem> probs(count);
   std::vector<int> small, tiled;
   {
-    std::vector<std::pair<std::pair<int64_t, int64_t>, int>> keys;  // ((offset, n*65536+m), cloud)
+    std::map<std::pair<int64_t, int64_t>, int> keys;  // (offset, n*65536+m) -> cloud
     for (int32_t i = 0; i < count; ++i) {
       const mag_batch_desc& d = desc[i];
       probs[i].w_offset = d.w_offset;
@@ -2943,14 +2943,7 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
         continue;
       }
       const std::pair<int64_t, int64_t> key(d.point_offset, (int64_t)d.n * 65536 + d.m);
-      int cid = -1;
-      for (auto& k : keys)
-        if (k.first == key) cid = k.second;
-      if (cid < 0) {
-        cid = (int)keys.size();
-        keys.push_back({key, cid});
-      }
-      probs[i].cloud = cid;
+      probs[i].cloud = keys.emplace(key, (int)keys.size()).first->second;
       // more than a factor block: the tile kernels (unless a launch shape of
       // the one-CTA kernel, or FP64 distances, are asked for)
       if (ctx->opt.batch_shape == 0 && ctx->opt.exact_distances && d.n >= kBatchTiledMin && d.m <= 512)
