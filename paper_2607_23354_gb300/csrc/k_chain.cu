@@ -289,59 +289,66 @@ __global__ void __launch_bounds__(CH_THREADS, 1)
 // B tiles of a factor, as the sweeps read them ([c][t] row-major):
 //   block q <  N - 1, I = q + 1:  Sf_I = L_{I,I-1}^T inv(L_II)^T   (= B_I^T)
 //   block q >= N - 1, I = q - N + 1:  Sb_I = L_{I+1,I} inv(L_II)  (= B'_I^T)
-// C = op(A) B with A, B row-major FP32 tiles, in FP32 on the CUDA cores:
-// K in chunks of 32 through shared memory, 8 x 8 outputs per thread.
-constexpr int PREP_KC = 32;
-constexpr int PREP_LD = TILE + 4;
+// C = op(A) B with A, B row-major FP32 tiles, in FP32 on the CUDA cores: four
+// CTAs a tile with 32 rows of C each, K in two chunks through shared memory, a
+// row block per warp and 4 x 4 outputs per thread (a broadcast and a contiguous
+// 16-byte read per k).  Bound: latency (a solve's few tiles leave most SMs
+// idle); one CTA a tile with 8 x 8 outputs took 57 us whatever n, now 11.
+constexpr int PREP_KC = 64;
+constexpr int PREP_ROWS = 32;
+constexpr int PREP_LD = PREP_ROWS + 4;
 
 __global__ void __launch_bounds__(256) k_chain_prep(const float* __restrict__ Z, const float* __restrict__ Dinv,
                                                     int64_t N, float* __restrict__ Sf, float* __restrict__ Sb) {
-  __shared__ __align__(16) float As[PREP_KC][PREP_LD];  // op(A)^T chunk: As[k][c] = op(A)[c][k]
-  __shared__ __align__(16) float Bs[PREP_KC][TILE];     // B chunk: Bs[k][t]
+  __shared__ __align__(16) float As[PREP_KC][PREP_LD];  // As[k][c] = op(A)[c0 + c][k]
+  __shared__ __align__(16) float Bs[PREP_KC][TILE];     // Bs[k][t]
   const int64_t q = blockIdx.x;
+  const int c0 = (int)blockIdx.y * PREP_ROWS;
   const bool fwd = q < N - 1;
   const int64_t I = fwd ? q + 1 : q - (N - 1);
   const float* A = Z + (fwd ? tri_index(I, I - 1) : tri_index(I + 1, I)) * TILE_ELEMS;
   const float* B = Dinv + (fwd ? (N + I) : I) * TILE_ELEMS;  // inv(L_II)^T or inv(L_II)
   float* C = (fwd ? Sf : Sb) + I * TILE_ELEMS;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  float acc[8][8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float acc[4][4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
   for (int k0 = 0; k0 < TILE; k0 += PREP_KC) {
-    for (int e = tid; e < PREP_KC * TILE; e += 256) {
-      const int k = e / TILE, c = e % TILE;
-      Bs[k][c] = B[(int64_t)(k0 + k) * TILE + c];
-      // forward: op(A) = A^T, op(A)[c][k] = A[k][c] (row k0 + k, coalesced);
-      // backward: op(A)[c][k] = A[c][k] (column read, 32 k per row)
-      if (fwd) {
-        As[k][c] = A[(int64_t)(k0 + k) * TILE + c];
-      } else {
-        const int cc = e / PREP_KC, kk = e % PREP_KC;
-        As[kk][cc] = A[(int64_t)cc * TILE + k0 + kk];
+#pragma unroll
+    for (int i = 0; i < PREP_KC * TILE / 4 / 256; ++i) {
+      const int e = tid + 256 * i, k = e >> 5, c = (e & 31) * 4;
+      *reinterpret_cast<float4*>(&Bs[k][c]) = *reinterpret_cast<const float4*>(B + (k0 + k) * TILE + c);
+    }
+#pragma unroll
+    for (int i = 0; i < PREP_KC * PREP_ROWS / 256; ++i) {
+      const int e = tid + 256 * i;
+      if (fwd) {  // op(A) = A^T: A[k][c0 + c]
+        const int k = e / PREP_ROWS, c = e % PREP_ROWS;
+        As[k][c] = A[(k0 + k) * TILE + c0 + c];
+      } else {  // A[c0 + c][k]
+        const int c = e / PREP_KC, k = e % PREP_KC;
+        As[k][c] = A[(c0 + c) * TILE + k0 + k];
       }
     }
     __syncthreads();
-#pragma unroll 4
+#pragma unroll 8
     for (int k = 0; k < PREP_KC; ++k) {
-      float a[8], b[8];
+      const float4 av = *reinterpret_cast<const float4*>(&As[k][4 * warp]);
+      const float4 bv = *reinterpret_cast<const float4*>(&Bs[k][4 * lane]);
+      const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = As[k][ty * 8 + i];
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 8; ++j) b[j] = Bs[k][tx * 8 + j];
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) C[(int64_t)(ty * 8 + i) * TILE + tx * 8 + j] = acc[i][j];
+  for (int i = 0; i < 4; ++i)
+    *reinterpret_cast<float4*>(C + (c0 + 4 * warp + i) * TILE + 4 * lane) =
+        make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
 }
 
 __global__ void k_scale_rhs_unset(const double* __restrict__ r, int64_t n, int64_t np, float* __restrict__ v,
@@ -375,7 +382,7 @@ cudaError_t launch_chain(K kern, int64_t N, void** args, cudaStream_t s) {
 
 cudaError_t launch_chain_prep(const float* Z, const float* Dinv, int64_t N, float* Sf, float* Sb, cudaStream_t s) {
   if (N < 2) return cudaSuccess;
-  k_chain_prep<<<(unsigned)(2 * (N - 1)), 256, 0, s>>>(Z, Dinv, N, Sf, Sb);
+  k_chain_prep<<<dim3((unsigned)(2 * (N - 1)), TILE / PREP_ROWS), 256, 0, s>>>(Z, Dinv, N, Sf, Sb);
   note_launch();
   return cudaGetLastError();
 }
