@@ -364,6 +364,7 @@ __device__ __forceinline__ void potrf_tile(float* __restrict__ tile, float* __re
 #pragma unroll 1
   for (int kb = 0; kb < NPB; ++kb) {
     const int o = kb * PB;
+    if (kb == NPB - 1) launch_next();  // the panel solve's set-up takes as long as the rest of this
     // the panel's row blocks in M: A's kb .. 3, then W's 0 .. kb (M's blocks
     // 4 .. 4 + kb): blocks kb + pw.  Warps 1, 2, 3 and 5 follow the diagonal
     // warp, away from its scheduler.

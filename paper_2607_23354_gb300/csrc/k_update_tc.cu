@@ -816,25 +816,31 @@ __global__ void __launch_bounds__(TRSM_THREADS, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t ntiles = N - K - 1;
   if (tid == 0) {
-    s_skip = (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) != 0;
     s_next = (int)atomicAdd(counter, 1u);
     abort_flag = 0;
     mbar_init(&done_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (s_skip || s_next >= ntiles) return;  // uniform: nothing claimed, nothing allocated
+  if (s_next >= ntiles) {  // uniform: nothing claimed, nothing allocated
+    wait_previous();
+    return;
+  }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_sh)),
                  "r"(TRSM_TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // the first tile is older than the diagonal tile's factor, which may still run
   float4 x[16];
-  trsm_load(Dinv + K * TILE_ELEMS, x);
-  trsm_split(x, b_hi, b_lo, bexp);
   int64_t tile = s_next;
   trsm_load(Z + tile_index(K + 1 + tile, K, wcap) * TILE_ELEMS, x);
+  trsm_split(x, a_hi, a_lo, aexp);
+  wait_previous();
+  trsm_load(Dinv + K * TILE_ELEMS, x);
+  if (tid == 0) s_skip = (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) != 0;
+  trsm_split(x, b_hi, b_lo, bexp);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -842,9 +848,11 @@ __global__ void __launch_bounds__(TRSM_THREADS, 1)
   const uint64_t deadline = globaltimer() + timeout_ns;
   uint32_t phase = 0;
   const float pscale = (float)(1 << FP16_SCALE_LOG2);
-  while (tile < ntiles) {
+  bool split_done = true;
+  while (tile < ntiles && !s_skip) {  // uniform
     const int64_t I = K + 1 + tile;
-    trsm_split(x, a_hi, a_lo, aexp);
+    if (!split_done) trsm_split(x, a_hi, a_lo, aexp);
+    split_done = false;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (tid == 0) s_next = (int)atomicAdd(counter, 1u);
     __syncthreads();
@@ -1087,10 +1095,10 @@ cudaError_t launch_trsm_tc(float* Z, const float* Dinv, int64_t K, int64_t N, in
   if (e != cudaSuccess) return e;
   if ((int64_t)grid > ntiles) grid = (int)ntiles;
   if (grid < 1) grid = 1;
-  k_trsm_tc<<<grid, TRSM_THREADS, smem, s>>>(Z, Dinv, K, N, k0, width, mode == UPD_FP16X3 ? 1 : 0,
-                                              static_cast<__half*>(hi), static_cast<__half*>(lo), counter, st,
-                                              10000000000ull, wcap,
-                                              mode == UPD_FP16 ? static_cast<__half*>(lh) : nullptr);
+  e = launch_after(k_trsm_tc, dim3(grid), dim3(TRSM_THREADS), smem, s, Z, Dinv, K, N, k0, width,
+                   mode == UPD_FP16X3 ? 1 : 0, static_cast<__half*>(hi), static_cast<__half*>(lo), counter, st,
+                   (uint64_t)10000000000ull, wcap, mode == UPD_FP16 ? static_cast<__half*>(lh) : nullptr);
+  if (e != cudaSuccess) return e;
   note_launch();
   return cudaGetLastError();
 }

@@ -88,6 +88,30 @@ struct DevStatus {
   unsigned long long hash_bits;    // checksum of the points (launch_hash)
 };
 
+// ------------------------------------------------- programmatic launches
+// A kernel launched with launch_after may start before the kernel ahead of it
+// on the stream has ended, once every block of that kernel has called
+// launch_next (or returned): its own set-up and reads of older data run
+// meanwhile.  It calls wait_previous in every block before it touches anything
+// the kernel ahead writes (or reads, where it writes), and before launch_next:
+// then whatever the kernel ahead itself waited for is complete too.
+#ifdef __CUDACC__
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid, c.blockDim = block, c.dynamicSmemBytes = smem, c.stream = s;
+  cudaLaunchAttribute a[1];
+  a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = a;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kern, P(args)...);
+}
+#endif
+
 // ---------------------------------------------------------------- launchers
 // Every launcher enqueues on `s` and returns cudaGetLastError().
 
