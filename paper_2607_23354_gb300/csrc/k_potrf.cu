@@ -347,17 +347,22 @@ __device__ __forceinline__ void potrf_tile(float* __restrict__ tile, float* __re
   PotrfSmem& S = *reinterpret_cast<PotrfSmem*>(potrf_smem);
   float* W = S.M + TILE * LDP;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+#pragma unroll
+  for (int i = 0; i < TILE * TILE / 4 / POTRF_THREADS; ++i) {  // I's blocks on and above the diagonal
+    const int e = tid + i * POTRF_THREADS, r = e >> 5, c = (e & 31) * 4;
+    if (c / PB >= r / PB)
+      *reinterpret_cast<float4*>(W + r * LDP + c) = make_float4(c == r ? 1.0f : 0.0f, c + 1 == r ? 1.0f : 0.0f,
+                                                                c + 2 == r ? 1.0f : 0.0f, c + 3 == r ? 1.0f : 0.0f);
+  }
+  wait_previous();
   // set by earlier kernels of the stream: uniform across the CTA
   if (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) return;
-  // A's blocks on and below the diagonal, I's on and above it
+  // A's blocks on and below the diagonal
 #pragma unroll
   for (int i = 0; i < TILE * TILE / 4 / POTRF_THREADS; ++i) {
     const int e = tid + i * POTRF_THREADS, r = e >> 5, c = (e & 31) * 4;
     if (c / PB <= r / PB)
       *reinterpret_cast<float4*>(S.M + r * LDP + c) = reinterpret_cast<const float4*>(tile)[e];
-    if (c / PB >= r / PB)
-      *reinterpret_cast<float4*>(W + r * LDP + c) = make_float4(c == r ? 1.0f : 0.0f, c + 1 == r ? 1.0f : 0.0f,
-                                                                c + 2 == r ? 1.0f : 0.0f, c + 3 == r ? 1.0f : 0.0f);
   }
   __syncthreads();
 
@@ -440,7 +445,8 @@ cudaError_t launch_potrf_f32(float* Z, float* Dinv, float* DinvT, int64_t K, Dev
   cudaError_t e = cudaFuncSetAttribute(k_potrf_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sizeof(PotrfSmem));
   if (e != cudaSuccess) return e;
-  k_potrf_f32<<<1, POTRF_THREADS, sizeof(PotrfSmem), s>>>(Z, Dinv, DinvT, K, st);
+  e = launch_after(k_potrf_f32, dim3(1), dim3(POTRF_THREADS), sizeof(PotrfSmem), s, Z, Dinv, DinvT, K, st);
+  if (e != cudaSuccess) return e;
   note_launch();
   return cudaGetLastError();
 }

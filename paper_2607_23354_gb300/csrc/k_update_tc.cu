@@ -565,6 +565,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(UPD_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
   const uint64_t deadline = globaltimer() + p.timeout_ns;
+  wait_previous();
   // both CTAs must hold the accumulator at the same TMEM address; after an
   // earlier launch gave up waiting, this one does no work either
   if (threadIdx.x == 0) {
@@ -625,7 +626,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(UPD_THREADS, 1)
           mbar_arrive_remote(r0_tq_empty + ts * 8u);
         }
         if (++ts == TQ) ts = 0, tph ^= 1u;
-        if (q < 0) break;
+        if (q < 0) {
+          launch_next();  // the last tasks' products and epilogue remain
+          break;
+        }
         int64_t I, J;
         decode_task(q, p, &I, &J);
         const int ya = (int)((I + rank - p.k0) * TILE), yb = (int)((J + rank - p.k0) * TILE);
@@ -873,6 +877,7 @@ __global__ void __launch_bounds__(TRSM_THREADS, 1)
       mma_commit(&done_bar);
     }
     const int64_t next = s_next;
+    if (next >= ntiles) launch_next();
     if (next < ntiles) trsm_load(Z + tile_index(K + 1 + next, K, wcap) * TILE_ELEMS, x);
     const bool waited = mbar_wait(&done_bar, phase, &abort_flag, deadline);
     phase ^= 1u;
@@ -987,7 +992,8 @@ cudaError_t launch_mode(const UpdMaps& maps, const CMap& cmap, const UpdParams& 
 }
 
 template <int MODE>
-cudaError_t launch_mode2(const UpdMaps& maps, const CMap& cmap, const UpdParams& p, int grid, cudaStream_t s) {
+cudaError_t launch_mode2(const UpdMaps& maps, const CMap& cmap, const UpdParams& p, int grid, bool after,
+                         cudaStream_t s) {
   constexpr int OPS = ModeCfg<MODE>::SPLIT ? 2 : 1;
   constexpr int CH = ModeCfg<MODE>::CHUNK;
   const size_t smem = (size_t)stages2_of<MODE>() * OPS * chunks2_of<MODE>() * 2 * 128 * CH + EPI_STAGING + 1024;
@@ -998,7 +1004,12 @@ cudaError_t launch_mode2(const UpdMaps& maps, const CMap& cmap, const UpdParams&
   grid &= ~1;  // whole clusters
   if (grid < 2) grid = 2;
   const CUtensorMap* c = reinterpret_cast<const CUtensorMap*>(cmap.m);
-  kern<<<grid, UPD_THREADS, smem, s>>>(m[0], m[2], *c, p);
+  if (after) {
+    e = launch_after(kern, dim3(grid), dim3(UPD_THREADS), smem, s, m[0], m[2], *c, p);
+    if (e != cudaSuccess) return e;
+  } else {
+    kern<<<grid, UPD_THREADS, smem, s>>>(m[0], m[2], *c, p);
+  }
   note_launch();
   return cudaGetLastError();
 }
@@ -1057,17 +1068,17 @@ int64_t update_tasks(int64_t N, int64_t j0, int64_t j1, bool pairs, std::vector<
 }
 
 cudaError_t launch_update_tc(const UpdMaps& maps, const CMap& cmap, UpdParams p, int mode, int grid, bool pairs,
-                             cudaStream_t s) {
+                             bool after, cudaStream_t s) {
   if (p.ntasks <= 0 || p.kc_hi <= p.kc_lo) return cudaSuccess;
   if (p.wcap <= 0) p.wcap = p.N;
   if (pairs) {
     if ((int64_t)grid > 2 * p.ntasks) grid = (int)(2 * p.ntasks);
     switch (mode) {
-      case UPD_TF32X3: return launch_mode2<UPD_TF32X3>(maps, cmap, p, grid, s);
-      case UPD_TF32: return launch_mode2<UPD_TF32>(maps, cmap, p, grid, s);
-      case UPD_BF16: return launch_mode2<UPD_BF16>(maps, cmap, p, grid, s);
-      case UPD_FP16X3: return launch_mode2<UPD_FP16X3>(maps, cmap, p, grid, s);
-      case UPD_FP16: return launch_mode2<UPD_FP16>(maps, cmap, p, grid, s);
+      case UPD_TF32X3: return launch_mode2<UPD_TF32X3>(maps, cmap, p, grid, after, s);
+      case UPD_TF32: return launch_mode2<UPD_TF32>(maps, cmap, p, grid, after, s);
+      case UPD_BF16: return launch_mode2<UPD_BF16>(maps, cmap, p, grid, after, s);
+      case UPD_FP16X3: return launch_mode2<UPD_FP16X3>(maps, cmap, p, grid, after, s);
+      case UPD_FP16: return launch_mode2<UPD_FP16>(maps, cmap, p, grid, after, s);
       default: return cudaErrorInvalidValue;
     }
   }

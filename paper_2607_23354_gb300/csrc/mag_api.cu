@@ -638,7 +638,8 @@ int tc_update(TcFactor& F, int b, int64_t k0, int kc_lo, int kc_hi, int64_t j0, 
     grid = (int)std::min<int64_t>(units * (F.pairs ? 2 : 1), 1 << 30);
   }
   TRY(prof_begin(ctx, cat, st));
-  CU(launch_update_tc(ctx->maps[b], *F.cmap, up, F.mode, grid, F.pairs, st));
+  // the trailing update beside a panel leaves no SM to a launch that would wait
+  CU(launch_update_tc(ctx->maps[b], *F.cmap, up, F.mode, grid, F.pairs, max_tasks == 0, st));
   TRY(prof_end(ctx, st));
   ++*F.launches;
   *F.flops += update_flops(F.N, k0 + kc_lo, k0 + kc_hi, j0, j1);

@@ -268,7 +268,7 @@ int64_t update_tasks(int64_t N, int64_t j0, int64_t j1, bool pairs, std::vector<
 // pairs: the CTA-pair (cta_group::2) kernel with a pair task table; grid is
 // rounded down to whole clusters of two CTAs.
 cudaError_t launch_update_tc(const UpdMaps& maps, const CMap& cmap, UpdParams p, int mode, int grid, bool pairs,
-                             cudaStream_t s);
+                             bool after, cudaStream_t s);
 
 // Panel copy of column K (tiles I in (K, N)) for the tensor-core update:
 // row (I - k0)*TILE + r, column (K - k0)*TILE + c of the row-major panel
