@@ -21,7 +21,7 @@
 // Per tile column K: the diagonal tile (FP64, k_potrf_f64), the digits of
 // inv(L_KK) and of the panel's tiles, the panel solve L_IK = A_IK inv(L_KK)^T,
 // the digits of the solved panel and the trailing update C_IJ -= L_IK L_JK^T.
-// n = 5001: 123 ms with FP64 products throughout, 20.9 ms this way (12.8 of
+// n = 5001: 123 ms with FP64 products throughout, 15.8 ms this way (8.5 of
 // them the 40 diagonal tiles); backward error 5e-16 -> 0.6e-16.
 #include <cuda_fp16.h>
 
@@ -36,29 +36,31 @@ namespace {
 
 // ---------------------------------------------------------- diagonal tile
 // The elimination of [A; I] of k_potrf.cu in FP64, in four panels of 32
-// columns, four columns at a time.  A's lower and W = inv(L)^T's upper
-// triangle share one 128 x 128 array, W's diagonal blocks have their own.
-// Bound: the FP64 pipe (555,000 SM cycles of warp operations, two thirds of
-// them the trailing updates) and, within a panel, the pivots' chain.
+// columns, four columns at a time, by a cluster of eight CTAs: each holds one
+// block of 32 rows, A's four (becoming L) and those of W = inv(L)^T.  Per panel
+// the CTA of the diagonal block factors it and hands it to the others' shared
+// memory, the blocks below it (and W's up to it) are solved, A's
+// go round in the same way, and every CTA updates its remaining columns.  Bound:
+// the FP64 pipe, 16 SM cycles a warp operation and 64 on one of its quarters:
+// the panels' chain of pivots (about 30 us a panel), then the trailing updates
+// (98,000 cycles on the busiest of eight CTAs, 555,000 on one).  214 us a tile;
+// one CTA took 343, an elimination column by column about 1,000.
 constexpr int PB = 32;
 constexpr int NPB = TILE / PB;
-constexpr int LDM = TILE + 2;
+constexpr int LDR = TILE + 2;
 constexpr int LDW = PB + 2;
 constexpr int P64_THREADS = 512;
-constexpr int PANEL_WARPS = NPB + 1;
-constexpr int BG_WARPS = P64_THREADS / 32 - PANEL_WARPS;
+constexpr int P64_CTAS = 2 * NPB;
 
 struct Potrf64Smem {
-  double M[TILE * LDM];          // block (i, j): A, becoming L (i >= j); W (i < j)
-  double Wd[NPB][PB * LDW];      // W's diagonal blocks
-  double rinv[TILE];             // 1 / L[c][c]
+  double R[PB * LDR];         // the CTA's rows
+  double D[PB * LDW];         // the panel's diagonal block of L
+  double X[NPB][PB * LDW];    // the panel's blocks of L below it, by row block
+  double rinv[PB];            // 1 / L[c][c] of the panel
 };
 
-__device__ __forceinline__ void bar_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(int id, int threads) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+__device__ __forceinline__ void st_remote_f64(uint32_t cluster_addr, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr), "d"(v) : "memory");
 }
 
 // s = sqrt(p) and its reciprocal, p > 0: the FP32 seed, two Newton steps, s
@@ -112,90 +114,109 @@ __device__ __forceinline__ void pivot_factor64(const double* a, int j, Pivot64& 
   q.bad = (int)b0 | (int)b1 << 1 | (int)b2 << 2 | (int)b3 << 3;
 }
 
-// A panel row's steps (DIAG: the diagonal block's rows); own: this lane's 32
-// entries, Ld: the panel's diagonal block of M.
+// A panel's steps for a block of 32 rows (DIAG: the diagonal block's) by four
+// warps, a row per lane: warp w owns column groups w and w + 4 of the eight.
+// The owner of a group scales its four columns and writes them to the row; the
+// others follow after a barrier of the four.  The owner of the next group
+// updates that one first and leaves its other until it has written.  (An SM
+// quarter issues a warp's FP64 operation in 64 cycles: a warp alone took 20 us
+// for its 528, 28 with the pivots.)  own: this lane's 32 entries, Ld: the panel's
+// diagonal block of L (row stride ld), rinv its reciprocals.
 template <bool DIAG>
-__device__ __forceinline__ void panel_rows64(Potrf64Smem& S, int o, double* own, int lane, int64_t K, DevStatus* st) {
-  constexpr int NBAR = 32 * PANEL_WARPS;
-  const double* Ld = S.M + o * LDM + o;
-  double a[PB];
+__device__ __forceinline__ void panel_rows64(double* own, const double* Ld, int ld, double* rinv, int w, int lane,
+                                             int row, DevStatus* st) {
+  double a[2][4];
 #pragma unroll
-  for (int c = 0; c < PB; ++c) a[c] = own[c];
-  Pivot64 q;
-  q.bad = 0;
-#pragma unroll 1
-  for (int g = 0; g < PB / 4; ++g) {
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) a[s][c] = own[16 * s + 4 * w + c];
+  // slot s (group w + 4 s) -= group g's columns
+  auto update = [&](double(&v)[4], int s, int g) {
     const int j = 4 * g;
-    if (DIAG) {
-      pivot_factor64(a, j, q);
-    } else {
-      bar_sync(1 + g, NBAR);
-      q.r0 = S.rinv[o + j], q.r1 = S.rinv[o + j + 1], q.r2 = S.rinv[o + j + 2], q.r3 = S.rinv[o + j + 3];
-      const double* r1 = Ld + (j + 1) * LDM + j;
-      q.l10 = r1[0];
-      q.l20 = r1[LDM], q.l21 = r1[LDM + 1];
-      q.l30 = r1[2 * LDM], q.l31 = r1[2 * LDM + 1], q.l32 = r1[2 * LDM + 2];
+    const double2 x01 = *reinterpret_cast<const double2*>(own + j), x23 = *reinterpret_cast<const double2*>(own + j + 2);
+    const double* Lq = Ld + (16 * s + 4 * w) * ld + j;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const double2 v01 = *reinterpret_cast<const double2*>(Lq + c * ld);
+      const double2 v23 = *reinterpret_cast<const double2*>(Lq + c * ld + 2);
+      v[c] = fma(-x23.y, v23.y, fma(-x23.x, v23.x, fma(-x01.y, v01.y, fma(-x01.x, v01.x, v[c]))));
     }
-    double x0 = a[0] * q.r0;
-    double x1 = fma(-x0, q.l10, a[1]) * q.r1;
-    double x2 = fma(-x1, q.l21, fma(-x0, q.l20, a[2])) * q.r2;
-    double x3 = fma(-x2, q.l32, fma(-x1, q.l31, fma(-x0, q.l30, a[3]))) * q.r3;
+  };
+  // group g = w + 4 s: its columns
+  auto eliminate = [&](double(&v)[4], int g) {
+    const int j = 4 * g;
+    Pivot64 q;
+    q.bad = 0;
+    if (DIAG) {
+      pivot_factor64(v, j, q);
+    } else {
+      q.r0 = rinv[j], q.r1 = rinv[j + 1], q.r2 = rinv[j + 2], q.r3 = rinv[j + 3];
+      const double* r1 = Ld + (j + 1) * ld + j;
+      q.l10 = r1[0];
+      q.l20 = r1[ld], q.l21 = r1[ld + 1];
+      q.l30 = r1[2 * ld], q.l31 = r1[2 * ld + 1], q.l32 = r1[2 * ld + 2];
+    }
+    double x0 = v[0] * q.r0;
+    double x1 = fma(-x0, q.l10, v[1]) * q.r1;
+    double x2 = fma(-x1, q.l21, fma(-x0, q.l20, v[2])) * q.r2;
+    double x3 = fma(-x2, q.l32, fma(-x1, q.l31, fma(-x0, q.l30, v[3]))) * q.r3;
     if (DIAG) {
       x0 = lane < j ? 0.0 : (lane == j ? q.s0 : x0);
       x1 = lane < j + 1 ? 0.0 : (lane == j + 1 ? q.s1 : x1);
       x2 = lane < j + 2 ? 0.0 : (lane == j + 2 ? q.s2 : x2);
       x3 = lane < j + 3 ? 0.0 : (lane == j + 3 ? q.s3 : x3);
-    }
-    own[j] = x0, own[j + 1] = x1, own[j + 2] = x2, own[j + 3] = x3;
-    if (DIAG) {
       if (lane == 0) {
-        S.rinv[o + j] = q.r0, S.rinv[o + j + 1] = q.r1, S.rinv[o + j + 2] = q.r2, S.rinv[o + j + 3] = q.r3;
+        rinv[j] = q.r0, rinv[j + 1] = q.r1, rinv[j + 2] = q.r2, rinv[j + 3] = q.r3;
         if (q.bad) {
           atomicOr(&st->flags, ST_NOTPD);
-          atomicMin(&st->notpd_index, (int)(K * TILE + o + j) + __ffs(q.bad));
-        }
-      }
-      __syncwarp();
-      bar_arrive(1 + g, NBAR);
-    }
-    // the remaining columns, rotated by four; beyond the panel's end nothing
-    // is needed any more
-#pragma unroll
-    for (int c4 = 0; c4 < PB - 4; c4 += 4) {
-      if (j + 4 + c4 < PB) {
-        const double* Lq = Ld + (j + 4 + c4) * LDM + j;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const double2 v01 = *reinterpret_cast<const double2*>(Lq + c * LDM);
-          const double2 v23 = *reinterpret_cast<const double2*>(Lq + c * LDM + 2);
-          a[c4 + c] = fma(-x3, v23.y, fma(-x2, v23.x, fma(-x1, v01.y, fma(-x0, v01.x, a[c4 + c + 4]))));
+          atomicMin(&st->notpd_index, row + j + __ffs(q.bad));
         }
       }
     }
+    own[j] = x0, own[j + 1] = x1, own[j + 2] = x2, own[j + 3] = x3;
+  };
+  auto meet = [] { asm volatile("bar.sync 1, 128;" ::: "memory"); };
+  if (w == 0) eliminate(a[0], 0);
+  meet();
+#pragma unroll 1
+  for (int g = 0; g < PB / 4 - 1; ++g) {
+    const int next = g + 1;
+    if (w == (next & 3)) {
+      if (next < 4) {
+        update(a[0], 0, g);
+        eliminate(a[0], next);
+      } else {
+        update(a[1], 1, g);
+        eliminate(a[1], next);
+      }
+    }
+    if (w > g && w != next) update(a[0], 0, g);
+    if (w + 4 > g && w + 4 != next) update(a[1], 1, g);
+    meet();
   }
 }
 
-// 8 x 32 outputs: C -= P Q^T, K = 32 (P: row stride ldp; Q, C in M).  The sums
-// start from C: the partial sums shrink towards the Schur complement, where a
-// sum taken apart rises to C's size and cancels (backward error 1.9e-16 for
+// 8 x 32 outputs: C -= P Q^T, K = 32 (P, C: rows of R; Q: a block of X).  The
+// sums start from C: the partial sums shrink towards the Schur complement, where
+// a sum taken apart rises to C's size and cancels (backward error 1.9e-16 for
 // 0.5e-16 at 128 points of the unit cube).
-__device__ __forceinline__ void trailing_job64(const double* P, int ldp, const double* Q, double* C, int lane) {
-  const double* p = P + (lane >> 3) * ldp;
-  const double* q = Q + (lane & 7) * LDM;
-  double* c = C + (lane >> 3) * LDM + (lane & 7);
+__device__ __forceinline__ void trailing_job64(const double* P, const double* Q, double* C, int lane) {
+  const double* p = P + (lane >> 3) * LDR;
+  const double* q = Q + (lane & 7) * LDW;
+  double* c = C + (lane >> 3) * LDR + (lane & 7);
   double acc[2][4];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = c[4 * i * LDM + 8 * j];
+    for (int j = 0; j < 4; ++j) acc[i][j] = c[4 * i * LDR + 8 * j];
 #pragma unroll 4
   for (int k = 0; k < PB; ++k) {
     double b[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = q[8 * j * LDM + k];
+    for (int j = 0; j < 4; ++j) b[j] = q[8 * j * LDW + k];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const double a = -p[4 * i * ldp + k];
+      const double a = -p[4 * i * LDR + k];
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[i][j] = fma(a, b[j], acc[i][j]);
     }
@@ -203,92 +224,91 @@ __device__ __forceinline__ void trailing_job64(const double* P, int ldp, const d
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) c[4 * i * LDM + 8 * j] = acc[i][j];
+    for (int j = 0; j < 4; ++j) c[4 * i * LDR + 8 * j] = acc[i][j];
 }
 
-// Quarter h (8 rows) of the trailing update with panel kb of column block jb,
-// row block number b of: A's jb .. 3, then W's 0 .. kb.
-__device__ __forceinline__ void trailing_block64(Potrf64Smem& S, int kb, int jb, int b, int h, int lane) {
-  const int ib = jb + b;
-  const double* Q = S.M + jb * PB * LDM + kb * PB;
-  if (ib < NPB) {
-    double* row = S.M + (ib * PB + 8 * h) * LDM;
-    trailing_job64(row + kb * PB, LDM, Q, row + jb * PB, lane);
-  } else {
-    const int wb = ib - NPB;
-    double* row = S.M + (wb * PB + 8 * h) * LDM;
-    if (wb == kb)
-      trailing_job64(S.Wd[kb] + 8 * h * LDW, LDW, Q, row + jb * PB, lane);
-    else
-      trailing_job64(row + kb * PB, LDM, Q, row + jb * PB, lane);
+// The CTA's block of 32 x 32 (row stride LDR) into dst of every CTA of the cluster.
+__device__ __forceinline__ void hand_round(const double* src, double* dst, int tid) {
+  const uint32_t d = smem_u32(dst);
+#pragma unroll
+  for (int i = 0; i < PB * PB / P64_THREADS; ++i) {
+    const int e = tid + i * P64_THREADS, r = e / PB, c = e % PB;
+    const double v = src[r * LDR + c];
+#pragma unroll
+    for (int k = 0; k < P64_CTAS; ++k) st_remote_f64(map_to_rank(d + (r * LDW + c) * 8, k), v);
   }
 }
 
-__global__ void __launch_bounds__(P64_THREADS, 1)
+__global__ void __cluster_dims__(P64_CTAS, 1, 1) __launch_bounds__(P64_THREADS, 1)
     k_potrf_f64(double* __restrict__ Z, double* __restrict__ Dinv, double* __restrict__ DinvT, int64_t K,
                 DevStatus* st) {
   extern __shared__ __align__(16) unsigned char p64_smem[];
   Potrf64Smem& S = *reinterpret_cast<Potrf64Smem*>(p64_smem);
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  if (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) return;  // uniform
+  const int rank = (int)blockIdx.x, blk = rank & (NPB - 1);
+  const bool isW = rank >= NPB;
+  // set by earlier kernels (this one sets none before the first cluster barrier): uniform over the cluster
+  if (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) return;
   double* tile = Z + tri_index(K, K) * TILE_ELEMS;
-#pragma unroll 8
-  for (int e = tid; e < TILE * TILE / 2; e += P64_THREADS) {
-    const int r = e >> 6, c = (e & 63) * 2;
-    const double2 v = c / PB <= r / PB ? reinterpret_cast<const double2*>(tile)[e] : make_double2(0.0, 0.0);
-    *reinterpret_cast<double2*>(S.M + r * LDM + c) = v;
+#pragma unroll
+  for (int i = 0; i < PB * TILE / 2 / P64_THREADS; ++i) {
+    const int e = tid + i * P64_THREADS, r = e >> 6, c = (e & 63) * 2;
+    double2 v = make_double2(0.0, 0.0);
+    if (isW) {
+      if (c == blk * PB + (r & ~1)) (r & 1 ? v.y : v.x) = 1.0;
+    } else if (c < (blk + 1) * PB) {
+      v = *reinterpret_cast<const double2*>(tile + (blk * PB + r) * TILE + c);
+    }
+    *reinterpret_cast<double2*>(S.R + r * LDR + c) = v;
   }
-  for (int e = tid; e < NPB * PB * PB; e += P64_THREADS) {
-    const int b = e / (PB * PB), r = e / PB % PB, c = e % PB;
-    S.Wd[b][r * LDW + c] = r == c ? 1.0 : 0.0;
-  }
-  __syncthreads();
+  cluster_sync_all();
 #pragma unroll 1
   for (int kb = 0; kb < NPB; ++kb) {
     const int o = kb * PB;
-    // the panel's warps: A's row blocks kb .. 3, W's 0 .. kb - 1 (warp = row
-    // block), W's kb-th on warp 4 + (kb + 1) % 4, away from the diagonal's scheduler
-    const int wk = NPB + ((kb + 1) & 3);
-    if (w < NPB) {
-      double* own = S.M + (w * PB + lane) * LDM + o;
-      if (w == kb)
-        panel_rows64<true>(S, o, own, lane, K, st);
-      else
-        panel_rows64<false>(S, o, own, lane, K, st);
-    } else if (w == wk) {
-      panel_rows64<false>(S, o, S.Wd[kb] + lane * LDW, lane, K, st);
-    } else if (kb > 0) {
-      // the rest of the previous panel's trailing update
-      const int bw = w < wk ? w - NPB : w - PANEL_WARPS;
-      int job = bw;
-#pragma unroll 1
-      for (int jb = kb + 1; jb < NPB; ++jb) {
-        const int jobs = 4 * (NPB - jb + kb);
-        for (; job < jobs; job += BG_WARPS) trailing_block64(S, kb - 1, jb, job >> 2, job & 3, lane);
-        job -= jobs;
+    if (rank == kb) {
+      if (w < 4) panel_rows64<true>(S.R + lane * LDR + o, S.R + o, LDR, S.rinv, w, lane, (int)(K * TILE + o), st);
+      __syncthreads();
+      hand_round(S.R + o, S.D, tid);
+      if (tid < PB) {
+        const double v = S.rinv[tid];
+        for (int k = 0; k < P64_CTAS; ++k)
+          if (k != rank) st_remote_f64(map_to_rank(smem_u32(&S.rinv[tid]), k), v);
+      }
+    }
+    cluster_sync_all();
+    const bool mine = isW ? blk <= kb : blk > kb;
+    if (mine && w < 4) panel_rows64<false>(S.R + lane * LDR + o, S.D, LDW, S.rinv, w, lane, 0, st);
+    __syncthreads();
+    if (mine && !isW) hand_round(S.R + o, S.X[blk], tid);
+    cluster_sync_all();
+    if (mine) {
+      // A's blocks up to the diagonal, W's all: a quarter (8 rows) of a product a job
+      const int last = isW ? NPB - 1 : blk;
+      for (int job = w; job < 4 * (last - kb); job += P64_THREADS / 32) {
+        const int jb = kb + 1 + (job >> 2);
+        double* row = S.R + 8 * (job & 3) * LDR;
+        trailing_job64(row + o, S.X[jb], row + jb * PB, lane);
       }
     }
     __syncthreads();
-    if (kb < NPB - 1) {
-      trailing_block64(S, kb, kb + 1, w >> 2, w & 3, lane);  // the next panel's four row blocks
-      __syncthreads();
+  }
+  if (!isW) {
+    for (int e = tid; e < PB * TILE; e += P64_THREADS) {
+      const int r = e >> 7, c = e & 127;
+      tile[(blk * PB + r) * TILE + c] = c <= blk * PB + r ? S.R[r * LDR + c] : 0.0;
     }
+    return;
   }
-  double* Y = Dinv + K * TILE_ELEMS;
-  double* YT = DinvT + K * TILE_ELEMS;
-  // W[c][r] = inv(L)[r][c]
-  auto wv = [&](int c, int r) -> double {
-    const int bc = c / PB, br = r / PB;
-    return bc == br ? S.Wd[bc][(c % PB) * LDW + r % PB] : (br > bc ? S.M[c * LDM + r] : 0.0);
-  };
-  for (int e = tid; e < TILE * TILE; e += P64_THREADS) {
-    const int r = e >> 7, c = e & 127;
-    tile[e] = c <= r ? S.M[r * LDM + c] : 0.0;
-    YT[e] = c >= r ? wv(r, c) : 0.0;
+  // W[c][r] = inv(L)[r][c], c = blk PB ..
+  double* Y = Dinv + K * TILE_ELEMS + blk * PB;
+  double* YT = DinvT + K * TILE_ELEMS + blk * PB * TILE;
+  for (int e = tid; e < PB * TILE; e += P64_THREADS) {
+    const int i = e >> 7, r = e & 127;
+    YT[e] = r >= blk * PB + i ? S.R[i * LDR + r] : 0.0;
   }
-  for (int e = tid; e < TILE * TILE; e += P64_THREADS) {
-    const int r = e >> 7, c = e & 127;
-    Y[e] = c <= r ? wv(c, r) : 0.0;
+  for (int e = tid; e < PB * TILE; e += P64_THREADS) {
+    const int r = e >> 5, i = e & 31;
+    Y[r * TILE + i] = r >= blk * PB + i ? S.R[i * LDR + r] : 0.0;
   }
 }
 
@@ -533,7 +553,7 @@ cudaError_t launch_potrf_f64(double* Z, double* Dinv, double* DinvT, int64_t K, 
   cudaError_t e = cudaFuncSetAttribute(k_potrf_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sizeof(Potrf64Smem));
   if (e != cudaSuccess) return e;
-  k_potrf_f64<<<1, P64_THREADS, sizeof(Potrf64Smem), s>>>(Z, Dinv, DinvT, K, st);
+  k_potrf_f64<<<P64_CTAS, P64_THREADS, sizeof(Potrf64Smem), s>>>(Z, Dinv, DinvT, K, st);
   note_launch();
   return cudaGetLastError();
 }
