@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(FX_THREADS, fx_ctas(KIND))
     const int64_t e = tile_off + (int64_t)r * TILE + 4 * lane;
     *reinterpret_cast<double2*>(Dd + e) = make_double2(ddv[0], ddv[1]);
     *reinterpret_cast<double2*>(Dd + e + 2) = make_double2(ddv[2], ddv[3]);
-  });
+  }, (int)blockIdx.y, (int)gridDim.y);
   finish_min(mind2b, mq, qe, flags, warpmin, st);
 }
 
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(FX_THREADS, fx_ctas(KIND))
       for (int o = 16; o > 0; o >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, o);
       if (lane == 0 && gr < n) atomicAdd(rowsum + gr, (double)rs);
     }
-  });
+  }, (int)blockIdx.y, (int)gridDim.y);
 #pragma unroll
   for (int c = 0; c < 4; ++c) colpart[warp][4 * lane + c] = cs[c];
   finish_min(mind2b, mq, sc.e, flags, warpmin, st);  // synchronizes
@@ -625,6 +625,18 @@ cudaError_t launch_generate_dist(const double* X, int64_t n, int m, double t, in
 
 namespace {
 
+// CTAs a tile: a tile's 16 rows a warp take 45 us, so while all of a launch's
+// CTAs are resident at once its rows are shared by two or four (n = 300, m = 6:
+// 52 -> 19 us).
+unsigned row_slices(int64_t tiles, int kind) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 1;
+  const int64_t resident = (int64_t)sms * fx_ctas(kind);
+  return 4 * tiles <= resident ? 4u : (2 * tiles <= resident ? 2u : 1u);
+}
+
 template <int KIND, bool WF, bool WD, bool EXP>
 cudaError_t launch_gen_q(const fx_coord* Xq, const double* X, int64_t n, int m, const FxScale& sc, double t,
                          unsigned tiles, float* Zf, double* Zd, double* rowsum, DevStatus* st, cudaStream_t s,
@@ -633,7 +645,7 @@ cudaError_t launch_gen_q(const fx_coord* Xq, const double* X, int64_t n, int m, 
   const size_t smem = fx_tile_smem(m);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<tiles, FX_THREADS, smem, s>>>(Xq, X, n, m, sc, t, Zf, Zd, rowsum, st, kind, tiny, kc, t0, W);
+  kern<<<dim3(tiles, row_slices(tiles, KIND)), FX_THREADS, smem, s>>>(Xq, X, n, m, sc, t, Zf, Zd, rowsum, st, kind, tiny, kc, t0, W);
   note_launch();
   return cudaGetLastError();
 }
@@ -727,7 +739,7 @@ cudaError_t launch_dist_q(const void* Xq, const double* X, int64_t n, int m, int
   auto kern = kd == 0 ? k_dist_q<0> : (kd == 1 ? k_dist_q<1> : k_dist_q<2>);
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  kern<<<(unsigned)tiles, FX_THREADS, smem, s>>>(q, X, n, m, e, Dd, st);
+  kern<<<dim3((unsigned)tiles, row_slices(tiles, kd)), FX_THREADS, smem, s>>>(q, X, n, m, e, Dd, st);
   note_launch();
   return cudaGetLastError();
 }

@@ -21,7 +21,8 @@
 //         p = r - r^2/2 + r^3/6 - r^4/24 + r^5/120, r = f ln2/256 < 2^-8.5, the
 //         cubic and later terms in 32 bits.  Omitted terms and truncations stay
 //         below 2^-57.5 relative, so the rounding to FP64 dominates: within
-//         0.55 units in the last place.
+//         0.55 units in the last place (and t d 2^-11 for t's own rounding to
+//         64 bits: 0.53 measured below t d = 64).
 //
 // The functions are host functions too: tests compare them with
 // arbitrary-precision arithmetic on the CPU.
@@ -49,9 +50,9 @@ constexpr int FX_MAX_DIM = 512;          // d^2 < 512 2^118 fits 128 bits
 // with LB = fx_limb_of(m).  31 + 30 bits while four dimensions' products fit
 // the 64-bit sums, 30 + 29 bits for 16 dimensions and, with the sums emptied
 // every 16, any more.  The finer grid at m <= 4 is for the pairs too close for
-// it (fx_close), which are common in few dimensions: the 8-component cloud of
-// 16,384 points in R^3 sends 20% of its warps to FP64 with 59 bits, 0.3% with
-// 61 (generation 2.35 and 1.7 ms).
+// it (fx_close), which are common in few dimensions and cost their whole warp
+// the FP64 differences: the generation of the 8-component cloud of 16,384 points
+// in R^3 takes 2.35 ms with 59 bits, 1.64 with 61.
 constexpr int FX_LOW_DIM = 4;
 constexpr int FX_SPILL = 16;
 FX_HD int fx_limb_of(int m) { return m <= FX_LOW_DIM ? 31 : 30; }
@@ -345,7 +346,7 @@ __device__ __forceinline__ void load_fx_table(fx_u64* tab) {
 // 4 lane + 3.  KIND: 0 for m <= FX_LOW_DIM, 1 for m <= FX_SPILL, 2 beyond.
 // Beyond FX_SPILL two rows are accumulated together, where the column reads
 // would set the pace; below, one (they hide behind the finishing work).  smem:
-// fx_tile_smem bytes.
+// fx_tile_smem bytes.  slice of slices (1, 2 or 4): that part of the rows only.
 constexpr int FX_THREADS = 256;
 inline int fx_kind(int m) { return m <= FX_LOW_DIM ? 0 : (m <= FX_SPILL ? 1 : 2); }
 // CTAs per SM the kernels over tiles are compiled for: one row at a time fits
@@ -357,7 +358,7 @@ inline size_t fx_tile_smem(int m) { return 2 * (size_t)128 * (m < FX_CHUNK ? m :
 
 template <int KIND, int THREADS = FX_THREADS, class F>
 __device__ __forceinline__ void fx_tile_pairs(const fx_coord* __restrict__ Xq, int64_t n, int m, int64_t row0,
-                                              int64_t col0, fx_coord* smem, F&& f) {
+                                              int64_t col0, fx_coord* smem, F&& f, int slice = 0, int slices = 1) {
   constexpr int R = KIND < 2 ? 1 : 2, LB = KIND == 0 ? 31 : 30, NW = THREADS / 32;
   const int mc = m < FX_CHUNK ? m : FX_CHUNK;
   fx_coord* xr = smem;              // [128][mc] row points (broadcast reads)
@@ -376,7 +377,7 @@ __device__ __forceinline__ void fx_tile_pairs(const fx_coord* __restrict__ Xq, i
     __syncthreads();
   }
 #pragma unroll 1
-  for (int i = 0; i < 128 / NW; i += R) {
+  for (int i = 128 / NW * slice / slices; i < 128 / NW * (slice + 1) / slices; i += R) {
     FxSquare q[R][4];
     FxSums s[R][4];
 #pragma unroll
