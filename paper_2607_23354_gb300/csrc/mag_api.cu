@@ -473,7 +473,10 @@ template <typename T>
 int factor_blocked(mag_ctx* ctx, T* Z, T* Dinv, int* launches, double* flops) {
   const Layout& L = ctx->lay;
   cudaStream_t s = ctx->stream;
-  const bool digits = sizeof(T) == 8 && grow_buffer(ctx, &ctx->dg, &ctx->dg_bytes, factor64_scratch_bytes(L.N), 0);
+  const size_t need = factor64_scratch_bytes(L.N);
+  const bool fits = ctx->opt.workspace_limit_bytes <= 0 ||
+                    (double)(ctx->ws_bytes + need) <= ctx->opt.workspace_limit_bytes;
+  const bool digits = sizeof(T) == 8 && fits && grow_buffer(ctx, &ctx->dg, &ctx->dg_bytes, need, 0);
   for (int64_t K = 0; K < L.N; ++K) {
     CU(launch_potrf_diag<T>(Z, Dinv, K, L.n, ctx->st(), s));
     if (digits)
@@ -2887,6 +2890,8 @@ int batch_tiled(mag_ctx* ctx, const mag_batch_desc* desc, const std::vector<int>
     size_t fre = 0, tot = 0;
     CU(cudaMemGetInfo(&fre, &tot));
     budget = std::max<size_t>(budget, std::min<size_t>(kBatchTiledBytes, (fre + budget) / 2));
+    if (ctx->opt.workspace_limit_bytes > 0)  // smaller groups; a problem alone may exceed it, as one CTA's scratch does
+      budget = (size_t)std::min<double>((double)budget, ctx->opt.workspace_limit_bytes);
   }
   for (size_t i = 0; i < ids.size();) {
     size_t bytes = 0, k = i;
