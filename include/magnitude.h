@@ -170,7 +170,10 @@ typedef struct mag_options {
                              stalls is replaced by the split factor
                              (mag_info.fallback = 3); -1 never; 1 whenever
                              the contraction is <= 16 (any n)              */
-  int32_t batch_shape;    /* mag_solve_batch launch shape: 0 (default) tuned
+  int32_t batch_shape;    /* mag_solve_batch launch shape: 0 (default):
+                             problems of 97 points or more (m <= 512, exact
+                             distances) through the tile kernels together, the
+                             rest one CTA each in a launch shape tuned
                              per size class (ceil(log2 max n)) on the first
                              batch of that class with at least twice the
                              largest grid of problems -- each shape solves a
@@ -193,14 +196,14 @@ typedef struct mag_options {
                              1 the same with FP32 tiles always; 2 the sweeps
                              with one progress counter and the full tile
                              product per step                               */
-  int32_t exact_distances;  /* distances of a multi-t call (mag_solve_multi,
-                             mag_sweep_tplus) from coordinates quantized to
+  int32_t exact_distances;  /* distances (every solve, residual, gradient and
+                             dense matrix) from coordinates quantized to
                              a common grid, as exact integer sums on the
                              integer pipe (1, default; pairs closer than
                              sqrt(m) 2^53 times the grid step take FP64
                              differences), or FP64 differences for all
                              pairs (0).  Either way within the FP64
-                             differences' rounding of d; m <= 32 and finite
+                             differences' rounding of d; m <= 512 and finite
                              coordinates, else FP64                          */
   int32_t reserved4;
 } mag_options;
@@ -452,8 +455,9 @@ typedef struct mag_batch_desc {
 
 /* a10: many independent solves (uneven n, any t) in one persistent launch
  * sequence.  desc: HOST array of count descriptors; points, w_out: device;
- * mag_out: device, count doubles.  Each problem is factored in FP32 and
- * refined in FP64 to ctx's ir_tol.  status_out (device, count int32, may be
+ * mag_out: device, count doubles.  Each problem is factored in FP32 (from 97
+ * points in split FP16 products with FP32 sums) and refined to ctx's ir_tol
+ * with residuals of FP64 accuracy or better.  status_out (device, count int32, may be
  * NULL) receives a per-problem mag_status.  Returns MAG_OK when every
  * problem converged, else the first failing status. */
 int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, const double* points,

@@ -908,7 +908,7 @@ __global__ void __launch_bounds__(1024) k_reduce_w(const double* __restrict__ w,
 // the kernel.  Tiles leave their row and column sums in P (slot of the other
 // block, like the residual's), added by k_grad_finish; the order of every sum
 // is fixed.  A thread per row over all columns, with FP64 distances, a division
-// and twice the pairs, took 31 ms at n = 8192, m = 16 on 64 of the 152 SMs; 3.9
+// and twice the pairs, took 31 ms at n = 8192, m = 16 on 64 of the 152 SMs; 4.2
 // now.
 constexpr int GRAD_THREADS = 512;
 constexpr int GRAD_LD = TILE + 2;
