@@ -96,8 +96,8 @@ __global__ void __launch_bounds__(RES_THREADS) k_resid_mf(const double* __restri
 
 // Stored-tile residual: Zw from the FP64 lower tiles (Z_IJ for I >= J; the
 // diagonal tiles are stored in full).  CTA (t, J) works on column block J:
-// t = 0 takes the diagonal tile; t >= 1 the strip of RS_STRIP tiles (I, J),
-// I in [J+1+(t-1)S, J+1+tS).  For each tile it stores the row contributions
+// t = 0 takes the diagonal tile; t >= 1 the strip of S tiles (I, J), I in
+// [J+1+(t-1)S, J+1+tS).  For each tile it stores the row contributions
 // Z_IJ w_J (rows of block I) as partial P[I][J][r]; over the strip it
 // accumulates the transposed contributions Z_IJ^T w_I (rows of block J) in
 // registers and stores their sum once as P[J][J+t][c], so the cross-lane
@@ -108,15 +108,27 @@ __global__ void __launch_bounds__(RES_THREADS) k_resid_mf(const double* __restri
 // 16 columns 16k + 2cg, 16k + 2cg + 1 (k < 8); warp wp and row slot rs cover
 // tile rows 16 wp + 4 i + rs (i < 4).  Each load instruction reads four
 // 128-byte row segments.
+//
+// S: eight tiles while that leaves every SM a strip, else as few as spread the
+// tiles over all SMs (a tile is 9 us of the FP64 pipe: with strips of eight, 24
+// tile rows took 96 us on a third of the SMs; a sweep of 3,000 points, 97
+// evaluations, 45.0 -> 41.5 ms).
 constexpr int RS_STRIP = 8;
+int strip_tiles(int64_t N) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return RS_STRIP;
+  return (int)std::min<int64_t>(RS_STRIP, (num_lower_tiles(N) + sms - 1) / sms);
+}
 
 __global__ void __launch_bounds__(256) k_resid_stored(const double* __restrict__ Zd, int64_t n, int64_t N,
                                                       const double* __restrict__ w,
-                                                      double* __restrict__ P) {
+                                                      double* __restrict__ P, int strip) {
   __shared__ double colp[8][TILE];
   const int64_t J = blockIdx.y;
   const int64_t t = blockIdx.x;
-  const int64_t nstrips = (N - 1 - J + RS_STRIP - 1) / RS_STRIP;
+  const int64_t nstrips = (N - 1 - J + strip - 1) / strip;
   if (t > nstrips) return;  // uniform
   const int tid = threadIdx.x, wp = tid >> 5, l = tid & 31, cg = l & 7, rs = l >> 3;
   double wc[16];
@@ -126,8 +138,8 @@ __global__ void __launch_bounds__(256) k_resid_stored(const double* __restrict__
     wc[2 * k] = col < n ? w[col] : 0.0;
     wc[2 * k + 1] = col + 1 < n ? w[col + 1] : 0.0;
   }
-  const int64_t I0 = t == 0 ? J : J + 1 + (t - 1) * RS_STRIP;
-  const int64_t I1 = t == 0 ? J + 1 : (I0 + RS_STRIP < N ? I0 + RS_STRIP : N);
+  const int64_t I0 = t == 0 ? J : J + 1 + (t - 1) * strip;
+  const int64_t I1 = t == 0 ? J + 1 : (I0 + strip < N ? I0 + strip : N);
   double cs[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) cs[k] = 0.0;
@@ -239,11 +251,12 @@ __global__ void k_split_ff(const double* __restrict__ w, int64_t n, int64_t np, 
 }
 
 __global__ void __launch_bounds__(256) k_resid_stored_ff(const double* __restrict__ Zd, int64_t n, int64_t N,
-                                                         const float2* __restrict__ wf, double* __restrict__ P) {
+                                                         const float2* __restrict__ wf, double* __restrict__ P,
+                                                         int strip) {
   __shared__ ffp colp[8][TILE];
   const int64_t J = blockIdx.y;
   const int64_t t = blockIdx.x;
-  const int64_t nstrips = (N - 1 - J + RS_STRIP - 1) / RS_STRIP;
+  const int64_t nstrips = (N - 1 - J + strip - 1) / strip;
   if (t > nstrips) return;  // uniform
   const int tid = threadIdx.x, wp = tid >> 5, l = tid & 31, cg = l & 7, rs = l >> 3;
   float2 wc[16];
@@ -253,8 +266,8 @@ __global__ void __launch_bounds__(256) k_resid_stored_ff(const double* __restric
     wc[2 * k] = wf[col];  // wf is zero-padded to a whole tile row
     wc[2 * k + 1] = wf[col + 1];
   }
-  const int64_t I0 = t == 0 ? J : J + 1 + (t - 1) * RS_STRIP;
-  const int64_t I1 = t == 0 ? J + 1 : (I0 + RS_STRIP < N ? I0 + RS_STRIP : N);
+  const int64_t I0 = t == 0 ? J : J + 1 + (t - 1) * strip;
+  const int64_t I1 = t == 0 ? J + 1 : (I0 + strip < N ? I0 + strip : N);
   ffp cs[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) cs[k] = ffp{0.0f, 0.0f};
@@ -737,12 +750,12 @@ __global__ void k_resid_sym_finish(const double* __restrict__ P, int64_t n, int6
 __global__ void k_resid_stored_finish(const double* __restrict__ P, int64_t n, int64_t N, int64_t np,
                                       const double* __restrict__ w, const double* __restrict__ b,
                                       const double* __restrict__ rowsum, double* __restrict__ r,
-                                      DevStatus* st) {
+                                      DevStatus* st, int strip) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double ra = 0.0, za = 0.0, wa = 0.0;
   if (j < n) {
     const int64_t I = j / TILE, rr = j % TILE;
-    const int64_t slots = I + 1 + (N - 1 - I + RS_STRIP - 1) / RS_STRIP;
+    const int64_t slots = I + 1 + (N - 1 - I + strip - 1) / strip;
     double s = 0.0, c = 0.0;
     for (int64_t J = 0; J < slots; ++J) {
       const double v = P[(I * N + J) * TILE + rr];
@@ -1318,12 +1331,13 @@ cudaError_t launch_residual_stored(const double* Zd, int64_t n, int64_t N, const
                                    const double* b, const double* rowsum, double* r, double* P, int64_t np,
                                    DevStatus* st, cudaStream_t s) {
   if (N > 65535) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)((N - 1 + RS_STRIP - 1) / RS_STRIP + 1), (unsigned)N);
-  k_resid_stored<<<grid, 256, 0, s>>>(Zd, n, N, w, P);
+  const int strip = strip_tiles(N);
+  const dim3 grid((unsigned)((N - 1 + strip - 1) / strip + 1), (unsigned)N);
+  k_resid_stored<<<grid, 256, 0, s>>>(Zd, n, N, w, P, strip);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_resid_stored_finish<<<blocks_for(np, 256), 256, 0, s>>>(P, n, N, np, w, b, rowsum, r, st);
+  k_resid_stored_finish<<<blocks_for(np, 256), 256, 0, s>>>(P, n, N, np, w, b, rowsum, r, st, strip);
   note_launch();
   return cudaGetLastError();
 }
@@ -1337,12 +1351,13 @@ cudaError_t launch_residual_stored_ff(const double* Zd, int64_t n, int64_t N, co
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const dim3 grid((unsigned)((N - 1 + RS_STRIP - 1) / RS_STRIP + 1), (unsigned)N);
-  k_resid_stored_ff<<<grid, 256, 0, s>>>(Zd, n, N, wf, P);
+  const int strip = strip_tiles(N);
+  const dim3 grid((unsigned)((N - 1 + strip - 1) / strip + 1), (unsigned)N);
+  k_resid_stored_ff<<<grid, 256, 0, s>>>(Zd, n, N, wf, P, strip);
   note_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_resid_stored_finish<<<blocks_for(np, 256), 256, 0, s>>>(P, n, N, np, w, b, rowsum, r, st);
+  k_resid_stored_finish<<<blocks_for(np, 256), 256, 0, s>>>(P, n, N, np, w, b, rowsum, r, st, strip);
   note_launch();
   return cudaGetLastError();
 }

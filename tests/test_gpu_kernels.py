@@ -292,3 +292,16 @@ def test_batch_tiles_statuses():
     assert ok[0].all() and ok[6].all()
     assert not ok[1].any() and not ok[2].any() and not ok[3].any() and not ok[4].any()
     assert np.allclose(out[0][1][ok], out[1][1][ok], rtol=1e-12)
+
+
+# The stored-tile residuals by strip length (1, 1, 2, 4, 5 and 8 tiles): a solve
+# refined with them, judged by the residual entry point's own pass over the
+# points (the library's bound of 1e-14).
+@pytest.mark.parametrize("n", [129, 300, 2300, 4000, 4500, 6300])
+def test_stored_residual_strips(ctx, n):
+    X = _dev(workloads.unit_cube_cloud(n=n, m=6, seed=n))
+    w, mag, info = ctx.solve(X, 3.0)
+    _, norms = ctx.residual(X, 3.0, w)
+    assert info["fallback"] == 0
+    assert norms["r_norm_inf"] <= 1e-14 * norms["z_norm_inf"] * norms["w_norm_inf"]
+    assert abs(mag - float(w.sum())) <= n * 2.0 ** -53 * float(w.abs().sum())
