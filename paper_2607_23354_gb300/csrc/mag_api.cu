@@ -2481,6 +2481,9 @@ int mag_solve_rhs(mag_ctx* ctx, const double* points, int64_t n, int32_t m, doub
     unsigned long long h = 0;
     TRY(points_hash(ctx, points, n, m, &h));
     if (h == ctx->fac_hash) {
+      // the coordinates in xq may be those of other points that lay at this
+      // address meanwhile (mag_residual, mag_grad)
+      ctx->xq_ok = false;
       TRY(reset_status(ctx));
       double overall = INFINITY;
       bool escalate = false;

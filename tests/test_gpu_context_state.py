@@ -1,0 +1,61 @@
+"""What a context keeps between calls (the factor, the quantized coordinates,
+side buffers, the report of a batch) must not reach a later call with other
+points: each test mixes entry points on one context and checks the results
+against plain FP64 arithmetic."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+M = pytest.importorskip("paper_2607_23354_gb300")
+
+
+def _dev(X):
+    return torch.from_numpy(np.ascontiguousarray(X)).cuda()
+
+
+def _rel(X, t, x, b):
+    """||b - Z x|| / (||Z|| ||x||) in FP64, Z from the points."""
+    d = torch.cdist(X, X, compute_mode="donot_use_mm_for_euclid_dist")
+    Z = torch.exp(-t * d)
+    return float((b - Z @ x).abs().max() / (Z.sum(1).max() * x.abs().max()))
+
+
+# A solve with a kept factor refines with the points it was given: in between,
+# another entry point quantizes other points at the same address (changed in
+# place and restored, or the temporary FP64 copies of FP32 points).  The other
+# points are 1e-6 away, so a refinement with them converges, to a residual of
+# about 1e-7 here; 1e-14 is the library's tolerance, doubled for the check's own
+# FP64 rounding.
+@pytest.mark.parametrize("options", [dict(precision="fp64"), dict(residual_mode="matrix_free")])
+@pytest.mark.parametrize("between", ["residual", "grad"])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_kept_factor_refines_with_its_own_points(options, between, fp32):
+    rng = np.random.default_rng(4)
+    n, t = 700, 2.0
+    A = _dev(rng.random((n, 6)))
+    B = A + 1e-6 * _dev(rng.standard_normal((n, 6)))
+    if fp32:
+        A, B = A.float(), B.float()
+    b = _dev(rng.standard_normal(n))
+    c = M.Context(M.Options(**options))
+
+    def other(P):
+        if between == "residual":
+            c.residual(P, t, b)
+        else:
+            c.grad(P, t, w=b)
+
+    c.solve(A, t)
+    if fp32:
+        other(B)
+    else:
+        keep = A.clone()
+        A.copy_(B)
+        other(A)
+        A.copy_(keep)
+    x, info = c.solve_rhs(A, t, b)
+    c.close()
+    assert info["factor_reused"] == 1 or fp32  # the copies' address is the allocator's choice
+    assert _rel(A.double(), t, x, b) <= 2e-14
