@@ -313,6 +313,12 @@ int ensure_workspace(mag_ctx* ctx, int64_t n, bool f32, bool f64, int64_t zf_til
     ctx->ws = p;
     ctx->ws_bytes = L.total;
   }
+  // the kept factor is addressed through the layout that it was made in
+  if (L.n != ctx->lay.n || L.f32 != ctx->lay.f32 || L.f64 != ctx->lay.f64 || L.dist != ctx->lay.dist ||
+      L.zf_tiles != ctx->lay.zf_tiles || L.W != ctx->lay.W) {
+    ctx->fac_valid = false;
+    ctx->chain_ready = ctx->lh_ready = false;
+  }
   ctx->lay = L;
   return MAG_OK;
 }

@@ -59,3 +59,29 @@ def test_kept_factor_refines_with_its_own_points(options, between, fp32):
     c.close()
     assert info["factor_reused"] == 1 or fp32  # the copies' address is the allocator's choice
     assert _rel(A.double(), t, x, b) <= 2e-14
+
+
+# A kept factor is given up when an entry point lays the workspace out for more
+# points (its tiles would be looked for at the other layout's offsets).
+@pytest.mark.parametrize("between", ["min_distance", "residual", "similarity_matrix"])
+def test_kept_factor_and_a_larger_layout(between):
+    rng = np.random.default_rng(9)
+    X, Y = _dev(rng.random((300, 4))), _dev(rng.random((2000, 4)))
+    b = _dev(rng.standard_normal(300))
+    c = M.Context()
+    c.solve(X, 3.0)
+    if between == "min_distance":
+        c.min_distance(Y)
+    elif between == "residual":
+        c.residual(Y, 3.0, Y[:, 0])
+    else:
+        c.similarity_matrix(Y, 3.0)
+    x, info = c.solve_rhs(X, 3.0, b)
+    assert info["factor_reused"] == 0
+    assert _rel(X, 3.0, x, b) <= 2e-14
+    # and is used again without such a call
+    c.solve(X, 3.0)
+    x, info = c.solve_rhs(X, 3.0, b)
+    c.close()
+    assert info["factor_reused"] == 1
+    assert _rel(X, 3.0, x, b) <= 2e-14
