@@ -165,12 +165,6 @@ __device__ __forceinline__ fx_u64 fixed60(fx_u64 z, int shift) {
   return fx_make(fx_lo(v) & 0x3fffffffu, (uint32_t)(v >> 30));
 }
 
-// The same rounded to FP32: the conversion rounds 32 bits with the rest as a
-// sticky bit (z's own error is far below it); shift < 70.
-__device__ __forceinline__ float float_of(fx_u64 z, int shift) {
-  return __uint_as_float(__float_as_uint(__uint2float_rn(fx_hi(z) | 1u)) - ((uint32_t)(31 + shift) << 23));
-}
-
 // One tile (I, J) of a cloud: the distances once, then every problem's entries.
 // Entries below e^-46 take the FP32 exponential and count as zero in the
 // residual (below its unit).
@@ -241,7 +235,7 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
             int shift;
             const fx_u64 z = fx_exp_fixed(dm[c], kd[c] + kg, g, fxtab, &shift);
             zi[c] = fixed60(z, shift);
-            zf[c] = float_of(z, shift);
+            zf[c] = fx_float_of(z, shift);
           }
         } else if ((unit >> c & 1) && gr < n) {
           zi[c] = 1ull << 62;  // 1

@@ -279,6 +279,18 @@ FX_HD fx_u64 fx_pack_any(fx_u64 z, int shift) {
   if (ex < 1) return 0;
   return ((fx_u64)(uint32_t)ex << 52) + (fx_make(ml, mh) >> 11) + ((ml >> 10) & 1u);
 }
+// The same rounded to FP32 (z in (0.25, 1] 2^63): the conversion rounds 32 bits
+// with the rest as a sticky bit, z's own error being far below it.  0 below
+// 2^-125, where the exponent field would run out.
+FX_HD float fx_float_of(fx_u64 z, int shift) {
+  if (shift >= 124) return 0.0f;
+#ifdef __CUDA_ARCH__
+  const float f = __uint2float_rn(fx_hi(z) | 1u);
+#else
+  const float f = (float)(fx_hi(z) | 1u);
+#endif
+  return fx_float(fx_bits(f) - ((uint32_t)(31 + shift) << 23));
+}
 FX_HD fx_u64 fx_exp_neg(fx_u64 dm, int k, fx_u64 g, const fx_u64* T) {
   int shift;
   const fx_u64 z = fx_exp_fixed(dm, k, g, T, &shift);

@@ -51,6 +51,19 @@ extern "C" void fx_exps(long n, const fx_u64* d, const double* t, fx_u64* o, fx_
     o[i] = fx_exp_neg_d(d[i], kg, g, T), gs[i] = g, kgs[i] = kg;
   }
 }
+extern "C" void fx_floats(long n, const double* d, double t, float* o) {
+  fx_u64 g;
+  int kg;
+  fx_scale_t(t, &g, &kg);
+  for (long i = 0; i < n; ++i) {
+    union { double d; fx_u64 u; } x;
+    x.d = d[i];
+    int shift;
+    const fx_u64 frac = (x.u & 0xfffffffffffffull) | 0x10000000000000ull;
+    const fx_u64 z = fx_exp_fixed(frac << 10, (int)(x.u >> 52) - 1023 + kg, g, T, &shift);
+    o[i] = fx_float_of(z, shift);
+  }
+}
 """
 
 
@@ -112,6 +125,20 @@ def test_exponential(lib):
         ti = D(int(g[i])) * D(2) ** (int(kg[i]) - 63) * D(2).ln() / 256
         assert abs(ti - D(float(t[i]))) <= D(float(t[i])) * D(2) ** -64
         assert _ulps(o[i], (-ti * D(float(d[i]))).exp()) <= D("0.55")
+
+
+# The FP32 entries of the batch's factor over every argument a pair can have: the
+# pairs too close for the quantized coordinates come here whatever their t d.
+# One rounding and the sticky bit's 2^-32; 0 (nothing else) from 2^-124 down.
+def test_float_entries(lib):
+    x = np.concatenate([np.linspace(1e-12, 90.0, 4001), 10.0 ** np.linspace(1.9, 12.0, 4001), [86.0, 88.7, 89.0, 1e6]])
+    for t in (0.7, 1e5):
+        d, o = np.ascontiguousarray(x / t), np.zeros(x.size, np.float32)
+        lib.fx_floats(ctypes.c_long(d.size), _ptr(d), ctypes.c_double(t), _ptr(o))
+        ref = np.exp(-(t * d).astype(np.longdouble))
+        small = ref < 2.0 ** -123
+        assert np.all(np.abs(o[~small] - ref[~small]) <= (2.0 ** -24 + 2.0 ** -30) * ref[~small])
+        assert np.all((o[small] == 0.0) | (np.abs(o[small] - ref[small]) <= 2.0 ** -24 * ref[small] + 2.0 ** -148))
 
 
 def test_table_is_generated():

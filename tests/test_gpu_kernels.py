@@ -305,3 +305,23 @@ def test_stored_residual_strips(ctx, n):
     assert info["fallback"] == 0
     assert norms["r_norm_inf"] <= 1e-14 * norms["z_norm_inf"] * norms["w_norm_inf"]
     assert abs(mag - float(w.sum())) <= n * 2.0 ** -53 * float(w.abs().sum())
+
+
+# Pairs of a batch that are too close for the quantized coordinates and yet far
+# apart in t d: two clusters 10 apart with nearly all in-cluster distances below
+# 0.1 (close is below sqrt(3) 2^-8 of 16 at m = 3), t d from 5 up to 1e8.  Every
+# problem stays with the batch's own factor.
+def test_batch_close_pairs_at_large_t(ctx):
+    rng = np.random.default_rng(12)
+    s = 10.0 ** rng.uniform(-3, -1.6, (260, 1))
+    X = rng.standard_normal((260, 3)) * s
+    X[130:] += 10.0
+    dmin = ctx.min_distance(_dev(X))[0]
+    ts = [f / dmin for f in (5.0, 50.0, 90.0, 300.0, 1e4, 1e6)]
+    ws, mags, sts = ctx.solve_batch([_dev(X)], ts)
+    assert int(sts.abs().sum()) == 0
+    assert ctx.last_batch_info["fallback"] == 0
+    for t, w, mag in zip(ts, ws, mags[0]):
+        w = w.cpu().numpy()
+        assert oracle.relative_residual(X, t, w) <= 1e-14
+        assert abs(mag.item() - w.sum()) <= 260 * 2.0 ** -53 * np.abs(w).sum()
