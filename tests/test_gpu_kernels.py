@@ -325,3 +325,27 @@ def test_batch_close_pairs_at_large_t(ctx):
         w = w.cpu().numpy()
         assert oracle.relative_residual(X, t, w) <= 1e-14
         assert abs(mag.item() - w.sum()) <= 260 * 2.0 ** -53 * np.abs(w).sum()
+
+
+# Pivots that have cancelled to a few units in the last place, as the second of
+# a pair at every place of a pivot block and in every panel, with a first one
+# that is not 1 (an earlier point near both): the factor is refused, or its
+# diagonal is positive and its backward error within the bound above.
+@pytest.mark.parametrize("p", [2, 3, 4, 5, 6, 7, 31, 33, 35, 67, 97, 126, 127])
+def test_cancelled_pivots(ctx, p):
+    rng = np.random.default_rng(p)
+    refused = 0
+    for _ in range(64):
+        X = np.zeros((128, 2))
+        X[:, 0] = 16.0 * np.arange(128)
+        X[p - 1] = X[p - 2] + rng.uniform(0.02, 0.6, 2)
+        X[p] = X[p - 1] + 10.0 ** rng.uniform(-7.5, -5.0) * rng.standard_normal(2)
+        try:
+            L = ctx.cholesky_factor(_dev(X), 1.0, "fp32").double()
+        except M.MagnitudeError as e:
+            assert e.status == M.MAG_ENOTPD
+            refused += 1
+            continue
+        assert bool((torch.diagonal(L) > 0).all())
+        assert float((L @ L.T - _z(_dev(X), 1.0)).abs().max()) <= (128 + 5) * 2.0 ** -23
+    assert refused < 64
