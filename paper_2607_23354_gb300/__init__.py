@@ -209,6 +209,24 @@ class Options:
         return o
 
 
+def _batch_descriptors(shapes, ts):
+    """Every cloud (n, m, entries) at every t as the rows of mag_batch_desc, in host
+    memory whatever PyTorch's default device, and each problem's n.  One int64
+    array (n and m share a word): a struct and a slice at a time took 3 us a
+    problem."""
+    ts = torch.tensor(ts, dtype=torch.float64, device="cpu")
+    n = torch.tensor([s[0] for s in shapes], dtype=torch.int64, device="cpu")
+    m = torch.tensor([s[1] for s in shapes], dtype=torch.int64, device="cpu")
+    size = torch.tensor([s[2] for s in shapes], dtype=torch.int64, device="cpu")
+    ns = n.repeat_interleave(len(ts))
+    desc = torch.empty(len(n), len(ts), 4, dtype=torch.int64, device="cpu")
+    desc[:, :, 0] = (size.cumsum(0) - size)[:, None]
+    desc[:, :, 1] = (ns.cumsum(0) - ns).reshape(len(n), len(ts))
+    desc[:, :, 2] = (n + (m << 32))[:, None]
+    desc[:, :, 3] = ts.view(torch.int64)
+    return desc, ns.tolist()
+
+
 class Context:
     """A mag_ctx bound to a CUDA device and stream (owns the solver workspace)."""
 
@@ -403,22 +421,11 @@ class Context:
         """Solve every cloud at every t.  clouds: list of (n_i x m) tensors on
         this device; ts: list of t values.  Returns (list of w per (cloud, t),
         mags tensor [len(clouds), len(ts)], statuses)."""
-        flat = [c.to(torch.float64).contiguous() for c in clouds]
+        flat, ts = [c.to(torch.float64).contiguous() for c in clouds], [float(t) for t in ts]
         P = torch.cat([c.reshape(-1) for c in flat]) if flat else torch.empty(0, dtype=torch.float64,
                                                                             device=self.device)
-        # mag_batch_desc as the rows of one int64 array (n and m share a word): a
-        # struct and a slice at a time took 3 us a problem
-        ts = torch.tensor([float(t) for t in ts], dtype=torch.float64)
-        n = torch.tensor([c.shape[0] for c in flat], dtype=torch.int64)
-        m = torch.tensor([c.shape[1] for c in flat], dtype=torch.int64)
-        size = torch.tensor([c.numel() for c in flat], dtype=torch.int64)
-        ns = n.repeat_interleave(len(ts))
-        count, w_off = len(ns), int(ns.sum())
-        desc = torch.empty(len(flat), len(ts), 4, dtype=torch.int64)
-        desc[:, :, 0] = (size.cumsum(0) - size)[:, None]
-        desc[:, :, 1] = (ns.cumsum(0) - ns).reshape(len(flat), len(ts))
-        desc[:, :, 2] = (n + (m << 32))[:, None]
-        desc[:, :, 3] = ts.view(torch.int64)
+        desc, ns = _batch_descriptors([(c.shape[0], c.shape[1], c.numel()) for c in flat], ts)
+        count, w_off = len(ns), sum(ns)
         D = ctypes.cast(desc.data_ptr(), ctypes.POINTER(mag_batch_desc))
         W = torch.empty(w_off, dtype=torch.float64, device=self.device)
         M = torch.empty(count, dtype=torch.float64, device=self.device)
@@ -431,7 +438,7 @@ class Context:
         # per-problem failures are reported in S; raise only for a call-level error
         if st != MAG_OK and not bool((S == st).any()):
             self._check(st)
-        ws = list(torch.unsafe_split_with_sizes(W, ns.tolist())) if count else []
+        ws = list(torch.unsafe_split_with_sizes(W, ns)) if count else []
         return ws, M.reshape(len(flat), len(ts)), S.reshape(len(flat), len(ts))
 
 
