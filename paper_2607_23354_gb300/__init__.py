@@ -17,6 +17,7 @@ import ctypes
 import dataclasses
 import os
 import threading
+from array import array
 from dataclasses import dataclass, fields
 
 import torch
@@ -211,20 +212,32 @@ class Options:
 
 def _batch_descriptors(shapes, ts):
     """Every cloud (n, m, entries) at every t as the rows of mag_batch_desc, in host
-    memory whatever PyTorch's default device, and each problem's n.  One int64
-    array (n and m share a word): a struct and a slice at a time took 3 us a
-    problem."""
+    memory whatever PyTorch's default device: (owner, address, each problem's n).
+    The rows are int64 words (n and m share one), formed as lists for few problems
+    and as tensors for many: 1.4 against 113 us for one problem, 104 against 120 for
+    256, 295 against 134 for 1,024 (a struct each: 3 us a problem)."""
+    k = len(ts)
+    if len(shapes) * k <= 256:
+        bits = array("q", array("d", ts).tobytes())
+        words, ns, p, w = array("q"), [], 0, 0
+        for n, m, size in shapes:
+            for t in bits:
+                words.extend((p, w, n | m << 32, t))
+                ns.append(n)
+                w += n
+            p += size
+        return words, words.buffer_info()[0], ns
     ts = torch.tensor(ts, dtype=torch.float64, device="cpu")
     n = torch.tensor([s[0] for s in shapes], dtype=torch.int64, device="cpu")
     m = torch.tensor([s[1] for s in shapes], dtype=torch.int64, device="cpu")
     size = torch.tensor([s[2] for s in shapes], dtype=torch.int64, device="cpu")
-    ns = n.repeat_interleave(len(ts))
-    desc = torch.empty(len(n), len(ts), 4, dtype=torch.int64, device="cpu")
+    ns = n.repeat_interleave(k)
+    desc = torch.empty(len(n), k, 4, dtype=torch.int64, device="cpu")
     desc[:, :, 0] = (size.cumsum(0) - size)[:, None]
-    desc[:, :, 1] = (ns.cumsum(0) - ns).reshape(len(n), len(ts))
+    desc[:, :, 1] = (ns.cumsum(0) - ns).reshape(len(n), k)
     desc[:, :, 2] = (n + (m << 32))[:, None]
     desc[:, :, 3] = ts.view(torch.int64)
-    return desc, ns.tolist()
+    return desc, desc.data_ptr(), ns.tolist()
 
 
 class Context:
@@ -424,9 +437,9 @@ class Context:
         flat, ts = [c.to(torch.float64).contiguous() for c in clouds], [float(t) for t in ts]
         P = torch.cat([c.reshape(-1) for c in flat]) if flat else torch.empty(0, dtype=torch.float64,
                                                                             device=self.device)
-        desc, ns = _batch_descriptors([(c.shape[0], c.shape[1], c.numel()) for c in flat], ts)
+        desc, address, ns = _batch_descriptors([(c.shape[0], c.shape[1], c.numel()) for c in flat], ts)
         count, w_off = len(ns), sum(ns)
-        D = ctypes.cast(desc.data_ptr(), ctypes.POINTER(mag_batch_desc))
+        D = ctypes.cast(address, ctypes.POINTER(mag_batch_desc))  # desc owns it
         W = torch.empty(w_off, dtype=torch.float64, device=self.device)
         M = torch.empty(count, dtype=torch.float64, device=self.device)
         S = torch.empty(count, dtype=torch.int32, device=self.device)

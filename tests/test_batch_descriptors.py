@@ -8,6 +8,8 @@ import torch
 
 M = pytest.importorskip("paper_2607_23354_gb300")
 
+# 1 to 256 problems are formed as lists, more as tensors
+
 
 class _Library:
     def mag_solve_batch(self, h, desc, count, points, w, mags, status, info):
@@ -24,7 +26,8 @@ def _solve_batch(clouds, ts):
 
 
 @pytest.mark.parametrize("sizes,ts", [([(3, 2)], [0.5]), ([(5, 4)], [1.0, 2.0]), ([(7, 1), (2, 9), (300, 16)], [1e-3, 7.0, 1e5]),
-                                      ([(2 + i, 3) for i in range(700)], [2.0, 3.0])])
+                                      ([(2 + i, 3) for i in range(128)], [2.0, 3.0]),
+                                      ([(2 + i, 3) for i in range(257)], [2.0]), ([(2 + i, 3) for i in range(700)], [2.0, 3.0])])
 @pytest.mark.parametrize("default", ["cpu", "meta"])
 def test_descriptors(sizes, ts, default):
     clouds = [torch.zeros(n, m, dtype=torch.float64) for n, m in sizes]
