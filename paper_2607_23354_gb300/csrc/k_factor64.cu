@@ -13,16 +13,24 @@
 //
 // for l = 0..7 (36 products).  The leading digit is at most 64, so |D_l| < 8 *
 // 128 * 2^14 = 2^24 and the sums are exact whatever their order; the levels are
-// combined in integers and rounded to FP64 once.  What is dropped (l > 7) is
-// about 2^-67 of the product of the two rows' largest entries, against 2^-53 of
-// every partial sum in FP64 arithmetic.  (Seven digits of 55 bits: backward
-// errors 10 to 40% above the FP64 products'.)
+// combined in integers and rounded to FP64 once.  The other 28 digit products (l
+// > 7) are left out: about 2^-57.5 of the product of the two rows' largest
+// entries (rms, 128 normal entries), against 2^-53 of every partial sum in FP64
+// arithmetic.  (Seven digits of 55 bits: backward errors 10 to 40% above the FP64
+// products'.)  That is a bound by rows, not by entries: an entry whose terms are
+// far below its rows' largest has its sum taken in FP64 (k_oz_gemm), so that
+// |Z - L L^T| stays a few units of |L| |L^T| entry by entry.  n = 300, six clouds
+// in R^6 to R^20, t = 1 to 6: at most 2.3e-15 of |L| |L^T|, FP64 products 8.0e-15
+// (by digits alone 0.03 at worst).
 //
 // Per tile column K: the diagonal tile (FP64, k_potrf_f64), the digits of
 // inv(L_KK) and of the panel's tiles, the panel solve L_IK = A_IK inv(L_KK)^T,
 // the digits of the solved panel and the trailing update C_IJ -= L_IK L_JK^T.
 // n = 5001: 123 ms with FP64 products throughout, 15.8 ms this way (8.5 of
-// them the 40 diagonal tiles); backward error 5e-16 -> 0.6e-16.
+// them the 40 diagonal tiles); backward error 5e-16 -> 0.6e-16.  The sums in FP64
+// cost nothing where the entries of Z are within a few decades; n = 4000: 11.4
+// ms, N(0, I_10) at t = 6 19.8, N(0, I_6) at t = 6 36.5 (a third of the entries;
+// FP64 products 87.9).
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -316,12 +324,15 @@ __global__ void __cluster_dims__(P64_CTAS, 1, 1) __launch_bounds__(P64_THREADS, 
 constexpr int NDIG = 8;
 constexpr int64_t CHUNK_BYTES = 128 * 128;                     // 128 rows x 64 FP16 columns
 constexpr int64_t DIGIT_BYTES = 2 * NDIG * CHUNK_BYTES;        // a tile's digits: [K chunk][digit][128 rows]
-constexpr int64_t DIGIT_STRIDE = DIGIT_BYTES + 1024;           // then 128 row exponents
+constexpr int64_t DIGIT_STRIDE = DIGIT_BYTES + 1024;           // then 128 row exponents and 128 row weights
 
-// Digits of the FP64 tiles of column K: slot 0 from `first` (inv(L_KK), when
-// given), the following slots from tiles (I, K), I = K + 1 ....  Row r of a
-// tile is x = X 2^(e_r - 62), |X| < 2^62, X = sum_i d_i 256^(7 - i).  A row
-// whose largest entry is below 2^-450 counts as zero.
+// Digits of the FP64 tiles of column K: slot 0 from `first` (inv(L_KK) without
+// its diagonal, when given), the following slots from tiles (I, K), I = K + 1
+// ....  Row r of a tile is x = X 2^(e_r - 62), |X| < 2^62, X = sum_i d_i
+// 256^(7 - i).  A row whose largest entry is below 2^-450 counts as zero.  A
+// row's weight is the exponent that its errors are judged by (k_oz_gemm): e_r,
+// nothing for a row of zeros, 64 more where the digits leave out the row.
+constexpr int WEIGHT_NONE = -16384;
 __global__ void __launch_bounds__(256) k_digits(const double* __restrict__ first, const double* __restrict__ Z,
                                                 int64_t K, unsigned char* __restrict__ out, const DevStatus* st) {
   if (st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) return;
@@ -334,15 +345,21 @@ __global__ void __launch_bounds__(256) k_digits(const double* __restrict__ first
   for (int r = warp; r < TILE; r += 8) {
     const double2 v01 = *reinterpret_cast<const double2*>(src + r * TILE + 4 * lane);
     const double2 v23 = *reinterpret_cast<const double2*>(src + r * TILE + 4 * lane + 2);
-    const unsigned long long b[4] = {
+    unsigned long long b[4] = {
         (unsigned long long)__double_as_longlong(v01.x), (unsigned long long)__double_as_longlong(v01.y),
         (unsigned long long)__double_as_longlong(v23.x), (unsigned long long)__double_as_longlong(v23.y)};
     unsigned mx = 0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) mx = max(mx, (unsigned)(b[q] >> 52) & 0x7ffu);
+    for (int q = 0; q < 4; ++q) {
+      if (first && slot == 0 && 4 * lane + q == r) b[q] = 0;
+      mx = max(mx, (unsigned)(b[q] >> 52) & 0x7ffu);
+    }
     mx = __reduce_max_sync(0xffffffffu, mx);
     const bool zero = mx < 1023 - 450;
-    if (lane == 0) exps[r] = zero ? 0 : (int)mx - 1022;
+    if (lane == 0) {
+      exps[r] = zero ? 0 : (int)mx - 1022;
+      exps[TILE + r] = mx == 0 ? WEIGHT_NONE : (int)mx - 1022 + (zero ? 64 : 0);
+    }
     __half d[NDIG][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -374,16 +391,54 @@ __global__ void __launch_bounds__(256) k_digits(const double* __restrict__ first
   }
 }
 
+// The least exponent among the entries of each half tile of Z (64 columns),
+// rows and columns of the padding left out.
+__global__ void __launch_bounds__(256) k_least_exponent(const double* __restrict__ Z, int64_t n, int* __restrict__ least) {
+  __shared__ int part[8];
+  const int64_t q = blockIdx.x >> 1;
+  const int h = blockIdx.x & 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int64_t I, J;
+  tri_coords(q, &I, &J);
+  const int64_t col = J * TILE + 64 * h + 2 * lane;
+  int e = 0x7ff;
+#pragma unroll 4
+  for (int r = warp; r < TILE; r += 8) {
+    const double2 z = *reinterpret_cast<const double2*>(Z + q * TILE_ELEMS + r * TILE + 64 * h + 2 * lane);
+    if (I * TILE + r < n) {
+      if (col < n) e = min(e, (__double2hiint(z.x) >> 20) & 0x7ff);
+      if (col + 1 < n) e = min(e, (__double2hiint(z.y) >> 20) & 0x7ff);
+    }
+  }
+  e = __reduce_min_sync(0xffffffffu, e);
+  if (lane == 0) part[warp] = e;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) e = min(e, part[k]);
+    least[blockIdx.x] = e - 1023;
+  }
+}
+
 // ---------------------------------------------------------------- products
 // 128 x 64 outputs (half h of a tile) of A B^T from the digits, K = 128 in two
 // chunks of 64 columns: 128 KB of A's digits and 64 KB of B's in shared memory
 // at a time, the eight levels in 8 x 64 TMEM columns.  ASSIGN: tile (I, K) of
-// the panel, A = its own digits (slot 1 + i), B = inv(L_KK) (slot 0); else the
-// trailing update of tile (I, J), A and B the panel's digits.
+// the panel, A = its own digits (slot 1 + i), B = inv(L_KK) without its
+// diagonal (slot 0), whose part is one FP64 product an entry; else the trailing
+// update of tile (I, J), A and B the panel's digits.
+//
+// What the digits drop is a fraction of the rows' largest entries max_a max_b,
+// about 2^-57, while the factor's error is to stay a fraction of |L| |L^T| entry
+// by entry, which is at least Z_ij.  Rows whose entries span many decades
+// (points in few dimensions at large t) leave some entries below: where neither
+// the half tile's least Z_ij nor |C_ij| (in the panel |a_ij inv_jj|) reaches
+// 2^-8 max_a max_b, an entry's sum is taken in FP64, a warp each.  The test runs
+// beside the products.  The panel's halves read all of a row of A there, so the
+// two CTAs of a tile are a cluster and write once both have read.
 constexpr int OZ_THREADS = 256;
 constexpr uint32_t OZ_TMEM = 512;
 constexpr int OZ_SMEM = NDIG * (128 * 128 + 64 * 128);
 constexpr int OZ_LD = 66;
+constexpr int OZ_MARGIN = 8;
 
 __device__ __forceinline__ void mma_f16_128x64(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate) {
   constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
@@ -402,21 +457,28 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+__device__ __forceinline__ int exponent_of(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) - 1023; }
+
+// least: k_least_exponent's; inv: inv(L_KK) (ASSIGN)
 template <bool ASSIGN>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    k_oz_gemm(double* __restrict__ Z, int64_t N, int64_t K, const unsigned char* __restrict__ digits, DevStatus* st,
-              uint64_t timeout_ns) {
+    k_oz_gemm(double* __restrict__ Z, int64_t N, int64_t K, const unsigned char* __restrict__ digits,
+              const int* __restrict__ least, const double* __restrict__ inv, DevStatus* st, uint64_t timeout_ns) {
   extern __shared__ __align__(1024) unsigned char oz_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)oz_raw + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t full_bar, done_bar[2];  // done_bar[c]: the products of chunk c
   __shared__ uint32_t tmem_base_sh;
   __shared__ int abort_flag;
-  __shared__ int ea[128], eb[64];
-  __shared__ int skip;
+  __shared__ int ea[128], eb[64], wa[128], wb[64];  // row exponents and weights
+  __shared__ uint2 low[128];                        // a row's columns 2 l (x) and 2 l + 1 (y) that need FP64 sums
+  __shared__ int skip, any_low;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) skip = (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) != 0;
   __syncthreads();
-  if (skip) return;  // uniform across the CTA
+  if (skip) {  // uniform across the CTA
+    if (ASSIGN) cluster_sync_all();  // the other half's CTA may have gone on
+    return;
+  }
   const int h = blockIdx.x & 1;
   int64_t I, J;
   const unsigned char *da, *db;
@@ -433,6 +495,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   }
   if (tid == 0) {
     abort_flag = 0;
+    any_low = 0;
     mbar_init(&full_bar, 1);
     mbar_init(&done_bar[0], 1);
     mbar_init(&done_bar[1], 1);
@@ -444,13 +507,22 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if (tid < 128) ea[tid] = reinterpret_cast<const int*>(da + DIGIT_BYTES)[tid];
-  if (tid >= 128 && tid < 192) eb[tid - 128] = reinterpret_cast<const int*>(db + DIGIT_BYTES)[64 * h + tid - 128];
+  const int* xa = reinterpret_cast<const int*>(da + DIGIT_BYTES);
+  const int* xb = reinterpret_cast<const int*>(db + DIGIT_BYTES) + 64 * h;
+  if (tid < 128)
+    ea[tid] = xa[tid], wa[tid] = xa[TILE + tid], low[tid] = make_uint2(0, 0);
+  else if (tid < 192)
+    eb[tid - 128] = xb[tid - 128], wb[tid - 128] = xb[TILE + tid - 128];
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base_sh;
   const uint64_t deadline = globaltimer() + timeout_ns;
+  const int64_t tile = tri_index(I, J);
+  double* C = Z + tile * TILE_ELEMS + 64 * h;
+  // the inverse's diagonal for this lane's columns 2 lane, 2 lane + 1
+  double2 iv = make_double2(1.0, 1.0);
+  if (ASSIGN) iv = make_double2(inv[(64 * h + 2 * lane) * (TILE + 1)], inv[(64 * h + 2 * lane + 1) * (TILE + 1)]);
   if (tid == 0) {
     bool ok = true;
     for (int c = 0; c < 2 && ok; ++c) {
@@ -480,8 +552,22 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         }
       mma_commit(&done_bar[c]);
     }
+  } else if (warp > 0) {
+    const int b0 = wb[2 * lane], b1 = wb[2 * lane + 1], bmax = __reduce_max_sync(0xffffffffu, max(b0, b1));
+    const int zmin = least[2 * tile + h] + OZ_MARGIN;
+    for (int r = warp - 1; r < TILE; r += OZ_THREADS / 32 - 1) {
+      const int w = wa[r];
+      if (w + bmax <= zmin) continue;  // uniform
+      const double2 c = *reinterpret_cast<const double2*>(C + r * TILE + 2 * lane);
+      const unsigned x = __ballot_sync(0xffffffffu, w + b0 > max(zmin, exponent_of(c.x) + exponent_of(iv.x) + OZ_MARGIN));
+      const unsigned y = __ballot_sync(0xffffffffu, w + b1 > max(zmin, exponent_of(c.y) + exponent_of(iv.y) + OZ_MARGIN));
+      if (lane == 0 && (x | y)) low[r] = make_uint2(x, y), *(volatile int*)&any_low = 1;
+    }
   }
   __syncwarp();
+  double2 old[16];  // rows warp + 8 i: on their way while the products run
+#pragma unroll
+  for (int i = 0; i < 16; ++i) old[i] = *reinterpret_cast<const double2*>(C + (warp + 8 * i) * TILE + 2 * lane);
   const bool waited = mbar_wait(&done_bar[1], 0, &abort_flag, deadline);
   const bool fine = __syncthreads_and(waited ? 1 : 0) != 0;  // one decision for the whole CTA
   tc_fence_after();
@@ -521,20 +607,70 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if (fine && any_low) {  // uniform
+    const double* A = Z + tri_index(I, K) * TILE_ELEMS;
+    const double* B = (ASSIGN ? inv : Z + tri_index(J, K) * TILE_ELEMS) + 64 * h * TILE;
+    for (int r = warp; r < TILE; r += OZ_THREADS / 32) {
+      const uint2 m = low[r];
+      if (!(m.x | m.y)) continue;  // uniform
+      const double2 a0 = reinterpret_cast<const double2*>(A + r * TILE)[lane];
+      const double2 a1 = reinterpret_cast<const double2*>(A + r * TILE)[lane + 32];
+      auto part = [&](int c) {  // this lane's columns 2 lane, 2 lane + 1 and the same beyond 64
+        double2 b0 = reinterpret_cast<const double2*>(B + c * TILE)[lane];
+        double2 b1 = reinterpret_cast<const double2*>(B + c * TILE)[lane + 32];
+        if (ASSIGN) {  // the columns before the diagonal
+          const int k = 64 * h + c - 2 * lane;
+          b0 = make_double2(k > 0 ? b0.x : 0.0, k > 1 ? b0.y : 0.0);
+          b1 = make_double2(k > 64 ? b1.x : 0.0, k > 65 ? b1.y : 0.0);
+        }
+        return fma(a1.y, b1.y, fma(a1.x, b1.x, fma(a0.y, b0.y, a0.x * b0.x)));
+      };
+#pragma unroll 1
+      for (int p = 0; p < 2; ++p) {
+        unsigned set = p ? m.y : m.x;
+        auto next = [&] {
+          const int c = 2 * (__ffs((int)set) - 1) + p;
+          set &= set - 1;
+          return c;
+        };
+        // four sums together share the reduction's last levels: 5.5 operations
+        // of the FP64 pipe a sum, 9 apart
+#pragma unroll 1
+        while (__popc(set) >= 4) {
+          const int c0 = next(), c1 = next(), c2 = next(), c3 = next();
+          const double s0 = part(c0), s1 = part(c1), s2 = part(c2), s3 = part(c3);
+          const bool up = (lane & 16) != 0, odd = (lane & 8) != 0;
+          double u0 = (up ? s2 : s0) + __shfl_xor_sync(0xffffffffu, up ? s0 : s2, 16);
+          double u1 = (up ? s3 : s1) + __shfl_xor_sync(0xffffffffu, up ? s1 : s3, 16);
+          double u = (odd ? u1 : u0) + __shfl_xor_sync(0xffffffffu, odd ? u0 : u1, 8);
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+          if ((lane & 7) == 0) stage[r * OZ_LD + (up ? (odd ? c3 : c2) : (odd ? c1 : c0))] = u;
+        }
+#pragma unroll 1
+        while (set) {
+          const int c = next();
+          double u = part(c);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+          if (lane == 0) stage[r * OZ_LD + c] = u;
+        }
+      }
+      __syncwarp();  // the row's entries are read below by this warp
+    }
+  }
+  if (ASSIGN) cluster_sync_all();
   if (fine) {
-    double* C = Z + tri_index(I, J) * TILE_ELEMS + 64 * h;
-#pragma unroll 4
+#pragma unroll
     for (int i = 0; i < 16; ++i) {
       const int r = warp + 8 * i;
       const double2 v = *reinterpret_cast<const double2*>(stage + r * OZ_LD + 2 * lane);
-      double2* p = reinterpret_cast<double2*>(C + r * TILE + 2 * lane);
-      if (ASSIGN) {
-        *p = v;
-      } else {
-        double2 c = *p;
+      double2 c = old[i];
+      if (ASSIGN)
+        c.x = fma(c.x, iv.x, v.x), c.y = fma(c.y, iv.y, v.y);
+      else
         c.x -= v.x, c.y -= v.y;
-        *p = c;
-      }
+      *reinterpret_cast<double2*>(C + r * TILE + 2 * lane) = c;
     }
   }
   if (tid == 0 && abort_flag) atomicOr(&st->flags, ST_TIMEOUT);
@@ -547,7 +683,21 @@ constexpr uint64_t kOzTimeout = 10000000000ull;
 
 }  // namespace
 
-size_t factor64_scratch_bytes(int64_t N) { return (size_t)(N + 1) * DIGIT_STRIDE; }
+// the digits of a panel and of an inverse, then the half tiles' least exponents
+size_t factor64_scratch_bytes(int64_t N) {
+  return (size_t)(N + 1) * DIGIT_STRIDE + 2 * (size_t)num_lower_tiles(N) * sizeof(int);
+}
+static int* least_of(void* scratch, int64_t N) {
+  return reinterpret_cast<int*>(static_cast<unsigned char*>(scratch) + (N + 1) * DIGIT_STRIDE);
+}
+
+cudaError_t launch_factor64_begin(const double* Z, int64_t n, int64_t N, void* scratch, cudaStream_t s) {
+  const int64_t tiles = num_lower_tiles(N);
+  if (2 * tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  k_least_exponent<<<(unsigned)(2 * tiles), 256, 0, s>>>(Z, n, least_of(scratch, N));
+  note_launch();
+  return cudaGetLastError();
+}
 
 cudaError_t launch_potrf_f64(double* Z, double* Dinv, double* DinvT, int64_t K, DevStatus* st, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(k_potrf_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -569,15 +719,22 @@ cudaError_t launch_factor64_panel(double* Z, const double* Dinv, int64_t K, int6
   if (e != cudaSuccess) return e;
   k_digits<<<(unsigned)(below + 1), 256, 0, s>>>(Dinv + K * TILE_ELEMS, Z, K, dg, st);
   note_launch();
-  k_oz_gemm<true><<<(unsigned)(2 * below), OZ_THREADS, smem, s>>>(Z, N, K, dg, st, kOzTimeout);
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)(2 * below)), c.blockDim = dim3(OZ_THREADS), c.dynamicSmemBytes = smem, c.stream = s;
+  cudaLaunchAttribute pair[1];
+  pair[0].id = cudaLaunchAttributeClusterDimension;
+  pair[0].val.clusterDim.x = 2, pair[0].val.clusterDim.y = 1, pair[0].val.clusterDim.z = 1;
+  c.attrs = pair, c.numAttrs = 1;
+  e = cudaLaunchKernelEx(&c, k_oz_gemm<true>, Z, N, K, (const unsigned char*)dg, (const int*)least_of(scratch, N),
+                         Dinv + K * TILE_ELEMS, st, kOzTimeout);
+  if (e != cudaSuccess) return e;
   note_launch();
   k_digits<<<(unsigned)below, 256, 0, s>>>(nullptr, Z, K, dg, st);
   note_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_factor64_update(double* Z, int64_t K, int64_t N, const void* scratch, DevStatus* st,
-                                   cudaStream_t s) {
+cudaError_t launch_factor64_update(double* Z, int64_t K, int64_t N, void* scratch, DevStatus* st, cudaStream_t s) {
   const int64_t below = N - K - 1, tiles = num_lower_tiles(below);
   if (below <= 0) return cudaSuccess;
   if (2 * tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
@@ -585,7 +742,7 @@ cudaError_t launch_factor64_update(double* Z, int64_t K, int64_t N, const void* 
   cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   k_oz_gemm<false><<<(unsigned)(2 * tiles), OZ_THREADS, smem, s>>>(Z, N, K, static_cast<const unsigned char*>(scratch),
-                                                                  st, kOzTimeout);
+                                                                  least_of(scratch, N), nullptr, st, kOzTimeout);
   note_launch();
   return cudaGetLastError();
 }

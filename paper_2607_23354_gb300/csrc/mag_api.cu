@@ -483,6 +483,7 @@ int factor_blocked(mag_ctx* ctx, T* Z, T* Dinv, int* launches, double* flops) {
   const bool fits = ctx->opt.workspace_limit_bytes <= 0 ||
                     (double)(ctx->ws_bytes + need) <= ctx->opt.workspace_limit_bytes;
   const bool digits = sizeof(T) == 8 && fits && grow_buffer(ctx, &ctx->dg, &ctx->dg_bytes, need, 0);
+  if (digits) CU(launch_factor64_begin((const double*)Z, L.n, L.N, ctx->dg, s));
   for (int64_t K = 0; K < L.N; ++K) {
     CU(launch_potrf_diag<T>(Z, Dinv, K, L.n, ctx->st(), s));
     if (digits)

@@ -349,3 +349,18 @@ def test_cancelled_pivots(ctx, p):
         assert bool((torch.diagonal(L) > 0).all())
         assert float((L @ L.T - _z(_dev(X), 1.0)).abs().max()) <= (128 + 5) * 2.0 ** -23
     assert refused < 64
+
+
+# The FP64 factor entry by entry, where the entries of a row span many decades and
+# the panels hold little of some: |L L^T - Z| <= (n + 1) u |L| |L^T|, plus 4 u,
+# by the theorem above with the product it is stated with, from clouds whose
+# panels pass by digits alone to ones that need FP64 products.
+@pytest.mark.parametrize("n", [129, 300])
+@pytest.mark.parametrize("cloud,m,t", [("cube", 6, 1.0), ("cube", 6, 6.0), ("cube", 20, 6.0), ("normal", 2, 3.0),
+                                       ("normal", 6, 3.0), ("normal", 6, 6.0), ("normal", 12, 6.0), ("normal", 20, 5.0)])
+def test_fp64_factor_by_entry(ctx, n, cloud, m, t):
+    rng = np.random.default_rng(m)
+    X = _dev(rng.random((n, m)) if cloud == "cube" else rng.standard_normal((n, m)))
+    L = ctx.cholesky_factor(X, t, "fp64").cpu().numpy().astype(np.longdouble)
+    Z = ctx.similarity_matrix(X, t, "fp64").cpu().numpy()
+    assert np.all(np.abs(L @ L.T - Z) <= (n + 5) * 2.0 ** -53 * (np.abs(L) @ np.abs(L).T))
