@@ -468,9 +468,10 @@ __global__ void __launch_bounds__(SYM_THREADS, 1)
 // COMP (the residual entry points): every sum compensated beyond chains of
 // four FMAs -- a row's lane sums and a column's groups of four rows by TwoSum
 // with the errors carried along, P as (sum, error) pairs, the row sums of Z
-// exact in 128-bit fixed point up to 2^-64 an entry -- which costs five FP64
-// operations a pair instead of two and still stays below the integer work's
-// time.  The solver's own residual (COMP false) takes FMA chains and FP32 norms.
+// exact in 128-bit fixed point up to 2^-64 an entry and added up as integers, so
+// that the norms do not depend on the order of the tiles either -- which costs
+// five FP64 operations a pair instead of two and still stays below the integer
+// work's time.  The solver's own residual (COMP false) takes FMA chains and FP32 norms.
 constexpr int SYMQ_LD = 33;
 
 // s + c <- s + c + x with the rounding of s collected in c
@@ -480,6 +481,15 @@ __device__ __forceinline__ void add_comp(double& s, double& c, double x) {
   s = t;
 }
 
+// A row sum of Z in units of 2^-63 as two words, h 2^32 + l: exact, in any order
+// (2^32 entries at most in each).
+__device__ __forceinline__ void add_row_sum(double* rowsum, int64_t row, fx_u64 l, fx_u64 h) {
+  fx_u64* p = reinterpret_cast<fx_u64*>(rowsum) + 2 * row;
+  atomicAdd(p, l);
+  atomicAdd(p + 1, h);
+}
+
+// rowsum: n doubles; COMP: n pairs of words
 template <int KIND, bool COMP>
 __global__ void __launch_bounds__(FX_THREADS, 2)
     k_resid_sym_q(const fx_coord* __restrict__ Xq, const double* __restrict__ X, int64_t n, int m, FxScale sc,
@@ -589,8 +599,7 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
         zl += ol;
         zh += zl < ol ? 1u : 0u;
       }
-      // units of 2^-63, 2^64 of them in zh: to FP64 from the two halves
-      if (lane == 0 && gr < n) atomicAdd(rowsum + gr, fma((double)zh, 2.0, (double)zl * 0x1p-63));
+      if (lane == 0 && gr < n) add_row_sum(rowsum, gr, zl & 0xffffffffull, (zl >> 32) + ((fx_u64)zh << 32));
     } else {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) zv += __shfl_xor_sync(0xffffffffu, zv, o);
@@ -637,8 +646,7 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
         e += colerr[k][c];
       }
       reinterpret_cast<double2*>(P)[(J * N + I) * TILE + c] = make_double2(s, e);
-      if (col0 + c < n)
-        atomicAdd(rowsum + col0 + c, fma((double)zcol_h[c], 0x1p-31, (double)zcol_l[c] * 0x1p-63));
+      if (col0 + c < n) add_row_sum(rowsum, col0 + c, zcol_l[c], zcol_h[c]);
     } else {
       double v = 0.0;
       float z = 0.0f;
@@ -657,8 +665,8 @@ __global__ void __launch_bounds__(FX_THREADS, 2)
 // norms; eight threads a row, each every eighth partial.
 __global__ void __launch_bounds__(256) k_resid_comp_finish(const double2* __restrict__ P, int64_t n, int64_t N,
                                                            const double* __restrict__ w, const double* __restrict__ b,
-                                                           const double* __restrict__ rowsum, double* __restrict__ r,
-                                                           DevStatus* st) {
+                                                           const ulonglong2* __restrict__ rowsum,
+                                                           double* __restrict__ r, DevStatus* st) {
   __shared__ double2 part[8][32];
   const int row = threadIdx.x & 31, k = threadIdx.x >> 5;
   const int64_t j = (int64_t)blockIdx.x * 32 + row;
@@ -687,7 +695,8 @@ __global__ void __launch_bounds__(256) k_resid_comp_finish(const double2* __rest
     const double rj = (bj - s) - e;
     r[j] = rj;
     ra = fabs(rj);
-    za = rowsum[j];
+    const ulonglong2 z = rowsum[j];
+    za = fma((double)z.y, 0x1p-31, (double)z.x * 0x1p-63);
     wa = fabs(w[j]);
   }
 #pragma unroll
@@ -1300,7 +1309,7 @@ cudaError_t launch_residual_sym(const double* X, int64_t n, int m, double t, con
 
 size_t residual_comp_bytes(int64_t n) {
   const size_t N = (size_t)((n + TILE - 1) / TILE);
-  return N * N * TILE * sizeof(double2) + N * TILE * sizeof(double);
+  return N * N * TILE * sizeof(double2) + N * TILE * sizeof(ulonglong2);
 }
 
 cudaError_t launch_residual_comp(const void* Xq, const double* X, int64_t n, int m, int qe, double t, const double* w,
@@ -1310,7 +1319,7 @@ cudaError_t launch_residual_comp(const void* Xq, const double* X, int64_t n, int
   if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
   double* P = static_cast<double*>(scratch);
   double* rowsum = P + 2 * N * N * TILE;
-  cudaError_t e = cudaMemsetAsync(rowsum, 0, (size_t)n * sizeof(double), s);
+  cudaError_t e = cudaMemsetAsync(rowsum, 0, (size_t)n * sizeof(ulonglong2), s);
   if (e != cudaSuccess) return e;
   const FxScale sc = fx_scale(t, qe);
   const size_t sq = (size_t)TILE * SYMQ_LD * sizeof(double) + fx_tile_smem(m);
@@ -1322,7 +1331,8 @@ cudaError_t launch_residual_comp(const void* Xq, const double* X, int64_t n, int
   note_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_resid_comp_finish<<<blocks_for(n, 32), 256, 0, s>>>(reinterpret_cast<const double2*>(P), n, N, w, b, rowsum, r, st);
+  k_resid_comp_finish<<<blocks_for(n, 32), 256, 0, s>>>(reinterpret_cast<const double2*>(P), n, N, w, b,
+                                                          reinterpret_cast<const ulonglong2*>(rowsum), r, st);
   note_launch();
   return cudaGetLastError();
 }

@@ -364,3 +364,17 @@ def test_fp64_factor_by_entry(ctx, n, cloud, m, t):
     L = ctx.cholesky_factor(X, t, "fp64").cpu().numpy().astype(np.longdouble)
     Z = ctx.similarity_matrix(X, t, "fp64").cpu().numpy()
     assert np.all(np.abs(L @ L.T - Z) <= (n + 5) * 2.0 ** -53 * (np.abs(L) @ np.abs(L).T))
+
+
+# The norms of the residual entry point add the tiles' row sums of Z in any order:
+# exactly, so that equal calls give equal bits (n = 3000: 24 tiles a row) and the
+# row sum is the exact one, rounded (2^-64 dropped of every entry).
+def test_residual_norms_are_the_same_every_time(ctx):
+    rng = np.random.default_rng(21)
+    X = rng.standard_normal((3000, 5))
+    w = rng.standard_normal(3000)
+    norms = [ctx.residual(_dev(X), 0.8, _dev(w))[1] for _ in range(24)]
+    assert all(v == norms[0] for v in norms)
+    Z = ctx.similarity_matrix(_dev(X), 0.8).cpu().numpy().astype(np.longdouble)
+    z = Z.sum(1).max()
+    assert abs(norms[0]["z_norm_inf"] - z) <= 3 * 2.0 ** -53 * z
