@@ -288,6 +288,42 @@ Layout plan(const mag_ctx* ctx, int64_t n, bool f32, bool f64, bool dist = false
   return L;
 }
 
+// Side buffers hold nothing from one call to the next (partial sums, digits of a
+// panel, the batch's workspaces): a call that needs their memory gets it back.
+size_t side_bytes(const mag_ctx* ctx) { return ctx->rp_bytes + ctx->btws_bytes + ctx->dg_bytes + ctx->bws_bytes; }
+void release_side(mag_ctx* ctx, void** keep = nullptr) {
+  struct {
+    void** p;
+    size_t* bytes;
+  } all[] = {{&ctx->rp, &ctx->rp_bytes}, {&ctx->btws, &ctx->btws_bytes}, {&ctx->dg, &ctx->dg_bytes},
+             {&ctx->bws, &ctx->bws_bytes}};
+  cudaStreamSynchronize(ctx->stream);
+  for (auto& b : all)
+    if (b.p != keep && *b.p) {
+      cudaFree(*b.p);
+      *b.p = nullptr;
+      *b.bytes = 0;
+    }
+}
+// cudaMalloc, with the side buffers' memory (but *keep's) when there is no other.
+cudaError_t device_alloc(mag_ctx* ctx, void** p, size_t bytes, void** keep = nullptr) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation || side_bytes(ctx) == 0) return e;
+  cudaGetLastError();
+  release_side(ctx, keep);
+  return cudaMalloc(p, bytes);
+}
+// Whether *p (a side buffer of `have` bytes) may grow to `need` beside the
+// workspace under options.workspace_limit_bytes; the others are given back for it.
+bool within_limit(mag_ctx* ctx, void** p, size_t have, size_t need) {
+  const double limit = ctx->opt.workspace_limit_bytes;
+  const size_t size = std::max(have, need);
+  if (limit <= 0 || (double)(ctx->ws_bytes + side_bytes(ctx) - have + size) <= limit) return true;
+  if ((double)(ctx->ws_bytes + size) > limit) return false;
+  release_side(ctx, p);
+  return true;
+}
+
 int ensure_workspace(mag_ctx* ctx, int64_t n, bool f32, bool f64, int64_t zf_tiles = -1) {
   Layout L = plan(ctx, n, f32, f64, ctx->dist_active && zf_tiles < 0, zf_tiles);
   if (ctx->opt.workspace_limit_bytes > 0 && (double)L.total > ctx->opt.workspace_limit_bytes)
@@ -304,7 +340,7 @@ int ensure_workspace(mag_ctx* ctx, int64_t n, bool f32, bool f64, int64_t zf_til
     ctx->fac_valid = false;   // and the factor
     ctx->chain_ready = ctx->lh_ready = false;
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, L.total);
+    cudaError_t e = device_alloc(ctx, &p, L.total);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return fail(ctx, MAG_ENOMEM, "cudaMalloc(%.3g GB) failed: %s", L.total / 1e9,
@@ -334,14 +370,22 @@ bool grow_buffer(mag_ctx* ctx, void** p, size_t* have, size_t need, size_t margi
     cudaGetLastError();
     return false;
   }
-  if ((double)fre + (double)*have < (double)need + (double)margin) return false;
+  if ((double)fre + (double)*have < (double)need + (double)margin) {
+    if ((double)fre + (double)*have + (double)side_bytes(ctx) < (double)need + (double)margin) return false;
+    release_side(ctx, p);
+    if (cudaMemGetInfo(&fre, &tot) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if ((double)fre + (double)*have < (double)need + (double)margin) return false;
+  }
   if (*p) {
     cudaStreamSynchronize(ctx->stream);
     cudaFree(*p);
     *p = nullptr;
     *have = 0;
   }
-  if (cudaMalloc(p, need) != cudaSuccess) {
+  if (device_alloc(ctx, p, need, p) != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
     return false;
@@ -359,7 +403,7 @@ int ensure_aux(mag_ctx* ctx, int64_t n) {
     ctx->aux = nullptr;
     ctx->aux_np = 0;
   }
-  cudaError_t e = cudaMalloc((void**)&ctx->aux, (size_t)A_COUNT * np * sizeof(double));
+  cudaError_t e = device_alloc(ctx, (void**)&ctx->aux, (size_t)A_COUNT * np * sizeof(double));
   if (e != cudaSuccess) {
     cudaGetLastError();
     ctx->aux = nullptr;
@@ -473,16 +517,15 @@ double update_flops(int64_t N, int64_t k0, int64_t k1, int64_t j0, int64_t j1) {
   return tiles * (double)(k1 - k0) * 2.0 * TILE * TILE * TILE;
 }
 
-// FP64 products by digits on the tensor cores while their scratch (230 KB a
+// FP64 products by digits on the tensor cores while their scratch (257 KB a
 // tile row) fits; else, and for FP32, on the CUDA cores.
 template <typename T>
 int factor_blocked(mag_ctx* ctx, T* Z, T* Dinv, int* launches, double* flops) {
   const Layout& L = ctx->lay;
   cudaStream_t s = ctx->stream;
   const size_t need = factor64_scratch_bytes(L.N);
-  const bool fits = ctx->opt.workspace_limit_bytes <= 0 ||
-                    (double)(ctx->ws_bytes + need) <= ctx->opt.workspace_limit_bytes;
-  const bool digits = sizeof(T) == 8 && fits && grow_buffer(ctx, &ctx->dg, &ctx->dg_bytes, need, 0);
+  const bool digits = sizeof(T) == 8 && within_limit(ctx, &ctx->dg, ctx->dg_bytes, need) &&
+                      grow_buffer(ctx, &ctx->dg, &ctx->dg_bytes, need, 0);
   if (digits) CU(launch_factor64_begin((const double*)Z, L.n, L.N, ctx->dg, s));
   for (int64_t K = 0; K < L.N; ++K) {
     CU(launch_potrf_diag<T>(Z, Dinv, K, L.n, ctx->st(), s));
@@ -853,7 +896,7 @@ int plan_out_of_core(mag_ctx* ctx, int64_t n, int prec, int64_t* pool_tiles) {
     cudaGetLastError();
     fre = 0;
   }
-  double avail = 0.95 * ((double)fre + (double)ctx->ws_bytes);
+  double avail = 0.95 * ((double)fre + (double)(ctx->ws_bytes + side_bytes(ctx)));
   if (o.workspace_limit_bytes > 0) avail = std::min(avail, o.workspace_limit_bytes);
   const Layout incore = plan(ctx, n, true, false);
   if (o.out_of_core == 0 && (double)incore.total <= avail) return MAG_OK;
@@ -1367,7 +1410,7 @@ void begin_dist_reuse(mag_ctx* ctx, int64_t n) {
     return;
   }
   const Layout with = plan(ctx, n, true, true, true);
-  ctx->dist_active = (double)with.total <= 0.8 * ((double)fre + (double)ctx->ws_bytes);
+  ctx->dist_active = (double)with.total <= 0.8 * ((double)fre + (double)(ctx->ws_bytes + side_bytes(ctx)));
 }
 void end_dist_reuse(mag_ctx* ctx) {
   ctx->dist_active = false;
@@ -1589,7 +1632,7 @@ int probe_fp16(mag_ctx* ctx, const double* X, int32_t m, double t, bool stored, 
       ctx->probe_z = nullptr;
       ctx->probe_bytes = 0;
     }
-    cudaError_t e = cudaMalloc((void**)&ctx->probe_z, bytes);
+    cudaError_t e = device_alloc(ctx, (void**)&ctx->probe_z, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
       ctx->probe_z = nullptr;
@@ -1691,7 +1734,7 @@ int gmres_ir(mag_ctx* ctx, int prec, const double* X, int32_t m, double t, const
       ctx->gm = nullptr;
       ctx->gm_bytes = 0;
     }
-    cudaError_t e = cudaMalloc((void**)&ctx->gm, need);
+    cudaError_t e = device_alloc(ctx, (void**)&ctx->gm, need);
     if (e != cudaSuccess) {
       cudaGetLastError();
       ctx->gm = nullptr;
@@ -2137,7 +2180,7 @@ int solve_impl(mag_ctx* ctx, const double* X, int64_t n, int32_t m, double t, co
     size_t fre = 0, tot = 0;
     const Layout with = plan(ctx, n, true, true);
     if (cudaMemGetInfo(&fre, &tot) == cudaSuccess) {
-      const double avail = (double)fre + (double)ctx->ws_bytes;
+      const double avail = (double)fre + (double)(ctx->ws_bytes + side_bytes(ctx));
       stored = (double)with.total <= 0.5 * avail;
     } else {
       cudaGetLastError();
@@ -2528,9 +2571,8 @@ int mag_residual(mag_ctx* ctx, const double* points, int64_t n, int32_t m, doubl
   const size_t need = residual_comp_bytes(n);
   int qe = 0;
   const void* Xq = nullptr;
-  const bool fits = ctx->opt.workspace_limit_bytes <= 0 ||
-                    (double)(ctx->ws_bytes + need) <= ctx->opt.workspace_limit_bytes;
-  if (fits && quantize_points(ctx, points, n, m, &qe, &Xq) && grow_buffer(ctx, &ctx->rp, &ctx->rp_bytes, need, 7 * need))
+  if (within_limit(ctx, &ctx->rp, ctx->rp_bytes, need) && quantize_points(ctx, points, n, m, &qe, &Xq) &&
+      grow_buffer(ctx, &ctx->rp, &ctx->rp_bytes, need, 7 * need))
     CU(launch_residual_comp(Xq, points, n, m, qe, t, w, b, r, ctx->rp, ctx->st(), s));
   else
     CU(launch_residual_mf(points, n, m, t, w, b, r, ctx->part(), L.chunks, n, ctx->st(), s));
@@ -2720,13 +2762,15 @@ int mag_grad(mag_ctx* ctx, const double* points, int64_t n, int32_t m, double t,
     CU(cudaMemcpyAsync(lam, wv, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
   }
   if (!ctx->ws) TRY(ensure_workspace(ctx, n, false, false));
-  // partial sums of the tiles, a band of row blocks at a time within 1 GB
+  // partial sums of the tiles, a band of row blocks at a time within 1 GB (one
+  // row block whatever the limits)
   const int64_t N = (n + TILE - 1) / TILE;
   const size_t band = grad_band_bytes(n, m), head = grad_head_bytes(n);
   int64_t bands = std::max<int64_t>(1, std::min<int64_t>(N, (int64_t)(((size_t)1 << 30) / band)));
   int qe = 0;
   const void* Xq = nullptr;
   if (!quantize_points(ctx, points, n, m, &qe, &Xq)) Xq = nullptr;
+  while (bands > 1 && !within_limit(ctx, &ctx->rp, ctx->rp_bytes, head + (size_t)bands * band)) bands = (bands + 1) / 2;
   if (!grow_buffer(ctx, &ctx->rp, &ctx->rp_bytes, head + (size_t)bands * band, 0)) {
     bands = 1;
     if (!grow_buffer(ctx, &ctx->rp, &ctx->rp_bytes, head + band, 0))
@@ -2899,9 +2943,12 @@ int batch_tiled(mag_ctx* ctx, const mag_batch_desc* desc, const std::vector<int>
   if (want > budget) {
     size_t fre = 0, tot = 0;
     CU(cudaMemGetInfo(&fre, &tot));
-    budget = std::max<size_t>(budget, std::min<size_t>(kBatchTiledBytes, (fre + budget) / 2));
-    if (ctx->opt.workspace_limit_bytes > 0)  // smaller groups; a problem alone may exceed it, as one CTA's scratch does
-      budget = (size_t)std::min<double>((double)budget, ctx->opt.workspace_limit_bytes);
+    budget = std::max<size_t>(budget, std::min<size_t>(kBatchTiledBytes, (fre + side_bytes(ctx)) / 2));
+    if (ctx->opt.workspace_limit_bytes > 0) {
+      // smaller groups; a problem alone may exceed the limit, as one CTA's scratch does
+      budget = (size_t)std::min((double)budget, std::max(0.0, ctx->opt.workspace_limit_bytes - (double)ctx->ws_bytes));
+      within_limit(ctx, &ctx->btws, ctx->btws_bytes, std::min(budget, want));
+    }
   }
   for (size_t i = 0; i < ids.size();) {
     size_t bytes = 0, k = i;
@@ -3032,7 +3079,7 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
         ctx->bws = nullptr;
         ctx->bws_bytes = 0;
       }
-      cudaError_t e = cudaMalloc(&ctx->bws, off);
+      cudaError_t e = device_alloc(ctx, &ctx->bws, off);
       if (e != cudaSuccess) {
         cudaGetLastError();
         ctx->bws = nullptr;

@@ -85,3 +85,49 @@ def test_kept_factor_and_a_larger_layout(between):
     c.close()
     assert info["factor_reused"] == 1
     assert _rel(X, 3.0, x, b) <= 2e-14
+
+
+# A batch leaves its workspace (1.8 GB) in the context: a solve for which the free
+# memory alone is too little takes it back and stays in core.
+def test_side_buffers_are_given_back_to_a_solve():
+    rng = np.random.default_rng(3)
+    c = M.Context()
+    clouds = [_dev(rng.standard_normal((2048, 8))) for _ in range(48)]
+    c.solve_batch(clouds, [1.0])
+    X = _dev(rng.random((8192, 8)))
+    need = c.workspace_bytes(8192, 8)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    assert need > 0.9e9
+    hog = torch.empty(int(torch.cuda.mem_get_info()[0] - 0.5e9), dtype=torch.uint8, device="cuda")
+    try:
+        w, mag, info = c.solve(X, 5.0)
+        _, dx = c.grad(X, 5.0, w=w)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    assert info["slabs"] == 0 and bool(torch.isfinite(dx).all())
+    assert _rel(X, 5.0, w, torch.ones_like(w)) <= 2e-14
+    _, mags, sts = c.solve_batch(clouds[:2], [1.0])  # and the batch takes its own again
+    c.close()
+    assert int(sts.abs().sum()) == 0
+
+
+# Partial sums and digits keep to the workspace limit together with the workspace,
+# with the same results as without one.
+def test_side_buffers_under_a_workspace_limit():
+    rng = np.random.default_rng(5)
+    X, w = _dev(rng.random((3000, 6))), _dev(rng.standard_normal(3000))
+    g = torch.full((3000,), 0.7, dtype=torch.float64, device="cuda")  # constant: no solve
+    clouds = [_dev(rng.standard_normal((n, 6))) for n in (1500, 700, 300, 1500)]
+    out = []
+    for limit in (0.0, 4e7):
+        c = M.Context(M.Options(workspace_limit_bytes=limit))
+        r, norms = c.residual(X, 2.0, w)
+        dt, dx = c.grad(X, 2.0, w=w, dL_dw=g)
+        ws, mags, sts = c.solve_batch(clouds, [0.5, 2.0])
+        assert int(sts.abs().sum()) == 0
+        out.append((r, dx, torch.tensor([dt, norms["r_norm_inf"], norms["z_norm_inf"]]), torch.cat(ws), mags))
+        c.close()
+    for a, b in zip(*out):
+        assert float((a - b).abs().max()) <= 1e-11 * float(a.abs().max())
