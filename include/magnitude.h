@@ -267,7 +267,10 @@ typedef struct mag_info {
                               at least one update launch was in flight; the
                               look-ahead streams overlap, so ms_update, a sum
                               of intervals, counts shared stretches twice    */
-  int32_t batch_threads;   /* mag_solve_batch: threads per CTA of the launch   */
+  int32_t batch_threads;   /* mag_solve_batch: threads per CTA of the launch of
+                              the one-CTA kernel; this and the next two and
+                              batch_left_looking are 0 when no problem of the
+                              call went through it                           */
   int32_t batch_ctas_per_sm; /* ... the CTAs per SM of its shape              */
   int32_t batch_tensor_cores; /* ... 1: the factor's trailing update on the
                               tensor cores (split TF32), 0: CUDA cores      */

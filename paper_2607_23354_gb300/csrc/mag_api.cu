@@ -96,7 +96,6 @@ struct mag_ctx {
   size_t bws_bytes = 0;
   int batch_tuned[12] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};  // launch shape per
                                      // size class ceil(log2 nmax) of the batch kernel (-1: not tuned)
-  int batch_shape_used = 0;
   UpdMaps maps[2];                   // TMA descriptors of the two panel buffers
   const void* maps_base[2] = {nullptr, nullptr};
   int maps_mode[2] = {-1, -1};
@@ -3019,6 +3018,7 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
     return probs[a].n != probs[b].n ? probs[a].n > probs[b].n : probs[a].cloud < probs[b].cloud;
   };
   std::vector<int> st_host(count, MAG_BATCH_OK);
+  int shape_used = -1;  // launch shape of the one-CTA kernel, if it runs
   if (!tiled.empty()) {
     std::stable_sort(tiled.begin(), tiled.end(), by_size);
     TRY(batch_tiled(ctx, desc, tiled, probs, points, w_out, mag_out, &st_host, &small));
@@ -3138,7 +3138,7 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
       }
       ctx->batch_tuned[cls] = shape;
     }
-    ctx->batch_shape_used = shape;
+    shape_used = shape;
     CU(cudaMemsetAsync(d_q, 0, sizeof(int), s));
     CU(cudaMemsetAsync(d_st, 0, (size_t)count * sizeof(int), s));
     CU(launch_batch_solve(shape, d_pr, d_or, (int)small.size(), d_D, d_cf, d_sf, d_sd, nmax, w_out,
@@ -3176,10 +3176,11 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
   if (info) {
     info->fallback = fallbacks;
     info->kernel_launches = g_kernel_launches.load() - l0;
-    info->batch_threads = kBatchShapes[ctx->batch_shape_used].threads;
-    info->batch_ctas_per_sm = kBatchShapes[ctx->batch_shape_used].ctas_per_sm;
-    info->batch_tensor_cores = kBatchShapes[ctx->batch_shape_used].tensor_cores;
-    info->batch_left_looking = kBatchShapes[ctx->batch_shape_used].left_looking;
+    if (shape_used >= 0) {  // else zeros
+      const BatchShape& b = kBatchShapes[shape_used];
+      info->batch_threads = b.threads, info->batch_ctas_per_sm = b.ctas_per_sm;
+      info->batch_tensor_cores = b.tensor_cores, info->batch_left_looking = b.left_looking;
+    }
   }
   return first;
 }

@@ -131,3 +131,18 @@ def test_side_buffers_under_a_workspace_limit():
         c.close()
     for a, b in zip(*out):
         assert float((a - b).abs().max()) <= 1e-11 * float(a.abs().max())
+
+
+# A batch reports the launch shape of its own one-CTA launch, or none.
+def test_batch_reports_its_own_launch():
+    rng = np.random.default_rng(8)
+    small, large = [_dev(rng.standard_normal((n, 5))) for n in (40, 300)]
+    keys = ("batch_threads", "batch_ctas_per_sm", "batch_tensor_cores", "batch_left_looking")
+    c = M.Context()
+    seen = []
+    for clouds in ([large], [small, large], [large]):
+        c.solve_batch(clouds, [1.0])
+        seen.append([c.last_batch_info[k] for k in keys])
+    c.close()
+    assert seen[0] == seen[2] == [0, 0, 0, 0]
+    assert seen[1][0] in (256, 512) and seen[1][1] >= 1
