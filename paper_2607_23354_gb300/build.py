@@ -41,7 +41,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     nvcc = _nvcc()
     sources = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
-    headers = sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + sorted(glob.glob(os.path.join(INCLUDE, "*.h")))
+    headers = [h for d, p in ((CSRC, "*.cuh"), (CSRC, "*.inc"), (INCLUDE, "*.h")) for h in sorted(glob.glob(os.path.join(d, p)))]
     objs = []
     jobs = []
     for src in sources:
