@@ -421,11 +421,13 @@ class Context:
         dx = torch.empty(n, m, dtype=torch.float64, device=self.device)
         dt = ctypes.c_double(0.0)
         info = mag_info()
-        wp = _P(0) if w is None else _P(w.to(torch.float64).contiguous().data_ptr())
+        # converted copies live until the call returns
+        if w is not None:
+            w = w.to(device=self.device, dtype=torch.float64).contiguous()
+        wp = _P(0) if w is None else _P(w.data_ptr())
         if dL_dw is not None:
             dL_dw = dL_dw.to(device=self.device, dtype=torch.float64).contiguous()
         gp = _P(0) if dL_dw is None else _P(dL_dw.data_ptr())
-        keep = (w, dL_dw)  # noqa: F841  (keep converted tensors alive during the call)
         self._check(self._lib.mag_grad(self._h, _P(X.data_ptr()), n, m, float(t), wp, gp, ctypes.byref(dt),
                                        _P(dx.data_ptr()), ctypes.byref(info)))
         return dt.value, dx

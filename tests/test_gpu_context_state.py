@@ -146,3 +146,16 @@ def test_batch_reports_its_own_launch():
     c.close()
     assert seen[0] == seen[2] == [0, 0, 0, 0]
     assert seen[1][0] in (256, 512) and seen[1][1] >= 1
+
+
+# FP32 w and dL/dw are converted for the call: the copy of the one must not take the
+# memory of the other's.
+def test_gradient_of_converted_vectors():
+    rng = np.random.default_rng(2)
+    X = _dev(rng.random((400, 5)))
+    w, g = _dev(rng.standard_normal(400)).float(), _dev(rng.standard_normal(400)).float()
+    c = M.Context()
+    dt, dx = c.grad(X, 1.5, w=w, dL_dw=g)
+    dt64, dx64 = c.grad(X, 1.5, w=w.double(), dL_dw=g.double())
+    c.close()
+    assert dt == dt64 and torch.equal(dx, dx64)
