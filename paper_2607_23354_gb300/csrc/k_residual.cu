@@ -931,11 +931,60 @@ __global__ void __launch_bounds__(1024) k_reduce_w(const double* __restrict__ w,
 // block, like the residual's), added by k_grad_finish; the order of every sum
 // is fixed.  A thread per row over all columns, with FP64 distances, a division
 // and twice the pairs, took 31 ms at n = 8192, m = 16 on 64 of the 152 SMs; 4.2
-// now.
+// now.  A ragged tile leaves out the rows and groups of 32 columns without points
+// (all of a tile for few points took 1.14 ms at m = 64 where the thread per row had
+// taken 84 us for 2 points and 664 for 50; now a call with 2, 32, 50 and 100
+// points 173, 403, 655 and 1001 us).
 constexpr int GRAD_THREADS = 512;
 constexpr int GRAD_LD = TILE + 2;
 constexpr int GRAD_MC = 16;  // dimensions staged per chunk
 constexpr size_t GRAD_STAGE = (2 * GRAD_MC + 2 * (GRAD_THREADS / 32)) * (size_t)TILE * sizeof(double);  // 64 KB
+
+// A dimension's row sums (rows GRAD_THREADS / 32 apart at x) and column sums
+// (columns 32 apart at y) of a thread's 8 x 4 coefficients: all of them (ALL), or
+// the first ni rows and nj columns, and the column sums only if asked for.
+template <bool ALL>
+__device__ __forceinline__ void grad_sums(const double (&g)[8][4], const double* x, const double* y, int ni, int nj,
+                                          bool cols, double (&rs)[8], double (&cs)[4]) {
+  double b[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    b[j] = y[32 * j];
+    cs[j] = 0.0;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    rs[i] = 0.0;
+    if (!ALL && i >= ni) continue;
+    const double a = x[GRAD_THREADS / 32 * i];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (!ALL && j >= nj) continue;
+      const double diff = a - b[j];
+      rs[i] = fma(g[i][j], diff, rs[i]);
+      if (ALL || cols) cs[j] = fma(g[i][j], diff, cs[j]);
+    }
+  }
+}
+
+// R row sums over 32 lanes: halve the rows with the lanes, then the remaining
+// levels; lane 32 / R k ends with row k, GRAD_THREADS / 32 apart in out.
+template <int R>
+__device__ __forceinline__ void reduce_rows(double (&rs)[8], double* __restrict__ out, int lane) {
+#pragma unroll
+  for (int h = R / 2, o = 16; h > 0; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < R / 2; ++i)
+      if (i < h) {
+        const double send = up ? rs[i] : rs[i + h], keep = up ? rs[i + h] : rs[i];
+        rs[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+  }
+#pragma unroll
+  for (int o = 16 / R; o > 0; o >>= 1) rs[0] += __shfl_xor_sync(0xffffffffu, rs[0], o);
+  if ((lane & (32 / R - 1)) == 0) out[GRAD_THREADS / 32 * (lane / (32 / R))] = rs[0];
+}
 
 template <bool FX, int KIND>
 __global__ void __launch_bounds__(GRAD_THREADS, 1)
@@ -963,8 +1012,8 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1)
   }
   double wc[4], lc[4];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const int64_t gc = col0 + 4 * lane + c;
+  for (int c = 0; c < 4; ++c) {  // this lane's columns in the loops below
+    const int64_t gc = col0 + (FX ? 4 * lane + c : lane + 32 * c);
     wc[c] = gc < n ? w[gc] : 0.0;
     lc[c] = gc < n ? lam[gc] : 0.0;
   }
@@ -1024,11 +1073,11 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1)
       double tsum = 0.0;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const int64_t gc = col0 + 4 * lane + c;
+        const int64_t gc = col0 + lane + 32 * c;
         double g = 0.0;
         if (gr < n && gc < n && gr != gc)
           g = by_differences(gr, gc, fma(s_l[r], wc[c], lc[c] * s_w[r]), &tsum);
-        G[r * GRAD_LD + 4 * lane + c] = g;
+        G[r * GRAD_LD + lane + 32 * c] = g;
       }
       add_comp(ts, te, tsum);
     }
@@ -1058,6 +1107,11 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1)
   for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) g[i][j] = G[(warp + NW * i) * GRAD_LD + lane + 32 * j];
+  // rows and column groups with points: a ragged tile's others hold zeros
+  const bool whole = row0 + TILE <= n && col0 + TILE <= n;
+  const int64_t left = n - row0 - warp, right = n - col0;
+  const int ni = left <= 0 ? 0 : (left > TILE - NW ? 8 : (int)((left + NW - 1) / NW));
+  const int nj = right >= TILE ? 4 : (int)((right + 31) / 32);
   double* prow = P + ((I - I0) * 2 * N + J) * m * TILE;          // this tile's row sums
   double* pcol = P + ((I - I0) * 2 * N + N + J) * m * TILE;      // and column sums
   for (int l0 = 0; l0 < m; l0 += GRAD_MC) {
@@ -1069,39 +1123,17 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1)
       xc[l * TILE + r] = col0 + r < n ? X[(col0 + r) * m + l0 + l] : 0.0;
     }
     __syncthreads();
+    if (I == J && ni == 0) continue;  // no rows: nothing reads this warp's sums
     for (int l = 0; l < mc; ++l) {
-      double rs[8], cs[4], b[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        b[j] = xc[l * TILE + lane + 32 * j];
-        cs[j] = 0.0;
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const double a = xr[l * TILE + warp + NW * i];
-        rs[i] = 0.0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const double diff = a - b[j];
-          rs[i] = fma(g[i][j], diff, rs[i]);
-          cs[j] = fma(g[i][j], diff, cs[j]);
-        }
-      }
-      // eight row sums over 32 lanes: halve the rows with the lanes, then the
-      // last two levels; lane 4 k ends with row k' = its three top bits
-#pragma unroll
-      for (int h = 4, o = 16; h > 0; h >>= 1, o >>= 1) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (i < h) {
-            const double send = up ? rs[i] : rs[i + h], keep = up ? rs[i + h] : rs[i];
-            rs[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-          }
-      }
-      rs[0] += __shfl_xor_sync(0xffffffffu, rs[0], 2);
-      rs[0] += __shfl_xor_sync(0xffffffffu, rs[0], 1);
-      if ((lane & 3) == 0) prow[(l0 + l) * TILE + warp + NW * (lane >> 2)] = rs[0];
+      double rs[8], cs[4];
+      if (whole)
+        grad_sums<true>(g, xr + l * TILE + warp, xc + l * TILE + lane, 8, 4, true, rs, cs);
+      else
+        grad_sums<false>(g, xr + l * TILE + warp, xc + l * TILE + lane, ni, nj, I != J, rs, cs);
+      if (!whole && ni <= 4)
+        reduce_rows<4>(rs, prow + (l0 + l) * TILE + warp, lane);
+      else
+        reduce_rows<8>(rs, prow + (l0 + l) * TILE + warp, lane);
       if (I != J) {
         double* cp = colp + (l & 1) * NW * TILE;
 #pragma unroll

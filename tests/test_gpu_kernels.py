@@ -378,3 +378,23 @@ def test_residual_norms_are_the_same_every_time(ctx):
     Z = ctx.similarity_matrix(_dev(X), 0.8).cpu().numpy().astype(np.longdouble)
     z = Z.sum(1).max()
     assert abs(norms[0]["z_norm_inf"] - z) <= 3 * 2.0 ** -53 * z
+
+
+# Gradients of few points: FP64 differences up to 32, tiles whose last rows and
+# columns are empty (one to four groups of each), the second tile of a pair ragged.
+# Bound as for test_gradient_sums.
+@pytest.mark.parametrize("n", [2, 15, 16, 17, 31, 32, 33, 64, 65, 100, 135, 200])
+@pytest.mark.parametrize("m", [3, 17, 64])
+def test_gradient_of_few_points(ctx, n, m):
+    rng = np.random.default_rng(n + 1000 * m)
+    X, w = rng.standard_normal((n, m)), rng.standard_normal(n)
+    t, c = 1.5 / np.sqrt(m), 0.75
+    dt, dx = ctx.grad(_dev(X), t, w=_dev(w), dL_dw=_dev(np.full(n, c)))
+    D = X[:, None, :] - X[None, :, :]
+    d = np.sqrt((D.astype(np.longdouble) ** 2).sum(-1)).astype(np.float64)
+    Z, s = np.exp(-t * d), 2.0 * c * np.outer(w, w)
+    e = 2.0 ** -53 * ((m / 2 + 12) * (1 + t * d) + n)
+    assert abs(dt - (0.5 * d * Z * s).sum()) <= (0.5 * e * d * Z * abs(s)).sum()
+    np.fill_diagonal(d, 1.0)
+    G = t * Z * s / d
+    assert np.all(np.abs(dx.cpu().numpy() - (G[:, :, None] * D).sum(1)) <= ((e * abs(G))[:, :, None] * abs(D)).sum(1))
