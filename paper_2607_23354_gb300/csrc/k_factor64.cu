@@ -18,8 +18,9 @@
 // entries (rms, 128 normal entries), against 2^-53 of every partial sum in FP64
 // arithmetic.  (Seven digits of 55 bits: backward errors 10 to 40% above the FP64
 // products'.)  That is a bound by rows, not by entries: an entry whose terms are
-// far below its rows' largest has its sum taken in FP64 (k_oz_gemm), so that
-// |Z - L L^T| stays a few units of |L| |L^T| entry by entry.  n = 300, six clouds
+// far below its rows' largest has its sum taken in FP64 where L is the result
+// (entries; a solve refines its weighting, for which the bound by rows is
+// enough), so that |Z - L L^T| stays a few units of |L| |L^T| entry by entry.  n = 300, six clouds
 // in R^6 to R^20, t = 1 to 6: at most 2.3e-15 of |L| |L^T|, FP64 products 8.0e-15
 // (by digits alone 0.03 at worst).
 //
@@ -433,7 +434,7 @@ __global__ void __launch_bounds__(256) k_least_exponent(const double* __restrict
 // the half tile's least Z_ij nor |C_ij| (in the panel |a_ij inv_jj|) reaches
 // 2^-8 max_a max_b, an entry's sum is taken in FP64, a warp each.  The test runs
 // beside the products.  The panel's halves read all of a row of A there, so the
-// two CTAs of a tile are a cluster and write once both have read.
+// two CTAs of a tile are then a cluster and write once both have read.
 constexpr int OZ_THREADS = 256;
 constexpr uint32_t OZ_TMEM = 512;
 constexpr int OZ_SMEM = NDIG * (128 * 128 + 64 * 128);
@@ -459,7 +460,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
 
 __device__ __forceinline__ int exponent_of(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) - 1023; }
 
-// least: k_least_exponent's; inv: inv(L_KK) (ASSIGN)
+// least: k_least_exponent's (null: every entry by digits); inv: inv(L_KK) (ASSIGN)
 template <bool ASSIGN>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_gemm(double* __restrict__ Z, int64_t N, int64_t K, const unsigned char* __restrict__ digits,
@@ -476,7 +477,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   if (tid == 0) skip = (*(volatile int*)&st->flags & (ST_NOTPD | ST_NONFINITE | ST_DUPLICATE | ST_TIMEOUT)) != 0;
   __syncthreads();
   if (skip) {  // uniform across the CTA
-    if (ASSIGN) cluster_sync_all();  // the other half's CTA may have gone on
+    if (ASSIGN && least) cluster_sync_all();  // the other half's CTA may have gone on
     return;
   }
   const int h = blockIdx.x & 1;
@@ -552,7 +553,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         }
       mma_commit(&done_bar[c]);
     }
-  } else if (warp > 0) {
+  } else if (warp > 0 && least) {
     const int b0 = wb[2 * lane], b1 = wb[2 * lane + 1], bmax = __reduce_max_sync(0xffffffffu, max(b0, b1));
     const int zmin = least[2 * tile + h] + OZ_MARGIN;
     for (int r = warp - 1; r < TILE; r += OZ_THREADS / 32 - 1) {
@@ -659,7 +660,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       __syncwarp();  // the row's entries are read below by this warp
     }
   }
-  if (ASSIGN) cluster_sync_all();
+  if (ASSIGN && least) cluster_sync_all();
   if (fine) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -708,8 +709,8 @@ cudaError_t launch_potrf_f64(double* Z, double* Dinv, double* DinvT, int64_t K, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_factor64_panel(double* Z, const double* Dinv, int64_t K, int64_t N, void* scratch, DevStatus* st,
-                                  cudaStream_t s) {
+cudaError_t launch_factor64_panel(double* Z, const double* Dinv, int64_t K, int64_t N, void* scratch, bool entries,
+                                  DevStatus* st, cudaStream_t s) {
   unsigned char* dg = static_cast<unsigned char*>(scratch);
   cudaError_t e;
   const int64_t below = N - K - 1;
@@ -724,9 +725,9 @@ cudaError_t launch_factor64_panel(double* Z, const double* Dinv, int64_t K, int6
   cudaLaunchAttribute pair[1];
   pair[0].id = cudaLaunchAttributeClusterDimension;
   pair[0].val.clusterDim.x = 2, pair[0].val.clusterDim.y = 1, pair[0].val.clusterDim.z = 1;
-  c.attrs = pair, c.numAttrs = 1;
-  e = cudaLaunchKernelEx(&c, k_oz_gemm<true>, Z, N, K, (const unsigned char*)dg, (const int*)least_of(scratch, N),
-                         Dinv + K * TILE_ELEMS, st, kOzTimeout);
+  c.attrs = pair, c.numAttrs = entries ? 1 : 0;
+  e = cudaLaunchKernelEx(&c, k_oz_gemm<true>, Z, N, K, (const unsigned char*)dg,
+                         entries ? (const int*)least_of(scratch, N) : nullptr, Dinv + K * TILE_ELEMS, st, kOzTimeout);
   if (e != cudaSuccess) return e;
   note_launch();
   k_digits<<<(unsigned)below, 256, 0, s>>>(nullptr, Z, K, dg, st);
@@ -734,7 +735,8 @@ cudaError_t launch_factor64_panel(double* Z, const double* Dinv, int64_t K, int6
   return cudaGetLastError();
 }
 
-cudaError_t launch_factor64_update(double* Z, int64_t K, int64_t N, void* scratch, DevStatus* st, cudaStream_t s) {
+cudaError_t launch_factor64_update(double* Z, int64_t K, int64_t N, void* scratch, bool entries, DevStatus* st,
+                                   cudaStream_t s) {
   const int64_t below = N - K - 1, tiles = num_lower_tiles(below);
   if (below <= 0) return cudaSuccess;
   if (2 * tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
@@ -742,7 +744,8 @@ cudaError_t launch_factor64_update(double* Z, int64_t K, int64_t N, void* scratc
   cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   k_oz_gemm<false><<<(unsigned)(2 * tiles), OZ_THREADS, smem, s>>>(Z, N, K, static_cast<const unsigned char*>(scratch),
-                                                                  least_of(scratch, N), nullptr, st, kOzTimeout);
+                                                                  entries ? least_of(scratch, N) : nullptr, nullptr, st,
+                                                                  kOzTimeout);
   note_launch();
   return cudaGetLastError();
 }

@@ -518,25 +518,26 @@ double update_flops(int64_t N, int64_t k0, int64_t k1, int64_t j0, int64_t j1) {
 }
 
 // FP64 products by digits on the tensor cores while their scratch (257 KB a
-// tile row) fits; else, and for FP32, on the CUDA cores.
+// tile row) fits; else, and for FP32, on the CUDA cores.  entries: see
+// launch_factor64_panel.
 template <typename T>
-int factor_blocked(mag_ctx* ctx, T* Z, T* Dinv, int* launches, double* flops) {
+int factor_blocked(mag_ctx* ctx, T* Z, T* Dinv, bool entries, int* launches, double* flops) {
   const Layout& L = ctx->lay;
   cudaStream_t s = ctx->stream;
   const size_t need = factor64_scratch_bytes(L.N);
   const bool digits = sizeof(T) == 8 && within_limit(ctx, &ctx->dg, ctx->dg_bytes, need) &&
                       grow_buffer(ctx, &ctx->dg, &ctx->dg_bytes, need, 0);
-  if (digits) CU(launch_factor64_begin((const double*)Z, L.n, L.N, ctx->dg, s));
+  if (digits && entries) CU(launch_factor64_begin((const double*)Z, L.n, L.N, ctx->dg, s));
   for (int64_t K = 0; K < L.N; ++K) {
     CU(launch_potrf_diag<T>(Z, Dinv, K, L.n, ctx->st(), s));
     if (digits)
-      CU(launch_factor64_panel((double*)Z, (const double*)Dinv, K, L.N, ctx->dg, ctx->st(), s));
+      CU(launch_factor64_panel((double*)Z, (const double*)Dinv, K, L.N, ctx->dg, entries, ctx->st(), s));
     else
       CU(launch_trsm_col<T>(Z, Dinv, K, L.N, ctx->st(), s));
     if (K + 1 < L.N) {
       TRY(prof_begin(ctx));
       if (digits)
-        CU(launch_factor64_update((double*)Z, K, L.N, ctx->dg, ctx->st(), s));
+        CU(launch_factor64_update((double*)Z, K, L.N, ctx->dg, entries, ctx->st(), s));
       else
         CU(launch_syrk_simt<T>(Z, L.N, K, K + 1, K + 1, L.N, ctx->st(), s));
       TRY(prof_end(ctx));
@@ -1417,7 +1418,8 @@ void end_dist_reuse(mag_ctx* ctx) {
   ctx->dist_valid = false;
 }
 
-int run_factor(mag_ctx* ctx, int prec, SolveResult* R) {
+// entries: the factor itself is the result (factor_blocked)
+int run_factor(mag_ctx* ctx, int prec, SolveResult* R, bool entries = false) {
   cudaStream_t s = ctx->stream;
   const Layout& L = ctx->lay;
   ctx->chain_ready = ctx->lh_ready = false;
@@ -1431,9 +1433,9 @@ int run_factor(mag_ctx* ctx, int prec, SolveResult* R) {
   CU(cudaEventRecord(ctx->ev[0], s));
   ctx->prof_used = 0;
   if (prec == MAG_PREC_FP64)
-    TRY(factor_blocked<double>(ctx, ctx->zd(), ctx->dinvd(), &R->update_launches, &R->update_flops));
+    TRY(factor_blocked<double>(ctx, ctx->zd(), ctx->dinvd(), entries, &R->update_launches, &R->update_flops));
   else if (prec == MAG_PREC_FP32)
-    TRY(factor_blocked<float>(ctx, ctx->zf(), ctx->dinvf(), &R->update_launches, &R->update_flops));
+    TRY(factor_blocked<float>(ctx, ctx->zf(), ctx->dinvf(), entries, &R->update_launches, &R->update_flops));
   else
     TRY(factor_tc(ctx, upd_mode(prec), &R->update_launches, &R->update_flops, lh));
   if (chain) CU(launch_chain_prep(ctx->zf(), ctx->dinvf(), L.N, ctx->chain_s, ctx->chain_s + L.N * TILE_ELEMS, s));
@@ -2394,7 +2396,7 @@ int mag_cholesky_factor(mag_ctx* ctx, const double* points, int64_t n, int32_t m
   ctx->fac_valid = false;
   TRY(ensure_workspace(ctx, n, !f64, f64));
   TRY(generate(ctx, points, m, t, !f64, f64, &R));
-  TRY(run_factor(ctx, prec, &R));
+  TRY(run_factor(ctx, prec, &R, true));
   const Layout& L = ctx->lay;
   if (f64)
     CU(launch_unpack<double>(ctx->zd(), n, L.N, false, (double*)L_out, ctx->stream));

@@ -200,14 +200,16 @@ cudaError_t launch_potrf_f32(float* Z, float* Dinv, float* DinvT, int64_t K, Dev
 // The FP64 one (k_factor64.cu), and the rest of a tile column of the FP64
 // factor with its products on the FP16 tensor cores: the panel solve (and the
 // digits of the solved panel, left in scratch) and the trailing update from
-// them.  launch_factor64_begin first, on the n x n matrix itself.  scratch:
+// them.  entries: every entry of L as accurate as by FP64 products, not only the
+// rows; launch_factor64_begin first then, on the n x n matrix itself.  scratch:
 // factor64_scratch_bytes(N).
 cudaError_t launch_potrf_f64(double* Z, double* Dinv, double* DinvT, int64_t K, DevStatus* st, cudaStream_t s);
 size_t factor64_scratch_bytes(int64_t N);
 cudaError_t launch_factor64_begin(const double* Z, int64_t n, int64_t N, void* scratch, cudaStream_t s);
-cudaError_t launch_factor64_panel(double* Z, const double* Dinv, int64_t K, int64_t N, void* scratch, DevStatus* st,
-                                  cudaStream_t s);
-cudaError_t launch_factor64_update(double* Z, int64_t K, int64_t N, void* scratch, DevStatus* st, cudaStream_t s);
+cudaError_t launch_factor64_panel(double* Z, const double* Dinv, int64_t K, int64_t N, void* scratch, bool entries,
+                                  DevStatus* st, cudaStream_t s);
+cudaError_t launch_factor64_update(double* Z, int64_t K, int64_t N, void* scratch, bool entries, DevStatus* st,
+                                   cudaStream_t s);
 // Panel solve: tiles (I, K) for I in [K+1, N): A_IK <- A_IK inv(L_KK)^T.
 template <typename T>
 cudaError_t launch_trsm_col(T* Z, const T* Dinv, int64_t K, int64_t N, DevStatus* st,
