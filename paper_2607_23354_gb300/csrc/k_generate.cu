@@ -1,5 +1,12 @@
 // K1: fused distance + exp generator of Z = exp[-t d] (Sec. 2), packed lower tiles.
 //
+// k_generate_q, k_dist_q + k_generate_from_dist and k_dense_q form the pairs in
+// 64-bit fixed point from the quantized coordinates (mag_fx.cuh), without an FP64
+// operation but for pairs too close for those.  k_generate, below, serves the
+// points that admit no quantization (m > 512, a non-finite coordinate, every
+// dimension constant, a scale beyond 2^+-400, exact_distances = 0, no memory for
+// the copy):
+//
 // One CTA per lower tile (I, J).  Coordinates of the tile's 128 row points and
 // 128 column points are staged in shared memory in chunks of MC coordinates;
 // every pair difference x_jl - x_kl is taken in FP64 and squared/accumulated
@@ -7,7 +14,7 @@
 // not cancel).  The FP32 tile (factor input) takes sqrt/exp in FP32 from the
 // FP64 d^2; the FP64 tile (FP64 factor or stored residual) takes them in FP64.
 //
-// Thread layout (512 threads): warp w handles tile rows w + 16 i (i < 8),
+// Thread layout of k_generate (512 threads): warp w handles tile rows w + 16 i (i < 8),
 // lane l handles tile columns 4 l + q (q < 4), so each thread stores its four
 // entries of a row with one 16-byte store (FP32: a float4; FP64: two
 // double2) and a warp's stores cover one whole tile row.  The column points
@@ -450,13 +457,9 @@ __global__ void __launch_bounds__(FX_THREADS, fx_ctas(KIND))
       } else {
         fx_u64 s = 0, db = 0;
         int j = 0;
-        bool done = false;
         if (fx_close(q[c], m)) {
           db = (fx_u64)__double_as_longlong(sqrt_pos(close_square(X, gr, gc, m, &flags, &mind2b)));
-          if (EXP) {
-            zd = __longlong_as_double((long long)fx_exp_neg_d(db, sc.kg, sc.g, fxtab));
-            done = true;
-          }
+          if (EXP) zd = __longlong_as_double((long long)fx_exp_neg_d(db, sc.kg, sc.g, fxtab));
         } else {
           if (q[c].h < mq.h || (q[c].h == mq.h && q[c].l < mq.l)) mq = q[c];
           const FxRoot rt = fx_root_start(q[c]);
@@ -465,7 +468,6 @@ __global__ void __launch_bounds__(FX_THREADS, fx_ctas(KIND))
           if (EXP && td > tiny) {
             zf = exp_neg_tiny_f(td);
             zd = f32_to_f64_nonneg(zf);
-            done = true;
           } else {
             s = fx_root(rt);
             j = rt.j;
@@ -475,7 +477,6 @@ __global__ void __launch_bounds__(FX_THREADS, fx_ctas(KIND))
               db = fx_dist_bits(s, j, sc.e);
           }
         }
-        (void)done;
         if (!EXP) zd = mat_entry(kind, t, kc, __longlong_as_double((long long)db), exptab);
         if (WF || !WD) zf = !EXP && kind == MAT_DEFLATED ? __double2float_rn(zd) : f64_to_f32_nonneg(zd);
       }

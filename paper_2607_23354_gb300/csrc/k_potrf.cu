@@ -34,7 +34,7 @@
 // trailing updates 5,500.  One lane scaling and publishing a column at a time,
 // with warp-serial block inverses and register-tiled FP32 block products, took
 // 107,000.  57 us a launch before, 22 now (event to event, alone); a solve of
-// n = 16384 points in R^3 22.8 ms before, 17.2 now.  Backward error of a tile's
+// n = 16384 points in R^3 22.8 ms before, 17.2 with it alone.  Backward error of a tile's
 // factor: 1.1e-7 of ||Z|| before, 0.7e-7 now (Z of [0,1]^8, t = 1).
 #include <cuda_bf16.h>
 

@@ -1,14 +1,19 @@
 // K4: FP64 residual r = b - Z w of iterative refinement, with Z regenerated
-// on the fly from the points (matrix free: nothing of size n^2 is read), and
-// the norms the stopping test needs: ||r||inf, ||Z||inf (max row sum, Z > 0),
-// ||w||inf.  K5: the FP64 solution update.  K6: Mag = 1^T w (compensated),
-// min_j w_j and the sign information.  K7: the fused gradient reductions.
+// on the fly from the points (matrix free: nothing of size n^2 is read) or read
+// from the stored FP64 tiles, and the norms the stopping test needs: ||r||inf,
+// ||Z||inf (max row sum, Z > 0), ||w||inf.  K5: the FP64 solution update.  K6: Mag
+// = 1^T w (compensated), min_j w_j and the sign information.  K7: the fused
+// gradient reductions.
 //
-// Accuracy: every pair is d^2 = sum_l (x_jl - x_kl)^2 in FP64, Z_jk =
-// exp(-t sqrt(d^2)) in FP64, and each row sum is accumulated with Kahan
-// compensation per thread and then combined across column chunks with
-// Neumaier's rule, so the residual is good to a few units of FP64 rounding
-// relative to ||Z||inf ||w||inf (the refinement target is 1e-14).
+// Matrix free, every pair of the lower triangle once: k_resid_sym_q, entries in
+// fixed point from the quantized coordinates (mag_fx.cuh; with compensated sums
+// for the residual entry point), k_resid_sym from FP64 differences where the
+// points admit none or Z is not exp(-t d).  k_resid_mf visits every entry of the
+// square (no scratch of size n^2 / 128: mag_residual_noalloc, and mag_residual
+// where its partial sums do not fit): d^2 and exp in FP64, each row sum with Kahan
+// compensation per thread and Neumaier's rule across column chunks.  All are good
+// to a few units of FP64 rounding relative to ||Z||inf ||w||inf (the refinement
+// target is 1e-14).
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -470,8 +475,11 @@ __global__ void __launch_bounds__(SYM_THREADS, 1)
 // with the errors carried along, P as (sum, error) pairs, the row sums of Z
 // exact in 128-bit fixed point up to 2^-64 an entry and added up as integers, so
 // that the norms do not depend on the order of the tiles either -- which costs
-// five FP64 operations a pair instead of two and still stays below the integer
-// work's time.  The solver's own residual (COMP false) takes FMA chains and FP32 norms.
+// six FP64 operations a pair (two FMAs, 1.75 for the columns' groups, 1.7 for a
+// row's lanes, 0.5 for the columns' warps).  No pipe is full (FP64 60%, ALU 35%,
+// FMA 26% at n = 16,384, m = 8): two CTAs of 128 registers do not hide the
+// latencies.  n = 30,000, m = 8: 54 ms with FP64 differences for the whole square,
+// 8.3 now.  The solver's own residual (COMP false) takes FMA chains and FP32 norms.
 constexpr int SYMQ_LD = 33;
 
 // s + c <- s + c + x with the rounding of s collected in c

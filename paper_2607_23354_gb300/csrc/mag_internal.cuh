@@ -142,8 +142,8 @@ cudaError_t launch_generate_dist(const double* X, int64_t n, int m, double t, in
 // launch_range_ordered (k_mindist.cu): per dimension min and max of X in the
 // order-preserving encoding of ordered_value, range[2l], range[2l+1], and
 // range[2m] = 1 if a coordinate is not finite (2m + 1 words).
-// launch_quantize: Xq[i m + l] = round(2^e (X[i m + l] - min_l)) as two 30-bit
-// limbs (8 bytes a coordinate).
+// launch_quantize: Xq[i m + l] = round(2^e (X[i m + l] - min_l)) as two limbs
+// (fx_limb_of: 31 + 30 bits for m <= 4, else 30 + 29; 8 bytes a coordinate).
 // launch_dist_q: FP64 distances Dd of the packed lower tiles (m <= 512) from Xq
 // (pairs closer than sqrt(m) 2^(53-e) from the FP64 differences of X), min
 // d^2 and ST_DUPLICATE into st as the generator.

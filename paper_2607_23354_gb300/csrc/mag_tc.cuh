@@ -111,10 +111,13 @@ __device__ __forceinline__ void cluster_sync_all() {
 }
 
 // A 128-row x 128-column FP16 operand in the layout the K-major SWIZZLE_128B
-// descriptors read: chunks of 64 columns (16 KB each), row r at byte 128 r of
+// descriptors read: two chunks of 64 columns (16 KB each), row r at byte 128 r of
 // its chunk, 16-byte unit u (columns 8u .. 8u + 7 of the chunk) at unit
-// u ^ (r & 7).
+// u ^ (r & 7).  Within a chunk, then by the unit of the whole row (0 .. 15).
 __device__ __forceinline__ uint32_t swizzled_unit(int r, int u) { return (uint32_t)(r * 128 + ((u ^ (r & 7)) << 4)); }
+__device__ __forceinline__ uint32_t operand_unit(int r, int u16) {
+  return (uint32_t)((u16 >> 3) * 16384) + swizzled_unit(r, u16 & 7);
+}
 
 // Untiled bulk copy to shared memory (16-byte aligned addresses, a multiple of
 // 16 bytes), completing on `bar`.
@@ -126,15 +129,6 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 }
 
 // ------------------------------------------- FP32 tiles as FP16 operands
-// A 128-row x 128-column FP16 operand in the layout the K-major SWIZZLE_128B
-// descriptors read: two chunks of 64 columns (16 KB each), row r at byte
-// 128 r of its chunk, 16-byte unit u (columns 8u .. 8u + 7 of the chunk) at
-// unit u ^ (r & 7).
-__device__ __forceinline__ uint32_t trsm_unit_offset(int r, int u16) {
-  const int chunk = u16 >> 3, u = u16 & 7;
-  return (uint32_t)(chunk * 16384 + r * 128 + ((u ^ (r & 7)) << 4));
-}
-
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
 
 // Power-of-two exponent e with max |x| * 2^e in [2^13, 2^14): 0 for a row of
@@ -181,7 +175,7 @@ __device__ __forceinline__ void trsm_split(const float4 (&x)[16], unsigned char*
       h[q] = __float2half_rn(v[q]);
       l[q] = __float2half_rn(v[q] - __half2float(h[q]));
     }
-    const uint32_t off = trsm_unit_offset(r, lane & 15);
+    const uint32_t off = operand_unit(r, lane & 15);
     *reinterpret_cast<uint4*>(hi + off) = *reinterpret_cast<const uint4*>(h);
     *reinterpret_cast<uint4*>(lo + off) = *reinterpret_cast<const uint4*>(l);
     if ((lane & 15) == 0) rexp[r] = e;
