@@ -63,18 +63,11 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// 1 / sqrt(p) from r near it by one Newton step; r (1 + s) leaves 1.5 s^2.
-__device__ __forceinline__ float rsqrt_newton(float p, float r) {
-  const float e = fmaf(-0.5f * p * r, r, 0.5f);
-  return fmaf(r, e, r);
-}
-// The same for an r taken from a quantity that rounds apart from p: where the
-// pivot has cancelled so far that they differ by 2^-11 or more (or in sign), r
-// starts again from p itself.  p is the same in every lane.
-__device__ __forceinline__ float rsqrt_pivot(float p, float r) {
-  const float e = fmaf(-0.5f * p * r, r, 0.5f);
-  if (fabsf(e) < 0x1p-12f) return fmaf(r, e, r);
-  return rsqrt_newton(p, rsqrt_ftz(p));
+// r ~ 1 / sqrt(p) improved by one Newton step; e (half the seed's relative
+// error in p r^2) returned for the test of the seed
+__device__ __forceinline__ float rsqrt_newton(float p, float r, float* e) {
+  *e = fmaf(-0.5f * p * r, r, 0.5f);
+  return fmaf(r, *e, r);
 }
 __device__ __forceinline__ void bar_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
@@ -90,34 +83,45 @@ struct Pivot {
   int bad;  // bit i: pivot i is not positive
 };
 
-// A pivot that is not positive, or below FP32's normal range, is reported;
-// the entries after it are then meaningless (NaN or infinite) and the factor
-// is dropped.
-__device__ __forceinline__ void pivot_factor(float d00, float d10, float d20, float d30, float d11, float d21,
-                                             float d31, float d22, float d32, float d33, Pivot& q) {
-  constexpr float kMinPivot = 1.17549435e-38f;
-  // a pair's second pivot p1 = d11 - d10^2 / d00 is approximated as
-  // 1 / sqrt = sqrt(d00) / sqrt(d00 d11 - d10^2), so that both roots start
-  // together; the Newton step takes it to the pivot itself, the entry that is
-  // scaled, and that one is judged
-  const float e1 = fmaf(d00, d11, -d10 * d10);
-  const float s0 = rsqrt_ftz(d00), s1 = rsqrt_ftz(e1);
-  q.r0 = rsqrt_newton(d00, s0);
+// The factor with the second pivots' roots from the seeds s1, s3 (PAIRED: of the
+// pairs' determinants) or from the pivots themselves.  True where both seeds are
+// within 2^-11 of the pivots'.
+template <bool PAIRED>
+__device__ __forceinline__ bool pivot_steps(float d00, float d10, float d20, float d30, float d11, float d21, float d31,
+                                            float d22, float d32, float d33, Pivot& q) {
+  constexpr float kMinPivot = 1.17549435e-38f, kSeed = 0x1p-12f;
+  float e0, e1, e2, e3;
+  const float s0 = rsqrt_ftz(d00), s1 = PAIRED ? rsqrt_ftz(fmaf(d00, d11, -d10 * d10)) : 0.0f;
+  q.r0 = rsqrt_newton(d00, s0, &e0);
   q.l10 = d10 * q.r0, q.l20 = d20 * q.r0, q.l30 = d30 * q.r0;
   const float p1 = fmaf(-q.l10, q.l10, d11);
-  q.r1 = rsqrt_pivot(p1, (d00 * s0) * s1);
+  q.r1 = rsqrt_newton(p1, PAIRED ? (d00 * s0) * s1 : rsqrt_ftz(p1), &e1);
   q.l21 = fmaf(-q.l20, q.l10, d21) * q.r1, q.l31 = fmaf(-q.l30, q.l10, d31) * q.r1;
   const float p2 = fmaf(-q.l21, q.l21, fmaf(-q.l20, q.l20, d22));
   const float s32 = fmaf(-q.l31, q.l21, fmaf(-q.l30, q.l20, d32));
   const float s33 = fmaf(-q.l31, q.l31, fmaf(-q.l30, q.l30, d33));
-  const float e3 = fmaf(p2, s33, -s32 * s32);
-  const float s2 = rsqrt_ftz(p2), s3 = rsqrt_ftz(e3);
-  q.r2 = rsqrt_newton(p2, s2);
+  const float s2 = rsqrt_ftz(p2), s3 = PAIRED ? rsqrt_ftz(fmaf(p2, s33, -s32 * s32)) : 0.0f;
+  q.r2 = rsqrt_newton(p2, s2, &e2);
   q.l32 = s32 * q.r2;
   const float p3 = fmaf(-q.l32, q.l32, s33);
-  q.r3 = rsqrt_pivot(p3, (p2 * s2) * s3);
+  q.r3 = rsqrt_newton(p3, PAIRED ? (p2 * s2) * s3 : rsqrt_ftz(p3), &e3);
   q.bad = (int)!(d00 >= kMinPivot) | (int)!(p1 >= kMinPivot) << 1 | (int)!(p2 >= kMinPivot) << 2 |
           (int)!(p3 >= kMinPivot) << 3;
+  return fabsf(e1) < kSeed && fabsf(e3) < kSeed;
+}
+
+// A pivot that is not positive, or below FP32's normal range, is reported;
+// the entries after it are then meaningless (NaN or infinite) and the factor
+// is dropped.  A pair's second pivot d11 - d10^2 / d00 is first approximated as
+// 1 / sqrt = sqrt(d00) / sqrt(d00 d11 - d10^2), so that both roots start
+// together, and a Newton step takes it to the pivot itself, the entry that is
+// scaled and judged.  The two round apart: where the pivot has cancelled so far
+// that they differ by 2^-11 or more (or in sign), the block starts again from the
+// pivots.  The arguments are the same in every lane.
+__device__ __forceinline__ void pivot_factor(float d00, float d10, float d20, float d30, float d11, float d21,
+                                             float d31, float d22, float d32, float d33, Pivot& q) {
+  if (!pivot_steps<true>(d00, d10, d20, d30, d11, d21, d31, d22, d32, d33, q))
+    pivot_steps<false>(d00, d10, d20, d30, d11, d21, d31, d22, d32, d33, q);
 }
 
 // x - y z
