@@ -476,8 +476,8 @@ __global__ void __launch_bounds__(SYM_THREADS, 1)
 // exact in 128-bit fixed point up to 2^-64 an entry and added up as integers, so
 // that the norms do not depend on the order of the tiles either -- which costs
 // six FP64 operations a pair (two FMAs, 1.75 for the columns' groups, 1.7 for a
-// row's lanes, 0.5 for the columns' warps).  No pipe is full (FP64 60%, ALU 35%,
-// FMA 26% at n = 16,384, m = 8): two CTAs of 128 registers do not hide the
+// row's lanes, 0.5 for the columns' warps).  No pipe is full (FP64 54%, ALU 37%,
+// FMA 27% at n = 16,384, m = 8): two CTAs of 128 registers do not hide the
 // latencies.  n = 30,000, m = 8: 54 ms with FP64 differences for the whole square,
 // 8.3 now.  The solver's own residual (COMP false) takes FMA chains and FP32 norms.
 constexpr int SYMQ_LD = 33;

@@ -3013,12 +3013,13 @@ int mag_solve_batch(mag_ctx* ctx, const mag_batch_desc* desc, int32_t count, con
       const std::pair<int64_t, int64_t> key(d.point_offset, (int64_t)d.n * 65536 + d.m);
       probs[i].cloud = keys.emplace(key, (int)keys.size()).first->second;
       // from 97 points the tile kernels (unless a launch shape of the one-CTA
-      // kernel, or FP64 distances, are asked for): there they are no slower
-      // whatever the number of problems, below that for many of them.  1, 8,
-      // 150 and 1,200 problems in R^16, one CTA each against tiles: n = 64 337,
-      // 351, 827, 5131 against 350, 388, 880, 5794 us; n = 88 407, 437, 931, 5157
-      // against 366, 393, 887, 5224; n = 97 440, 471, 968, 6099 against 367, 398,
-      // 898, 6066; n = 129 538, 563, 1126, 6355 against 421, 457, 1102, 6478
+      // kernel, or FP64 distances, are asked for): there few problems gain up to
+      // a fifth and the fullest batches lose 2% at most (just past a tile),
+      // below it many problems lose more.  1, 8, 150 and 1,200 problems in R^16,
+      // one CTA each against tiles: n = 64 337, 351, 827, 5131 against 350, 388,
+      // 880, 5794 us; n = 88 407, 437, 931, 5157 against 366, 393, 887, 5224; n =
+      // 97 440, 471, 968, 6099 against 367, 398, 898, 6066; n = 129 538, 563,
+      // 1126, 6355 against 421, 457, 1102, 6478
       if (ctx->opt.batch_shape == 0 && ctx->opt.exact_distances && d.n >= kBatchTiledMin && d.m <= 512)
         tiled.push_back(i);
       else
