@@ -138,9 +138,9 @@ __global__ void __launch_bounds__(GEN_THREADS, 1)
           if (WD) zd = mat_entry(kind, t, kc, dd, exptab);
           if (WF)
             zf = WD ? (kind == MAT_DEFLATED ? __double2float_rn(zd) : f64_to_f32_nonneg(zd))
-                    : (kind == MAT_EXP ? expf(-tf * sqrtf((float)v))
-                                       : (kind == MAT_SHIFTED_DIST ? 1.0f - tf * sqrtf((float)v)
-                                                                   : fmaf((float)kc, expm1f(-tf * sqrtf((float)v)), 1.0f)));
+                    : (kind == MAT_EXP ? expf(-td_f32(tf, t, v))
+                                       : (kind == MAT_SHIFTED_DIST ? 1.0f - td_f32(tf, t, v)
+                                                                   : fmaf((float)kc, expm1f(-td_f32(tf, t, v)), 1.0f)));
         }
       }
       zfv[q] = zf;

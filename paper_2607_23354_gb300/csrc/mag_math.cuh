@@ -203,17 +203,22 @@ __device__ __forceinline__ double nl1_exact(int N) {
   return __longlong_as_double((long long)(((unsigned long long)(top + EXPT_L1E + 1022) << 52) + mant));
 }
 
+// 2^-126 <= x < 2^127 for x >= 0: FP32 holds it.
+__device__ __forceinline__ bool in_f32_range(double x) {
+  return ((unsigned)__double2hiint(x) >> 20) - (1023u - 126u) <= 252u;
+}
+__device__ __forceinline__ double exp_neg_product(double a, const double* tab) {
+  return (unsigned long long)__double_as_longlong(a) < 0x4050000000000000ull ? exp_neg_small(a, tab) : exp_neg(-a, tab);
+}
+
 // exp(-t d) for t > 0, d >= 0 (NaN propagates): N from the FP32 product of
 // t and d rounded on the integer pipe (within 2^-21 relative of t d, moving
 // N by less than 0.006), then the reduction without rounding t d; for t d
-// of about 63.5 or more the product is formed and exp_neg takes it.
+// of about 63.5 or more, and where t or d lies outside FP32's range, the product
+// is formed and exp_neg takes it.
 __device__ __forceinline__ double exp_neg_td(double t, double d, const double* tab) {
   const float af = f64_to_f32_nonneg(t) * f64_to_f32_nonneg(d);
-  if (!(af < 63.5f)) {
-    const double a = t * d;
-    return (unsigned long long)__double_as_longlong(a) < 0x4050000000000000ull ? exp_neg_small(a, tab)
-                                                                               : exp_neg(-a, tab);
-  }
+  if (!(af < 63.5f) || !in_f32_range(t) || !in_f32_range(d)) return exp_neg_product(t * d, tab);
   float kf;
   const int N = exp_reduce_n(af, &kf);
   return exp_neg_core(N, kf, fma(-t, d, nl1_exact(N)), tab);
@@ -288,7 +293,7 @@ __device__ __forceinline__ double f32_to_f64_nonneg(float v) {
 // exp(-t d) below e^-46 (exp_neg_tiny_f) from FP64 d >= 0 and tf = t rounded
 // to FP32: d rounded on the integer pipe, the product and the exponential on
 // the FP32 pipe.  Returns the FP32 entry; its FP64 copy is
-// f32_to_f64_nonneg of it.  d of 2^126 or more (or NaN) takes t d in FP64.
+// f32_to_f64_nonneg of it.  t or d (d^2) outside FP32's range take t d in FP64.
 __device__ __forceinline__ float exp_neg_tiny_td(float tf, double t, double d);
 // The same from d^2 (the square root on the FP32 pipe as well).
 __device__ __forceinline__ float exp_neg_tiny_td2(float tf, double t, double d2);
@@ -323,14 +328,19 @@ __device__ __forceinline__ double sqrt_pos(double v) {
 }
 
 __device__ __forceinline__ float exp_neg_tiny_td(float tf, double t, double d) {
-  if ((unsigned long long)__double_as_longlong(d) >= 0x47D0000000000000ull)  // 2^126, inf, NaN
+  if (!in_f32_range(d) || !in_f32_range(t))  // inf and NaN too
     return d != d ? (float)d : exp_neg_tiny_f((float)fmin(t * d, 100.0));
   return exp_neg_tiny_f(tf * f64_to_f32_nonneg(d));
 }
 __device__ __forceinline__ float exp_neg_tiny_td2(float tf, double t, double d2) {
-  if ((unsigned long long)__double_as_longlong(d2) >= 0x47D0000000000000ull)
+  if (!in_f32_range(d2) || !in_f32_range(t))
     return d2 != d2 ? (float)d2 : exp_neg_tiny_f((float)fmin(t * sqrt(d2), 100.0));
   return exp_neg_tiny_f(tf * sqrtf(f64_to_f32_nonneg(d2)));
+}
+// t d in FP32 from d^2, at most 2^100
+__device__ __forceinline__ float td_f32(float tf, double t, double d2) {
+  if (!in_f32_range(d2) || !in_f32_range(t)) return (float)fmin(t * sqrt(d2), 0x1p100);
+  return tf * sqrtf((float)d2);
 }
 
 // Doubles in an order-preserving unsigned encoding (atomic min / max of

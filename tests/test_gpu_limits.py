@@ -225,3 +225,38 @@ def test_adjoint_solve_reuses_the_forward_factor(ctx):
     dto, dxo = oracle.grad_loss(X2, t, 2 * w.cpu().numpy(), w=w.cpu().numpy())
     assert dt == pytest.approx(dto, rel=1e-8)
     assert np.abs(dx.cpu().numpy() - dxo).max() <= 1e-7 * np.abs(dxo).max()
+
+
+# ------------------------------------------------- scales far outside FP32's range
+
+# Points scaled by 2^k and t by 2^-k give the same matrix: every step but the
+# rounding of t d outside FP32's range scales exactly, so entries agree to (1 + t d)
+# units, and results to the solver's tolerance; with the quantized coordinates
+# (|k| < 400), beyond them and with FP64 differences, for few points and for tiles.
+@pytest.mark.parametrize("k", [-480, -430, -300, -140, 140, 300, 430, 480])
+@pytest.mark.parametrize("exact", [True, False])
+@pytest.mark.parametrize("n", [20, 60, 150])
+def test_scaled_points_and_t(k, exact, n):
+    rng = np.random.default_rng(n)
+    X, w = rng.standard_normal((n, 4)), rng.standard_normal(n)
+    t = 1.5
+    c = M.Context(M.Options(exact_distances=exact))
+    out = []
+    for s in (0, k):
+        Y, ts = _dev(np.ldexp(X, s)), float(np.ldexp(t, -s))
+        dt, dx = c.grad(Y, ts, w=_dev(w))
+        ws, mags, sts = c.solve_batch([Y], [ts, 40 * ts])
+        assert int(sts.abs().sum()) == 0
+        v, mag, _ = c.solve(Y, ts)
+        out.append([c.similarity_matrix(Y, ts), c.similarity_matrix(Y, 40 * ts), c.similarity_matrix(Y, ts, "fp32").double(),
+                    c.residual(Y, ts, _dev(w))[0], dx * 2.0 ** s, torch.tensor(float(np.ldexp(dt, -s))), torch.cat(ws), v,
+                    mags[0]])
+    c.close()
+    for i, (a, b) in enumerate(zip(*out)):
+        if i == 0 or i == 1:
+            a, b = a[a > 1e-280], b[a > 1e-280]
+            assert bool(((a - b).abs() <= 2.0 ** -51 * (1 - torch.log(a)) * a).all())
+        elif i == 2:
+            assert float((a - b).abs().max()) <= 2.0 ** -22
+        else:
+            assert float((a - b).abs().max()) <= 1e-11 * float(a.abs().max())
