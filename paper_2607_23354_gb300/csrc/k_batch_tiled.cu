@@ -1021,7 +1021,7 @@ template <int KIND>
 static cudaError_t launch_bt_generate_t(const TiledBatch& B, const double* points, const int2* tasks, int count,
                                         int mmax, cudaStream_t s) {
   const int smem = (int)fx_tile_smem(mmax);
-  cudaError_t e = dynamic_smem(k_bt_generate<KIND>, smem);
+  cudaError_t e = dynamic_smem(k_bt_generate<KIND>, (int)FX_TILE_SMEM_MAX);
   if (e != cudaSuccess) return e;
   k_bt_generate<KIND><<<(unsigned)count, FX_THREADS, smem, s>>>(tasks, B.clouds, B.probs, points,
                                                                static_cast<const fx_coord*>(B.Xq), B.Zf, B.Zi,

@@ -658,7 +658,7 @@ cudaError_t launch_gen_q(const fx_coord* Xq, const double* X, int64_t n, int m, 
                          int kind, float tiny, double kc, int64_t t0, int64_t W) {
   auto kern = k_generate_q<KIND, WF, WD, EXP>;
   const size_t smem = fx_tile_smem(m);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_TILE_SMEM_MAX);
   if (e != cudaSuccess) return e;
   kern<<<dim3(tiles, row_slices(tiles, KIND)), FX_THREADS, smem, s>>>(Xq, X, n, m, sc, t, Zf, Zd, rowsum, st, kind, tiny, kc, t0, W);
   note_launch();
@@ -709,7 +709,7 @@ static cudaError_t launch_dense_t(const fx_coord* Xq, const double* X, int64_t n
                                   unsigned tiles, DevStatus* st, cudaStream_t s) {
   auto kern = k_dense_q<KIND, T>;
   const size_t smem = fx_tile_smem(m);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_TILE_SMEM_MAX);
   if (e != cudaSuccess) return e;
   kern<<<tiles, FX_THREADS, smem, s>>>(Xq, X, n, m, sc, Z, st);
   note_launch();
@@ -752,7 +752,7 @@ cudaError_t launch_dist_q(const void* Xq, const double* X, int64_t n, int m, int
   const fx_coord* q = static_cast<const fx_coord*>(Xq);
   const int kd = fx_kind(m);
   auto kern = kd == 0 ? k_dist_q<0> : (kd == 1 ? k_dist_q<1> : k_dist_q<2>);
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_TILE_SMEM_MAX);
   if (err != cudaSuccess) return err;
   kern<<<dim3((unsigned)tiles, row_slices(tiles, kd)), FX_THREADS, smem, s>>>(q, X, n, m, e, Dd, st);
   note_launch();

@@ -481,6 +481,7 @@ __global__ void __launch_bounds__(SYM_THREADS, 1)
 // latencies.  n = 30,000, m = 8: 54 ms with FP64 differences for the whole square,
 // 8.3 now.  The solver's own residual (COMP false) takes FMA chains and FP32 norms.
 constexpr int SYMQ_LD = 33;
+constexpr size_t SYMQ_ROWS = (size_t)TILE * SYMQ_LD * sizeof(double);
 
 // s + c <- s + c + x with the rounding of s collected in c
 __device__ __forceinline__ void add_comp(double& s, double& c, double x) {
@@ -1297,7 +1298,8 @@ cudaError_t launch_residual_mf(const double* X, int64_t n, int m, double t, cons
     // large m: eight column points per stage need more than the default
     // 48 KB of static (8 KB exp table) plus dynamic shared memory; at most
     // 8 x 2049 doubles = 131 KB
-    cudaError_t e = cudaFuncSetAttribute(k_resid_mf<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_resid_mf<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         8 * (MAG_MAX_DIM + 1) * (int)sizeof(double));  // any thread's m
     if (e != cudaSuccess) return e;
   }
   if (m <= 8)
@@ -1328,10 +1330,10 @@ cudaError_t launch_residual_sym(const double* X, int64_t n, int m, double t, con
   if (e != cudaSuccess) return e;
   if (Xq && kind == MAT_EXP && m <= FX_MAX_DIM) {
     const FxScale sc = fx_scale(t, qe);
-    const size_t sq = (size_t)TILE * SYMQ_LD * sizeof(double) + fx_tile_smem(m);
+    const size_t sq = SYMQ_ROWS + fx_tile_smem(m);
     const int kd = fx_kind(m);
     auto kern = kd == 0 ? k_resid_sym_q<0, false> : (kd == 1 ? k_resid_sym_q<1, false> : k_resid_sym_q<2, false>);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sq);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SYMQ_ROWS + FX_TILE_SMEM_MAX));
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)tiles, FX_THREADS, sq, s>>>(static_cast<const fx_coord*>(Xq), X, n, m, sc, w, P, rowsum, N);
   } else {
@@ -1362,10 +1364,10 @@ cudaError_t launch_residual_comp(const void* Xq, const double* X, int64_t n, int
   cudaError_t e = cudaMemsetAsync(rowsum, 0, (size_t)n * sizeof(ulonglong2), s);
   if (e != cudaSuccess) return e;
   const FxScale sc = fx_scale(t, qe);
-  const size_t sq = (size_t)TILE * SYMQ_LD * sizeof(double) + fx_tile_smem(m);
+  const size_t sq = SYMQ_ROWS + fx_tile_smem(m);
   const int kd = fx_kind(m);
   auto kern = kd == 0 ? k_resid_sym_q<0, true> : (kd == 1 ? k_resid_sym_q<1, true> : k_resid_sym_q<2, true>);
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sq);
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SYMQ_ROWS + FX_TILE_SMEM_MAX));
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)tiles, FX_THREADS, sq, s>>>(static_cast<const fx_coord*>(Xq), X, n, m, sc, w, P, rowsum, N);
   note_launch();
@@ -1493,8 +1495,8 @@ template <bool FX, int KIND>
 static cudaError_t launch_grad_t(const fx_coord* Xq, const double* X, int64_t n, int m, const FxScale& sc, double t,
                                  const double* w, const double* lam, double* P, double* part_t, int64_t N, int64_t I0,
                                  int64_t I1, cudaStream_t s) {
-  const size_t fx = fx_tile_smem(m);
-  const size_t smem = (size_t)TILE * GRAD_LD * sizeof(double) + (fx > GRAD_STAGE ? fx : GRAD_STAGE);
+  static_assert(FX_TILE_SMEM_MAX <= GRAD_STAGE, "one size, whatever m: the limit set below is the process's");
+  const size_t smem = (size_t)TILE * GRAD_LD * sizeof(double) + GRAD_STAGE;
   auto kern = k_grad_tile<FX, KIND>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

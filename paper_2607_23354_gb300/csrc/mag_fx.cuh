@@ -366,6 +366,10 @@ inline int fx_kind(int m) { return m <= FX_LOW_DIM ? 0 : (m <= FX_SPILL ? 1 : 2)
 // (n = 16,384, m = 8: 1.79 against 1.95 ms); two rows need 128.
 constexpr int fx_ctas(int kind) { return kind < 2 ? 3 : 2; }
 constexpr int FX_CHUNK = 32;  // dimensions staged at a time
+// A kernel's limit on dynamic shared memory is the process's, not the call's: every
+// launch sets it to what its largest m takes, so that a call from another thread
+// cannot lower it between this one's setting and its launch.
+constexpr size_t FX_TILE_SMEM_MAX = 2 * (size_t)128 * FX_CHUNK * sizeof(fx_coord);
 inline size_t fx_tile_smem(int m) { return 2 * (size_t)128 * (m < FX_CHUNK ? m : FX_CHUNK) * sizeof(fx_coord); }
 
 template <int KIND, int THREADS = FX_THREADS, class F>

@@ -2,6 +2,8 @@
 side buffers, the report of a batch) must not reach a later call with other
 points: each test mixes entry points on one context and checks the results
 against plain FP64 arithmetic."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -159,3 +161,38 @@ def test_gradient_of_converted_vectors():
     dt64, dx64 = c.grad(X, 1.5, w=w.double(), dL_dw=g.double())
     c.close()
     assert dt == dt64 and torch.equal(dx, dx64)
+
+
+# Contexts of two threads, each on its own stream, with points of different
+# dimension: the kernels' shared memory depends on it, and their limit on it is one
+# for the process.  Errors of a launch come back as MagnitudeError.
+@pytest.mark.parametrize("call", ["similarity_matrix", "residual", "solve_batch", "residual_many_dimensions"])
+def test_threads_with_different_dimensions(call):
+    errors = []
+
+    def work(m, seed):
+        try:
+            rng = np.random.default_rng(seed)
+            n = 130 if call == "solve_batch" else 60
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                X, w = _dev(rng.standard_normal((n, m))), _dev(rng.standard_normal(n))
+                c = M.Context(stream=stream)
+                for _ in range(400):
+                    if call == "similarity_matrix":
+                        c.similarity_matrix(X, 0.2)
+                    elif call == "solve_batch":
+                        c.solve_batch([X], [0.5])
+                    else:
+                        c.residual(X, 0.2, w)
+                c.close()
+        except Exception as e:  # noqa: BLE001 (reported by the test's own thread)
+            errors.append(e)
+
+    dims = (1000, 1900) if call == "residual_many_dimensions" else (17, 32)
+    threads = [threading.Thread(target=work, args=(m, i)) for i, m in enumerate(dims)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
